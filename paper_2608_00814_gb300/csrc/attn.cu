@@ -124,20 +124,6 @@ struct AttnArgs {
   uint32_t* status;         // step status word (pipeline waits that give up)
 };
 
-OOS_DEV uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-// not .aligned: the threads of a warp may arrive at different points
-OOS_DEV void cluster_arrive_release() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
-OOS_DEV void cluster_wait_acquire() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-// address of the same shared-memory location in block `rank` of the cluster
-OOS_DEV uint32_t dsmem_addr(const void* p, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr(p)), "r"(rank));
-  return r;
-}
 // D[tmem] (+)= A[tmem] * B[smem]: A (M = 128 rows, one per lane) as packed
 // bf16 pairs, K index 2c and 2c + 1 in column c (low half first)
 OOS_DEV void tc_mma_bf16_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {

@@ -29,7 +29,7 @@ OOS_DEV unsigned long long wait_limit(const uint32_t* status) {
 
 OOS_DEV unsigned long long globaltimer() {
   unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t)::"memory");
   return t;
 }
 
@@ -116,6 +116,20 @@ OOS_DEV void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::
 
 // ---- shared-memory addresses and mbarriers
 OOS_DEV uint32_t smem_addr(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
+
+// ---- thread-block clusters
+// not .aligned: the threads of a warp may arrive at different points
+OOS_DEV void cluster_arrive_release() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+OOS_DEV void cluster_wait_acquire() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// arrival that orders nothing but the thread's own completed reads: it does not
+// wait for stores in flight
+OOS_DEV void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); }
+// address of the same shared-memory location in block `rank` of the cluster
+OOS_DEV uint32_t dsmem_addr(const void* p, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr(p)), "r"(rank));
+  return r;
+}
 
 OOS_DEV void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");

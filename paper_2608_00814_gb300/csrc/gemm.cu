@@ -4,10 +4,9 @@
 // f in the MMA's M = 128 slot and the T tree nodes in N ("swap-AB": T <= 128
 // is far too small for M).  Weights are the only large operand; each is read
 // from HBM exactly once per step.  Per CTA: one TMA producer thread streams
-// 128 x 64 weight tiles and the matching 64-wide slice of X through an
-// S-stage shared-memory ring; one thread issues tcgen05.mma into a TMEM
-// accumulator (two buffers, so the epilogue of one tile overlaps the MMAs of
-// the next); four epilogue warps drain TMEM with tcgen05.ld.
+// weight tiles of 64 k and the matching 64-wide slice of X through a
+// shared-memory ring; one thread issues tcgen05.mma into a TMEM accumulator;
+// eight epilogue warps drain TMEM with tcgen05.ld.
 // The layer's elementwise steps run in the GEMM epilogues (see below); the LM
 // head keeps a per-node running (max, argmax, second max) so logits never
 // reach memory.
@@ -20,17 +19,17 @@
 
 // Step timeline (built only with -DOOS_TIMELINE, see timeline.py): per GEMM
 // launch of a step and per CTA, the globaltimer at entry (0), at the end of the
-// dependency wait (1), when the last accumulator is ready (2), at the last
-// arrival count (4), when the finishing may start (5) and at exit (3).  A
-// launch's slot comes from its arrival-counter block, one per (layer, GEMM).
+// dependency wait (1), when the last accumulator is ready (2), when it is
+// staged for the cluster (4), when every split's is (5) and at exit (3).  One
+// slot per (layer, GEMM).
 #ifdef OOS_TIMELINE
 namespace oos {
 __device__ unsigned long long g_tl_gemm[1024][160][6];
 }
-#define TL_GEMM(ev)                                                                                   \
-  do {                                                                                                \
-    if (!ARGMAX && a.cnt && blockIdx.x < 160)                                                        \
-      oos::g_tl_gemm[((uintptr_t)a.cnt >> 10) & 1023][blockIdx.x][ev] = oos::globaltimer();          \
+#define TL_GEMM(ev)                                                                   \
+  do {                                                                                \
+    if (!ARGMAX && blockIdx.x < 160)                                                  \
+      oos::g_tl_gemm[a.tl_slot & 1023][blockIdx.x][ev] = oos::globaltimer();          \
   } while (0)
 #else
 #define TL_GEMM(ev) \
@@ -40,45 +39,55 @@ __device__ unsigned long long g_tl_gemm[1024][160][6];
 
 namespace oos {
 
-// Epilogues fused into the weight GEMMs (bf16 path).  Stream-K leaves a tile's
-// reduction split over up to a few CTAs: each writes its fp32 partial tile,
-// and the LAST contributor to arrive (a per-tile arrival counter) adds the
-// slices in slice order -- a fixed order, so results are deterministic -- and
-// applies the layer's elementwise step to the finished tile:
+// Epilogues fused into the weight GEMMs (bf16 path):
 //   EPI_QKV   : input RMSNorm scale, bias, per-head q/k RMSNorm, RoPE at
 //               ctx + depth; q (hi/lo bf16) to the query buffer, k/v to cache
 //               slot ctx + t.
 //   EPI_RESID : x += W.a (O- and down-projections), then y = g (.) x for the
 //               next RMSNorm (hi/lo bf16) and per-tile sums of x^2.
-//   EPI_SILU  : gate and up tiles are interleaved (tile 2i = gate rows of
-//               block i, 2i+1 = up rows); act = silu(r g) * (r u).
-//   EPI_ARGMAX: LM head -- whole tiles round-robin, logits scaled by the final
-//               RMSNorm factor and folded into a per-node running top-2.
+//   EPI_SILU  : a tile holds the same rows of gate and up; act = silu(r g) * (r u).
+//   EPI_ARGMAX: LM head -- logits scaled by the final RMSNorm factor and folded
+//               into a per-node running top-2.
 // RMSNorm is split across kernels by linearity: a producer stores y = g (.) x
-// and sum(x^2) per 128-feature chunk; the consumer GEMM computes W.y and
-// multiplies column t by r_t = rsqrt(sum x_t^2 / H + eps) in its epilogue.
+// and sum(x^2) per feature tile; the consumer GEMM computes W.y and multiplies
+// column t by r_t = rsqrt(sum x_t^2 / H + eps) in its epilogue.
+//
+// Work split.  Every matrix is cut into tiles of `rows` weight rows (a multiple
+// of 8 up to the MMA's 128; the accumulator lanes past it hold sums of whatever
+// follows in shared memory and are never read), chosen so that the tiles fill
+// the SMs about once (make_plan):
+//   QKV, RESID: a thread-block cluster of `split` CTAs shares a tile, each CTA
+//     one k-range of it.  Each stages its fp32 sums in its own shared memory
+//     (over the ring, idle by then); after a cluster barrier CTA i pulls every
+//     split's rows of its share of the tokens, adds them in split order (so the
+//     result is the same from run to run) and finishes them.  Everything else
+//     the epilogue reads (residual, rotary factors, norm sums) is loaded while
+//     the weights stream.
+//   SILU, ARGMAX: whole-K tiles, dealt round-robin (the weights of the next tile
+//     stream while one is finished).
 enum { EPI_QKV = 0, EPI_RESID = 1, EPI_SILU = 2, EPI_ARGMAX = 3 };
 
-// A work tile is SUB weight subtiles of 128 rows (the MMA's M) that share every
-// staged activation slice.  The gate/up GEMM and the LM head use SUB = 2 (per
-// weight byte half the activation traffic, more weight bytes in flight, and
-// gate + up rows of one block in one CTA); the smaller QKV, O and down GEMMs
-// use SUB = 1 so each tile has fewer stream-K contributors.  Subtile s of work
-// tile w is the 128-row tile SUB*w + s of the stacked weight.
+// A work tile is SUB weight subtiles that share every staged activation slice:
+// gate and up rows, or 2 x 128 rows of the LM head.
 template <int EPI>
-struct SubOf {
-  static constexpr int v = (EPI == 2 || EPI == 3) ? 2 : 1;
+struct EpiOf {
+  static constexpr int sub = (EPI == EPI_SILU || EPI == EPI_ARGMAX) ? 2 : 1;
+  // k-segments of a tile with an accumulator each, added in fp32 by the
+  // epilogue: the tensor core truncates every addition to its accumulator, an
+  // error that grows with the chain, so the chains are kept short
+  static constexpr int segs = EPI == EPI_ARGMAX ? 1 : 2;
+  static constexpr bool cluster = EPI == EPI_QKV || EPI == EPI_RESID;
 };
 
 struct GemmArgs {
-  int seg_tiles[3];   // cumulative 128-row tile counts per weight segment
-  int interleave2;    // 128-row tile 2i -> segment 0 block i, tile 2i+1 -> segment 1 block i
-  int n_tiles;        // 128-row tiles of the stacked weight
-  int n_work, kbt, total;   // work tiles (SUB subtiles each), k-blocks per tile, n_work * kbt
-  int N;              // output rows (features / vocab) of the stacked weight
+  int seg_tiles[3];   // EPI_QKV: cumulative tile counts of the q, k, v matrices
+  int rows;           // weight rows per subtile
+  int n_work, kbt;    // work tiles, k-blocks per tile
+  int split;          // CTAs sharing a tile (cluster size)
+  int stages;         // ring depth
+  int N;              // output rows (features / vocab; intermediate rows for EPI_SILU)
   int T;              // valid columns (tree nodes)
-  float* part;        // partial tiles [slice][kMaxT][n_work * SUB * 128]
-  int* cnt;           // arrival counter per work tile (zeroed at every step start)
+  int tl_slot;        // timeline slot (layer * 4 + kind)
   uint32_t* status;
   // RMSNorm scale of the GEMM input (EPI_QKV, EPI_SILU, EPI_ARGMAX)
   const float* ss_in;   // [chunk][kMaxT]
@@ -98,33 +107,50 @@ struct GemmArgs {
   float* ss_out;
   // EPI_SILU
   __nv_bfloat16* act_out;
-  int I;
   // EPI_ARGMAX
   float* am_v1;
   int32_t* am_i;
   float* am_v2;
 };
 
-template <int BN, int kSub>
+constexpr int kEpiWarps = 8;
+constexpr int kEpiThreads = kEpiWarps * 32;
+constexpr int kGemmThreads = 64 + kEpiThreads;
+constexpr int kMaxStages = 12;
+constexpr int kGemmSmemMax = 227 * 1024;
+
+template <int BN, int EPI>
 struct TcCfg {
-  static constexpr int A_BYTES = kTile * kBK * 2;              // 16 KB per 128-row weight subtile
+  static constexpr int kSub = EpiOf<EPI>::sub;
   static constexpr int B_BYTES = BN * kBK * 2;                 // one activation half (hi or lo)
-  static constexpr int STAGE = kSub * A_BYTES + 2 * B_BYTES;
   static constexpr int BAR_BYTES = 256;
-  static constexpr int EPI_BYTES = kMaxT * 4 + 64;             // input RMSNorm factors, flags
-  static constexpr int RED_BYTES = 4 * BN * 12 + BN * 12;      // argmax cross-warp scratch + running state
-  static constexpr int FIXED = 1024 /*align slack*/ + BAR_BYTES + EPI_BYTES + RED_BYTES;
-  static constexpr int S_RAW = (227 * 1024 - FIXED) / STAGE;
-  static constexpr int S = S_RAW > 8 ? 8 : S_RAW;
+  static constexpr int EPI_BYTES = kMaxT * 4;                  // input RMSNorm factors
+  static constexpr int RED_BYTES = EPI == EPI_ARGMAX ? 5 * BN * 12 : 0;   // argmax cross-warp scratch + running state
+  static constexpr int HEAD = (BAR_BYTES + EPI_BYTES + RED_BYTES + 1023) / 1024 * 1024;   // what precedes the ring
+  static constexpr int FIXED = 1024 /*align slack*/ + HEAD;
   // The hi and lo activation halves sit in one slot, hi rows then lo rows, so
   // one MMA with N = 2 BN multiplies both ("paired": half the MMAs, the weight
   // subtile read from shared memory once); the accumulator then holds the hi
   // products in columns [0, BN) and the lo products in [BN, 2 BN).  Paired
-  // when two buffers of kSub such accumulators fit the 512 TMEM columns.
-  static constexpr bool PAIRED = 2 * kSub * 2 * BN <= 512;
-  static constexpr int SUB_COLS = PAIRED ? 2 * BN : BN;                      // accumulator columns per subtile
-  static constexpr int NCOLS = (2 * kSub * SUB_COLS) < 32 ? 32 : 2 * kSub * SUB_COLS;   // 2 buffers
-  static constexpr int SMEM = FIXED + S * STAGE;
+  // when the accumulator buffers then fit the 512 TMEM columns.
+  static constexpr int BUFS = 2;
+  static constexpr bool PAIRED = BUFS * kSub * 2 * BN <= 512;
+  static constexpr int SUB_COLS = PAIRED ? 2 * BN : BN;        // accumulator columns per subtile
+  static constexpr int NCOLS = BUFS * kSub * SUB_COLS < 32 ? 32 : BUFS * kSub * SUB_COLS;
+  static int stage_bytes(int rows) { return kSub * rows * kBK * 2 + 2 * B_BYTES; }
+  static int stages(int rows) {
+    const int s = (kGemmSmemMax - FIXED) / stage_bytes(rows);
+    return s > kMaxStages ? kMaxStages : s;
+  }
+  // ring, or what the MMAs touch past the last weight subtile, or the staged tile
+  static int smem(int rows) {
+    const int s = stages(rows);
+    int ring = s * stage_bytes(rows);
+    const int reach = (s * kSub - 1) * rows * kBK * 2 + kTile * kBK * 2;
+    if (ring < reach) ring = reach;
+    if (EpiOf<EPI>::cluster && ring < BN * kTile * 4) ring = BN * kTile * 4;
+    return FIXED + ring;
+  }
 };
 
 struct Top2s {
@@ -145,86 +171,16 @@ OOS_DEV Top2s t2_merge(Top2s a, Top2s b) {
   return r;
 }
 
-OOS_DEV void epi_bar() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
-
-
-// Finishing a subtile: warp w of the four epilogue warps owns token rows
-// t = t0 + 4k + w, lane l owns the four features 4l..4l+3 of the subtile, so a
-// token's 128 features sit in one warp (RMSNorm sums, q/k norm and the RoPE
-// pair exchange are warp shuffles) and every slice load is a coalesced float4.
-// All loads of a pass are issued before any result is stored.
-constexpr int kFinRows = 4;    // token rows per warp per pass (16 tokens per pass)
+OOS_DEV void epi_bar() { asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory"); }
 
 OOS_DEV float4 f4_add(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
-OOS_DEV float4 f4_ldcg(const float* p) { return __ldcg(reinterpret_cast<const float4*>(p)); }
-
-// Where a finishing pass reads the partial sums of output (token t, feature f)
-// from: partial s of nc, the stream-K slices in global memory,
-// [slice][kMaxT][n_part] (feature f of the stacked weight).
-struct GSrc {
-  const float* p;
-  size_t slice;
-  int ld;
-  OOS_DEV float4 ld4(int s, int t, int f) const { return f4_ldcg(p + (size_t)s * slice + (size_t)t * ld + f); }
-};
-
-// acc[k] = (init ? init row : 0) + sum over nc slices of the partial tile rows,
-// rows t = t0 + nw k + w below T (the end of the token range; w is this warp's
-// index among the nw warps finishing the tile).  Slices are
-// fetched BATCH at a time -- every load of a group is issued before any is
-// added -- and added in slice order, so the sum is the same for every finisher.
-template <int R, int BATCH, typename Src>
-OOS_DEV void load_tile_rows(float4 (&acc)[R], const Src& src, int nc, int col, int t0, int T,
-                            const float* __restrict__ init, int init_ld, int init_col, int w, int nw) {
-#pragma unroll
-  for (int k = 0; k < R; ++k) {
-    const int t = t0 + nw * k + w;
-    acc[k] = (init && t < T) ? *reinterpret_cast<const float4*>(init + (size_t)t * init_ld + init_col)
-                             : make_float4(0.f, 0.f, 0.f, 0.f);
-  }
-  for (int s0 = 0; s0 < nc; s0 += BATCH) {
-    float4 v[BATCH][R];
-#pragma unroll
-    for (int q = 0; q < BATCH; ++q) {
-#pragma unroll
-      for (int k = 0; k < R; ++k) {
-        const int t = t0 + nw * k + w;
-        v[q][k] = (s0 + q < nc && t < T) ? src.ld4(s0 + q, t, col) : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < BATCH; ++q)
-#pragma unroll
-      for (int k = 0; k < R; ++k) acc[k] = f4_add(acc[k], v[q][k]);
-  }
-}
-
-// gate (col) and up (col + up_off) rows of a SwiGLU pair, two slices per batch
-template <int R, typename Src>
-OOS_DEV void load_pair_rows(float4 (&g)[R], float4 (&u)[R], const Src& src, int nc, int col, int up_off, int t0,
-                            int T, int w, int nw) {
-#pragma unroll
-  for (int k = 0; k < R; ++k) g[k] = u[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int s0 = 0; s0 < nc; s0 += 2) {
-    float4 vg[2][R], vu[2][R];
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-#pragma unroll
-      for (int k = 0; k < R; ++k) {
-        const int t = t0 + nw * k + w;
-        const bool ok = s0 + q < nc && t < T;
-        vg[q][k] = ok ? src.ld4(s0 + q, t, col) : make_float4(0.f, 0.f, 0.f, 0.f);
-        vu[q][k] = ok ? src.ld4(s0 + q, t, col + up_off) : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < 2; ++q)
-#pragma unroll
-      for (int k = 0; k < R; ++k) {
-        g[k] = f4_add(g[k], vg[q][k]);
-        u[k] = f4_add(u[k], vu[q][k]);
-      }
-  }
+OOS_DEV float4 ld_cluster_f4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(addr)
+               : "memory");
+  return v;
 }
 
 OOS_DEV float4 bf16x4(const __nv_bfloat16* p) {
@@ -233,178 +189,211 @@ OOS_DEV float4 bf16x4(const __nv_bfloat16* p) {
   return make_float4(__bfloat162float(h[0]), __bfloat162float(h[1]), __bfloat162float(h[2]), __bfloat162float(h[3]));
 }
 
-// EPI_RESID on 128-row tile `tile`, tokens [tb, te), by warp w of nw: x += W.a;
-// y = g (.) x; per-tile sums of x^2
-template <typename Src>
-OOS_DEV void finish_resid(const GemmArgs& a, const Src& src, int tile, int nc, int tb, int te, int w, int nw) {
+// RMSNorm factors of tokens [tb, te) into rms[], by the epilogue warps (w of
+// kEpiWarps): lanes take the chunk sums, four tokens of a warp in flight.
+OOS_DEV void input_rms(const GemmArgs& a, float* rms, int tb, int te, int w) {
   const int l = threadIdx.x & 31;
-  const int f = tile * kTile + 4 * l;
-  const float4 g = bf16x4(a.gain + f);
-  for (int t0 = tb; t0 < te; t0 += nw * kFinRows) {
-    float4 acc[kFinRows];
-    load_tile_rows<kFinRows, 8>(acc, src, nc, f, t0, te, a.x, a.N, f, w, nw);   // x + sum of the partials
+  for (int t0 = tb + 4 * w; t0 < te; t0 += 4 * kEpiWarps) {
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int c = l; c < a.ss_chunks; c += 32) {
 #pragma unroll
-    for (int k = 0; k < kFinRows; ++k) {
-      const int t = t0 + nw * k + w;
-      if (t >= te) break;
-      const float4 xv = acc[k];
+      for (int k = 0; k < 4; ++k)
+        if (t0 + k < te) s[k] += __ldcg(a.ss_in + (size_t)c * kMaxT + t0 + k);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s[k] = warp_sum(s[k]);
+    if (l == 0) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (t0 + k < te) rms[t0 + k] = rsqrtf(s[k] * a.inv_dim + a.eps);
+    }
+  }
+}
+
+// Finishing a tile of QKV or RESID: warp w of the eight epilogue warps owns
+// token rows t = t0 + w + 8k, k < kFinRows, of a pass, lane l the four features
+// 4l..4l+3 of the tile, so a token's features sit in one warp (RMSNorm sums,
+// q/k norm and the RoPE pair exchange are warp shuffles).
+constexpr int kFinRows = 4;
+constexpr int kFinPass = kFinRows * kEpiWarps;
+constexpr int kMaxSplit = 8;
+
+// acc[k] = sum over the cluster's CTAs, in rank order, of their staged row of
+// token t0 + w + 8k (peer[s]: shared-memory address of CTA s's stage)
+OOS_DEV void pull_rows(float4 (&acc)[kFinRows], const uint32_t (&peer)[kMaxSplit], int split, int t0, int te, int w,
+                       bool live) {
+  const uint32_t off = (uint32_t)(threadIdx.x & 31) * 16;
+#pragma unroll
+  for (int k = 0; k < kFinRows; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+  for (int s0 = 0; s0 < kMaxSplit; s0 += 4) {
+    if (s0 >= split) break;
+    float4 v[4][kFinRows];
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+#pragma unroll
+      for (int k = 0; k < kFinRows; ++k) {
+        const int t = t0 + w + kEpiWarps * k;
+        v[s][k] = (s0 + s < split && t < te && live) ? ld_cluster_f4(peer[s0 + s] + (uint32_t)t * (kTile * 4) + off)
+                                                     : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+#pragma unroll
+      for (int k = 0; k < kFinRows; ++k) acc[k] = f4_add(acc[k], v[s][k]);
+  }
+}
+
+// what a finishing pass of RESID reads from global memory
+struct ResidRows {
+  float4 x[kFinRows];
+};
+OOS_DEV void resid_load(const GemmArgs& a, ResidRows& r, int f, bool live, int t0, int te, int w) {
+#pragma unroll
+  for (int k = 0; k < kFinRows; ++k) {
+    const int t = t0 + w + kEpiWarps * k;
+    r.x[k] = (t < te && live) ? __ldcg(reinterpret_cast<const float4*>(a.x + (size_t)t * a.N + f))
+                              : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+}
+// x += W.a; y = g (.) x; per-tile sums of x^2
+OOS_DEV void resid_finish(const GemmArgs& a, const ResidRows& r, const float4 (&acc)[kFinRows], float4 g, int tile, int f,
+                          bool live, bool st, int t0, int te, int w) {
+  const int l = threadIdx.x & 31;
+#pragma unroll
+  for (int k = 0; k < kFinRows; ++k) {
+    const int t = t0 + w + kEpiWarps * k;
+    if (t >= te) break;
+    const float4 xv = f4_add(r.x[k], acc[k]);
+    if (live && st) {
       *reinterpret_cast<float4*>(a.x + (size_t)t * a.N + f) = xv;
       store_act4(a.y_out, (size_t)t * a.N + f, (size_t)kMaxT * a.N,
                  make_float4(g.x * xv.x, g.y * xv.y, g.z * xv.z, g.w * xv.w));
-      const float sq = warp_sum(xv.x * xv.x + xv.y * xv.y + xv.z * xv.z + xv.w * xv.w);
-      if (l == 0) a.ss_out[(size_t)tile * kMaxT + t] = sq;
     }
+    const float sq = warp_sum(live ? xv.x * xv.x + xv.y * xv.y + xv.z * xv.z + xv.w * xv.w : 0.f);
+    if (l == 0 && st) a.ss_out[(size_t)tile * kMaxT + t] = sq;
   }
 }
 
-// EPI_SILU on work tile wt (subtile 0 = gate rows of block wt, subtile 1 = up
-// rows), tokens [tb, te), by warp w of nw
-template <typename Src>
-OOS_DEV void finish_silu(const GemmArgs& a, const Src& src, int wt, int nc, const float* rms, int tb, int te, int w,
-                         int nw) {
-  const int l = threadIdx.x & 31;
-  const int i = wt * kTile + 4 * l;
-  constexpr int R = 8;   // 8 token rows per warp per pass
-  for (int t0 = tb; t0 < te; t0 += nw * R) {
-    float4 gv[R], uv[R];
-    // gate and up slices of a pass in one batch of loads
-    load_pair_rows<R>(gv, uv, src, nc, 2 * wt * kTile + 4 * l, kTile, t0, te, w, nw);
+// what a finishing pass of QKV reads from global memory: the rotary factors
+struct QkvRows {
+  float2 cs[kFinRows][4];
+};
+OOS_DEV void qkv_load(const GemmArgs& a, QkvRows& r, int kind, int t0, int te, int w) {
+  const int m0 = 4 * (threadIdx.x & 15);   // rotary frequency index of this lane's first feature
 #pragma unroll
-    for (int k = 0; k < R; ++k) {
-      const int t = t0 + nw * k + w;
-      if (t >= te) break;
-      const float r = rms[t];
-      const float g4[4] = {gv[k].x * r, gv[k].y * r, gv[k].z * r, gv[k].w * r};
-      const float u4[4] = {uv[k].x * r, uv[k].y * r, uv[k].z * r, uv[k].w * r};
-      float o4[4];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) o4[c] = g4[c] / (1.f + expf(-g4[c])) * u4[c];
-      store_act4(a.act_out, (size_t)t * a.I + i, (size_t)kMaxT * a.I, make_float4(o4[0], o4[1], o4[2], o4[3]));
-    }
+  for (int k = 0; k < kFinRows; ++k) {
+    const int t = t0 + w + kEpiWarps * k;
+    const bool ok = kind < 2 && t < te;
+    const float4* p = reinterpret_cast<const float4*>(a.rope + (size_t)t * (kTile / 2) + m0);
+    const float4 u = ok ? __ldcg(p) : make_float4(1.f, 0.f, 1.f, 0.f);
+    const float4 v = ok ? __ldcg(p + 1) : make_float4(1.f, 0.f, 1.f, 0.f);
+    r.cs[k][0] = make_float2(u.x, u.y);
+    r.cs[k][1] = make_float2(u.z, u.w);
+    r.cs[k][2] = make_float2(v.x, v.y);
+    r.cs[k][3] = make_float2(v.z, v.w);
   }
 }
-
-// EPI_QKV on 128-row tile `tile` = one head (q heads, then k heads, then v
-// heads), tokens [tb, te), by warp w of nw
-template <typename Src>
-OOS_DEV void finish_qkv(const GemmArgs& a, const Src& src, int tile, int nc, const float* rms, int tb, int te, int w,
-                        int nw) {
+// one head (kind 0: q, 1: k, 2: v) of the tokens of a pass
+OOS_DEV void qkv_finish(const GemmArgs& a, const QkvRows& r, const float4 (&acc)[kFinRows], float4 b4, bool norm,
+                        float4 g4, int kind, int h, int ctx, const float* rms, bool st, int t0, int te, int w) {
   const int l = threadIdx.x & 31;
-  int kind, h;
-  if (tile < a.nq) { kind = 0; h = tile; }
-  else if (tile < a.nq + a.nkv) { kind = 1; h = tile - a.nq; }
-  else { kind = 2; h = tile - a.nq - a.nkv; }
-  const __nv_bfloat16* bias = kind == 0 ? a.bq : kind == 1 ? a.bk : a.bv;
-  const __nv_bfloat16* gn = kind == 0 ? a.gq : kind == 1 ? a.gk : nullptr;
-  const float4 b4 = bias ? bf16x4(bias + h * kTile + 4 * l) : make_float4(0.f, 0.f, 0.f, 0.f);
-  const float4 g4 = gn ? bf16x4(gn + 4 * l) : make_float4(1.f, 1.f, 1.f, 1.f);
-  const int ctx = *a.ctx;
-  const int m0 = 4 * (l & 15);      // rotary frequency index of this lane's first feature
   const bool first_half = l < 16;   // features 0..63 pair with 64..127 held by lane ^ 16
-  for (int t0 = tb; t0 < te; t0 += nw * kFinRows) {
-    // the pass's rotary factors, loaded ahead of (and so together with) the partial sums
-    float2 cs[kFinRows][4];
 #pragma unroll
-    for (int k = 0; k < kFinRows; ++k) {
-      const int t = t0 + nw * k + w;
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-        cs[k][c] = (kind < 2 && t < te) ? __ldcg(a.rope + t * (kTile / 2) + m0 + c) : make_float2(1.f, 0.f);
+  for (int k = 0; k < kFinRows; ++k) {
+    const int t = t0 + w + kEpiWarps * k;
+    if (t >= te) break;
+    const float rt = rms[t];
+    float v[4] = {acc[k].x * rt + b4.x, acc[k].y * rt + b4.y, acc[k].z * rt + b4.z, acc[k].w * rt + b4.w};
+    if (norm) {   // per-head RMSNorm over the head's 128 features
+      const float ss = warp_sum(v[0] * v[0] + v[1] * v[1] + v[2] * v[2] + v[3] * v[3]);
+      const float rn = rsqrtf(ss * (1.f / kTile) + a.eps);
+      v[0] *= rn * g4.x;
+      v[1] *= rn * g4.y;
+      v[2] *= rn * g4.z;
+      v[3] *= rn * g4.w;
     }
-    float4 acc[kFinRows];
-    load_tile_rows<kFinRows, 8>(acc, src, nc, tile * kTile + 4 * l, t0, te, nullptr, 0, 0, w, nw);
+    if (kind < 2) {   // rotate-half RoPE at position ctx + depth(t)
 #pragma unroll
-    for (int k = 0; k < kFinRows; ++k) {
-      const int t = t0 + nw * k + w;
-      if (t >= te) break;
-      const float r = rms[t];
-      float v[4] = {acc[k].x * r + b4.x, acc[k].y * r + b4.y, acc[k].z * r + b4.z, acc[k].w * r + b4.w};
-      if (gn) {   // per-head RMSNorm over the head's 128 features
-        const float ss = warp_sum(v[0] * v[0] + v[1] * v[1] + v[2] * v[2] + v[3] * v[3]);
-        const float rn = rsqrtf(ss * (1.f / kTile) + a.eps);
-        v[0] *= rn * g4.x;
-        v[1] *= rn * g4.y;
-        v[2] *= rn * g4.z;
-        v[3] *= rn * g4.w;
+      for (int c = 0; c < 4; ++c) {
+        const float other = __shfl_xor_sync(0xffffffffu, v[c], 16);
+        v[c] = first_half ? v[c] * r.cs[k][c].x - other * r.cs[k][c].y : v[c] * r.cs[k][c].x + other * r.cs[k][c].y;
       }
-      if (kind < 2) {   // rotate-half RoPE at position ctx + depth(t)
+    }
+    if (!st) {
+      asm volatile("" ::"f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]));
+    } else if (kind == 0) {   // q as hi/lo halves in the cache's 16-bit format: the attention product sees ~16-bit q
+      const size_t qi = ((size_t)t * a.nq + h) * kTile + 4 * l, lo_off = (size_t)kMaxT * a.nq * kTile;
+      if (a.kv_f16) store_act4_h(reinterpret_cast<__half*>(a.q_out), qi, lo_off, make_float4(v[0], v[1], v[2], v[3]));
+      else store_act4(a.q_out, qi, lo_off, make_float4(v[0], v[1], v[2], v[3]));
+    } else {           // K/V in the cache's format (bf16, or binary16)
+      __nv_bfloat16* dst = (kind == 1 ? a.kc : a.vc) + ((size_t)(ctx + t) * a.nkv + h) * kTile;
+      uint2 o;
+      if (a.kv_f16) {
+        __half hv[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const float other = __shfl_xor_sync(0xffffffffu, v[c], 16);
-          v[c] = first_half ? v[c] * cs[k][c].x - other * cs[k][c].y : v[c] * cs[k][c].x + other * cs[k][c].y;
-        }
+        for (int c = 0; c < 4; ++c) hv[c] = __float2half_rn(v[c]);
+        o = *reinterpret_cast<const uint2*>(hv);
+      } else {
+        __nv_bfloat16 bv[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) bv[c] = __float2bfloat16_rn(v[c]);
+        o = *reinterpret_cast<const uint2*>(bv);
       }
-      if (kind == 0) {   // q as hi/lo halves in the cache's 16-bit format: the attention product sees ~16-bit q
-        const size_t qi = ((size_t)t * a.nq + h) * kTile + 4 * l, lo_off = (size_t)kMaxT * a.nq * kTile;
-        if (a.kv_f16) store_act4_h(reinterpret_cast<__half*>(a.q_out), qi, lo_off, make_float4(v[0], v[1], v[2], v[3]));
-        else store_act4(a.q_out, qi, lo_off, make_float4(v[0], v[1], v[2], v[3]));
-      } else {           // K/V in the cache's format (bf16, or binary16)
-        __nv_bfloat16* dst = (kind == 1 ? a.kc : a.vc) + ((size_t)(ctx + t) * a.nkv + h) * kTile;
-        uint2 o;
-        if (a.kv_f16) {
-          __half hv[4];
-#pragma unroll
-          for (int c = 0; c < 4; ++c) hv[c] = __float2half_rn(v[c]);
-          o = *reinterpret_cast<const uint2*>(hv);
-        } else {
-          __nv_bfloat16 bv[4];
-#pragma unroll
-          for (int c = 0; c < 4; ++c) bv[c] = __float2bfloat16_rn(v[c]);
-          o = *reinterpret_cast<const uint2*>(bv);
-        }
-        *reinterpret_cast<uint2*>(dst + 4 * l) = o;
-      }
+      *reinterpret_cast<uint2*>(dst + 4 * l) = o;
     }
   }
 }
 
 template <int BN, int EPI>
-__global__ void __launch_bounds__(192, 1)
+__global__ void __launch_bounds__(kGemmThreads, 1)
     k_gemm_tc(const __grid_constant__ CUtensorMap wm0, const __grid_constant__ CUtensorMap wm1,
-              const __grid_constant__ CUtensorMap wm2, const __grid_constant__ CUtensorMap am, GemmArgs a) {
-  constexpr int kSub = SubOf<EPI>::v;
-  using C = TcCfg<BN, kSub>;
-  constexpr int S = C::S;
+              const __grid_constant__ CUtensorMap wm2, const __grid_constant__ CUtensorMap am,
+              const __grid_constant__ GemmArgs a) {
+  using C = TcCfg<BN, EPI>;
+  constexpr int kSub = C::kSub;
   constexpr bool ARGMAX = EPI == EPI_ARGMAX;
+  constexpr bool CLUSTER = EpiOf<EPI>::cluster;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  // stage layout: [A subtile 0 | A subtile 1 | B hi | B lo]
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + S * C::STAGE);
-  uint64_t* empty = full + S;
-  uint64_t* accf = empty + S;
+  // [barriers | RMSNorm factors | argmax state], then from `ring` on the weight
+  // subtiles of every stage and after them the activation slices (hi, lo)
+  const int S = a.stages;
+  const int a_bytes = a.rows * kBK * 2;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem);
+  uint64_t* empty = full + kMaxStages;
+  uint64_t* accf = empty + kMaxStages;
   uint64_t* acce = accf + 2;
   uint64_t* drain = acce + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  float* rms = reinterpret_cast<float*>(smem + S * C::STAGE + C::BAR_BYTES);       // [kMaxT]
-  Top2s* red = reinterpret_cast<Top2s*>(smem + S * C::STAGE + C::BAR_BYTES + C::EPI_BYTES);   // [4][BN]
+  static_assert((2 * kMaxStages + 5) * 8 + 12 <= C::BAR_BYTES, "barrier block");
+  float* rms = reinterpret_cast<float*>(smem + C::BAR_BYTES);                                  // [kMaxT]
+  Top2s* red = reinterpret_cast<Top2s*>(smem + C::BAR_BYTES + C::EPI_BYTES);                   // [4][BN]
   Top2s* run = red + 4 * BN;                                                                   // [BN]
+  unsigned char* ring = smem + C::HEAD;
+  unsigned char* ring_x = ring + S * kSub * a_bytes;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int G = gridDim.x, cta = blockIdx.x;
   if (threadIdx.x == 0) TL_GEMM(0);
 
-  // this CTA's work: units [u0, u1) (stream-K) or work tiles cta, cta+G, ... (LM head)
-  long long u0, u1;
-  if (!ARGMAX) {
-    u0 = (long long)cta * a.total / G;
-    u1 = (long long)(cta + 1) * a.total / G;
+  // this CTA's work: k-blocks [kb0, kb0 + n_units) of tile `first` (cluster), or
+  // all k-blocks of tiles first, first + step, ...
+  int first, step, kb0, nkb, n_units;
+  uint32_t rank = 0;
+  if (CLUSTER) {
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    first = blockIdx.x / a.split;
+    step = 0;
+    kb0 = a.kbt * (int)rank / a.split;
+    nkb = n_units = a.kbt * ((int)rank + 1) / a.split - kb0;
   } else {
-    const int my_tiles = cta < a.n_work ? (a.n_work - cta + G - 1) / G : 0;
-    u0 = 0;
-    u1 = (long long)my_tiles * a.kbt;
+    first = blockIdx.x;
+    step = gridDim.x;
+    kb0 = 0;
+    nkb = a.kbt;
+    n_units = first < a.n_work ? (a.n_work - first + step - 1) / step * a.kbt : 0;
   }
-  const int n_units = (int)(u1 - u0);
-  auto unit_tile = [&](int j, int& wt, int& kb) {
-    if (!ARGMAX) {
-      const long long u = u0 + j;
-      wt = (int)(u / a.kbt);
-      kb = (int)(u % a.kbt);
-    } else {
-      wt = cta + (j / a.kbt) * G;
-      kb = j % a.kbt;
-    }
-  };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
@@ -413,7 +402,7 @@ __global__ void __launch_bounds__(192, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&accf[b], 1);
-      mbar_init(&acce[b], 4);
+      mbar_init(&acce[b], kEpiWarps);
     }
     mbar_init(drain, 1);
     abort_flag[0] = 0;
@@ -422,7 +411,7 @@ __global__ void __launch_bounds__(192, 1)
   }
   if (warp == 2) tmem_alloc(tmem_slot, C::NCOLS);
   if (ARGMAX && threadIdx.x >= 64) {
-    for (int e = threadIdx.x - 64; e < BN; e += 128) run[e] = Top2s{-INFINITY, 0x7fffffff, -INFINITY};
+    for (int e = threadIdx.x - 64; e < BN; e += kEpiThreads) run[e] = Top2s{-INFINITY, 0x7fffffff, -INFINITY};
   }
   tc_fence_before();
   __syncthreads();
@@ -436,56 +425,66 @@ __global__ void __launch_bounds__(192, 1)
       tma_prefetch_desc(&am);
       const uint64_t pol_w = policy_evict_first();
       const uint64_t pol_a = policy_evict_last();
-      auto load_w = [&](int j, int stage) {
-        int wt, kb;
-        unit_tile(j, wt, kb);
+      const uint32_t stage_bytes = (uint32_t)(kSub * a_bytes + 2 * C::B_BYTES);
+      // weights of the unit at (tile, kb) into `stage`; rows past the matrix
+      // read zeros (TMA out-of-bounds fill)
+      auto load_w = [&](int tile, int kb, int stage) {
+        unsigned char* dst = ring + stage * kSub * a_bytes;
+        if (EPI == EPI_SILU) {
+          tma_load_2d(dst, &wm0, &full[stage], kb * kBK, tile * a.rows, pol_w);
+          tma_load_2d(dst + a_bytes, &wm1, &full[stage], kb * kBK, tile * a.rows, pol_w);
+        } else if (EPI == EPI_QKV) {
+          const CUtensorMap* wm = tile < a.seg_tiles[0] ? &wm0 : tile < a.seg_tiles[1] ? &wm1 : &wm2;
+          const int base = tile < a.seg_tiles[0] ? 0 : tile < a.seg_tiles[1] ? a.seg_tiles[0] : a.seg_tiles[1];
+          tma_load_2d(dst, wm, &full[stage], kb * kBK, (tile - base) * a.rows, pol_w);
+        } else {
 #pragma unroll
-        for (int sub = 0; sub < kSub; ++sub) {
-          const int tile = wt * kSub + sub;          // 128-row tile of the stacked weight
-          const CUtensorMap* wm = &wm0;
-          int row = tile * kTile;
-          if (a.interleave2) {
-            wm = (tile & 1) ? &wm1 : &wm0;
-            row = (tile >> 1) * kTile;
-          } else if (tile >= a.seg_tiles[0]) {
-            if (tile >= a.seg_tiles[1]) {
-              wm = &wm2;
-              row = (tile - a.seg_tiles[1]) * kTile;
-            } else {
-              wm = &wm1;
-              row = (tile - a.seg_tiles[0]) * kTile;
-            }
-          }
-          // a subtile past the last weight row reads zeros (TMA out-of-bounds fill)
-          tma_load_2d(smem + stage * C::STAGE + sub * C::A_BYTES, wm, &full[stage], kb * kBK, row, pol_w);
+          for (int sub = 0; sub < kSub; ++sub)
+            tma_load_2d(dst + sub * a_bytes, &wm0, &full[stage], kb * kBK, (tile * kSub + sub) * a.rows, pol_w);
         }
       };
-      auto load_x = [&](int j, int stage) {
-        int wt, kb;
-        unit_tile(j, wt, kb);
-        unsigned char* dst = smem + stage * C::STAGE + kSub * C::A_BYTES;
+      auto load_x = [&](int kb, int stage) {
+        unsigned char* dst = ring_x + stage * 2 * C::B_BYTES;
         tma_load_2d(dst, &am, &full[stage], kb * kBK, 0, pol_a);                   // hi rows
         tma_load_2d(dst + C::B_BYTES, &am, &full[stage], kb * kBK, kMaxT, pol_a);  // lo rows
       };
       // weights do not depend on the previous kernel: start streaming them
       // before waiting for it (programmatic dependent launch)
       const int n_pre = n_units < S ? n_units : S;
-      for (int j = 0; j < n_pre; ++j) {
-        mbar_arrive_expect_tx(&full[j], C::STAGE);
-        load_w(j, j);
+      {
+        int tile = first, kb = 0;
+        for (int j = 0; j < n_pre; ++j) {
+          mbar_arrive_expect_tx(&full[j], stage_bytes);
+          load_w(tile, kb0 + kb, j);
+          if (++kb == nkb) {
+            kb = 0;
+            tile += step;
+          }
+        }
       }
       pdl_wait();
       pdl_trigger();
       TL_GEMM(1);
-      for (int j = 0; j < n_pre; ++j) load_x(j, j);
+      int tile = first, kb = 0;
+      auto advance = [&]() {
+        if (++kb == nkb) {
+          kb = 0;
+          tile += step;
+        }
+      };
+      for (int j = 0; j < n_pre; ++j) {
+        load_x(kb0 + kb, j);
+        advance();
+      }
       int stage = n_pre % S;
       uint32_t phase = (n_pre == S) ? 1u : 0u;
       int issued = n_pre;
       for (int j = n_pre; j < n_units; ++j) {
         if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, a.status)) break;
-        mbar_arrive_expect_tx(&full[stage], C::STAGE);
-        load_w(j, stage);
-        load_x(j, stage);
+        mbar_arrive_expect_tx(&full[stage], stage_bytes);
+        load_w(tile, kb0 + kb, stage);
+        load_x(kb0 + kb, stage);
+        advance();
         ++issued;
         if (++stage == S) {
           stage = 0;
@@ -495,14 +494,14 @@ __global__ void __launch_bounds__(192, 1)
       {
         // every copy this thread issued has landed before the CTA can exit,
         // whoever gave up (immediate on the normal path, where all were consumed)
-        const int first = issued - S > 0 ? issued - S : 0;
-        for (int j = first; j < issued; ++j) {
+        for (int j = issued - S > 0 ? issued - S : 0; j < issued; ++j) {
           const unsigned long long t0 = globaltimer();
           while (!mbar_test(smem_addr(&full[j % S]), (uint32_t)((j / S) & 1)) && globaltimer() - t0 < kWaitLimitNs) {
           }
         }
       }
     }
+    __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
     if (lane == 0) {
@@ -510,47 +509,49 @@ __global__ void __launch_bounds__(192, 1)
       int stage = 0;
       uint32_t phase = 0;
       int acc = 0;
-      uint32_t acc_use[2] = {0, 0};
-      int j = 0;
+      uint32_t use = 0;   // accumulators handed over so far (two buffers in turn)
       bool ok = true;
-      while (j < n_units && ok) {
-        int wt, kb;
-        unit_tile(j, wt, kb);
-        int seg_end = j + (a.kbt - kb);       // units of this work tile owned here
-        if (seg_end > n_units) seg_end = n_units;
-        if (!mbar_wait(&acce[acc], (acc_use[acc] & 1u) ^ 1u, abort_flag, a.status)) break;
-        tc_fence_after();
-        const uint32_t d0 = tmem_base + (uint32_t)(acc * kSub * C::SUB_COLS);
-        for (int jj = j; jj < seg_end; ++jj) {
-          if (!mbar_wait(&full[stage], phase, abort_flag, a.status)) {
+      const int segs = nkb < EpiOf<EPI>::segs ? 1 : EpiOf<EPI>::segs;
+      for (int j = 0; j < n_units && ok; j += nkb) {
+        for (int sg = 0; sg < segs && ok; ++sg) {
+          if (!mbar_wait(&acce[acc], ((use >> 1) & 1u) ^ 1u, abort_flag, a.status)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t sbase = smem_addr(smem + stage * C::STAGE);
-          const uint64_t bh = smem_desc_sw128(sbase + kSub * C::A_BYTES);
-          const uint64_t bl = smem_desc_sw128(sbase + kSub * C::A_BYTES + C::B_BYTES);
+          const uint32_t d0 = tmem_base + (uint32_t)(acc * kSub * C::SUB_COLS);
+          const int n = nkb * (sg + 1) / segs - nkb * sg / segs;
+          for (int jj = 0; jj < n; ++jj) {
+            if (!mbar_wait(&full[stage], phase, abort_flag, a.status)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            const uint32_t wbase = smem_addr(ring + stage * kSub * a_bytes);
+            const uint32_t xbase = smem_addr(ring_x + stage * 2 * C::B_BYTES);
+            const uint64_t bh = smem_desc_sw128(xbase);
+            const uint64_t bl = smem_desc_sw128(xbase + C::B_BYTES);
 #pragma unroll
-          for (int k = 0; k < kBK / 16; ++k) {
+            for (int k = 0; k < kBK / 16; ++k) {
 #pragma unroll
-            for (int sub = 0; sub < kSub; ++sub) {
-              const uint64_t ad = smem_desc_sw128(sbase + sub * C::A_BYTES);
-              const uint32_t d = d0 + (uint32_t)(sub * C::SUB_COLS);
-              tc_mma_bf16(d, ad + 2 * k, bh + 2 * k, idesc, (jj > j || k > 0) ? 1u : 0u);
-              if (!C::PAIRED) tc_mma_bf16(d, ad + 2 * k, bl + 2 * k, idesc, 1u);
+              for (int sub = 0; sub < kSub; ++sub) {
+                const uint64_t ad = smem_desc_sw128(wbase + (uint32_t)(sub * a_bytes));
+                const uint32_t d = d0 + (uint32_t)(sub * C::SUB_COLS);
+                tc_mma_bf16(d, ad + 2 * k, bh + 2 * k, idesc, (jj > 0 || k > 0) ? 1u : 0u);
+                if (!C::PAIRED) tc_mma_bf16(d, ad + 2 * k, bl + 2 * k, idesc, 1u);
+              }
+            }
+            tc_commit(&empty[stage]);
+            if (++stage == S) {
+              stage = 0;
+              phase ^= 1u;
             }
           }
-          tc_commit(&empty[stage]);
-          if (++stage == S) {
-            stage = 0;
-            phase ^= 1u;
-          }
+          if (!ok) break;
+          tc_commit(&accf[acc]);
+          ++use;
+          acc ^= 1;
         }
-        if (!ok) break;
-        tc_commit(&accf[acc]);
-        ++acc_use[acc];
-        acc ^= 1;
-        j = seg_end;
       }
       // all issued MMAs complete before TMEM is released
       tc_commit(drain);
@@ -558,249 +559,282 @@ __global__ void __launch_bounds__(192, 1)
       while (!mbar_test(smem_addr(drain), 0) && globaltimer() - t0 < kWaitLimitNs) {
       }
     }
-  } else {
-    // ------------------------------------------------------------ epilogue (warps 2..5)
+    __syncwarp();
+  }
+
+  // -------------------------------------------------------------- epilogue (warps 2..9)
+  const int ew = warp - 2;              // epilogue warp 0..7
+  const int q = warp & 3;               // TMEM lane quarter this warp may access
+  const int half = ew >> 2;             // 16-token column chunks half, half + 2, ...
+  const int row = q * 32 + lane;        // weight row of the tile
+  const uint32_t lane_base = tmem_base + ((uint32_t)(q * 32) << 16);
+  // 16 accumulator columns (tokens) starting at column `col`: paired hi + lo products
+  auto acc16 = [&](uint32_t col, float (&v)[16]) {
+    if (C::PAIRED) {
+      float lo[16];
+      tmem_ld16_nowait(lane_base + col, v);
+      tmem_ld16_nowait(lane_base + col + BN, lo);
+      tmem_wait_ld();
+      reg_fence(v);
+      reg_fence(lo);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) v[i] += lo[i];
+    } else {
+      tmem_ld16(lane_base + col, v);
+    }
+  };
+
+  if (CLUSTER && warp >= 2) {
+    const int tile = first;
+    // tokens [tb, te) are finished here
+    const int tb = a.T * (int)rank / a.split, te = a.T * ((int)rank + 1) / a.split;
+    const int f = EPI == EPI_RESID ? tile * a.rows + 4 * lane : 4 * lane;
+    const bool live = 4 * lane < a.rows && (EPI != EPI_RESID || f < a.N);
+    const bool two = nkb >= 2;   // one accumulator per k-segment
+    int kind = 0, h = 0, ctx = 0;
+    bool norm = false, have = false;
+    float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f), g4 = make_float4(1.f, 1.f, 1.f, 1.f);
+    ResidRows rr;
+    QkvRows qr;
+    float* stage = reinterpret_cast<float*>(ring);   // [token][kTile]
+    if (EPI == EPI_RESID) {
+      if (live) g4 = bf16x4(a.gain + f);
+    } else {
+      if (tile < a.nq) { kind = 0; h = tile; }
+      else if (tile < a.nq + a.nkv) { kind = 1; h = tile - a.nq; }
+      else { kind = 2; h = tile - a.nq - a.nkv; }
+      const __nv_bfloat16* bias = kind == 0 ? a.bq : kind == 1 ? a.bk : a.bv;
+      const __nv_bfloat16* gn = kind == 0 ? a.gq : kind == 1 ? a.gk : nullptr;
+      if (bias) b4 = bf16x4(bias + h * kTile + f);
+      if (gn) g4 = bf16x4(gn + f);
+      norm = gn != nullptr;
+    }
+    // Pass -1 is a dry run of the whole epilogue before the dependency wait:
+    // no wait, barrier or store, values discarded.  The epilogue runs once per
+    // launch, and the step's other kernels have evicted its code from the SM's
+    // instruction caches since the previous layer; this fetches it while the
+    // warps have nothing else to do.
+#pragma unroll 1
+    for (int pass = -1;; ++pass) {
+      asm volatile("" : "+r"(pass));   // one copy of the body for every pass
+      const bool dry = pass < 0;
+      const int t0 = dry ? tb : tb + pass * kFinPass;
+      if (pass > 0 && t0 >= te) break;
+      if (pass == 0) {
+        pdl_wait();
+        pdl_trigger();
+      }
+      // what the finishing reads, while the weights stream
+      if (EPI == EPI_RESID) {
+        resid_load(a, rr, f, live, t0, te, ew);
+      } else {
+        qkv_load(a, qr, kind, t0, te, ew);
+        if (pass <= 0) {
+          ctx = *a.ctx;
+          input_rms(a, rms, tb, te, ew);
+        }
+      }
+      if (pass <= 0) {
+        if (!dry) {
+          have = mbar_wait(&accf[0], 0, abort_flag, a.status) && (!two || mbar_wait(&accf[1], 0, abort_flag, a.status));
+          have = __all_sync(0xffffffffu, have);
+          if (threadIdx.x == 64) TL_GEMM(2);
+          tc_fence_after();
+        }
+        // every MMA has read its operands: the ring is free for the sums
+        const bool put = have && row < a.rows;
+#pragma unroll 1
+        for (int cc = half; cc < BN / 16; cc += 2) {
+          if (cc * 16 >= a.T) break;
+          float v[16];
+          acc16((uint32_t)(cc * 16), v);
+          if (two) {
+            float v1[16];
+            acc16((uint32_t)(C::SUB_COLS + cc * 16), v1);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) v[i] += v1[i];
+          }
+          if (put) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) stage[(cc * 16 + i) * kTile + row] = v[i];
+          }
+        }
+        if (!dry) {
+          if (threadIdx.x == 64) TL_GEMM(4);
+          // Every thread of the cluster arrives twice, whatever happened before:
+          // when its sums are staged, and when it has pulled its share (a CTA's
+          // stage must outlive its readers).
+          cluster_arrive_release();
+          __syncwarp();
+          cluster_wait_acquire();
+          if (threadIdx.x == 64) TL_GEMM(5);
+        }
+      }
+      uint32_t peer[kMaxSplit];   // the dry run reads its own stage: the peers may not run yet
+#pragma unroll
+      for (int s = 0; s < kMaxSplit; ++s) peer[s] = dsmem_addr(stage, dry ? rank : (uint32_t)(s < a.split ? s : 0));
+      float4 acc[kFinRows];
+      pull_rows(acc, peer, a.split, t0, te, ew, live);
+      if (!dry && t0 + kFinPass >= te) {   // the last pull: before the stores, which the barrier need not await
+#pragma unroll
+        for (int k = 0; k < kFinRows; ++k) asm volatile("" ::"f"(acc[k].x), "f"(acc[k].y), "f"(acc[k].z), "f"(acc[k].w) : "memory");
+        cluster_arrive_relaxed();
+      }
+      if (EPI == EPI_RESID) resid_finish(a, rr, acc, g4, tile, f, live, have, t0, te, ew);
+      else qkv_finish(a, qr, acc, b4, norm, g4, kind, h, ctx, rms, have, t0, te, ew);
+    }
+    __syncwarp();
+    cluster_wait_acquire();
+  } else if (CLUSTER) {   // the producer's and the issuer's warps: their two arrivals
+    cluster_arrive_release();
+    __syncwarp();
+    cluster_wait_acquire();
+    cluster_arrive_release();
+    __syncwarp();
+    cluster_wait_acquire();
+  } else if (!ARGMAX && warp >= 2) {
+    // Gate and up of one row sit in the same lane, so act is formed in
+    // registers.  Tile -1 is a dry run, as above.
+    const bool two = nkb >= 2;
+    const bool odd = lane & 1;
+    uint32_t use = 0;   // tiles drained
+    uint32_t acc0 = 0;  // buffer of the tile's first k-segment (the second's is the other one)
+#pragma unroll 1
+    for (int it = -1;; ++it) {
+      asm volatile("" : "+r"(it));
+      const bool dry = it < 0;
+      const int tile = first + (dry ? 0 : it) * step;
+      if (it == 0) {
+        pdl_wait();
+        pdl_trigger();
+      }
+      if (it <= 0) {
+        input_rms(a, rms, 0, a.T, ew);
+        epi_bar();
+      }
+      if (!dry) {
+        if (it * nkb >= n_units) break;
+        const bool ok = two ? mbar_wait(&accf[0], use & 1u, abort_flag, a.status) &&
+                                  mbar_wait(&accf[1], use & 1u, abort_flag, a.status)
+                            : mbar_wait(&accf[acc0], (use >> 1) & 1u, abort_flag, a.status);
+        if (!__all_sync(0xffffffffu, ok)) break;
+        if (threadIdx.x == 64 && (it + 1) * nkb >= n_units) TL_GEMM(2);
+        tc_fence_after();
+      }
+      const uint32_t col0 = acc0 * (uint32_t)(kSub * C::SUB_COLS), col1 = (acc0 ^ 1u) * (uint32_t)(kSub * C::SUB_COLS);
+      const int fi = tile * a.rows + (row & ~1);
+      const bool live = row < a.rows && fi < a.N && !dry;
+#pragma unroll 1
+      for (int cc = half; cc < BN / 16; cc += 2) {
+        if (cc * 16 >= a.T) break;
+        float g[16], u[16];
+        acc16(col0 + cc * 16, g);
+        acc16(col0 + C::SUB_COLS + cc * 16, u);
+        if (two) {
+          float v[16];
+          acc16(col1 + cc * 16, v);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) g[i] += v[i];
+          acc16(col1 + C::SUB_COLS + cc * 16, v);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) u[i] += v[i];
+        }
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          const float r = rms[cc * 16 + i];
+          const float gr = g[i] * r;
+          u[i] = __fdividef(gr, 1.f + expf(-gr)) * (u[i] * r);   // 2 ulp; exp's infinity gives 0
+        }
+        // lane pairs swap tokens so that a store covers two neighbouring features
+#pragma unroll
+        for (int i = 0; i < 16; i += 2) {
+          const float mine = odd ? u[i + 1] : u[i];
+          const float other = __shfl_xor_sync(0xffffffffu, odd ? u[i] : u[i + 1], 1);
+          const float v0 = odd ? other : mine, v1 = odd ? mine : other;   // features row & ~1, row | 1
+          const int t = cc * 16 + i + (odd ? 1 : 0);
+          const __nv_bfloat162 hi = __floats2bfloat162_rn(v0, v1);
+          const __nv_bfloat162 lo = __floats2bfloat162_rn(v0 - __low2float(hi), v1 - __high2float(hi));
+          if (live && t < a.T) {
+            __nv_bfloat16* dst = a.act_out + (size_t)t * a.N + fi;
+            *reinterpret_cast<__nv_bfloat162*>(dst) = hi;
+            *reinterpret_cast<__nv_bfloat162*>(dst + (size_t)kMaxT * a.N) = lo;
+          }
+        }
+      }
+      if (!dry) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) {
+          mbar_arrive(&acce[acc0]);
+          if (two) mbar_arrive(&acce[acc0 ^ 1u]);
+        }
+        ++use;
+        if (!two) acc0 ^= 1u;
+      }
+    }
+  } else if (warp >= 2) {
     pdl_wait();
     pdl_trigger();
-    const int q = warp & 3;               // TMEM lane quarter this warp may access
-    const int row = q * 32 + lane;
-    const int e = threadIdx.x - 64;       // 0..127
-    // Abort decisions of the epilogue warps are taken on one sample of the
-    // flag, so all 128 threads leave together and no named barrier is left
-    // waiting for threads that have gone.
-    volatile int* epi_abort = abort_flag + 1;
-    auto epi_aborted = [&]() -> bool {
-      epi_bar();
-      if (e == 0) *epi_abort = *abort_flag;
-      epi_bar();
-      return *epi_abort != 0;
-    };
-    if (EPI != EPI_RESID) {
-      if (e < a.T) {
-        float s = 0.f;
-        for (int c = 0; c < a.ss_chunks; ++c) s += a.ss_in[(size_t)c * kMaxT + e];
-        rms[e] = rsqrtf(s * a.inv_dim + a.eps);
-      }
-      epi_bar();
-    }
-    const int n_part = a.n_work * kSub * kTile;
+    const int e = threadIdx.x - 64;       // 0..kEpiThreads-1
+    input_rms(a, rms, 0, a.T, ew);
+    epi_bar();
     int acc = 0;
-    uint32_t acc_use[2] = {0, 0};
-    int j = 0;
-    while (j < n_units) {
-      int wt, kb;
-      unit_tile(j, wt, kb);
-      int seg_end = j + (a.kbt - kb);
-      if (seg_end > n_units) seg_end = n_units;
-      mbar_wait(&accf[acc], acc_use[acc] & 1u, abort_flag, a.status);
-      if (e == 0 && seg_end >= n_units) TL_GEMM(2);
-      if (epi_aborted()) break;
+    uint32_t use = 0;
+    for (int j = 0, tile = first; j < n_units; j += nkb, tile += step) {
+      mbar_wait(&accf[acc], (use >> 1) & 1u, abort_flag, a.status);
+      // the barriers below need every epilogue warp on one path: all of them
+      // leave on one sample of the flag
+      epi_bar();
+      if (e == 0) abort_flag[1] = abort_flag[0];
+      epi_bar();
+      if (abort_flag[1]) break;
       tc_fence_after();
-      const uint32_t taddr0 = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * kSub * C::SUB_COLS);
-      // 16 accumulator columns (tokens) of subtile `sub`: paired hi + lo products
-      auto acc16 = [&](int sub, int cc, float (&v)[16]) {
-        tmem_ld16(taddr0 + sub * C::SUB_COLS + cc * 16, v);
-        if (C::PAIRED) {
-          float w[16];
-          tmem_ld16(taddr0 + sub * C::SUB_COLS + BN + cc * 16, w);
-#pragma unroll
-          for (int i = 0; i < 16; ++i) v[i] += w[i];
-        }
-      };
-      if (!ARGMAX) {
-        int c0, c1;
-        StreamK sk{a.n_work, a.kbt, a.total, G};
-        sk.contributors(wt, c0, c1);
-        // lane l holds row q*32 + l; a 4 x 4 shuffle transpose per 4 tokens gives
-        // each lane 4 consecutive rows of one token: one float4 store, not four
-        const int li = lane & 3;
+      const uint32_t col0 = (uint32_t)(acc * kSub * C::SUB_COLS);
 #pragma unroll 1
-        for (int sub = 0; sub < kSub; ++sub) {
-          float* dst = a.part + (size_t)(cta - c0) * kMaxT * n_part + (size_t)(wt * kSub + sub) * kTile + q * 32 +
-                       (lane & ~3);
-          // the subtile's accumulator row in batches of TMEM loads (up to 64
-          // tokens, hi and lo products when paired), one wait per batch
-          constexpr int NG = BN / 16 < 4 ? BN / 16 : 4;   // 16-token chunks per batch
+      for (int sub = 0; sub < kSub; ++sub) {
+        const int f = (tile * kSub + sub) * kTile + row;
 #pragma unroll 1
-          for (int c0g = 0; c0g < BN / 16; c0g += NG) {
-            if (c0g * 16 >= a.T) break;
-            float vv[NG][16], ww[C::PAIRED ? NG : 1][16];
+        for (int cc = half; cc < BN / 16; cc += 2) {
+          if (cc * 16 >= a.T) break;
+          float v[16];
+          acc16(col0 + sub * C::SUB_COLS + cc * 16, v);
 #pragma unroll
-            for (int k = 0; k < NG; ++k) {
-              tmem_ld16_nowait(taddr0 + sub * C::SUB_COLS + (c0g + k) * 16, vv[k]);
-              if (C::PAIRED) tmem_ld16_nowait(taddr0 + sub * C::SUB_COLS + BN + (c0g + k) * 16, ww[C::PAIRED ? k : 0]);
+          for (int i = 0; i < 16; ++i) {
+            Top2s s{f < a.N ? v[i] * rms[cc * 16 + i] : -INFINITY, f, -INFINITY};
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+              Top2s y;
+              y.v1 = __shfl_xor_sync(0xffffffffu, s.v1, o);
+              y.i1 = __shfl_xor_sync(0xffffffffu, s.i1, o);
+              y.v2 = __shfl_xor_sync(0xffffffffu, s.v2, o);
+              s = t2_merge(s, y);
             }
-            tmem_wait_ld();
-#pragma unroll
-            for (int k = 0; k < NG; ++k) {
-              reg_fence(vv[k]);
-              if (C::PAIRED) reg_fence(ww[C::PAIRED ? k : 0]);
-            }
-#pragma unroll
-          for (int k = 0; k < NG; ++k) {
-            const int cc = c0g + k;
-            if (cc * 16 >= a.T) break;
-            float v[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) v[i] = C::PAIRED ? vv[k][i] + ww[C::PAIRED ? k : 0][i] : vv[k][i];
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-              float x0 = v[4 * b], x1 = v[4 * b + 1], x2 = v[4 * b + 2], x3 = v[4 * b + 3];
-              const float y0 = __shfl_xor_sync(0xffffffffu, (li & 1) ? x0 : x1, 1);
-              const float y1 = __shfl_xor_sync(0xffffffffu, (li & 1) ? x2 : x3, 1);
-              if (li & 1) {
-                x0 = y0;
-                x2 = y1;
-              } else {
-                x1 = y0;
-                x3 = y1;
-              }
-              const float z0 = __shfl_xor_sync(0xffffffffu, (li & 2) ? x0 : x2, 2);
-              const float z1 = __shfl_xor_sync(0xffffffffu, (li & 2) ? x1 : x3, 2);
-              if (li & 2) {
-                x0 = z0;
-                x1 = z1;
-              } else {
-                x2 = z0;
-                x3 = z1;
-              }
-              const int t = cc * 16 + 4 * b + li;   // rows (lane & ~3) .. +3 of token t
-              if (t < a.T) *reinterpret_cast<float4*>(dst + (size_t)t * n_part) = make_float4(x0, x1, x2, x3);
-            }
-          }
-          }
-        }
-        // accumulators drained: hand the TMEM buffer back to the MMA issuer
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&acce[acc]);
-        // publish this contribution (finished at the end of the range)
-        __threadfence();
-        epi_bar();
-        if (e == 0) atomicAdd(&a.cnt[wt], 1);
-        if (e == 0 && seg_end >= n_units) TL_GEMM(4);
-      } else {
-#pragma unroll 1
-        for (int sub = 0; sub < kSub; ++sub) {
-          const int f = (wt * kSub + sub) * kTile + row;
-#pragma unroll 1
-          for (int cc = 0; cc < BN / 16; ++cc) {
-            if (cc * 16 >= a.T) break;
-            float v[16];
-            acc16(sub, cc, v);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              Top2s s{f < a.N ? v[i] * rms[cc * 16 + i] : -INFINITY, f, -INFINITY};
-#pragma unroll
-              for (int o = 16; o > 0; o >>= 1) {
-                Top2s y;
-                y.v1 = __shfl_xor_sync(0xffffffffu, s.v1, o);
-                y.i1 = __shfl_xor_sync(0xffffffffu, s.i1, o);
-                y.v2 = __shfl_xor_sync(0xffffffffu, s.v2, o);
-                s = t2_merge(s, y);
-              }
-              if (lane == 0) {
-                Top2s* slot = &red[q * BN + cc * 16 + i];
-                *slot = sub == 0 ? s : t2_merge(*slot, s);
-              }
+            if (lane == 0) {
+              Top2s* slot = &red[q * BN + cc * 16 + i];
+              *slot = sub == 0 ? s : t2_merge(*slot, s);
             }
           }
         }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&acce[acc]);
-        epi_bar();
-        if (e < a.T) {
-          Top2s r = run[e];
-#pragma unroll
-          for (int w = 0; w < 4; ++w) r = t2_merge(r, red[w * BN + e]);
-          run[e] = r;
-        }
-        epi_bar();
       }
-      ++acc_use[acc];
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&acce[acc]);
+      epi_bar();
+      if (e < a.T) {
+        Top2s r = run[e];
+#pragma unroll
+        for (int w = 0; w < 4; ++w) r = t2_merge(r, red[w * BN + e]);
+        run[e] = r;
+      }
+      epi_bar();
+      ++use;
       acc ^= 1;
-      j = seg_end;
     }
-    if (!ARGMAX && !epi_aborted()) {
-      // Finish every work tile this CTA touched: once all nc contributions of
-      // the tile have arrived, contributor i (in CTA order) finishes token rows
-      // [T*i/nc, T*(i+1)/nc) -- slices are still added in slice order, so the
-      // result does not depend on who finishes.  All contributors end their
-      // ranges at about the same time (balanced stream-K), and the grid never
-      // exceeds one CTA per SM, so every awaited CTA is resident.  Tiles are
-      // taken two at a time: both arrival counts are awaited first, then
-      // epilogue warps 0-1 finish the first tile and warps 2-3 the second, so
-      // the two latency-bound passes overlap instead of running back to back.
-      StreamK sk{a.n_work, a.kbt, a.total, G};
-      int jj = 0;
-      bool tl_first = true;
-      while (jj < n_units) {
-        // the next one or two work tiles of the range: (tile, contributors, token share)
-        auto next_tile = [&](int& wt, int& nc, int& tb, int& te) {
-          int kb;
-          unit_tile(jj, wt, kb);
-          int seg_end = jj + (a.kbt - kb);
-          if (seg_end > n_units) seg_end = n_units;
-          jj = seg_end;
-          int c0, c1;
-          sk.contributors(wt, c0, c1);
-          nc = c1 - c0 + 1;
-          const int share = cta - c0;
-          tb = (int)((long long)a.T * share / nc);
-          te = (int)((long long)a.T * (share + 1) / nc);
-        };
-        int wt0, nc0, tb0, te0, wt1 = -1, nc1 = 0, tb1 = 0, te1 = 0;
-        next_tile(wt0, nc0, tb0, te0);
-        if (jj < n_units) next_tile(wt1, nc1, tb1, te1);
-        const bool two = wt1 >= 0;
-        if (e == 0) {
-          const unsigned long long t0 = globaltimer();
-          const unsigned long long limit = wait_limit(a.status);
-          for (int i = 0; i < (two ? 2 : 1) && !*abort_flag; ++i) {
-            const int wt = i ? wt1 : wt0, nc = i ? nc1 : nc0;
-            while (*(volatile int*)&a.cnt[wt] < nc) {
-              if (*abort_flag || (*(volatile uint32_t*)a.status & ST_TIMEOUT)) {
-                *abort_flag = 1;
-                break;
-              }
-              if (globaltimer() - t0 > limit) {
-                atomicOr(a.status, ST_TIMEOUT);
-                *abort_flag = 1;
-                break;
-              }
-            }
-          }
-        }
-        if (epi_aborted()) break;
-        if (e == 0 && tl_first) TL_GEMM(5);
-        tl_first = false;
-        __threadfence();
-        const int ew = e >> 5;   // epilogue warp 0..3
-        const bool second = two && ew >= 2;
-        const int nw = two ? 2 : 4, w = two ? (ew & 1) : ew;
-        const int wt = second ? wt1 : wt0, nc = second ? nc1 : nc0, tb = second ? tb1 : tb0, te = second ? te1 : te0;
-        if (tb < te) {
-          const GSrc src{a.part, (size_t)kMaxT * n_part, n_part};
-          if (EPI == EPI_SILU) {
-            finish_silu(a, src, wt, nc, rms, tb, te, w, nw);
-          } else {
-#pragma unroll 1
-            for (int sub = 0; sub < kSub; ++sub) {
-              const int tile = wt * kSub + sub;
-              if (tile >= a.n_tiles) break;
-              if (EPI == EPI_RESID) finish_resid(a, src, tile, nc, tb, te, w, nw);
-              else finish_qkv(a, src, tile, nc, rms, tb, te, w, nw);
-            }
-          }
-        }
-      }
-    }
-    if (ARGMAX && e < a.T) {
+    if (e < a.T) {
       const Top2s r = run[e];
-      a.am_v1[(size_t)cta * kMaxT + e] = r.v1;
-      a.am_i[(size_t)cta * kMaxT + e] = r.i1;
-      a.am_v2[(size_t)cta * kMaxT + e] = r.v2;
+      a.am_v1[(size_t)blockIdx.x * kMaxT + e] = r.v1;
+      a.am_i[(size_t)blockIdx.x * kMaxT + e] = r.i1;
+      a.am_v2[(size_t)blockIdx.x * kMaxT + e] = r.v2;
     }
   }
   tc_fence_before();
@@ -864,8 +898,8 @@ bool encode_bf16_map(CUtensorMap* map, const void* ptr, int rank, const uint64_t
   return r == CUDA_SUCCESS;
 }
 
-bool encode_weight_map(CUtensorMap* map, const void* ptr, int rows, int K) {
-  return encode_2d(map, ptr, rows, K, kTile);
+bool encode_weight_map(CUtensorMap* map, const void* ptr, int rows, int K, int box_rows) {
+  return encode_2d(map, ptr, rows, K, box_rows);
 }
 bool encode_act_map(CUtensorMap* map, const void* ptr, int K, int box_rows) {
   return encode_2d(map, ptr, 2 * kMaxT, K, box_rows);   // hi rows [0, 128), lo rows [128, 256)
@@ -875,11 +909,10 @@ int bn_index(int T) { return T <= 16 ? 0 : T <= 32 ? 1 : T <= 64 ? 2 : 3; }
 
 template <int BN, int EPI>
 static cudaError_t set_smem() {
-  cudaError_t e = cudaFuncSetAttribute(k_gemm_tc<BN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       TcCfg<BN, SubOf<EPI>::v>::SMEM);
-  return e;
+  // the depth of the ring, and so the size, depends on the plan's tile rows:
+  // allow the most any plan takes
+  return cudaFuncSetAttribute(k_gemm_tc<BN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmemMax);
 }
-
 
 template <int BN>
 static cudaError_t set_smem_all() {
@@ -898,54 +931,140 @@ cudaError_t gemm_setup() {
   return e;
 }
 
+// clusters of `c` GEMM CTAs resident at once (one CTA per SM)
+static int gemm_max_clusters(int c) {
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3(c);
+  lc.blockDim = dim3(kGemmThreads);
+  lc.dynamicSmemBytes = kGemmSmemMax;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = c;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  lc.attrs = attr;
+  lc.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, (const void*)k_gemm_tc<64, EPI_RESID>, &lc) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
+}
+
+// Tile rows and k-split of a QKV (rows fixed at one head) or RESID GEMM: of the
+// splits whose clusters fit the GPU, the one whose CTAs move the fewest bytes
+// in sequence, weights and activations (for 64 nodes) together, with a charge
+// per split for the sums it pulls and one per extra wave for a second prologue
+// and epilogue (~8 us at ~80 KB/us).  Not every place the occupancy query
+// counts is free when the clusters arrive (odd sizes leave SM pairs half used,
+// and the previous kernel's CTAs go one by one), and a cluster left over runs
+// after all the others: 46 clusters of 3 took 98 us where 43 take 55, so a
+// margin is kept.
+GemmPlan plan_cluster(int N, int K, bool whole_heads) {
+  GemmPlan best = {};
+  long long best_cost = -1;
+  const int kbt = K / kBK;
+  for (int c = 1; c <= kMaxSplit && c <= kbt; ++c) {
+    int fit = gemm_max_clusters(c);
+    if (c > 1) fit -= (c & 1) ? (fit + 11) / 12 : 1;
+    if (fit < 1) continue;
+    int rows = kTile;
+    if (!whole_heads && N < kTile * fit) rows = ((N + fit - 1) / fit + 7) / 8 * 8;
+    const int n_work = (N + rows - 1) / rows;
+    const long long waves = (n_work + fit - 1) / fit;
+    const long long cost = waves * ((kbt + c - 1) / c) * (rows * 128 + 16384) + (long long)c * 16384 +
+                           (waves - 1) * 640 * 1024;
+    if (best_cost < 0 || cost < best_cost) {
+      best_cost = cost;
+      best = GemmPlan{rows, n_work, kbt, c, n_work * c};
+    }
+  }
+  return best;
+}
+
+// Whole-K tiles of equal rows that fill the SMs in as few rounds as the MMA's
+// 128 rows allow (gate/up: `rows` of each matrix per tile).
+GemmPlan plan_rows(int N, int K, int n_sms) {
+  const int rounds = (N + kTile * n_sms - 1) / (kTile * n_sms);
+  const int rows = ((N + rounds * n_sms - 1) / (rounds * n_sms) + 7) / 8 * 8;
+  const int n_work = (N + rows - 1) / rows;
+  return GemmPlan{rows, n_work, K / kBK, 1, n_work < n_sms ? n_work : n_sms};
+}
+
 template <int BN, int EPI>
-static cudaError_t launch_tc(Model& m, const GemmW& g, const CUtensorMap& amap, int grid, const GemmArgs& a,
-                             cudaStream_t st) {
+static cudaError_t launch_tc(Model& m, const GemmW& g, const CUtensorMap& amap, GemmArgs& a, cudaStream_t st) {
+  using C = TcCfg<BN, EPI>;
+  a.stages = C::stages(g.plan.rows);
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3(g.plan.grid);
+  lc.blockDim = dim3(kGemmThreads);
+  lc.dynamicSmemBytes = (size_t)C::smem(g.plan.rows);
+  lc.stream = st;
+  cudaLaunchAttribute attr[2];
+  int n = 0;
+  if (EpiOf<EPI>::cluster) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = g.plan.split;
+    attr[n].val.clusterDim.y = 1;
+    attr[n].val.clusterDim.z = 1;
+    ++n;
+  }
+  if (m.pdl) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n].val.programmaticStreamSerializationAllowed = 1;
+    ++n;
+  }
+  lc.attrs = attr;
+  lc.numAttrs = n;
   const CUtensorMap& w1 = g.n_seg > 1 ? g.map[1] : g.map[0];
   const CUtensorMap& w2 = g.n_seg > 2 ? g.map[2] : g.map[0];
-  return launch(m.pdl, k_gemm_tc<BN, EPI>, dim3(grid), dim3(192), (size_t)TcCfg<BN, SubOf<EPI>::v>::SMEM, st,
-                g.map[0], w1, w2, amap, a);
+  return cudaLaunchKernelEx(&lc, k_gemm_tc<BN, EPI>, g.map[0], w1, w2, amap, a);
 }
 
 template <int EPI>
-static cudaError_t dispatch_tc(Model& m, const GemmW& g, const CUtensorMap* amaps, int T, int grid, GemmArgs& a,
+static cudaError_t dispatch_tc(Model& m, const GemmW& g, const CUtensorMap* amaps, int T, GemmArgs& a,
                                cudaStream_t st) {
-  const int bi = bn_index(T);
-  switch (bi) {
-    case 0: return launch_tc<16, EPI>(m, g, amaps[0], grid, a, st);
-    case 1: return launch_tc<32, EPI>(m, g, amaps[1], grid, a, st);
-    case 2: return launch_tc<64, EPI>(m, g, amaps[2], grid, a, st);
-    default: return launch_tc<128, EPI>(m, g, amaps[3], grid, a, st);
+  switch (bn_index(T)) {
+    case 0: return launch_tc<16, EPI>(m, g, amaps[0], a, st);
+    case 1: return launch_tc<32, EPI>(m, g, amaps[1], a, st);
+    case 2: return launch_tc<64, EPI>(m, g, amaps[2], a, st);
+    default: return launch_tc<128, EPI>(m, g, amaps[3], a, st);
   }
 }
 
-int* gemm_counters(Model& m, int layer, int kind) { return m.ws.cnt + ((size_t)layer * 4 + kind) * kCntPer; }
-
-static GemmArgs base_args(Model& m, const GemmW& g, int T, int* cnt) {
+static GemmArgs base_args(Model& m, const GemmW& g, int T, int slot) {
   GemmArgs a;
   memset(&a, 0, sizeof(a));
-  for (int s = 0; s < 3; ++s) a.seg_tiles[s] = g.seg_tiles[s < g.n_seg ? s : g.n_seg - 1];
-  a.interleave2 = g.interleave2;
-  a.n_tiles = (g.N + kTile - 1) / kTile;
-  a.n_work = g.plan.n_tiles;
+  a.rows = g.plan.rows;
+  a.n_work = g.plan.n_work;
   a.kbt = g.plan.kbt;
-  a.total = g.plan.total;
+  a.split = g.plan.split;
   a.N = g.N;
   a.T = T;
-  a.part = m.ws.part;
-  a.cnt = cnt;
+  a.tl_slot = slot;
   a.status = m.ws.status;
   a.ss_in = m.ws.ss;
-  a.ss_chunks = (m.cfg.hidden + kTile - 1) / kTile;
   a.inv_dim = 1.0f / (float)m.cfg.hidden;
   a.eps = m.cfg.rms_eps;
   return a;
 }
 
+// number of sum-of-squares chunks the input of layer `layer`'s attention block
+// comes with (layer n_layers: the final norm's): the embedding writes one per
+// 128 features, a down projection one per tile
+int norm_chunks(const Model& m, int layer) {
+  return layer == 0 ? (m.cfg.hidden + kTile - 1) / kTile : m.g_down[layer - 1].plan.n_work;
+}
+
 cudaError_t launch_gemm_qkv(Model& m, int layer, void* kc, void* vc, int T, cudaStream_t st) {
   const auto& c = m.cfg;
   const oos_layer_weights& L = m.layers[layer];
-  GemmArgs a = base_args(m, m.g_qkv[layer], T, gemm_counters(m, layer, 0));
+  GemmArgs a = base_args(m, m.g_qkv[layer], T, layer * 4);
+  a.seg_tiles[0] = c.n_q_heads;
+  a.seg_tiles[1] = c.n_q_heads + c.n_kv_heads;
+  a.seg_tiles[2] = c.n_q_heads + 2 * c.n_kv_heads;
+  a.ss_chunks = norm_chunks(m, layer);
   a.nq = c.n_q_heads;
   a.nkv = c.n_kv_heads;
   a.bq = (const __nv_bfloat16*)(c.qkv_bias ? L.b_q : nullptr);
@@ -959,41 +1078,42 @@ cudaError_t launch_gemm_qkv(Model& m, int layer, void* kc, void* vc, int T, cuda
   a.vc = (__nv_bfloat16*)vc;
   a.ctx = m.ws.ctx;
   a.kv_f16 = c.kv_f16 ? 1 : 0;
-  return dispatch_tc<EPI_QKV>(m, m.g_qkv[layer], m.amap_xn, T, m.g_qkv[layer].plan.grid, a, st);
+  return dispatch_tc<EPI_QKV>(m, m.g_qkv[layer], m.amap_xn, T, a, st);
 }
 
-static cudaError_t launch_resid(Model& m, const GemmW& g, const CUtensorMap* amaps, const void* gain, int* cnt, int T,
+static cudaError_t launch_resid(Model& m, const GemmW& g, const CUtensorMap* amaps, const void* gain, int slot, int T,
                                 cudaStream_t st) {
-  GemmArgs a = base_args(m, g, T, cnt);
+  GemmArgs a = base_args(m, g, T, slot);
   a.x = m.ws.x;
   a.gain = (const __nv_bfloat16*)gain;
   a.y_out = (__nv_bfloat16*)m.ws.xn;
   a.ss_out = m.ws.ss;
-  return dispatch_tc<EPI_RESID>(m, g, amaps, T, g.plan.grid, a, st);
+  return dispatch_tc<EPI_RESID>(m, g, amaps, T, a, st);
 }
 
 cudaError_t launch_gemm_o(Model& m, int layer, int T, cudaStream_t st) {
-  return launch_resid(m, m.g_o[layer], m.amap_attn, m.layers[layer].mlp_norm, gemm_counters(m, layer, 1), T, st);
+  return launch_resid(m, m.g_o[layer], m.amap_attn, m.layers[layer].mlp_norm, layer * 4 + 1, T, st);
 }
 
 cudaError_t launch_gemm_down(Model& m, int layer, int T, cudaStream_t st) {
   const void* gain = layer + 1 < m.cfg.n_layers ? m.layers[layer + 1].attn_norm : m.w.final_norm;
-  return launch_resid(m, m.g_down[layer], m.amap_act, gain, gemm_counters(m, layer, 3), T, st);
+  return launch_resid(m, m.g_down[layer], m.amap_act, gain, layer * 4 + 3, T, st);
 }
 
 cudaError_t launch_gemm_gu(Model& m, int layer, int T, cudaStream_t st) {
-  GemmArgs a = base_args(m, m.g_gu[layer], T, gemm_counters(m, layer, 2));
+  GemmArgs a = base_args(m, m.g_gu[layer], T, layer * 4 + 2);
+  a.ss_chunks = m.g_o[layer].plan.n_work;
   a.act_out = (__nv_bfloat16*)m.ws.act;
-  a.I = m.cfg.intermediate;
-  return dispatch_tc<EPI_SILU>(m, m.g_gu[layer], m.amap_xn, T, m.g_gu[layer].plan.grid, a, st);
+  return dispatch_tc<EPI_SILU>(m, m.g_gu[layer], m.amap_xn, T, a, st);
 }
 
 cudaError_t launch_lm_head_tc(Model& m, int T, cudaStream_t st) {
-  GemmArgs a = base_args(m, m.g_lm, T, nullptr);
+  GemmArgs a = base_args(m, m.g_lm, T, 0);
+  a.ss_chunks = norm_chunks(m, m.cfg.n_layers);
   a.am_v1 = m.ws.lm_v1;
   a.am_i = m.ws.lm_i;
   a.am_v2 = m.ws.lm_v2;
-  return dispatch_tc<EPI_ARGMAX>(m, m.g_lm, m.amap_xn, T, m.lm_grid, a, st);
+  return dispatch_tc<EPI_ARGMAX>(m, m.g_lm, m.amap_xn, T, a, st);
 }
 
 // ------------------------------------------------------------ fp32 CUDA-core path

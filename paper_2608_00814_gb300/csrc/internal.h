@@ -14,57 +14,31 @@ namespace oos {
 
 constexpr int kMaxT = 128;          // largest tree (ancestor sets are 128-bit masks)
 constexpr int kTile = 128;          // weight rows per MMA (tcgen05 M)
-constexpr int kWorkRowsWide = 256;  // weight rows per work tile of the gate/up GEMM and LM head
+constexpr int kLmRows = 256;        // vocabulary rows per work tile of the LM head
 constexpr int kBK = 64;             // reduction elements per pipeline stage (128 bytes of bf16)
 constexpr int kMaxLayers = 128;
-constexpr int kMaxGridCTAs = 1024;  // upper bound on CTAs of a stream-K GEMM / LM head
-constexpr int kMaxSsChunks = 64;    // hidden <= 8192: RMSNorm partial sums per 128 features
-constexpr int kCntPer = 256;        // arrival counters per (layer, GEMM kind): one per work tile
+constexpr int kMaxGridCTAs = 1024;  // upper bound on CTAs of the LM head
+constexpr int kMaxHidden = 8192;    // bf16 models
+constexpr int kMaxInter = 32768;
+constexpr int kMaxHeads = 256;      // q + k + v heads
+constexpr int kMaxSsChunks = 256;   // RMSNorm partial sums per token: one per tile of the producing kernel
 
-// Stream-K partition of a weight GEMM: the (tile, k-block) units of all tiles,
-// tile-major, are cut into `grid` contiguous equal ranges, one per CTA.  CTA c
-// owns units [c*total/grid, (c+1)*total/grid).  Each CTA writes one fp32
-// partial tile per tile it touches, into slice (c - first contributor of the
-// tile); a reduce kernel adds the slices in slice order (deterministic).
-struct StreamK {
-  int n_tiles;
-  int kbt;     // k-blocks per tile
-  int total;   // n_tiles * kbt
-  int grid;    // CTAs
-  __host__ __device__ int cta_of_unit(long long u) const {
-    // largest c with floor(c*total/grid) <= u
-    return (int)(((u + 1) * (long long)grid + total - 1) / total) - 1;
-  }
-  __host__ __device__ void contributors(int tile, int& c0, int& c1) const {
-    c0 = cta_of_unit((long long)tile * kbt);
-    c1 = cta_of_unit((long long)tile * kbt + kbt - 1);
-  }
-  int max_slices() const {
-    int m = 1;
-    for (int t = 0; t < n_tiles; ++t) {
-      int a, b;
-      contributors(t, a, b);
-      m = (b - a + 1) > m ? (b - a + 1) : m;
-    }
-    return m;
-  }
+// Work split of a weight GEMM of the bf16 path (gemm.cu says how it is chosen)
+struct GemmPlan {
+  int rows;     // weight rows per subtile, a multiple of 8
+  int n_work;   // work tiles
+  int kbt;      // k-blocks per tile
+  int split;    // CTAs (a cluster) sharing a tile
+  int grid;     // CTAs
 };
 
-StreamK make_streamk(int n_rows, int K, int n_sms, int tile_rows);
-StreamK make_single_slice(int n_rows);   // one contributor per tile (CUDA-core GEMM)
-
-// One weight GEMM of the bf16 path: up to three row-stacked segments (q|k|v,
-// gate|up), each with its own TMA descriptor.
+// One weight GEMM of the bf16 path: up to three matrices (q|k|v, gate|up), each
+// with its own TMA descriptor.
 struct GemmW {
   CUtensorMap map[3];
-  const void* ptr[3];
-  int seg_tiles[3];   // cumulative tile counts at the end of each segment
   int n_seg;
-  int interleave2;    // gate/up: tiles alternate between the two segments
-  int sub;            // 128-row MMA subtiles per stream-K work tile (1 or 2)
-  int round_robin;    // LM head: whole work tiles dealt round-robin instead of stream-K
-  int N, K;
-  StreamK plan;
+  int N, K;     // output rows (gate/up: of one matrix), reduction length
+  GemmPlan plan;
 };
 
 struct Workspace {
@@ -78,8 +52,7 @@ struct Workspace {
   void* q;                   // [kMaxT][nq][d]
   void* attn;                // attention output [kMaxT][nq*d]
   void* act;                 // SwiGLU activation [kMaxT][I]
-  float* part;               // GEMM partial slices
-  size_t part_floats;
+  float* part;               // GEMM outputs before their epilogue kernel (fp32 path)
   float* lm_v1;              // LM-head partial states [kMaxGridCTAs][kMaxT]
   int32_t* lm_i;
   float* lm_v2;
@@ -87,9 +60,8 @@ struct Workspace {
   int32_t* argmax;           // [kMaxT]
   float* top1;
   float* top2;
-  float* ss;                 // sum of x^2 per 128-feature chunk [kMaxSsChunks][kMaxT] (bf16 path)
+  float* ss;                 // sum of x^2 per feature tile [kMaxSsChunks][kMaxT] (bf16 path)
   float2* rope;              // (cos, sin) per node and rotary pair [kMaxT][d/2] (bf16 path)
-  int* cnt;                  // GEMM arrival counters [layer][4 kinds][kCntPer], zeroed at every step start
   int32_t* chain_parent;     // [kMaxT]: -1, 0, 1, ... (the chains a prefill runs as trees)
   int32_t* pf_scratch;       // prefill's unused accept outputs: len, bonus, nodes[kMaxT], tokens[kMaxT]
 };
@@ -135,8 +107,6 @@ struct Model {
   };
   std::vector<KvMaps> kv_maps;
   int lm_grid;
-  // fp32 path plans (one slice)
-  StreamK p_qkv, p_o, p_gu, p_down;
   // CUDA graph of the last call shape
   cudaStream_t cap_stream = nullptr;
   cudaGraph_t graph = nullptr;          // the graph gexec was instantiated from
@@ -177,10 +147,9 @@ cudaError_t set_tree_prep_ctx(Model& m, cudaGraphExec_t ex, cudaGraphNode_t node
 cudaError_t launch_embed_norm(Model& m, const int32_t* tokens, int T, cudaStream_t st);
 cudaError_t launch_embed_tc(Model& m, const int32_t* tokens, int T, cudaStream_t st);
 cudaError_t launch_final_hidden(Model& m, float* hidden, int T, cudaStream_t st);
-cudaError_t launch_qkv_post(Model& m, int layer, const StreamK& plan, void* kc, void* vc, int T, cudaStream_t st);
-cudaError_t launch_resid_norm(Model& m, const StreamK& plan, const void* gain, float* hidden_out, int T,
-                              cudaStream_t st);
-cudaError_t launch_silu_mul(Model& m, const StreamK& plan, int T, cudaStream_t st);
+cudaError_t launch_qkv_post(Model& m, int layer, void* kc, void* vc, int T, cudaStream_t st);
+cudaError_t launch_resid_norm(Model& m, const void* gain, float* hidden_out, int T, cudaStream_t st);
+cudaError_t launch_silu_mul(Model& m, int T, cudaStream_t st);
 // n_valid: DEVICE count of real nodes (the rest is padding, never accepted), or nullptr for T
 cudaError_t launch_argmax_accept(Model& m, const int32_t* tokens, const int32_t* parent, int T, const int32_t* n_valid,
                                  int n_parts, int32_t* len, int32_t* nodes, int32_t* toks, int32_t* bonus,
@@ -193,13 +162,13 @@ cudaError_t launch_accept_walk(const int32_t* tokens, const int32_t* parent, con
                                cudaStream_t st);
 
 // ---- GEMMs (gemm.cu)
-bool encode_weight_map(CUtensorMap* map, const void* ptr, int rows, int K);
 // 16-bit (bf16, or binary16 when f16) tensor map with 128-byte swizzle: dims[0]
 // contiguous, strides[i] = bytes between consecutive indices of dim i + 1, box[]
 // elements per dim
 bool encode_bf16_map(CUtensorMap* map, const void* ptr, int rank, const uint64_t* dims, const uint64_t* strides,
                      const uint32_t* box, bool f16 = false);
 bool encode_act_map(CUtensorMap* map, const void* ptr, int K, int box_rows);
+bool encode_weight_map(CUtensorMap* map, const void* ptr, int rows, int K, int box_rows);
 int bn_index(int T);   // N-tile variant for T tree nodes: 0..3 -> 16/32/64/128
 cudaError_t gemm_setup();
 cudaError_t launch_gemm_qkv(Model& m, int layer, void* kc, void* vc, int T, cudaStream_t st);
@@ -207,7 +176,9 @@ cudaError_t launch_gemm_o(Model& m, int layer, int T, cudaStream_t st);
 cudaError_t launch_gemm_gu(Model& m, int layer, int T, cudaStream_t st);
 cudaError_t launch_gemm_down(Model& m, int layer, int T, cudaStream_t st);
 cudaError_t launch_lm_head_tc(Model& m, int T, cudaStream_t st);
-int* gemm_counters(Model& m, int layer, int kind);   // kind 0 qkv, 1 o, 2 gate/up, 3 down
+GemmPlan plan_cluster(int N, int K, bool whole_heads);   // after gemm_setup
+GemmPlan plan_rows(int N, int K, int n_sms);
+int norm_chunks(const Model& m, int layer);
 cudaError_t launch_gemm_f32(Model& m, const void* w0, const void* w1, const void* w2, int rows0, int rows1,
                             int rows2, int K, const void* x, int T, cudaStream_t st);
 cudaError_t launch_lm_head_f32(Model& m, int T, cudaStream_t st);

@@ -2,6 +2,7 @@
 // carve-out, TMA descriptors, the per-call launch sequence and CUDA-graph
 // replay.  Every step of the path runs in this library's kernels.
 #include <math.h>
+#include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
 
@@ -16,27 +17,9 @@ namespace oos {
 
 static size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-StreamK make_streamk(int n_rows, int K, int n_sms, int tile_rows) {
-  StreamK p;
-  p.n_tiles = (n_rows + tile_rows - 1) / tile_rows;
-  p.kbt = K / kBK;
-  p.total = p.n_tiles * p.kbt;
-  p.grid = std::min(std::min(n_sms, p.total), kMaxGridCTAs);
-  return p;
-}
-
-StreamK make_single_slice(int n_rows) {
-  StreamK p;
-  p.n_tiles = (n_rows + kTile - 1) / kTile;
-  p.kbt = 1;
-  p.total = p.n_tiles;
-  p.grid = p.n_tiles;
-  return p;
-}
-
 static int lm_grid_for(const oos_model_config& c, int n_sms) {
   if (c.dtype == OOS_DTYPE_BF16)
-    return std::min(std::min(n_sms, (c.vocab + kWorkRowsWide - 1) / kWorkRowsWide), kMaxGridCTAs);
+    return std::min(std::min(n_sms, (c.vocab + kLmRows - 1) / kLmRows), kMaxGridCTAs);
   return std::max(1, std::min(std::min(2 * n_sms, (c.vocab + 15) / 16), kMaxGridCTAs));
 }
 
@@ -63,19 +46,8 @@ size_t carve_workspace(const oos_model_config& c, int n_sms, uint8_t* base, Work
   w.q = take(halves * kMaxT * qd * es);
   w.attn = take(halves * kMaxT * qd * es);
   w.act = take(halves * kMaxT * I * es);
-  size_t pf = 0;
-  const int Nq = (int)(qd + 2 * kvd);
-  if (c.dtype == OOS_DTYPE_BF16) {
-    const int rows[4] = {kTile, kTile, kWorkRowsWide, kTile};
-    const StreamK ps[4] = {make_streamk(Nq, (int)H, n_sms, rows[0]), make_streamk((int)H, (int)qd, n_sms, rows[1]),
-                           make_streamk((int)(2 * I), (int)H, n_sms, rows[2]),
-                           make_streamk((int)H, (int)I, n_sms, rows[3])};
-    for (int i = 0; i < 4; ++i) pf = std::max(pf, (size_t)ps[i].max_slices() * kMaxT * ps[i].n_tiles * rows[i]);
-  } else {
-    pf = (size_t)kMaxT * std::max(std::max((size_t)Nq, H), 2 * I);
-  }
-  w.part_floats = pf;
-  w.part = (float*)take(pf * 4);
+  const size_t Nq = qd + 2 * kvd;
+  w.part = (float*)take(c.dtype == OOS_DTYPE_BF16 ? 0 : (size_t)kMaxT * std::max(std::max(Nq, H), 2 * I) * 4);
   const size_t lm = (size_t)kMaxGridCTAs * kMaxT;
   w.lm_v1 = (float*)take(lm * 4);
   w.lm_i = (int32_t*)take(lm * 4);
@@ -86,7 +58,6 @@ size_t carve_workspace(const oos_model_config& c, int n_sms, uint8_t* base, Work
   w.top2 = (float*)take(kMaxT * 4);
   w.ss = (float*)take((size_t)kMaxSsChunks * kMaxT * 4);
   w.rope = (float2*)take((size_t)kMaxT * (c.head_dim / 2) * 8);
-  w.cnt = (int*)take((size_t)c.n_layers * 4 * kCntPer * 4);
   w.chain_parent = (int32_t*)take(kMaxT * 4);
   w.pf_scratch = (int32_t*)take((2 + 2 * kMaxT) * 4);
   if (ws) *ws = w;
@@ -134,9 +105,7 @@ static bool shape_supported(const oos_model_config* c) {
   if (c->kv_f16 && c->dtype != OOS_DTYPE_BF16) return false;   // FP16 caches: bf16 models only
   if (c->dtype == OOS_DTYPE_BF16) {
     if (c->head_dim != 128 || c->hidden % 128 || c->intermediate % 128) return false;
-    if (c->hidden / 128 > kMaxSsChunks) return false;
-    if (2 * c->intermediate / kWorkRowsWide > kCntPer || (c->n_q_heads + 2 * c->n_kv_heads) > kCntPer ||
-        c->hidden / kTile > kCntPer)
+    if (c->hidden > kMaxHidden || c->intermediate > kMaxInter || c->n_q_heads + 2 * c->n_kv_heads > kMaxHeads)
       return false;
   }
   return true;
@@ -192,15 +161,15 @@ static int enqueue_layers(Model& m, const oos_kv_cache* kv, int ctx, const int32
       OOS_TRY(launch_gemm_down(m, l, T, st));
     } else {
       OOS_TRY(launch_gemm_f32(m, W.w_q, W.w_k, W.w_v, qd, kvd, kvd, c.hidden, m.ws.xn, T, st));
-      OOS_TRY(launch_qkv_post(m, l, m.p_qkv, kv->k[l], kv->v[l], T, st));
+      OOS_TRY(launch_qkv_post(m, l, kv->k[l], kv->v[l], T, st));
       OOS_TRY(launch_attention(m, l, kv->k[l], kv->v[l], kv->capacity, ctx_hint, T, st));
       OOS_TRY(launch_gemm_f32(m, W.w_o, nullptr, nullptr, c.hidden, 0, 0, qd, m.ws.attn, T, st));
-      OOS_TRY(launch_resid_norm(m, m.p_o, W.mlp_norm, nullptr, T, st));
+      OOS_TRY(launch_resid_norm(m, W.mlp_norm, nullptr, T, st));
       OOS_TRY(launch_gemm_f32(m, W.w_gate, W.w_up, nullptr, c.intermediate, c.intermediate, 0, c.hidden, m.ws.xn, T,
                               st));
-      OOS_TRY(launch_silu_mul(m, m.p_gu, T, st));
+      OOS_TRY(launch_silu_mul(m, T, st));
       OOS_TRY(launch_gemm_f32(m, W.w_down, nullptr, nullptr, c.hidden, 0, 0, c.intermediate, m.ws.act, T, st));
-      OOS_TRY(launch_resid_norm(m, m.p_down, next_gain, hid, T, st));
+      OOS_TRY(launch_resid_norm(m, next_gain, hid, T, st));
     }
   }
   return OOS_OK;
@@ -395,27 +364,24 @@ int oos_model_create(const oos_model_config* cfg, const oos_weights* w, void* wo
     const int H = c.hidden, I = c.intermediate, qd = c.n_q_heads * c.head_dim, kvd = c.n_kv_heads * c.head_dim;
     m->lm_grid = lm_grid_for(c, n_sms);
     if (c.dtype == OOS_DTYPE_BF16) {
-      auto mk = [&](GemmW& g, const void* const* ptrs, const int* rows, int nseg, int K, int interleave,
-                    int tile_rows) -> bool {
+      auto mk = [&](GemmW& g, const void* const* ptrs, const int* rows, int nseg, int K, const GemmPlan& plan) -> bool {
         memset(&g, 0, sizeof(g));
-        g.interleave2 = interleave;
-        int tiles = 0, N = 0;
-        for (int s = 0; s < nseg; ++s) {
-          if (!encode_weight_map(&g.map[s], ptrs[s], rows[s], K)) return false;
-          g.ptr[s] = ptrs[s];
-          tiles += (rows[s] + kTile - 1) / kTile;
-          g.seg_tiles[s] = tiles;
-          N += rows[s];
-        }
-        for (int s = nseg; s < 3; ++s) g.seg_tiles[s] = tiles;
+        for (int s = 0; s < nseg; ++s)
+          if (!encode_weight_map(&g.map[s], ptrs[s], rows[s], K, plan.rows)) return false;
         g.n_seg = nseg;
-        g.N = N;
+        g.N = rows[0];
         g.K = K;
-        g.plan = make_streamk(N, K, n_sms, tile_rows);
-        g.sub = tile_rows / kTile;
-        g.round_robin = 0;
-        return true;
+        g.plan = plan;
+        return plan.grid > 0;
       };
+      const GemmPlan p_qkv = plan_cluster(qd + 2 * kvd, H, true), p_o = plan_cluster(H, qd, false);
+      const GemmPlan p_gu = plan_rows(I, H, n_sms), p_down = plan_cluster(H, I, false);
+#ifdef OOS_TIMELINE
+      const GemmPlan* plans[4] = {&p_qkv, &p_o, &p_gu, &p_down};
+      for (int i = 0; i < 4; ++i)
+        fprintf(stderr, "plan %d: %d rows x %d tiles, split %d, %d CTAs\n", i, plans[i]->rows, plans[i]->n_work,
+                plans[i]->split, plans[i]->grid);
+#endif
       bool ok = true;
       m->g_qkv.resize(c.n_layers);
       m->g_o.resize(c.n_layers);
@@ -426,19 +392,16 @@ int oos_model_create(const oos_model_config* cfg, const oos_weights* w, void* wo
         const void* pq[3] = {L.w_q, L.w_k, L.w_v};
         const int rq[3] = {qd, kvd, kvd};
         const void* po[1] = {L.w_o};
-        const int ro[1] = {H};
+        const int rh[1] = {H};
         const void* pg[2] = {L.w_gate, L.w_up};
         const int rg[2] = {I, I};
         const void* pd[1] = {L.w_down};
-        const int rd[1] = {H};
-        ok = mk(m->g_qkv[l], pq, rq, 3, H, 0, kTile) && mk(m->g_o[l], po, ro, 1, qd, 0, kTile) &&
-             mk(m->g_gu[l], pg, rg, 2, H, 1, kWorkRowsWide) && mk(m->g_down[l], pd, rd, 1, I, 0, kTile);
+        ok = mk(m->g_qkv[l], pq, rq, 3, H, p_qkv) && mk(m->g_o[l], po, rh, 1, qd, p_o) &&
+             mk(m->g_gu[l], pg, rg, 2, H, p_gu) && mk(m->g_down[l], pd, rh, 1, I, p_down);
       }
-      const void* pl[1] = {c.vocab ? w->lm_head : nullptr};
+      const void* pl[1] = {w->lm_head};
       const int rl[1] = {c.vocab};
-      ok = ok && mk(m->g_lm, pl, rl, 1, H, 0, kWorkRowsWide);
-      m->g_lm.round_robin = 1;
-      m->g_lm.plan.grid = m->lm_grid;
+      ok = ok && mk(m->g_lm, pl, rl, 1, H, GemmPlan{kTile, (c.vocab + kLmRows - 1) / kLmRows, H / kBK, 1, m->lm_grid});
       const int boxes[4] = {16, 32, 64, 128};
       for (int b = 0; b < 4 && ok; ++b)
         ok = encode_act_map(&m->amap_xn[b], m->ws.xn, H, boxes[b]) &&
@@ -449,11 +412,6 @@ int oos_model_create(const oos_model_config* cfg, const oos_weights* w, void* wo
         rc = OOS_ECUDA;
         break;
       }
-    } else {
-      m->p_qkv = make_single_slice(qd + 2 * kvd);
-      m->p_o = make_single_slice(H);
-      m->p_gu = make_single_slice(2 * I);
-      m->p_down = make_single_slice(H);
     }
     if (c.use_graph && cudaStreamCreateWithFlags(&m->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
       rc = OOS_ECUDA;
@@ -541,18 +499,9 @@ int oos_launch_stage(oos_model* m, int32_t layer, int32_t stage, int32_t T, void
   if (c.dtype == OOS_DTYPE_BF16) {
     switch (stage) {
       case OOS_STAGE_QKV: return OOS_EINVAL;   // its epilogue writes the KV cache
-      case OOS_STAGE_O:
-      case OOS_STAGE_GATE_UP:
-      case OOS_STAGE_DOWN: {
-        // a lone GEMM: its arrival counters start from zero as in a verify step
-        const int kind = stage == OOS_STAGE_O ? 1 : stage == OOS_STAGE_GATE_UP ? 2 : 3;
-        e = cudaMemsetAsync(gemm_counters(*m, layer, kind), 0, kCntPer * sizeof(int), st);
-        if (e != cudaSuccess) break;
-        e = stage == OOS_STAGE_O ? launch_gemm_o(*m, layer, T, st)
-            : stage == OOS_STAGE_GATE_UP ? launch_gemm_gu(*m, layer, T, st)
-                                         : launch_gemm_down(*m, layer, T, st);
-        break;
-      }
+      case OOS_STAGE_O: e = launch_gemm_o(*m, layer, T, st); break;
+      case OOS_STAGE_GATE_UP: e = launch_gemm_gu(*m, layer, T, st); break;
+      case OOS_STAGE_DOWN: e = launch_gemm_down(*m, layer, T, st); break;
       default: e = launch_lm_head_tc(*m, T, st); break;
     }
   } else {

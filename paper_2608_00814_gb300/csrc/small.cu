@@ -133,10 +133,6 @@ __global__ void __launch_bounds__(256) k_embed_norm(const int32_t* __restrict__ 
 
 cudaError_t launch_embed_norm(Model& m, const int32_t* tokens, int T, cudaStream_t st) {
   const auto& c = m.cfg;
-  if (c.dtype == OOS_DTYPE_BF16)
-    return launch(m.pdl, k_embed_norm<__nv_bfloat16>, dim3(T), dim3(256), 0, st, tokens,
-                  (const __nv_bfloat16*)m.w.embed, (const __nv_bfloat16*)m.layers[0].attn_norm, c.hidden,
-                  c.vocab, c.rms_eps, m.ws.x, (__nv_bfloat16*)m.ws.xn);
   return launch(m.pdl, k_embed_norm<float>, dim3(T), dim3(256), 0, st, tokens, (const float*)m.w.embed,
                 (const float*)m.layers[0].attn_norm, c.hidden, c.vocab, c.rms_eps, m.ws.x, (float*)m.ws.xn);
 }
@@ -153,15 +149,11 @@ __global__ void __launch_bounds__(128) k_embed_tc(const int32_t* __restrict__ to
                                                   float* __restrict__ x, __nv_bfloat16* __restrict__ y,
                                                   float* __restrict__ ss, const int32_t* __restrict__ pos,
                                                   const double* __restrict__ inv_freq, int half_d,
-                                                  float2* __restrict__ rope, int* __restrict__ cnt, int n_cnt) {
+                                                  float2* __restrict__ rope) {
   __shared__ float red[32];
   pdl_wait();
   pdl_trigger();
   const int t = blockIdx.x, f = blockIdx.y * 128 + threadIdx.x;
-  {   // the step's GEMM arrival counters start from zero
-    const int nb = gridDim.x * gridDim.y, b = blockIdx.y * gridDim.x + blockIdx.x;
-    for (int i = b * blockDim.x + threadIdx.x; i < n_cnt; i += nb * blockDim.x) cnt[i] = 0;
-  }
   if (blockIdx.y == 0 && threadIdx.x < half_d) {
     const double two_pi = 6.283185307179586476925286766559;
     const double ang = (double)pos[t] * inv_freq[threadIdx.x];
@@ -186,7 +178,7 @@ cudaError_t launch_embed_tc(Model& m, const int32_t* tokens, int T, cudaStream_t
   return launch(m.pdl, k_embed_tc, dim3(T, (c.hidden + 127) / 128), dim3(128), 0, st, tokens,
                 (const __nv_bfloat16*)m.w.embed, (const __nv_bfloat16*)m.layers[0].attn_norm, c.hidden, c.vocab,
                 m.ws.x, (__nv_bfloat16*)m.ws.xn, m.ws.ss, (const int32_t*)m.ws.pos, (const double*)m.ws.inv_freq,
-                c.head_dim / 2, m.ws.rope, m.ws.cnt, c.n_layers * 4 * kCntPer);
+                c.head_dim / 2, m.ws.rope);
 }
 
 // bf16 path, checking output only: the final RMSNorm output in fp32,
@@ -207,17 +199,7 @@ __global__ void __launch_bounds__(256) k_final_hidden(const float* __restrict__ 
 cudaError_t launch_final_hidden(Model& m, float* hidden, int T, cudaStream_t st) {
   const auto& c = m.cfg;
   return launch(m.pdl, k_final_hidden, dim3(T), dim3(256), 0, st, (const float*)m.ws.x, (const float*)m.ws.ss,
-                (c.hidden + 127) / 128, (const __nv_bfloat16*)m.w.final_norm, c.hidden, c.rms_eps, hidden);
-}
-
-// sum of the fp32 partial slices of GEMM output (t, f)
-OOS_DEV float gather_partial(const float* __restrict__ part, const StreamK& plan, int N, int t, int f) {
-  int c0, c1;
-  plan.contributors(f / kTile, c0, c1);
-  float v = 0.f;
-  const size_t slice = (size_t)kMaxT * N;
-  for (int s = 0; s <= c1 - c0; ++s) v += part[s * slice + (size_t)t * N + f];
-  return v;
+                norm_chunks(m, c.n_layers), (const __nv_bfloat16*)m.w.final_norm, c.hidden, c.rms_eps, hidden);
 }
 
 // ============================================================ q/k/v epilogue
@@ -226,7 +208,6 @@ OOS_DEV float gather_partial(const float* __restrict__ part, const StreamK& plan
 // pos[t]; q goes to the query buffer, k and v to cache slot ctx + t.
 struct QkvPostArgs {
   const float* part;
-  StreamK plan;
   int N, nq, nkv, d;
   const void* bq;
   const void* bk;
@@ -249,8 +230,8 @@ __global__ void k_qkv_post(QkvPostArgs a) {
   pdl_trigger();
   const int t = blockIdx.x, hs = blockIdx.y, j = threadIdx.x, half = a.d / 2;
   const int f0 = hs * a.d + j, f1 = f0 + half;
-  float v0 = gather_partial(a.part, a.plan, a.N, t, f0);
-  float v1 = gather_partial(a.part, a.plan, a.N, t, f1);
+  float v0 = a.part[(size_t)t * a.N + f0];
+  float v1 = a.part[(size_t)t * a.N + f1];
   int kind, h;  // 0 = q, 1 = k, 2 = v
   if (hs < a.nq) { kind = 0; h = hs; }
   else if (hs < a.nq + a.nkv) { kind = 1; h = hs - a.nq; }
@@ -286,12 +267,11 @@ __global__ void k_qkv_post(QkvPostArgs a) {
   dst[j + half] = from_f32<E>(v1);
 }
 
-cudaError_t launch_qkv_post(Model& m, int layer, const StreamK& plan, void* kc, void* vc, int T, cudaStream_t st) {
+cudaError_t launch_qkv_post(Model& m, int layer, void* kc, void* vc, int T, cudaStream_t st) {
   const auto& c = m.cfg;
   const auto& L = m.layers[layer];
   QkvPostArgs a;
   a.part = m.ws.part;
-  a.plan = plan;
   a.nq = c.n_q_heads;
   a.nkv = c.n_kv_heads;
   a.d = c.head_dim;
@@ -309,7 +289,6 @@ cudaError_t launch_qkv_post(Model& m, int layer, const StreamK& plan, void* kc, 
   a.vc = vc;
   a.ctx = m.ws.ctx;
   dim3 grid(T, c.n_q_heads + 2 * c.n_kv_heads);
-  if (c.dtype == OOS_DTYPE_BF16) return launch(m.pdl, k_qkv_post<__nv_bfloat16>, grid, dim3(c.head_dim / 2), 0, st, a);
   return launch(m.pdl, k_qkv_post<float>, grid, dim3(c.head_dim / 2), 0, st, a);
 }
 
@@ -318,7 +297,7 @@ cudaError_t launch_qkv_post(Model& m, int layer, const StreamK& plan, void* kc, 
 // xn[t] = RMSNorm(x[t]) * gain (input of the next GEMM).  For the final norm
 // the fp32 normalised row is also written to hidden_out (when given).
 template <typename E>
-__global__ void __launch_bounds__(256) k_resid_norm(const float* __restrict__ part, StreamK plan, int H,
+__global__ void __launch_bounds__(256) k_resid_norm(const float* __restrict__ part, int H,
                                                     const E* __restrict__ gain, float eps, float* __restrict__ x,
                                                     E* __restrict__ xn, float* __restrict__ hidden_out) {
   __shared__ float red[32];
@@ -328,7 +307,7 @@ __global__ void __launch_bounds__(256) k_resid_norm(const float* __restrict__ pa
   float* xr = x + (size_t)t * H;
   float ss = 0.f;
   for (int f = threadIdx.x; f < H; f += blockDim.x) {
-    const float v = xr[f] + gather_partial(part, plan, H, t, f);
+    const float v = xr[f] + part[(size_t)t * H + f];
     xr[f] = v;
     ss += v * v;
   }
@@ -341,39 +320,32 @@ __global__ void __launch_bounds__(256) k_resid_norm(const float* __restrict__ pa
   }
 }
 
-cudaError_t launch_resid_norm(Model& m, const StreamK& plan, const void* gain, float* hidden_out, int T,
-                              cudaStream_t st) {
+cudaError_t launch_resid_norm(Model& m, const void* gain, float* hidden_out, int T, cudaStream_t st) {
   const auto& c = m.cfg;
-  if (c.dtype == OOS_DTYPE_BF16)
-    return launch(m.pdl, k_resid_norm<__nv_bfloat16>, dim3(T), dim3(256), 0, st, (const float*)m.ws.part, plan,
-                  c.hidden, (const __nv_bfloat16*)gain, c.rms_eps, m.ws.x, (__nv_bfloat16*)m.ws.xn, hidden_out);
-  return launch(m.pdl, k_resid_norm<float>, dim3(T), dim3(256), 0, st, (const float*)m.ws.part, plan, c.hidden,
+  return launch(m.pdl, k_resid_norm<float>, dim3(T), dim3(256), 0, st, (const float*)m.ws.part, c.hidden,
                 (const float*)gain, c.rms_eps, m.ws.x, (float*)m.ws.xn, hidden_out);
 }
 
 // ============================================================ SwiGLU
 // act[t][i] = silu(gate) * up, gate/up = rows i and I + i of the stacked GEMM.
 template <typename E>
-__global__ void __launch_bounds__(256) k_silu_mul(const float* __restrict__ part, StreamK plan, int I,
+__global__ void __launch_bounds__(256) k_silu_mul(const float* __restrict__ part, int I,
                                                   E* __restrict__ act) {
   pdl_wait();
   pdl_trigger();
   const int t = blockIdx.y;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < I) {
-    const float g = gather_partial(part, plan, 2 * I, t, i);
-    const float u = gather_partial(part, plan, 2 * I, t, I + i);
+    const float g = part[(size_t)t * 2 * I + i];
+    const float u = part[(size_t)t * 2 * I + I + i];
     store_act(act, (size_t)t * I + i, (size_t)kMaxT * I, g / (1.f + expf(-g)) * u);
   }
 }
 
-cudaError_t launch_silu_mul(Model& m, const StreamK& plan, int T, cudaStream_t st) {
+cudaError_t launch_silu_mul(Model& m, int T, cudaStream_t st) {
   const auto& c = m.cfg;
   dim3 grid((c.intermediate + 255) / 256, T);
-  if (c.dtype == OOS_DTYPE_BF16)
-    return launch(m.pdl, k_silu_mul<__nv_bfloat16>, grid, dim3(256), 0, st, (const float*)m.ws.part, plan,
-                  c.intermediate, (__nv_bfloat16*)m.ws.act);
-  return launch(m.pdl, k_silu_mul<float>, grid, dim3(256), 0, st, (const float*)m.ws.part, plan, c.intermediate,
+  return launch(m.pdl, k_silu_mul<float>, grid, dim3(256), 0, st, (const float*)m.ws.part, c.intermediate,
                 (float*)m.ws.act);
 }
 

@@ -8,8 +8,9 @@ stamps).
 
 Printed per GEMM kind (q/k/v, O, gate/up, down), averaged over the layers:
   main     first CTA entry -> the last CTA's last accumulator ready
-  tail     last accumulator ready -> last CTA exit, split into publish (-> the
-           last arrival count), poll (-> the last finisher released) and
+  tail     last accumulator ready -> last CTA exit; for the GEMMs whose tiles
+           are shared by a cluster split into stage (-> the last CTA's sums in
+           shared memory), barrier (-> the last cluster barrier passed) and
            finish (-> the last exit)
 and per layer the time from one kernel's last exit to the next one's
 (attention included), then the attention's phases (median over its blocks,
@@ -93,11 +94,10 @@ def main():
     for n, (start, b) in enumerate(launches):
         kind = kinds[n % 4]
         main_end = b[:, 2].max()
-        publish = b[:, 4].max()
-        pol = b[:, 5][b[:, 5] > 0]
-        released = pol.max() if len(pol) else publish
+        staged = max(b[:, 4].max(), main_end)     # 0 where a kernel has no such event
+        released = max(b[:, 5].max(), staged)
         exit_ = b[:, 3].max()
-        agg[kind].append(((main_end - start), (exit_ - main_end), (publish - main_end), (released - publish),
+        agg[kind].append(((main_end - start), (exit_ - main_end), (staged - main_end), (released - staged),
                           (exit_ - released)))
         if prev_exit is not None:
             gaps[kind].append(exit_ - prev_exit)
@@ -109,7 +109,7 @@ def main():
     for k in kinds:
         x = np.array(agg[k]) / 1e3
         gp = np.array(gaps[k]) / 1e3 if gaps[k] else np.zeros(1)
-        print("  %-8s main %6.2f  tail %6.2f [publish %5.2f  poll %5.2f  finish %5.2f]  previous exit -> exit %6.2f"
+        print("  %-8s main %6.2f  tail %6.2f [stage %5.2f  barrier %5.2f  finish %5.2f]  previous exit -> exit %6.2f"
               % (k, x[:, 0].mean(), x[:, 1].mean(), x[:, 2].mean(), x[:, 3].mean(), x[:, 4].mean(), gp.mean()))
     print("  (the O row's 'previous exit -> exit' includes the attention)")
 
