@@ -14,6 +14,7 @@ namespace oos {
 
 constexpr int kStaticBlocks = 512;   // vocabulary blocks per call (grid size)
 constexpr int kStaticMaxT = 128;     // rows of `hidden` per call
+constexpr int kStaticThreads = 256;
 
 struct StaticTop2 {
   float v1;
@@ -45,35 +46,147 @@ OOS_DEV StaticTop2 st_merge(StaticTop2 a, StaticTop2 b) {
   return r;
 }
 
-// Block b scans vocabulary rows [b*rows, (b+1)*rows): warp w takes rows
-// w, w+4, ..., lanes stride over the hidden dimension; every row's logit for
-// each of the T hidden rows updates that warp's running top-2.  The last block
-// to finish merges all blocks' states, in block order.
+// A task is `R` vocabulary rows by `TT` hidden rows, one warp.  The lanes split
+// the hidden dimension (VEC consecutive elements each in turn), so that every
+// logit is 32 short fp32 chains added as a tree; the R x TT products of the
+// loaded elements are formed in registers.
+//
+// What bounds it is FMA issue from about 8 hidden rows on, below that the weight
+// stream: per VEC elements a lane loads R + 2 TT 16-byte words for R * TT * VEC
+// FMAs.  R = 8 (bf16) or 4 (fp32) and TT <= 8 keep the sums and the loaded weights
+// in registers.  The warps of a block take the token groups of a row group side by side, so a row group
+// comes from HBM once and from L1 after that.
 template <typename E>
-__global__ void __launch_bounds__(128) k_lm_argmax_static(const E* __restrict__ W, int V, int H, int rows_per_block,
-                                                          const float* __restrict__ hidden, int T, StaticScratch* sc,
-                                                          int32_t* out_argmax, float* out_top1, float* out_top2) {
-  __shared__ StaticTop2 st[4][kStaticMaxT];
+struct StaticRows {
+  static constexpr int v = sizeof(E) == 2 ? 8 : 4;
+};
+// blocks an SM holds: from 6 tokens a task the sums and unpacked weights want
+// more than 128 registers
+constexpr int static_blocks_per_sm(int tt) { return tt >= 6 ? 1 : 2; }
+
+template <typename E, int VEC>
+struct StaticVec;   // VEC consecutive weights as loaded, and as floats
+template <>
+struct StaticVec<__nv_bfloat16, 8> {
+  uint4 u;
+  OOS_DEV void load(const __nv_bfloat16* p) { u = __ldg(reinterpret_cast<const uint4*>(p)); }
+  OOS_DEV float get(int i) const {
+    const uint32_t w = i < 2 ? u.x : i < 4 ? u.y : i < 6 ? u.z : u.w;
+    return __uint_as_float((i & 1) ? (w & 0xffff0000u) : (w << 16));
+  }
+};
+template <>
+struct StaticVec<float, 8> {
+  float4 a, b;
+  OOS_DEV void load(const float* p) {
+    a = __ldg(reinterpret_cast<const float4*>(p));
+    b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+  }
+  OOS_DEV float get(int i) const {
+    const float4 v = i < 4 ? a : b;
+    return (i & 3) == 0 ? v.x : (i & 3) == 1 ? v.y : (i & 3) == 2 ? v.z : v.w;
+  }
+};
+template <typename E>
+struct StaticVec<E, 1> {
+  float v;
+  OOS_DEV void load(const E* p) { v = to_f32(*p); }
+  OOS_DEV float get(int) const { return v; }
+};
+
+// Sums of v[0..N) over the warp.  At each step a lane keeps the half of the
+// values its lane bit selects, so N values cost about 2N shuffles, not 5N; on
+// return v[0..n) hold the sums of elements base..base+n-1.
+template <int N>
+OOS_DEV void warp_sums(float (&v)[N], int& base, int& n) {
+  const int lane = threadIdx.x & 31;
+  base = 0;
+  n = N;
+  int len = N;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    if (len % 2 == 0) {
+      const int h = len / 2;
+      const bool up = lane & o;
+#pragma unroll
+      for (int i = 0; i < N / 2; ++i) {
+        if (i < h) {
+          const float send = up ? v[i] : v[i + h], keep = up ? v[i + h] : v[i];
+          v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+      }
+      if (up) base += h;
+      len = h;
+    } else {
+#pragma unroll
+      for (int i = 0; i < N; ++i)
+        if (i < len) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+    }
+  }
+  n = len;
+}
+
+// Block b scans vocabulary rows [b*rows, (b+1)*rows) in tasks (row group, token
+// group), one warp each; every logit updates that warp's running top-2.  The
+// last block to finish merges all blocks' states, in block order.
+template <typename E, int TT, int VEC>
+__global__ void __launch_bounds__(kStaticThreads, static_blocks_per_sm(TT))
+    k_lm_argmax_static(const E* __restrict__ W, int V, int H, int rows_per_block, const float* __restrict__ hidden, int T,
+                       StaticScratch* sc, int32_t* out_argmax, float* out_top1, float* out_top2) {
+  constexpr int R = StaticRows<E>::v, WARPS = kStaticThreads / 32;
+  __shared__ StaticTop2 st[WARPS][kStaticMaxT];
+  __shared__ float lg[WARPS][R * TT];
   __shared__ int s_last;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int t = lane; t < T; t += 32) st[warp][t] = StaticTop2{-INFINITY, 0x7fffffff, -INFINITY};
-  __syncwarp();   // lane 0 below reads states the other lanes initialised
+  __syncwarp();
   const int r_begin = blockIdx.x * rows_per_block;
   const int r_end = min(V, r_begin + rows_per_block);
-  for (int r = r_begin + warp; r < r_end; r += 4) {
-    const E* w = W + (size_t)r * H;
-    for (int t = 0; t < T; ++t) {
-      const float* h = hidden + (size_t)t * H;
-      float acc = 0.f;
-      for (int k = lane; k < H; k += 32) acc += to_f32(w[k]) * h[k];
-      acc = warp_sum(acc);
-      if (lane == 0) st[warp][t] = st_merge(st[warp][t], StaticTop2{acc, r, -INFINITY});
+  const int groups = (T + TT - 1) / TT;
+  const int tasks = r_begin < r_end ? (r_end - r_begin + R - 1) / R * groups : 0;
+  const int chunks = H / VEC;
+  for (int task = warp; task < tasks; task += WARPS) {
+    const int r0 = r_begin + task / groups * R, t0 = task % groups * TT;
+    float acc[R * TT];
+#pragma unroll
+    for (int i = 0; i < R * TT; ++i) acc[i] = 0.f;
+    const E* w0 = W + (size_t)r0 * H;
+    const float* h0 = hidden + (size_t)t0 * H;
+    const int nr = min(R, r_end - r0), nt = min(TT, T - t0);   // rows past the end repeat the last one
+    // element offsets from the group's first rows: 32 bits, and kept as indexes,
+    // so that they do not take the registers of R + TT pointers
+#pragma unroll 1
+    for (int c = lane; c < chunks; c += 32) {
+      StaticVec<E, VEC> w[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) w[r].load(w0 + ((uint32_t)min(r, nr - 1) * (uint32_t)H + (uint32_t)(c * VEC)));
+#pragma unroll
+      for (int t = 0; t < TT; ++t) {
+        StaticVec<float, VEC> h;
+        h.load(h0 + ((uint32_t)min(t, nt - 1) * (uint32_t)H + (uint32_t)(c * VEC)));
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+          for (int i = 0; i < VEC; ++i) acc[r * TT + t] = fmaf(w[r].get(i), h.get(i), acc[r * TT + t]);
+      }
     }
+    int base, n;
+    warp_sums(acc, base, n);
+#pragma unroll
+    for (int i = 0; i < R * TT; ++i)
+      if (i < n) lg[warp][base + i] = acc[i];
+    __syncwarp();
+    if (lane < nt) {
+      StaticTop2 s = st[warp][t0 + lane];
+      for (int r = 0; r < nr; ++r) s = st_merge(s, StaticTop2{lg[warp][r * TT + lane], r0 + r, -INFINITY});
+      st[warp][t0 + lane] = s;
+    }
+    __syncwarp();
   }
   __syncthreads();
   for (int t = threadIdx.x; t < T; t += blockDim.x) {
     StaticTop2 r = st[0][t];
-    for (int w = 1; w < 4; ++w) r = st_merge(r, st[w][t]);
+    for (int w = 1; w < WARPS; ++w) r = st_merge(r, st[w][t]);
     sc->part[blockIdx.x][t] = r;
   }
   __threadfence();
@@ -121,6 +234,51 @@ static StaticScratch* scratch_for_current_device(cudaStream_t st) {
   return g_scratch_ptr[dev];
 }
 
+struct StaticCall {
+  const void* w;
+  int V, H;
+  const float* hidden;
+  int T;
+  StaticScratch* sc;
+  int32_t* argmax;
+  float *top1, *top2;
+  cudaStream_t st;
+};
+
+template <typename E, int TT, int VEC>
+static bool launch_static_tt(const StaticCall& c) {
+  // one wave; a block's rows are whole row groups
+  constexpr int R = StaticRows<E>::v;
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return false;
+  const int fit = static_blocks_per_sm(TT) * sms;
+  const int most = fit < kStaticBlocks ? fit : kStaticBlocks;
+  const int groups = c.V / R + (c.V % R != 0);
+  const int rows = (groups + most - 1) / most * R;
+  const int blocks = c.V / rows + (c.V % rows != 0);
+  k_lm_argmax_static<E, TT, VEC><<<blocks, kStaticThreads, 0, c.st>>>((const E*)c.w, c.V, c.H, rows, c.hidden, c.T, c.sc,
+                                                                     c.argmax, c.top1, c.top2);
+  return cudaGetLastError() == cudaSuccess;
+}
+
+template <typename E>
+static bool launch_static(const StaticCall& c) {
+  // 16-byte loads where every row of both matrices starts on a 16-byte
+  // boundary; any other shape or address goes element by element.  (Offsets
+  // within a row group are 32-bit: 8 rows of up to 2^29 elements.)
+  if (c.H % 8 == 0 && (((uintptr_t)c.w | (uintptr_t)c.hidden) & 15) == 0) {
+    const int groups = (c.T + 7) / 8, tt = (c.T + groups - 1) / groups;   // the fewest groups, evenly filled
+    if (tt <= 1) return launch_static_tt<E, 1, 8>(c);
+    if (tt <= 2) return launch_static_tt<E, 2, 8>(c);
+    if (tt <= 4) return launch_static_tt<E, 4, 8>(c);
+    if (tt <= 6) return launch_static_tt<E, 6, 8>(c);
+    return launch_static_tt<E, 8, 8>(c);
+  }
+  return launch_static_tt<E, 8, 1>(c);
+}
+
 }  // namespace oos
 
 using namespace oos;
@@ -135,13 +293,7 @@ extern "C" int oos_lm_head_argmax_static(int32_t dtype, int32_t vocab, int32_t h
   cudaStream_t st = (cudaStream_t)stream;
   StaticScratch* sc = scratch_for_current_device(st);
   if (!sc) return OOS_ECUDA;
-  const int blocks = vocab < kStaticBlocks ? vocab : kStaticBlocks;
-  const int rows = (vocab + blocks - 1) / blocks;
-  if (dtype == OOS_DTYPE_BF16)
-    k_lm_argmax_static<__nv_bfloat16><<<blocks, 128, 0, st>>>((const __nv_bfloat16*)lm_head, vocab, hidden_dim, rows,
-                                                             hidden, T, sc, out_argmax, out_top1, out_top2);
-  else
-    k_lm_argmax_static<float><<<blocks, 128, 0, st>>>((const float*)lm_head, vocab, hidden_dim, rows, hidden, T, sc,
-                                                      out_argmax, out_top1, out_top2);
-  return cudaGetLastError() == cudaSuccess ? OOS_OK : OOS_ECUDA;
+  StaticCall c{lm_head, vocab, hidden_dim, hidden, T, sc, out_argmax, out_top1, out_top2, st};
+  if (dtype == OOS_DTYPE_BF16) return launch_static<__nv_bfloat16>(c) ? OOS_OK : OOS_ECUDA;
+  return launch_static<float>(c) ? OOS_OK : OOS_ECUDA;
 }

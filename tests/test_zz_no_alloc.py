@@ -67,3 +67,32 @@ def test_static_argmax_rejects_oversized_T():
     with pytest.raises(B.OosError) as e:
         B.oos_lm_head_argmax_static(B.OOS_DTYPE_F32, 16, 4, x, x, 129, i, x, x)
     assert e.value.code == B.OOS_EINVAL
+
+
+@pytest.mark.parametrize("vocab,hidden,T,bf16,shift", [
+    (1, 8, 1, True, 0), (700, 1000, 3, True, 0), (701, 1000, 17, True, 0),   # row groups cut by the matrix end
+    (300, 24, 128, True, 0), (301, 24, 128, False, 0),                       # every token group size in use
+    (500, 1001, 9, True, 0), (500, 64, 9, True, 1), (333, 64, 33, False, 1),  # no 16-byte rows: element by element
+])
+def test_static_argmax_shapes(vocab, hidden, T, bf16, shift):
+    """Sizes at the edges of the kernel's row and token groups, and rows that
+    16-byte loads cannot read, against fp64 products of the same numbers."""
+    g = torch.Generator().manual_seed(vocab + T)
+    dt = torch.bfloat16 if bf16 else torch.float32
+    w = torch.randn(vocab * hidden + shift, generator=g).to(dt).cuda()[shift:].view(vocab, hidden)
+    h = torch.randn(T * hidden + shift, generator=g).cuda()[shift:].view(T, hidden)
+    arg = torch.full((T,), -7, dtype=torch.int32, device="cuda")
+    t1, t2 = torch.zeros(T, device="cuda"), torch.zeros(T, device="cuda")
+    B.oos_lm_head_argmax_static(B.OOS_DTYPE_BF16 if bf16 else B.OOS_DTYPE_F32, vocab, hidden, w, h, T, arg, t1, t2)
+    lg = h.cpu().double() @ w.cpu().double().T
+    top = lg.topk(min(2, vocab), -1)
+    # fp32 products and sums: 2^-24 a step over chains of hidden/32 and a tree, on
+    # sums of size sqrt(hidden)
+    tol = 2.0 ** -24 * (hidden / 32 + 16) * hidden ** 0.5 * 4
+    assert (t1.cpu().double() - top.values[:, 0]).abs().max() <= tol
+    if vocab > 1:
+        assert (t2.cpu().double() - top.values[:, 1]).abs().max() <= tol
+        sure = top.values[:, 0] - top.values[:, 1] > 2 * tol
+        assert torch.equal(arg.cpu()[sure], top.indices[:, 0][sure].int())
+    else:
+        assert int(arg[0]) == 0 and torch.isinf(t2).all()
