@@ -10,15 +10,17 @@
 // bank order, cut at the lane depth or before an EOS; a lane counts towards
 // the budget only when it creates a node.
 //
-// k_hint_match: for every bank position the longest n whose suffix ends
-// there (0 when nothing, or EOS, follows), as one byte; a warp per 256-position
-// chunk, 8 positions per lane; the maximum of each chunk and of each run of 256
-// chunks (a "span") is kept too, and the warp maxima give the n of the call.  k_hint_pack: one block descends the two summaries in bank order --
-// spans, then their chunks, then positions, 256 at a time, each level's hits
-// gathered in order by warp ballots -- so only spans and chunks that hold an
-// occurrence are read, and warp 0 inserts each lane into the tree held in
-// shared memory: a lane token looks for an existing child with one ballot over
-// the nodes.
+// k_hint_match: for every bank position the longest n whose suffix ends there (0
+// when nothing, or EOS, follows); a warp per 256-position chunk.  What it cannot
+// do without is reading the bank once, so it compares every token with y's last
+// one and looks at a position's neighbours only where that matches; the match
+// lengths (one byte each) are written only for chunks that hold one, the chunk
+// maximum always.
+// k_hint_pack: one block finds the chunks that hold an occurrence, in bank
+// order -- from the chunk maxima themselves in a bank of up to kHintFlat chunks,
+// through maxima of 256-chunk spans in a larger one -- gathers the occurrences of
+// eight chunks at a time and loads eight lanes at a time, one per warp; warp 0
+// inserts them into the tree held in shared memory.
 #include <stdint.h>
 
 #include "common.cuh"
@@ -27,15 +29,19 @@
 namespace oos {
 
 constexpr int kHintMaxN = 7;        // longest suffix tried
-constexpr int kHintThreads = 256;   // threads of both kernels
+constexpr int kHintThreads = 256;   // threads of both kernels, positions of a chunk, chunks of a span
+constexpr int kHintWarps = kHintThreads / 32;
+// Chunks whose maxima the packing block reads in one load of 16 bytes a thread.
+// Up to there (1 Mi tokens) the span maxima, the atomics that build them and the
+// copy that zeroes them are left out: three launches become two.
+constexpr int kHintFlat = kHintThreads * 16;
+constexpr int kHintUnroll = 4;      // chunks a warp has in flight
 
 // prefix_len_dev: the prefix length in device memory (the decode loop's
-// committed length), or nullptr to use prefix_len.  Each warp takes one
-// 256-position chunk at a time (grid-stride over chunks), each lane 8
-// consecutive positions: the lane reads bank[p0 - 8, p0 + 16) (vector loads
-// when the bank is 16-byte aligned), computes the 8 match lengths, stores
-// them as 8 bytes, and the chunk maximum is a warp reduction -- no block
-// barrier.  vec: the bank address is 16-byte aligned.
+// committed length), or nullptr to use prefix_len.  Lane l of a chunk's warp holds
+// positions 4l .. 4l+3 of both 128-position halves, so that a 16-byte load of the
+// warp is one contiguous run.  vec: the bank address is 16-byte aligned.
+// smax, best: nullptr in a bank of up to kHintFlat chunks.
 __global__ void __launch_bounds__(kHintThreads) k_hint_match(const int32_t* __restrict__ bank, int N, int eos,
                                                              const int32_t* __restrict__ prefix, int prefix_len,
                                                              const int32_t* __restrict__ prefix_len_dev, int vec,
@@ -49,64 +55,81 @@ __global__ void __launch_bounds__(kHintThreads) k_hint_match(const int32_t* __re
   // suf[j] is the token j places before y's last token
   if (threadIdx.x < nmax) suf[threadIdx.x] = prefix[prefix_len - 1 - threadIdx.x];
   __syncthreads();
-  int sfx[kHintMaxN];
-#pragma unroll
-  for (int j = 0; j < kHintMaxN; ++j) sfx[j] = j < nmax ? suf[j] : 0;
+  const int last = suf[0];
   const int lane = threadIdx.x & 31;
   const long long n_chunks = ((long long)N + kHintThreads - 1) / kHintThreads;
-  const long long n_warps = (long long)gridDim.x * (kHintThreads / 32);
+  const long long n_warps = (long long)gridDim.x * kHintWarps;
   int wbest = 0;
-  for (long long c = (long long)blockIdx.x * (kHintThreads / 32) + (threadIdx.x >> 5); c < n_chunks; c += n_warps) {
-    const long long p0 = c * kHintThreads + lane * 8;
-    int w[24];   // bank[p0 - 8 + i]; positions outside [0, N) are never compared
-    if (vec && p0 >= 8 && p0 + 16 <= N) {
-      const int4* src = reinterpret_cast<const int4*>(bank + p0 - 8);
+  for (long long c0 = (long long)blockIdx.x * kHintWarps + (threadIdx.x >> 5); c0 < n_chunks;
+       c0 += n_warps * kHintUnroll) {
+    // bit i: the lane's token i equals y's last one (positions past the bank never do)
+    uint32_t hits[kHintUnroll];
+    int4 v[kHintUnroll][2];
 #pragma unroll
-      for (int q = 0; q < 6; ++q) {
-        const int4 v = __ldcs(src + q);
-        w[4 * q] = v.x;
-        w[4 * q + 1] = v.y;
-        w[4 * q + 2] = v.z;
-        w[4 * q + 3] = v.w;
-      }
-    } else {
-#pragma unroll
-      for (int i = 0; i < 24; ++i) {
-        const long long q = p0 - 8 + i;
-        w[i] = (q >= 0 && q < N) ? bank[q] : 0;
+    for (int u = 0; u < kHintUnroll; ++u) {
+      const long long c = c0 + u * n_warps;
+      if (vec && (c + 1) * kHintThreads <= N) {
+        const int4* src = reinterpret_cast<const int4*>(bank + c * kHintThreads) + lane;
+        v[u][0] = __ldcs(src);
+        v[u][1] = __ldcs(src + 32);
       }
     }
-    uint32_t packed[2] = {0u, 0u};
-    int lmax = 0;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const long long p = p0 + i;
-      int m = 0;
-      // the next bank token must exist and not be EOS
-      if (p + 1 < N && w[9 + i] != eos) {
+    for (int u = 0; u < kHintUnroll; ++u) {
+      const long long c = c0 + u * n_warps;
+      hits[u] = 0u;
+      if (vec && (c + 1) * kHintThreads <= N) {
 #pragma unroll
-        for (int j = 0; j < kHintMaxN; ++j) {
-          if (m < j || j >= nmax || p - j < 0 || w[8 + i - j] != sfx[j]) break;
-          m = j + 1;
+        for (int h = 0; h < 2; ++h)
+          hits[u] |= ((v[u][h].x == last ? 1u : 0u) | (v[u][h].y == last ? 2u : 0u) | (v[u][h].z == last ? 4u : 0u) |
+                      (v[u][h].w == last ? 8u : 0u))
+                     << (4 * h);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const long long p = c * kHintThreads + (i >> 2) * 128 + lane * 4 + (i & 3);
+          if (p < N && bank[p] == last) hits[u] |= 1u << i;
         }
       }
-      packed[i >> 2] |= (uint32_t)m << (8 * (i & 3));
-      lmax = m > lmax ? m : lmax;
     }
-    if (p0 + 8 <= N) {
-      *reinterpret_cast<uint2*>(mlen + p0) = make_uint2(packed[0], packed[1]);
-    } else {
-      for (int i = 0; i < 8 && p0 + i < N; ++i) mlen[p0 + i] = (uint8_t)((packed[i >> 2] >> (8 * (i & 3))) & 255u);
-    }
+#pragma unroll 1
+    for (int u = 0; u < kHintUnroll; ++u) {
+      const long long c = c0 + u * n_warps;
+      if (c >= n_chunks) break;
+      uint32_t h = hits[0];   // a rotating window: no indexed registers
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) lmax = max(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
-    if (lane == 0) {
-      cmax[c] = (uint8_t)lmax;
-      if (lmax > 0) atomicMax(&smax[c / kHintThreads], lmax);
+      for (int k = 0; k + 1 < kHintUnroll; ++k) hits[k] = hits[k + 1];
+      int lmax = 0;
+      if (__any_sync(0xffffffffu, h != 0u)) {
+        uint32_t packed[2] = {0u, 0u};
+        while (h) {
+          const int i = __ffs(h) - 1;
+          h &= h - 1;
+          const long long p = c * kHintThreads + (i >> 2) * 128 + lane * 4 + (i & 3);
+          // the next bank token must exist and not be EOS
+          if (p + 1 >= N || bank[p + 1] == eos) continue;
+          int m = 1;
+          while (m < nmax && p - m >= 0 && bank[p - m] == suf[m]) ++m;
+          if (i < 4) packed[0] |= (uint32_t)m << (8 * i);
+          else packed[1] |= (uint32_t)m << (8 * (i - 4));
+          lmax = m > lmax ? m : lmax;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) lmax = max(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
+        if (lmax > 0) {
+          uint32_t* dst = reinterpret_cast<uint32_t*>(mlen + c * kHintThreads) + lane;
+          dst[0] = packed[0];
+          dst[32] = packed[1];
+        }
+      }
+      if (lane == 0) {
+        cmax[c] = (uint8_t)lmax;
+        if (smax && lmax > 0) atomicMax(&smax[c / kHintThreads], lmax);
+      }
+      wbest = max(wbest, lmax);
     }
-    wbest = max(wbest, lmax);
   }
-  if (lane == 0 && wbest > 0) atomicMax(best, wbest);
+  if (best && lane == 0 && wbest > 0) atomicMax(best, wbest);
 }
 
 // Whole block: the values of the threads whose `has` is set, in thread order,
@@ -131,14 +154,14 @@ OOS_DEV int ordered_select(bool has, int32_t value, int32_t* out, int* s_wcnt, i
   return *s_cnt;
 }
 
-// Insert one lane into the tree (warp 0, all lanes of the warp together).
-// Returns whether a node was created.  The caller stops when the lane or
-// node budget is spent.
+// Insert one lane into the tree (warp 0, all lanes of the warp together): walk
+// down its tokens while the tree has them, then append the rest under the node
+// reached, as far as the node budget goes -- a new node has no children to look
+// for.  Returns whether a node was created.
 OOS_DEV bool hint_insert(int32_t* s_tok, int32_t* s_par, int& T, int max_nodes, const int32_t* lane, int len) {
   const int lane_id = threadIdx.x & 31;
-  int cur = 0;
-  bool created = false;
-  for (int j = 0; j < len; ++j) {
+  int cur = 0, j = 0;
+  for (; j < len; ++j) {
     const int t = lane[j];
     // the child of cur with token t, if any (nodes are distinct per (parent, token))
     int found = -1;
@@ -147,21 +170,18 @@ OOS_DEV bool hint_insert(int32_t* s_tok, int32_t* s_par, int& T, int max_nodes, 
       const unsigned hit = __ballot_sync(0xffffffffu, i < T && s_par[i] == cur && s_tok[i] == t);
       if (hit) found = base + __ffs(hit) - 1;
     }
-    if (found >= 0) {
-      cur = found;
-      continue;
-    }
-    if (T >= max_nodes) break;
-    if (lane_id == 0) {
-      s_tok[T] = t;
-      s_par[T] = cur;
-    }
-    __syncwarp();
-    cur = T;
-    ++T;
-    created = true;
+    if (found < 0) break;
+    cur = found;
   }
-  return created;
+  const int add = min(len - j, max_nodes - T);
+  if (add <= 0) return false;
+  for (int k = lane_id; k < add; k += 32) {
+    s_tok[T + k] = lane[j + k];
+    s_par[T + k] = k == 0 ? cur : T + k - 1;
+  }
+  __syncwarp();
+  T += add;
+  return true;
 }
 
 __global__ void __launch_bounds__(kHintThreads) k_hint_pack(const int32_t* __restrict__ bank, int N, int eos,
@@ -177,16 +197,16 @@ __global__ void __launch_bounds__(kHintThreads) k_hint_pack(const int32_t* __res
                                                             int pad_to, int32_t* out_tok, int32_t* out_par,
                                                             int32_t* out_T, int32_t* out_info) {
   __shared__ int32_t s_tok[kMaxT], s_par[kMaxT];
-  __shared__ int32_t s_pos[kHintThreads];     // occurrences in the chunk being visited, in bank order
-  __shared__ int32_t s_chunk[kHintThreads];   // the span's chunks holding an occurrence, in order
-  __shared__ int32_t s_span[kHintThreads];    // this round's spans holding an occurrence, in order
-  __shared__ int32_t s_lane[kMaxT];           // the lane being inserted
-  __shared__ int s_wcnt[kHintThreads / 32];
-  __shared__ int s_n, s_nc, s_ns, s_done;
+  __shared__ int32_t s_pos[kHintWarps * kHintThreads];   // occurrences in the chunks being visited, in bank order
+  __shared__ int32_t s_chunk[kHintFlat];                 // chunks holding an occurrence, in order
+  __shared__ int32_t s_span[kHintThreads];               // this round's spans holding an occurrence, in order
+  __shared__ int32_t s_lane[kHintWarps][kMaxT];          // the lanes being inserted
+  __shared__ int s_len[kHintWarps];
+  __shared__ int s_wcnt[kHintWarps];
+  __shared__ int s_nc, s_ns, s_done;
   const int warp = threadIdx.x >> 5, lane_id = threadIdx.x & 31;
   pdl_wait();   // the match kernel's results
   pdl_trigger();
-  const int n = *best;
   if (prefix_len_dev) prefix_len = *prefix_len_dev;
   int T = 1, lanes = 0, hint_lanes = 0;       // warp 0's copies are the authoritative ones
   if (threadIdx.x == 0) {
@@ -194,50 +214,126 @@ __global__ void __launch_bounds__(kHintThreads) k_hint_pack(const int32_t* __res
     s_par[0] = -1;
     s_done = (max_lanes <= 0 || max_nodes <= 1) ? 1 : 0;
   }
-  __syncthreads();
-  // hint lanes: occurrences of the length-n suffix (match length >= n), bank order
-  const long long n_chunks = ((long long)N + kHintThreads - 1) / kHintThreads;
-  const long long n_spans = (n_chunks + kHintThreads - 1) / kHintThreads;
-  for (long long sb = 0; n > 0 && sb < n_spans; sb += kHintThreads) {
-    if (s_done) break;
-    const long long sp = sb + threadIdx.x;
-    const int ns = ordered_select(sp < n_spans && smax[sp] >= n, (int32_t)sp, s_span, s_wcnt, &s_ns);
-    for (int si = 0; si < ns; ++si) {
-      if (s_done) break;
-      const long long c = (long long)s_span[si] * kHintThreads + threadIdx.x;
-      const int nc = ordered_select(c < n_chunks && cmax[c] >= n, (int32_t)c, s_chunk, s_wcnt, &s_nc);
-      // visit the chunks: their occurrences in order, then warp 0 inserts their lanes
-      for (int ci = 0; ci < nc; ++ci) {
-        if (s_done) break;
-        const long long p = (long long)s_chunk[ci] * kHintThreads + threadIdx.x;
-        const int np = ordered_select(p < N && mlen[p] >= n, (int32_t)p, s_pos, s_wcnt, &s_n);
-        if (warp == 0) {
-          for (int k = 0; k < np; ++k) {
-            if (lanes >= max_lanes || T >= max_nodes) break;
-            // lane: up to depth tokens after the occurrence, stopping before an EOS
-            const long long q0 = (long long)s_pos[k] + 1;
-            int len = 0;
-            for (int j = 0; j < depth; ++j) {
-              const long long q = q0 + j;
-              if (q >= N) break;
-              const int t = bank[q];
-              if (t == eos) break;
-              if (lane_id == 0) s_lane[j] = t;
-              ++len;
+  const int n_chunks = (int)(((long long)N + kHintThreads - 1) / kHintThreads);
+
+  // the lanes of the occurrences (match length >= n) in the nc chunks of s_chunk
+  auto visit = [&](int nc, int n) {
+    for (int ci = 0; ci < nc && !s_done; ci += kHintWarps) {
+      // one chunk per warp, 8 positions per lane
+      const int c = ci + warp < nc ? s_chunk[ci + warp] : -1;
+      uint2 m = make_uint2(0u, 0u);
+      if (c >= 0) m = reinterpret_cast<const uint2*>(mlen + (size_t)c * kHintThreads)[lane_id];
+      uint32_t hit = 0u;
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if ((int)(((i < 4 ? m.x : m.y) >> (8 * (i & 3))) & 255u) >= n) hit |= 1u << i;
+      const int mine = c >= 0 ? __popc(hit) : 0;
+      int upto = mine;   // hits of lanes 0 .. lane_id
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, upto, o);
+        if (lane_id >= o) upto += y;
+      }
+      if (lane_id == 31) s_wcnt[warp] = upto;
+      __syncthreads();
+      int off = upto - mine, total = 0;
+      for (int w = 0; w < kHintWarps; ++w) {
+        if (w < warp) off += s_wcnt[w];
+        total += s_wcnt[w];
+      }
+      for (int i = 0; mine && i < 8; ++i)
+        if ((hit >> i) & 1u) s_pos[off++] = c * kHintThreads + lane_id * 8 + i;
+      __syncthreads();
+      for (int k = 0; k < total && !s_done; k += kHintWarps) {
+        // one lane per warp: up to depth tokens after the occurrence, stopping before an EOS
+        if (k + warp < total) {
+          const long long q0 = (long long)s_pos[k + warp] + 1;
+          int len = depth;
+          for (int j0 = 0; j0 < depth; j0 += 32) {
+            const int j = j0 + lane_id;
+            const int t = j < depth && q0 + j < N ? bank[q0 + j] : eos;
+            if (j < depth) s_lane[warp][j] = t;
+            const unsigned end = __ballot_sync(0xffffffffu, t == eos);
+            if (end) {
+              len = min(depth, j0 + __ffs(end) - 1);
+              break;
             }
-            __syncwarp();
-            if (hint_insert(s_tok, s_par, T, max_nodes, s_lane, len)) {
+          }
+          if (lane_id == 0) s_len[warp] = len;
+        }
+        __syncthreads();
+        if (warp == 0) {
+          for (int u = 0; u < kHintWarps && k + u < total; ++u) {
+            if (lanes >= max_lanes || T >= max_nodes) break;
+            if (hint_insert(s_tok, s_par, T, max_nodes, s_lane[u], s_len[u])) {
               ++lanes;
               ++hint_lanes;
             }
-            __syncwarp();
           }
           if (lane_id == 0 && (lanes >= max_lanes || T >= max_nodes)) s_done = 1;
         }
         __syncthreads();
       }
     }
+  };
+
+  int n = 0;   // the longest suffix with a counted occurrence
+  if (!smax) {
+    // every chunk maximum: 16 a thread
+    const int b0 = threadIdx.x * 16;
+    uint4 w = make_uint4(0u, 0u, 0u, 0u);
+    if (b0 < n_chunks) w = reinterpret_cast<const uint4*>(cmax)[threadIdx.x];
+    const uint32_t wd[4] = {w.x, w.y, w.z, w.w};
+    int mx[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      mx[i] = b0 + i < n_chunks ? (int)((wd[i >> 2] >> (8 * (i & 3))) & 255u) : 0;
+      n = max(n, mx[i]);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) n = max(n, __shfl_xor_sync(0xffffffffu, n, o));
+    if (lane_id == 0) s_wcnt[warp] = n;
+    __syncthreads();
+    for (int k = 0; k < kHintWarps; ++k) n = max(n, s_wcnt[k]);
+    __syncthreads();
+    if (n > 0) {
+      int mine = 0;
+#pragma unroll
+      for (int i = 0; i < 16; ++i) mine += mx[i] >= n ? 1 : 0;
+      int upto = mine;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, upto, o);
+        if (lane_id >= o) upto += y;
+      }
+      if (lane_id == 31) s_wcnt[warp] = upto;
+      __syncthreads();
+      int off = upto - mine, nc = 0;
+      for (int k = 0; k < kHintWarps; ++k) {
+        if (k < warp) off += s_wcnt[k];
+        nc += s_wcnt[k];
+      }
+#pragma unroll
+      for (int i = 0; i < 16; ++i)
+        if (mx[i] >= n) s_chunk[off++] = b0 + i;
+      __syncthreads();
+      visit(nc, n);
+    }
+  } else {
+    n = *best;
+    __syncthreads();
+    const int n_spans = (n_chunks + kHintThreads - 1) / kHintThreads;
+    for (int sb = 0; n > 0 && sb < n_spans && !s_done; sb += kHintThreads) {
+      const int sp = sb + threadIdx.x;
+      const int ns = ordered_select(sp < n_spans && smax[sp] >= n, sp, s_span, s_wcnt, &s_ns);
+      for (int si = 0; si < ns && !s_done; ++si) {
+        const int c = s_span[si] * kHintThreads + threadIdx.x;
+        const int nc = ordered_select(c < n_chunks && cmax[c] >= n, c, s_chunk, s_wcnt, &s_nc);
+        visit(nc, n);
+      }
+    }
   }
+  __syncthreads();
   // native lanes fill what the budgets leave
   if (warp == 0) {
     for (int i = 0; i < n_native; ++i) {
@@ -246,9 +342,9 @@ __global__ void __launch_bounds__(kHintThreads) k_hint_pack(const int32_t* __res
       len = len < depth ? len : depth;
       len = len < native_stride ? len : native_stride;
       len = len < 0 ? 0 : len;
-      for (int j = lane_id; j < len; j += 32) s_lane[j] = native[(size_t)i * native_stride + j];
+      for (int j = lane_id; j < len; j += 32) s_lane[0][j] = native[(size_t)i * native_stride + j];
       __syncwarp();
-      if (hint_insert(s_tok, s_par, T, max_nodes, s_lane, len)) ++lanes;
+      if (hint_insert(s_tok, s_par, T, max_nodes, s_lane[0], len)) ++lanes;
       __syncwarp();
     }
     for (int i = lane_id; i < T; i += 32) {
@@ -271,8 +367,6 @@ __global__ void __launch_bounds__(kHintThreads) k_hint_pack(const int32_t* __res
   }
 }
 
-// workspace: [best | pad to 256][mlen: one byte per position, padded to 256]
-//            [cmax: one byte per chunk, padded to 256][smax: one int per span]
 // Workspace: the call's n (best) and the span maxima first, so that one
 // zeroing copy covers both; then one match byte per position and the chunk maxima.
 static size_t hint_head_bytes(size_t spans) { return (4 + spans * 4 + 255) / 256 * 256; }
@@ -294,14 +388,19 @@ cudaError_t launch_hint_tree(const int32_t* bank, int N, int eos, const int32_t*
   int* smax = best + 1;
   uint8_t* mlen = (uint8_t*)ws + hint_head_bytes((size_t)n_spans);
   uint8_t* cmax = mlen + n_chunks * kHintThreads;
-  cudaError_t e = cudaMemsetAsync(best, 0, (size_t)(1 + n_spans) * sizeof(int), st);
-  if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
+  if (n_chunks <= kHintFlat) {
+    best = smax = nullptr;
+  } else {
+    e = cudaMemsetAsync(best, 0, (size_t)(1 + n_spans) * sizeof(int), st);
+    if (e != cudaSuccess) return e;
+  }
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  // one warp per 256-position chunk; enough blocks for every SM to hold several
+  // one warp per 256-position chunk, as many blocks as the SMs hold at once
   const long long want = (n_chunks + kHintThreads / 32 - 1) / (kHintThreads / 32);
-  const int grid = (int)(want < (long long)sms * 8 ? want : (long long)sms * 8);
+  const int grid = (int)(want < (long long)sms * 3 ? want : (long long)sms * 3);
   const int vec = ((uintptr_t)bank & 15) == 0 ? 1 : 0;
   // the packing block launches while the match kernel runs (programmatic
   // dependent launch) and waits for it before reading its results

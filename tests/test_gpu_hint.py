@@ -17,9 +17,11 @@ torch = pytest.importorskip("torch")
 from paper_2608_00814_gb300 import binding as B  # noqa: E402
 
 
-def _gpu(bank, eos, y, native, max_lanes, depth, max_nodes):
+def _gpu(bank, eos, y, native, max_lanes, depth, max_nodes, shift=0):
+    """shift: the bank starts that many tokens past an allocation's start."""
     dev = "cuda"
-    b = torch.as_tensor(np.asarray(bank, np.int32), device=dev)
+    b = torch.zeros(shift + len(bank), dtype=torch.int32, device=dev)[shift:]
+    b.copy_(torch.as_tensor(np.asarray(bank, np.int32)))
     p = torch.as_tensor(np.asarray(y, np.int32), device=dev)
     if native:
         stride = max(1, max(len(l) for l in native))
@@ -41,9 +43,9 @@ def _gpu(bank, eos, y, native, max_lanes, depth, max_nodes):
     return tok[:n].cpu().numpy(), par[:n].cpu().numpy(), info.cpu().numpy().tolist(), tok[n:].cpu().numpy()
 
 
-def _check(bank, eos, y, native, max_lanes, depth, max_nodes):
+def _check(bank, eos, y, native, max_lanes, depth, max_nodes, shift=0):
     r = hb.propose_tree(bank, eos, y, native, max_lanes, depth, max_nodes)
-    tok, par, info, rest = _gpu(bank, eos, y, native, max_lanes, depth, max_nodes)
+    tok, par, info, rest = _gpu(bank, eos, y, native, max_lanes, depth, max_nodes, shift)
     np.testing.assert_array_equal(tok, r["tokens"])
     np.testing.assert_array_equal(par, r["parents"])
     assert info == [r["match_n"], r["hint_lanes"], r["lanes"]]
@@ -109,3 +111,32 @@ def test_bank_over_several_spans(spots):
     y = np.concatenate([rng.integers(2, vocab, size=12), key]).tolist()
     r = _check(bank.tolist(), eos, y, [[5, 6]], 6, 8, 96)
     assert r["match_n"] == 7 and r["hint_lanes"] == len(spots)
+
+
+@pytest.mark.parametrize("n", [256, 257, 1 << 20, (1 << 20) + 1, (1 << 20) + 300])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_chunk_and_summary_edges(n, shift):
+    """Bank sizes at the edge of a chunk and of what the packing block reads
+    without span maxima, from an address aligned to 16 bytes and one that is not;
+    the suffix occurs at the first and last places it can and across chunk ends."""
+    rng = np.random.default_rng(n)
+    bank = rng.integers(10, 50000, size=n)
+    key = rng.integers(2, 10, size=7)                       # tokens the rest of the bank does not use
+    spots = sorted({0, 249, n // 2 // 256 * 256 - 3, n - 8} & set(range(0, n - 7)))
+    for at in spots:
+        bank[at:at + 7] = key
+    y = np.concatenate([rng.integers(10, 50000, size=5), key]).tolist()
+    r = _check(bank.tolist(), 1, y, [], 16, 9, 128, shift)
+    assert r["match_n"] == 7 and r["hint_lanes"] == len([p for p in spots if p == n - 8 or p + 7 < n])
+
+
+def test_dense_occurrences():
+    """Hundreds of occurrences per chunk, most repeating earlier lanes; the lane
+    budget is met only by the few that differ, far apart."""
+    bank = [5, 6] * 700
+    for i, at in enumerate((3, 601, 1199)):
+        bank[at] = 20 + i
+    r = _check(bank, 0, [6, 5], [[1, 2], [3]], 40, 5, 128)
+    assert r["hint_lanes"] > 3
+    _check(bank, 0, [6, 5], [[1, 2], [3]], 3, 128, 128)
+    _check(bank, 0, [6, 5], [], 128, 40, 50)
