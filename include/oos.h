@@ -206,8 +206,10 @@ int oos_hint_tree(const int32_t* bank, int32_t bank_len, int32_t eos, const int3
  *   kv            cache; slots [0, ctx_len) are read, slots [ctx_len,
  *                 ctx_len + n) receive the prompt's K/V.
  *   tokens        DEVICE int32[n], the prompt after the ctx_len cached positions.
- *   n             >= 1; any length that fits the cache: it runs as chains of at
- *                 most max_T tokens, each a tree pass of the verify kernels (a
+ *   n             >= 1; any length that fits the cache.  bf16 models take it in
+ *                 chunks of up to 2048 tokens (a workspace of that many rows is
+ *                 part of oos_workspace_bytes), a chunk of at most 128 and fp32
+ *                 models as chains of tree passes of the verify kernels (a
  *                 chain's tree attention is causal attention).
  *   out_next_token  DEVICE int32[1] or NULL: the greedy next token after the
  *                 prompt (argmax of the last position's logits, Eq. 1).

@@ -37,6 +37,10 @@
 // and their V rows are zeroed in shared memory before the P.V product, so
 // whatever the cache holds there cannot reach the output.
 //
+// Prefill runs the same kernel on a chunk of consecutive tokens (CAUSAL): row i
+// attends to every slot up to its own, ctx + i, so a block's keys end at its last
+// row's slot and the mask is a length, not an ancestor set.
+//
 // fp32 path: one block per (node, head), CUDA cores (small models only).
 #include <math.h>
 #include <string.h>
@@ -104,11 +108,15 @@ constexpr int kAttnThreads = 224;                         // 7 warps, roles belo
 static_assert(kAttnSmem <= 227 * 1024, "shared memory per block");
 static_assert(kMaxSplits <= 16, "cluster size");
 // TMEM columns (lane = query row): S[2] fp32 scores of a tile (P, bf16 pairs,
-// overwrites the first 64 columns of its S buffer), O fp32
+// overwrites the first 64 columns of its S buffer), O fp32.  Prefill keeps an O of
+// the even and one of the odd tiles: its blocks go through every key unsplit, the
+// tensor core truncates each addition to an accumulator, and two chains half as
+// long are closer to the sum (K/V error 5.3e-4 -> 5.2e-4 over 2048 tokens; the
+// verify step's chains are short, and reading a second O cost it 1 %)
 constexpr int kTmS = 0;                            // [2] x 128
-constexpr int kTmO = 2 * kAttnKeys;                // 128
+constexpr int kTmO = 2 * kAttnKeys;                // [2] x 128
 constexpr int kAttnTmemCols = 512;                 // allocation unit: a power of two
-static_assert(kTmO + kAttnD <= kAttnTmemCols, "TMEM columns");
+static_assert(kTmO + 2 * kAttnD <= kAttnTmemCols, "TMEM columns");
 
 struct AttnArgs {
   CUtensorMap kmap, vmap;   // cache [capacity][nkv][d] as (d, kv head, slot)
@@ -243,8 +251,8 @@ OOS_DEV void drain_wait(uint64_t* bar, uint32_t parity) {
 // warps 2..5 run the softmax (thread = query row = TMEM lane); all warps take
 // part in the merge.
 // F16: the KV cache (and q) are IEEE binary16 -- every product runs in f16;
-// otherwise bf16.
-template <bool F16>
+// otherwise bf16.  CAUSAL: a prefill chunk.
+template <bool F16, bool CAUSAL>
 __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_constant__ AttnArgs a) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -267,7 +275,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
   const int T = a.T, nq = a.nq, G = a.group, npc = a.npc, S = a.splits;
   const float scale_log2 = a.scale_log2;
   uint32_t* status = a.status;
-  const int rb = blockIdx.x, g = blockIdx.y, split = blockIdx.z;
+  // causal row blocks late in the chunk have the most keys: they start first
+  const int rb = CAUSAL ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x, g = blockIdx.y, split = blockIdx.z;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int node0 = rb * npc;
   const int rows = npc * G;                                   // query rows of the block
@@ -278,7 +287,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
   // only after its own dependency wait, so when this kernel starts the kernel
   // two launches back and everything before it are complete.
   const int ctx = *a.ctx_dev;
-  const int n_all = (ctx + T + kAttnKeys - 1) / kAttnKeys;   // tiles over slots [0, ctx + T)
+  const int n_keys = ctx + (CAUSAL ? min(T, node0 + npc) : T);
+  const int n_all = (n_keys + kAttnKeys - 1) / kAttnKeys;   // tiles over the block's keys, slots [0, n_keys)
   const int t0 = (int)((long long)split * n_all / S);
   const int n_tiles = (int)((long long)(split + 1) * n_all / S) - t0;
   // merge: rows [0, vrows) are dealt to the S blocks of the cluster, block j
@@ -433,8 +443,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
         const uint64_t vd = vdesc0 + (uint64_t)((b * kTileBytes) >> 4);
 #pragma unroll
         for (int kk = 0; kk < kAttnKeys / 16; ++kk)
-          tc_mma_bf16_ts(tmem_o, pt + 8 * kk, vd + (uint64_t)((kk * 16 * 128) >> 4), idesc_pv,
-                         (ti > 0 || kk > 0) ? 1u : 0u);
+          tc_mma_bf16_ts(tmem_o + (CAUSAL ? b * kAttnD : 0), pt + 8 * kk, vd + (uint64_t)((kk * 16 * 128) >> 4), idesc_pv,
+                         (ti > (CAUSAL ? 1 : 0) || kk > 0) ? 1u : 0u);
         tc_commit(&pvdone[b]);
         tc_commit(&vempty[b]);
       }
@@ -465,8 +475,10 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
         pdl_wait();
         pdl_trigger();
         waited = true;
-        anc0 = a.anc[2 * node];
-        anc1 = a.anc[2 * node + 1];
+        if (!CAUSAL) {
+          anc0 = a.anc[2 * node];
+          anc1 = a.anc[2 * node + 1];
+        }
       }
       const int tt = dry ? 0 : ti;
       const int b = tt & 1;
@@ -482,13 +494,16 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
       // valid keys of this row in the tile: committed slots, then the tree
       // slots of the node's ancestors (slot ctx + j for ancestor j); slots at
       // or past ctx + T are never ancestors (the dry pass takes the masked path)
-      const bool full_tile = !dry && key0 + kAttnKeys <= ctx;   // tile-uniform
+      const bool full_tile = !dry && key0 + kAttnKeys <= ctx + (CAUSAL ? node0 + 1 : 0);   // tile-uniform
       unsigned long long mlo = ~0ull, mhi = ~0ull;
       if (!full_tile) {
-        const int c = max(0, ctx - key0);                 // leading committed slots (< 128)
-        unsigned long long tlo, thi;
-        if (key0 >= ctx) shr128(anc0, anc1, key0 - ctx, tlo, thi);
-        else shl128(anc0, anc1, c, tlo, thi);
+        // leading valid slots: the committed ones (< 128), or those up to the row's own
+        const int c = CAUSAL ? max(0, min(kAttnKeys, ctx + node + 1 - key0)) : max(0, ctx - key0);
+        unsigned long long tlo = 0ull, thi = 0ull;
+        if (!CAUSAL) {
+          if (key0 >= ctx) shr128(anc0, anc1, key0 - ctx, tlo, thi);
+          else shl128(anc0, anc1, c, tlo, thi);
+        }
         const unsigned long long clo = c >= 64 ? ~0ull : (c == 0 ? 0ull : (~0ull >> (64 - c)));
         const unsigned long long chi = c <= 64 ? 0ull : (~0ull >> (128 - c));
         mlo = clo | tlo;
@@ -520,7 +535,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
         tc_fence_after();
         const float f = rescale ? exp2f(m_used - tmax) : 1.f;
 #pragma unroll 1
-        for (int c = 0; c < kAttnD / 32; ++c) {   // 32 columns at a time: the scores stay in registers
+        for (int c = 0; c < (CAUSAL ? 2 : 1) * kAttnD / 32; ++c) {   // 32 columns at a time: the scores stay in registers
           float ov[32];
           tmem_ld32_nowait(tmem_o + lane_off + c * 32, ov);
           tmem_wait_ld_regs(ov);
@@ -617,6 +632,16 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
     float ov[kAttnD];
     if (have_o) {
       tmem_ld128(tmem_o + lane_off, ov);
+      if (CAUSAL && n_tiles > 1) {
+#pragma unroll
+        for (int c = 0; c < kAttnD / 32; ++c) {
+          float o1[32];
+          tmem_ld32_nowait(tmem_o + kAttnD + lane_off + c * 32, o1);
+          tmem_wait_ld_regs(o1);
+#pragma unroll
+          for (int i = 0; i < 32; ++i) ov[c * 32 + i] += o1[i];
+        }
+      }
     } else {
 #pragma unroll
       for (int i = 0; i < kAttnD; ++i) ov[i] = 0.f;
@@ -770,18 +795,22 @@ __global__ void __launch_bounds__(128) k_attn_f32(const float* __restrict__ q, c
 
 int attn_nodes_per_block(int group) { return group >= kAttnRows ? 1 : kAttnRows / group; }
 
-bool attn_encode_q_maps(Model& m) {
+static bool encode_q_maps(const Model& m, const void* q, int nodes, CUtensorMap* hi, CUtensorMap* lo) {
   const auto& c = m.cfg;
   const int group = c.n_q_heads / c.n_kv_heads;
   // q [node][nq][d] viewed as (d, head in group, kv head, node); a box is the
   // (node, head in group) rows of one kv head, 64 of d at a time
-  const uint64_t dims[4] = {(uint64_t)kAttnD, (uint64_t)group, (uint64_t)c.n_kv_heads, (uint64_t)kMaxT};
+  const uint64_t dims[4] = {(uint64_t)kAttnD, (uint64_t)group, (uint64_t)c.n_kv_heads, (uint64_t)nodes};
   const uint64_t strides[3] = {(uint64_t)kAttnD * 2, (uint64_t)group * kAttnD * 2, (uint64_t)c.n_q_heads * kAttnD * 2};
   const uint32_t box[4] = {64, (uint32_t)group, 1, (uint32_t)attn_nodes_per_block(group)};
-  const __nv_bfloat16* q = (const __nv_bfloat16*)m.ws.q;
+  const __nv_bfloat16* qp = (const __nv_bfloat16*)q;
   const bool f16 = c.kv_f16 != 0;
-  return encode_bf16_map(&m.qmap_hi, q, 4, dims, strides, box, f16) &&
-         encode_bf16_map(&m.qmap_lo, q + (size_t)kMaxT * c.n_q_heads * kAttnD, 4, dims, strides, box, f16);
+  return encode_bf16_map(hi, qp, 4, dims, strides, box, f16) &&
+         encode_bf16_map(lo, qp + (size_t)nodes * c.n_q_heads * kAttnD, 4, dims, strides, box, f16);
+}
+bool attn_encode_q_maps(Model& m) {
+  return encode_q_maps(m, m.ws.q, kMaxT, &m.qmap_hi, &m.qmap_lo) &&
+         encode_q_maps(m, m.ws.pf_q, kPfTokens, &m.pf_qmap_hi, &m.pf_qmap_lo);
 }
 
 // clusters of `sp` attention blocks resident at once on this device (occupancy query, cached)
@@ -801,22 +830,25 @@ static int attn_max_clusters(int sp) {
     lc.attrs = attr;
     lc.numAttrs = 1;
     int n = 0;
-    cached[sp] = cudaOccupancyMaxActiveClusters(&n, (const void*)k_attn_tc<false>, &lc) == cudaSuccess && n > 0 ? n : -1;
+    cached[sp] = cudaOccupancyMaxActiveClusters(&n, (const void*)k_attn_tc<false, false>, &lc) == cudaSuccess && n > 0 ? n : -1;
     cudaGetLastError();
   }
   return cached[sp];
 }
 
-template <bool F16>
+template <bool F16, bool CAUSAL>
 static cudaError_t attn_setup_one() {
-  cudaError_t e = cudaFuncSetAttribute(k_attn_tc<F16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttnSmem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_attn_tc<F16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  cudaError_t e = cudaFuncSetAttribute(k_attn_tc<F16, CAUSAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttnSmem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_attn_tc<F16, CAUSAL>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   return e;
 }
 
 cudaError_t attn_setup() {
-  cudaError_t e = attn_setup_one<false>();
-  return e == cudaSuccess ? attn_setup_one<true>() : e;
+  cudaError_t e = attn_setup_one<false, false>();
+  if (e == cudaSuccess) e = attn_setup_one<true, false>();
+  if (e == cudaSuccess) e = attn_setup_one<false, true>();
+  return e == cudaSuccess ? attn_setup_one<true, true>() : e;
 }
 
 int attn_splits(Model& m, int ctx_hint, int T) {
@@ -833,16 +865,11 @@ int attn_splits(Model& m, int ctx_hint, int T) {
   return 1;
 }
 
-cudaError_t launch_attention(Model& m, int layer, const void* kc, const void* vc, int capacity, int ctx, int T,
-                             cudaStream_t st) {
+// one bf16-path launch over T nodes: a.qhi/qlo, a.out and a.out_lo_off are the caller's
+template <bool CAUSAL>
+static cudaError_t launch_attn_tc(Model& m, int layer, const void* kc, const void* vc, int capacity, int ctx, int T,
+                                  AttnArgs& a, cudaStream_t st) {
   const auto& c = m.cfg;
-  if (c.dtype != OOS_DTYPE_BF16) {
-    return launch(m.pdl, k_attn_f32, dim3(T, c.n_q_heads), dim3(128), 0, st, (const float*)m.ws.q, (const float*)kc,
-                  (const float*)vc, (const unsigned long long*)m.ws.anc, T, c.n_q_heads, c.n_kv_heads, c.head_dim,
-                  (const int32_t*)m.ws.ctx, 1.0f / sqrtf((float)c.head_dim), (float*)m.ws.attn);
-  }
-  AttnArgs a;
-  memset(&a, 0, sizeof(a));
   // this layer's cache over its whole capacity, (d, kv head, slot); encoded
   // again only when the cache buffers change
   {
@@ -864,8 +891,6 @@ cudaError_t launch_attention(Model& m, int layer, const void* kc, const void* vc
     a.kmap = km.kmap;
     a.vmap = km.vmap;
   }
-  a.qhi = m.qmap_hi;
-  a.qlo = m.qmap_lo;
   a.anc = m.ws.anc;
   a.ctx_dev = m.ws.ctx;
   a.T = T;
@@ -875,8 +900,6 @@ cudaError_t launch_attention(Model& m, int layer, const void* kc, const void* vc
   const int RB = (T + a.npc - 1) / a.npc;
   a.splits = attn_splits(m, ctx, T);
   a.scale_log2 = 1.4426950408889634f / sqrtf((float)kAttnD);
-  a.out = (__nv_bfloat16*)m.ws.attn;
-  a.out_lo_off = (size_t)kMaxT * c.n_q_heads * kAttnD;
   a.status = m.ws.status;
 
   cudaLaunchConfig_t lc = {};
@@ -893,7 +916,36 @@ cudaError_t launch_attention(Model& m, int layer, const void* kc, const void* vc
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   lc.attrs = attr;
   lc.numAttrs = m.pdl ? 2 : 1;
-  return c.kv_f16 ? cudaLaunchKernelEx(&lc, k_attn_tc<true>, a) : cudaLaunchKernelEx(&lc, k_attn_tc<false>, a);
+  return c.kv_f16 ? cudaLaunchKernelEx(&lc, k_attn_tc<true, CAUSAL>, a)
+                  : cudaLaunchKernelEx(&lc, k_attn_tc<false, CAUSAL>, a);
+}
+
+cudaError_t launch_attention(Model& m, int layer, const void* kc, const void* vc, int capacity, int ctx, int T,
+                             cudaStream_t st) {
+  const auto& c = m.cfg;
+  if (c.dtype != OOS_DTYPE_BF16) {
+    return launch(m.pdl, k_attn_f32, dim3(T, c.n_q_heads), dim3(128), 0, st, (const float*)m.ws.q, (const float*)kc,
+                  (const float*)vc, (const unsigned long long*)m.ws.anc, T, c.n_q_heads, c.n_kv_heads, c.head_dim,
+                  (const int32_t*)m.ws.ctx, 1.0f / sqrtf((float)c.head_dim), (float*)m.ws.attn);
+  }
+  AttnArgs a;
+  memset(&a, 0, sizeof(a));
+  a.qhi = m.qmap_hi;
+  a.qlo = m.qmap_lo;
+  a.out = (__nv_bfloat16*)m.ws.attn;
+  a.out_lo_off = (size_t)kMaxT * c.n_q_heads * kAttnD;
+  return launch_attn_tc<false>(m, layer, kc, vc, capacity, ctx, T, a, st);
+}
+
+cudaError_t launch_attention_pf(Model& m, int layer, const void* kc, const void* vc, int capacity, int ctx, int T,
+                                cudaStream_t st) {
+  AttnArgs a;
+  memset(&a, 0, sizeof(a));
+  a.qhi = m.pf_qmap_hi;
+  a.qlo = m.pf_qmap_lo;
+  a.out = (__nv_bfloat16*)m.ws.pf_attn;
+  a.out_lo_off = (size_t)kPfTokens * m.cfg.n_q_heads * kAttnD;
+  return launch_attn_tc<true>(m, layer, kc, vc, capacity, ctx, T, a, st);
 }
 
 }  // namespace oos

@@ -48,6 +48,10 @@ namespace oos {
 //   EPI_SILU  : a tile holds the same rows of gate and up; act = silu(r g) * (r u).
 //   EPI_ARGMAX: LM head -- logits scaled by the final RMSNorm factor and folded
 //               into a per-node running top-2.
+// A prefill chunk too small for the tiles of prefill.cu runs through the same
+// kernels in token tiles of 128 (CHUNK): the token tiles of a weight tile are
+// separate clusters (or CTAs).
+//
 // RMSNorm is split across kernels by linearity: a producer stores y = g (.) x
 // and sum(x^2) per feature tile; the consumer GEMM computes W.y and multiplies
 // column t by r_t = rsqrt(sum x_t^2 / H + eps) in its epilogue.
@@ -66,6 +70,10 @@ namespace oos {
 //   SILU, ARGMAX: whole-K tiles, dealt round-robin (the weights of the next tile
 //     stream while one is finished).
 enum { EPI_QKV = 0, EPI_RESID = 1, EPI_SILU = 2, EPI_ARGMAX = 3 };
+
+// token rows the activation buffers are laid out for; the lo halves follow them
+template <bool CHUNK>
+constexpr int kLdr = CHUNK ? kPfTokens : kMaxT;
 
 // A work tile is SUB weight subtiles that share every staged activation slice:
 // gate and up rows, or 2 x 128 rows of the LM head.
@@ -86,17 +94,17 @@ struct GemmArgs {
   int split;          // CTAs sharing a tile (cluster size)
   int stages;         // ring depth
   int N;              // output rows (features / vocab; intermediate rows for EPI_SILU)
-  int T;              // valid columns (tree nodes)
+  int T;              // valid columns (tree nodes; all token tiles together)
   int tl_slot;        // timeline slot (layer * 4 + kind)
   uint32_t* status;
   // RMSNorm scale of the GEMM input (EPI_QKV, EPI_SILU, EPI_ARGMAX)
-  const float* ss_in;   // [chunk][kMaxT]
+  const float* ss_in;   // [chunk][ldr]
   int ss_chunks;
   float inv_dim, eps;
   // EPI_QKV
   int nq, nkv;
   const __nv_bfloat16 *bq, *bk, *bv, *gq, *gk;
-  const float2* rope;   // [kMaxT][64] (cos, sin) of the step's positions
+  const float2* rope;   // [ldr][64] (cos, sin) of the step's positions
   __nv_bfloat16 *q_out, *kc, *vc;
   const int32_t* ctx;   // committed length of the step (device; K/V of node t go to slot *ctx + t)
   int kv_f16;           // the KV cache (and so q) are binary16 instead of bf16
@@ -189,16 +197,18 @@ OOS_DEV float4 bf16x4(const __nv_bfloat16* p) {
   return make_float4(__bfloat162float(h[0]), __bfloat162float(h[1]), __bfloat162float(h[2]), __bfloat162float(h[3]));
 }
 
-// RMSNorm factors of tokens [tb, te) into rms[], by the epilogue warps (w of
-// kEpiWarps): lanes take the chunk sums, four tokens of a warp in flight.
-OOS_DEV void input_rms(const GemmArgs& a, float* rms, int tb, int te, int w) {
+// RMSNorm factors of tokens [tb, te) of the token tile at tok0 into rms[], by the
+// epilogue warps (w of kEpiWarps): lanes take the chunk sums, four tokens of a
+// warp in flight.
+template <bool CHUNK>
+OOS_DEV void input_rms(const GemmArgs& a, float* rms, int tok0, int tb, int te, int w) {
   const int l = threadIdx.x & 31;
   for (int t0 = tb + 4 * w; t0 < te; t0 += 4 * kEpiWarps) {
     float s[4] = {0.f, 0.f, 0.f, 0.f};
     for (int c = l; c < a.ss_chunks; c += 32) {
 #pragma unroll
       for (int k = 0; k < 4; ++k)
-        if (t0 + k < te) s[k] += __ldcg(a.ss_in + (size_t)c * kMaxT + t0 + k);
+        if (t0 + k < te) s[k] += __ldcg(a.ss_in + (size_t)c * kLdr<CHUNK> + tok0 + t0 + k);
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) s[k] = warp_sum(s[k]);
@@ -216,7 +226,6 @@ OOS_DEV void input_rms(const GemmArgs& a, float* rms, int tb, int te, int w) {
 // q/k norm and the RoPE pair exchange are warp shuffles).
 constexpr int kFinRows = 4;
 constexpr int kFinPass = kFinRows * kEpiWarps;
-constexpr int kMaxSplit = 8;
 
 // acc[k] = sum over the cluster's CTAs, in rank order, of their staged row of
 // token t0 + w + 8k (peer[s]: shared-memory address of CTA s's stage)
@@ -248,17 +257,19 @@ OOS_DEV void pull_rows(float4 (&acc)[kFinRows], const uint32_t (&peer)[kMaxSplit
 struct ResidRows {
   float4 x[kFinRows];
 };
-OOS_DEV void resid_load(const GemmArgs& a, ResidRows& r, int f, bool live, int t0, int te, int w) {
+template <bool CHUNK>
+OOS_DEV void resid_load(const GemmArgs& a, ResidRows& r, int f, bool live, int tok0, int t0, int te, int w) {
 #pragma unroll
   for (int k = 0; k < kFinRows; ++k) {
     const int t = t0 + w + kEpiWarps * k;
-    r.x[k] = (t < te && live) ? __ldcg(reinterpret_cast<const float4*>(a.x + (size_t)t * a.N + f))
+    r.x[k] = (t < te && live) ? __ldcg(reinterpret_cast<const float4*>(a.x + (size_t)(tok0 + t) * a.N + f))
                               : make_float4(0.f, 0.f, 0.f, 0.f);
   }
 }
 // x += W.a; y = g (.) x; per-tile sums of x^2
+template <bool CHUNK>
 OOS_DEV void resid_finish(const GemmArgs& a, const ResidRows& r, const float4 (&acc)[kFinRows], float4 g, int tile, int f,
-                          bool live, bool st, int t0, int te, int w) {
+                          bool live, bool st, int tok0, int t0, int te, int w) {
   const int l = threadIdx.x & 31;
 #pragma unroll
   for (int k = 0; k < kFinRows; ++k) {
@@ -266,12 +277,12 @@ OOS_DEV void resid_finish(const GemmArgs& a, const ResidRows& r, const float4 (&
     if (t >= te) break;
     const float4 xv = f4_add(r.x[k], acc[k]);
     if (live && st) {
-      *reinterpret_cast<float4*>(a.x + (size_t)t * a.N + f) = xv;
-      store_act4(a.y_out, (size_t)t * a.N + f, (size_t)kMaxT * a.N,
+      *reinterpret_cast<float4*>(a.x + (size_t)(tok0 + t) * a.N + f) = xv;
+      store_act4(a.y_out, (size_t)(tok0 + t) * a.N + f, (size_t)kLdr<CHUNK> * a.N,
                  make_float4(g.x * xv.x, g.y * xv.y, g.z * xv.z, g.w * xv.w));
     }
     const float sq = warp_sum(live ? xv.x * xv.x + xv.y * xv.y + xv.z * xv.z + xv.w * xv.w : 0.f);
-    if (l == 0 && st) a.ss_out[(size_t)tile * kMaxT + t] = sq;
+    if (l == 0 && st) a.ss_out[(size_t)tile * kLdr<CHUNK> + tok0 + t] = sq;
   }
 }
 
@@ -279,13 +290,14 @@ OOS_DEV void resid_finish(const GemmArgs& a, const ResidRows& r, const float4 (&
 struct QkvRows {
   float2 cs[kFinRows][4];
 };
-OOS_DEV void qkv_load(const GemmArgs& a, QkvRows& r, int kind, int t0, int te, int w) {
+template <bool CHUNK>
+OOS_DEV void qkv_load(const GemmArgs& a, QkvRows& r, int kind, int tok0, int t0, int te, int w) {
   const int m0 = 4 * (threadIdx.x & 15);   // rotary frequency index of this lane's first feature
 #pragma unroll
   for (int k = 0; k < kFinRows; ++k) {
     const int t = t0 + w + kEpiWarps * k;
     const bool ok = kind < 2 && t < te;
-    const float4* p = reinterpret_cast<const float4*>(a.rope + (size_t)t * (kTile / 2) + m0);
+    const float4* p = reinterpret_cast<const float4*>(a.rope + (size_t)(tok0 + t) * (kTile / 2) + m0);
     const float4 u = ok ? __ldcg(p) : make_float4(1.f, 0.f, 1.f, 0.f);
     const float4 v = ok ? __ldcg(p + 1) : make_float4(1.f, 0.f, 1.f, 0.f);
     r.cs[k][0] = make_float2(u.x, u.y);
@@ -295,8 +307,9 @@ OOS_DEV void qkv_load(const GemmArgs& a, QkvRows& r, int kind, int t0, int te, i
   }
 }
 // one head (kind 0: q, 1: k, 2: v) of the tokens of a pass
+template <bool CHUNK>
 OOS_DEV void qkv_finish(const GemmArgs& a, const QkvRows& r, const float4 (&acc)[kFinRows], float4 b4, bool norm,
-                        float4 g4, int kind, int h, int ctx, const float* rms, bool st, int t0, int te, int w) {
+                        float4 g4, int kind, int h, int ctx, const float* rms, bool st, int tok0, int t0, int te, int w) {
   const int l = threadIdx.x & 31;
   const bool first_half = l < 16;   // features 0..63 pair with 64..127 held by lane ^ 16
 #pragma unroll
@@ -323,11 +336,11 @@ OOS_DEV void qkv_finish(const GemmArgs& a, const QkvRows& r, const float4 (&acc)
     if (!st) {
       asm volatile("" ::"f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]));
     } else if (kind == 0) {   // q as hi/lo halves in the cache's 16-bit format: the attention product sees ~16-bit q
-      const size_t qi = ((size_t)t * a.nq + h) * kTile + 4 * l, lo_off = (size_t)kMaxT * a.nq * kTile;
+      const size_t qi = ((size_t)(tok0 + t) * a.nq + h) * kTile + 4 * l, lo_off = (size_t)kLdr<CHUNK> * a.nq * kTile;
       if (a.kv_f16) store_act4_h(reinterpret_cast<__half*>(a.q_out), qi, lo_off, make_float4(v[0], v[1], v[2], v[3]));
       else store_act4(a.q_out, qi, lo_off, make_float4(v[0], v[1], v[2], v[3]));
     } else {           // K/V in the cache's format (bf16, or binary16)
-      __nv_bfloat16* dst = (kind == 1 ? a.kc : a.vc) + ((size_t)(ctx + t) * a.nkv + h) * kTile;
+      __nv_bfloat16* dst = (kind == 1 ? a.kc : a.vc) + ((size_t)(ctx + tok0 + t) * a.nkv + h) * kTile;
       uint2 o;
       if (a.kv_f16) {
         __half hv[4];
@@ -345,7 +358,7 @@ OOS_DEV void qkv_finish(const GemmArgs& a, const QkvRows& r, const float4 (&acc)
   }
 }
 
-template <int BN, int EPI>
+template <int BN, int EPI, bool CHUNK>
 __global__ void __launch_bounds__(kGemmThreads, 1)
     k_gemm_tc(const __grid_constant__ CUtensorMap wm0, const __grid_constant__ CUtensorMap wm1,
               const __grid_constant__ CUtensorMap wm2, const __grid_constant__ CUtensorMap am,
@@ -379,12 +392,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 
   // this CTA's work: k-blocks [kb0, kb0 + n_units) of tile `first` (cluster), or
   // all k-blocks of tiles first, first + step, ...
-  int first, step, kb0, nkb, n_units;
+  int first, step, kb0, nkb, n_units, tok0 = 0;
   uint32_t rank = 0;
   if (CLUSTER) {
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
     first = blockIdx.x / a.split;
     step = 0;
+    if (CHUNK) {
+      tok0 = first / a.n_work * kTile;
+      first %= a.n_work;
+    }
     kb0 = a.kbt * (int)rank / a.split;
     nkb = n_units = a.kbt * ((int)rank + 1) / a.split - kb0;
   } else {
@@ -392,8 +409,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     step = gridDim.x;
     kb0 = 0;
     nkb = a.kbt;
-    n_units = first < a.n_work ? (a.n_work - first + step - 1) / step * a.kbt : 0;
+    if (CHUNK) {   // one tile per CTA
+      tok0 = first / a.n_work * kTile;
+      first %= a.n_work;
+      n_units = a.kbt;
+    } else {
+      n_units = first < a.n_work ? (a.n_work - first + step - 1) / step * a.kbt : 0;
+    }
   }
+  const int T = CHUNK ? min(a.T - tok0, kMaxT) : a.T;   // tokens of this CTA's tiles
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
@@ -428,25 +452,30 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       const uint32_t stage_bytes = (uint32_t)(kSub * a_bytes + 2 * C::B_BYTES);
       // weights of the unit at (tile, kb) into `stage`; rows past the matrix
       // read zeros (TMA out-of-bounds fill)
+      auto load_sub = [&](const CUtensorMap* wm, unsigned char* dst, int kb, int row, int stage) {
+        tma_load_2d(dst, wm, &full[stage], kb * kBK, row, pol_w);
+        if (CHUNK && CLUSTER)   // the chunk's boxes are 64 rows high
+          tma_load_2d(dst + 64 * kBK * 2, wm, &full[stage], kb * kBK, row + 64, pol_w);
+      };
       auto load_w = [&](int tile, int kb, int stage) {
         unsigned char* dst = ring + stage * kSub * a_bytes;
         if (EPI == EPI_SILU) {
-          tma_load_2d(dst, &wm0, &full[stage], kb * kBK, tile * a.rows, pol_w);
-          tma_load_2d(dst + a_bytes, &wm1, &full[stage], kb * kBK, tile * a.rows, pol_w);
+          load_sub(&wm0, dst, kb, tile * a.rows, stage);
+          load_sub(&wm1, dst + a_bytes, kb, tile * a.rows, stage);
         } else if (EPI == EPI_QKV) {
           const CUtensorMap* wm = tile < a.seg_tiles[0] ? &wm0 : tile < a.seg_tiles[1] ? &wm1 : &wm2;
           const int base = tile < a.seg_tiles[0] ? 0 : tile < a.seg_tiles[1] ? a.seg_tiles[0] : a.seg_tiles[1];
-          tma_load_2d(dst, wm, &full[stage], kb * kBK, (tile - base) * a.rows, pol_w);
+          load_sub(wm, dst, kb, (tile - base) * a.rows, stage);
         } else {
 #pragma unroll
           for (int sub = 0; sub < kSub; ++sub)
-            tma_load_2d(dst + sub * a_bytes, &wm0, &full[stage], kb * kBK, (tile * kSub + sub) * a.rows, pol_w);
+            load_sub(&wm0, dst + sub * a_bytes, kb, (tile * kSub + sub) * a.rows, stage);
         }
       };
       auto load_x = [&](int kb, int stage) {
         unsigned char* dst = ring_x + stage * 2 * C::B_BYTES;
-        tma_load_2d(dst, &am, &full[stage], kb * kBK, 0, pol_a);                   // hi rows
-        tma_load_2d(dst + C::B_BYTES, &am, &full[stage], kb * kBK, kMaxT, pol_a);  // lo rows
+        tma_load_2d(dst, &am, &full[stage], kb * kBK, tok0, pol_a);                       // hi rows
+        tma_load_2d(dst + C::B_BYTES, &am, &full[stage], kb * kBK, kLdr<CHUNK> + tok0, pol_a);  // lo rows
       };
       // weights do not depend on the previous kernel: start streaming them
       // before waiting for it (programmatic dependent launch)
@@ -587,7 +616,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   if (CLUSTER && warp >= 2) {
     const int tile = first;
     // tokens [tb, te) are finished here
-    const int tb = a.T * (int)rank / a.split, te = a.T * ((int)rank + 1) / a.split;
+    const int tb = T * (int)rank / a.split, te = T * ((int)rank + 1) / a.split;
     const int f = EPI == EPI_RESID ? tile * a.rows + 4 * lane : 4 * lane;
     const bool live = 4 * lane < a.rows && (EPI != EPI_RESID || f < a.N);
     const bool two = nkb >= 2;   // one accumulator per k-segment
@@ -626,12 +655,12 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       }
       // what the finishing reads, while the weights stream
       if (EPI == EPI_RESID) {
-        resid_load(a, rr, f, live, t0, te, ew);
+        resid_load<CHUNK>(a, rr, f, live, tok0, t0, te, ew);
       } else {
-        qkv_load(a, qr, kind, t0, te, ew);
+        qkv_load<CHUNK>(a, qr, kind, tok0, t0, te, ew);
         if (pass <= 0) {
           ctx = *a.ctx;
-          input_rms(a, rms, tb, te, ew);
+          input_rms<CHUNK>(a, rms, tok0, tb, te, ew);
         }
       }
       if (pass <= 0) {
@@ -645,7 +674,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         const bool put = have && row < a.rows;
 #pragma unroll 1
         for (int cc = half; cc < BN / 16; cc += 2) {
-          if (cc * 16 >= a.T) break;
+          if (cc * 16 >= T) break;
           float v[16];
           acc16((uint32_t)(cc * 16), v);
           if (two) {
@@ -680,8 +709,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         for (int k = 0; k < kFinRows; ++k) asm volatile("" ::"f"(acc[k].x), "f"(acc[k].y), "f"(acc[k].z), "f"(acc[k].w) : "memory");
         cluster_arrive_relaxed();
       }
-      if (EPI == EPI_RESID) resid_finish(a, rr, acc, g4, tile, f, live, have, t0, te, ew);
-      else qkv_finish(a, qr, acc, b4, norm, g4, kind, h, ctx, rms, have, t0, te, ew);
+      if (EPI == EPI_RESID) resid_finish<CHUNK>(a, rr, acc, g4, tile, f, live, have, tok0, t0, te, ew);
+      else qkv_finish<CHUNK>(a, qr, acc, b4, norm, g4, kind, h, ctx, rms, have, tok0, t0, te, ew);
     }
     __syncwarp();
     cluster_wait_acquire();
@@ -709,7 +738,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         pdl_trigger();
       }
       if (it <= 0) {
-        input_rms(a, rms, 0, a.T, ew);
+        input_rms<CHUNK>(a, rms, tok0, 0, T, ew);
         epi_bar();
       }
       if (!dry) {
@@ -726,7 +755,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       const bool live = row < a.rows && fi < a.N && !dry;
 #pragma unroll 1
       for (int cc = half; cc < BN / 16; cc += 2) {
-        if (cc * 16 >= a.T) break;
+        if (cc * 16 >= T) break;
         float g[16], u[16];
         acc16(col0 + cc * 16, g);
         acc16(col0 + C::SUB_COLS + cc * 16, u);
@@ -754,10 +783,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
           const int t = cc * 16 + i + (odd ? 1 : 0);
           const __nv_bfloat162 hi = __floats2bfloat162_rn(v0, v1);
           const __nv_bfloat162 lo = __floats2bfloat162_rn(v0 - __low2float(hi), v1 - __high2float(hi));
-          if (live && t < a.T) {
-            __nv_bfloat16* dst = a.act_out + (size_t)t * a.N + fi;
+          if (live && t < T) {
+            __nv_bfloat16* dst = a.act_out + (size_t)(tok0 + t) * a.N + fi;
             *reinterpret_cast<__nv_bfloat162*>(dst) = hi;
-            *reinterpret_cast<__nv_bfloat162*>(dst + (size_t)kMaxT * a.N) = lo;
+            *reinterpret_cast<__nv_bfloat162*>(dst + (size_t)kLdr<CHUNK> * a.N) = lo;
           }
         }
       }
@@ -776,7 +805,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     pdl_wait();
     pdl_trigger();
     const int e = threadIdx.x - 64;       // 0..kEpiThreads-1
-    input_rms(a, rms, 0, a.T, ew);
+    input_rms<CHUNK>(a, rms, tok0, 0, T, ew);
     epi_bar();
     int acc = 0;
     uint32_t use = 0;
@@ -795,7 +824,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         const int f = (tile * kSub + sub) * kTile + row;
 #pragma unroll 1
         for (int cc = half; cc < BN / 16; cc += 2) {
-          if (cc * 16 >= a.T) break;
+          if (cc * 16 >= T) break;
           float v[16];
           acc16(col0 + sub * C::SUB_COLS + cc * 16, v);
 #pragma unroll
@@ -820,7 +849,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(&acce[acc]);
       epi_bar();
-      if (e < a.T) {
+      if (e < T) {
         Top2s r = run[e];
 #pragma unroll
         for (int w = 0; w < 4; ++w) r = t2_merge(r, red[w * BN + e]);
@@ -830,7 +859,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       ++use;
       acc ^= 1;
     }
-    if (e < a.T) {
+    if (e < T) {
       const Top2s r = run[e];
       a.am_v1[(size_t)blockIdx.x * kMaxT + e] = r.v1;
       a.am_i[(size_t)blockIdx.x * kMaxT + e] = r.i1;
@@ -898,7 +927,7 @@ bool encode_bf16_map(CUtensorMap* map, const void* ptr, int rank, const uint64_t
   return r == CUDA_SUCCESS;
 }
 
-bool encode_weight_map(CUtensorMap* map, const void* ptr, int rows, int K, int box_rows) {
+bool encode_rows_map(CUtensorMap* map, const void* ptr, int rows, int K, int box_rows) {
   return encode_2d(map, ptr, rows, K, box_rows);
 }
 bool encode_act_map(CUtensorMap* map, const void* ptr, int K, int box_rows) {
@@ -907,11 +936,11 @@ bool encode_act_map(CUtensorMap* map, const void* ptr, int K, int box_rows) {
 
 int bn_index(int T) { return T <= 16 ? 0 : T <= 32 ? 1 : T <= 64 ? 2 : 3; }
 
-template <int BN, int EPI>
+template <int BN, int EPI, bool CHUNK = false>
 static cudaError_t set_smem() {
   // the depth of the ring, and so the size, depends on the plan's tile rows:
   // allow the most any plan takes
-  return cudaFuncSetAttribute(k_gemm_tc<BN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmemMax);
+  return cudaFuncSetAttribute(k_gemm_tc<BN, EPI, CHUNK>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmemMax);
 }
 
 template <int BN>
@@ -928,11 +957,18 @@ cudaError_t gemm_setup() {
   if (e == cudaSuccess) e = set_smem_all<32>();
   if (e == cudaSuccess) e = set_smem_all<64>();
   if (e == cudaSuccess) e = set_smem_all<128>();
+  if (e == cudaSuccess) e = set_smem<128, EPI_QKV, true>();
+  if (e == cudaSuccess) e = set_smem<128, EPI_RESID, true>();
+  if (e == cudaSuccess) e = set_smem<128, EPI_SILU, true>();
   return e;
 }
 
-// clusters of `c` GEMM CTAs resident at once (one CTA per SM)
-static int gemm_max_clusters(int c) {
+// Clusters of `c` GEMM CTAs resident at once (one CTA per SM).  Not every place the
+// occupancy query counts is free when the clusters arrive (odd sizes leave SM
+// pairs half used, and the previous kernel's CTAs go one by one), and a cluster
+// left over runs after all the others: 46 clusters of 3 took 98 us where 43 take
+// 55, so a margin is kept.
+int gemm_fit(int c) {
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3(c);
   lc.blockDim = dim3(kGemmThreads);
@@ -945,10 +981,11 @@ static int gemm_max_clusters(int c) {
   lc.attrs = attr;
   lc.numAttrs = 1;
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, (const void*)k_gemm_tc<64, EPI_RESID>, &lc) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&n, (const void*)k_gemm_tc<64, EPI_RESID, false>, &lc) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
+  if (c > 1) n -= (c & 1) ? (n + 11) / 12 : 1;
   return n;
 }
 
@@ -956,18 +993,13 @@ static int gemm_max_clusters(int c) {
 // splits whose clusters fit the GPU, the one whose CTAs move the fewest bytes
 // in sequence, weights and activations (for 64 nodes) together, with a charge
 // per split for the sums it pulls and one per extra wave for a second prologue
-// and epilogue (~8 us at ~80 KB/us).  Not every place the occupancy query
-// counts is free when the clusters arrive (odd sizes leave SM pairs half used,
-// and the previous kernel's CTAs go one by one), and a cluster left over runs
-// after all the others: 46 clusters of 3 took 98 us where 43 take 55, so a
-// margin is kept.
+// and epilogue (~8 us at ~80 KB/us).
 GemmPlan plan_cluster(int N, int K, bool whole_heads) {
   GemmPlan best = {};
   long long best_cost = -1;
   const int kbt = K / kBK;
   for (int c = 1; c <= kMaxSplit && c <= kbt; ++c) {
-    int fit = gemm_max_clusters(c);
-    if (c > 1) fit -= (c & 1) ? (fit + 11) / 12 : 1;
+    const int fit = gemm_fit(c);
     if (fit < 1) continue;
     int rows = kTile;
     if (!whole_heads && N < kTile * fit) rows = ((N + fit - 1) / fit + 7) / 8 * 8;
@@ -992,20 +1024,22 @@ GemmPlan plan_rows(int N, int K, int n_sms) {
   return GemmPlan{rows, n_work, K / kBK, 1, n_work < n_sms ? n_work : n_sms};
 }
 
-template <int BN, int EPI>
-static cudaError_t launch_tc(Model& m, const GemmW& g, const CUtensorMap& amap, GemmArgs& a, cudaStream_t st) {
+// grid: CTAs, `split` times the tiles for the cluster GEMMs
+template <int BN, int EPI, bool CHUNK = false>
+static cudaError_t launch_tc(Model& m, const GemmW& g, const CUtensorMap& amap, int grid, GemmArgs& a, cudaStream_t st) {
   using C = TcCfg<BN, EPI>;
-  a.stages = C::stages(g.plan.rows);
+  a.stages = C::stages(a.rows);
+  const CUtensorMap* maps = CHUNK ? g.pf_map : g.map;
   cudaLaunchConfig_t lc = {};
-  lc.gridDim = dim3(g.plan.grid);
+  lc.gridDim = dim3(grid);
   lc.blockDim = dim3(kGemmThreads);
-  lc.dynamicSmemBytes = (size_t)C::smem(g.plan.rows);
+  lc.dynamicSmemBytes = (size_t)C::smem(a.rows);
   lc.stream = st;
   cudaLaunchAttribute attr[2];
   int n = 0;
   if (EpiOf<EPI>::cluster) {
     attr[n].id = cudaLaunchAttributeClusterDimension;
-    attr[n].val.clusterDim.x = g.plan.split;
+    attr[n].val.clusterDim.x = a.split;
     attr[n].val.clusterDim.y = 1;
     attr[n].val.clusterDim.z = 1;
     ++n;
@@ -1017,19 +1051,19 @@ static cudaError_t launch_tc(Model& m, const GemmW& g, const CUtensorMap& amap, 
   }
   lc.attrs = attr;
   lc.numAttrs = n;
-  const CUtensorMap& w1 = g.n_seg > 1 ? g.map[1] : g.map[0];
-  const CUtensorMap& w2 = g.n_seg > 2 ? g.map[2] : g.map[0];
-  return cudaLaunchKernelEx(&lc, k_gemm_tc<BN, EPI>, g.map[0], w1, w2, amap, a);
+  const CUtensorMap& w1 = g.n_seg > 1 ? maps[1] : maps[0];
+  const CUtensorMap& w2 = g.n_seg > 2 ? maps[2] : maps[0];
+  return cudaLaunchKernelEx(&lc, k_gemm_tc<BN, EPI, CHUNK>, maps[0], w1, w2, amap, a);
 }
 
 template <int EPI>
 static cudaError_t dispatch_tc(Model& m, const GemmW& g, const CUtensorMap* amaps, int T, GemmArgs& a,
                                cudaStream_t st) {
   switch (bn_index(T)) {
-    case 0: return launch_tc<16, EPI>(m, g, amaps[0], a, st);
-    case 1: return launch_tc<32, EPI>(m, g, amaps[1], a, st);
-    case 2: return launch_tc<64, EPI>(m, g, amaps[2], a, st);
-    default: return launch_tc<128, EPI>(m, g, amaps[3], a, st);
+    case 0: return launch_tc<16, EPI>(m, g, amaps[0], g.plan.grid, a, st);
+    case 1: return launch_tc<32, EPI>(m, g, amaps[1], g.plan.grid, a, st);
+    case 2: return launch_tc<64, EPI>(m, g, amaps[2], g.plan.grid, a, st);
+    default: return launch_tc<128, EPI>(m, g, amaps[3], g.plan.grid, a, st);
   }
 }
 
@@ -1057,7 +1091,7 @@ int norm_chunks(const Model& m, int layer) {
   return layer == 0 ? (m.cfg.hidden + kTile - 1) / kTile : m.g_down[layer - 1].plan.n_work;
 }
 
-cudaError_t launch_gemm_qkv(Model& m, int layer, void* kc, void* vc, int T, cudaStream_t st) {
+static GemmArgs qkv_args(Model& m, int layer, void* kc, void* vc, int T) {
   const auto& c = m.cfg;
   const oos_layer_weights& L = m.layers[layer];
   GemmArgs a = base_args(m, m.g_qkv[layer], T, layer * 4);
@@ -1078,6 +1112,11 @@ cudaError_t launch_gemm_qkv(Model& m, int layer, void* kc, void* vc, int T, cuda
   a.vc = (__nv_bfloat16*)vc;
   a.ctx = m.ws.ctx;
   a.kv_f16 = c.kv_f16 ? 1 : 0;
+  return a;
+}
+
+cudaError_t launch_gemm_qkv(Model& m, int layer, void* kc, void* vc, int T, cudaStream_t st) {
+  GemmArgs a = qkv_args(m, layer, kc, vc, T);
   return dispatch_tc<EPI_QKV>(m, m.g_qkv[layer], m.amap_xn, T, a, st);
 }
 
@@ -1105,6 +1144,42 @@ cudaError_t launch_gemm_gu(Model& m, int layer, int T, cudaStream_t st) {
   a.ss_chunks = m.g_o[layer].plan.n_work;
   a.act_out = (__nv_bfloat16*)m.ws.act;
   return dispatch_tc<EPI_SILU>(m, m.g_gu[layer], m.amap_xn, T, a, st);
+}
+
+// ---- a prefill chunk in token tiles of 128 (prefill.cu chooses between these
+// and its own tiles): 128 weight rows a tile (64 of gate and up), buffers of
+// kPfTokens rows, norm sums per 128 features as prefill.cu writes them
+static void chunk_args(Model& m, GemmArgs& a, int rows, int n_work, int split) {
+  a.rows = rows;
+  a.n_work = n_work;
+  a.split = split;
+  a.ss_in = m.ws.pf_ss;
+  a.ss_chunks = m.cfg.hidden / kTile;
+}
+static int chunk_tiles(const GemmArgs& a) { return a.n_work * ((a.T + kTile - 1) / kTile); }
+cudaError_t launch_chunk_qkv(Model& m, int layer, void* kc, void* vc, int T, int split, cudaStream_t st) {
+  GemmArgs a = qkv_args(m, layer, kc, vc, T);
+  chunk_args(m, a, kTile, m.cfg.n_q_heads + 2 * m.cfg.n_kv_heads, split);
+  a.rope = m.ws.pf_rope;
+  a.q_out = (__nv_bfloat16*)m.ws.pf_q;
+  return launch_tc<128, EPI_QKV, true>(m, m.g_qkv[layer], m.pf_xn_map, chunk_tiles(a) * split, a, st);
+}
+cudaError_t launch_chunk_resid(Model& m, int layer, bool down, const void* gain, int T, int split, cudaStream_t st) {
+  const GemmW& g = down ? m.g_down[layer] : m.g_o[layer];
+  GemmArgs a = base_args(m, g, T, layer * 4 + (down ? 3 : 1));
+  chunk_args(m, a, kTile, g.N / kTile, split);
+  a.x = m.ws.pf_x;
+  a.gain = (const __nv_bfloat16*)gain;
+  a.y_out = (__nv_bfloat16*)m.ws.pf_xn;
+  a.ss_out = m.ws.pf_ss;
+  return launch_tc<128, EPI_RESID, true>(m, g, down ? m.pf_act_map : m.pf_attn_map, chunk_tiles(a) * split, a, st);
+}
+cudaError_t launch_chunk_gu(Model& m, int layer, int T, cudaStream_t st) {
+  const GemmW& g = m.g_gu[layer];
+  GemmArgs a = base_args(m, g, T, layer * 4 + 2);
+  chunk_args(m, a, 64, g.N / 64, 1);
+  a.act_out = (__nv_bfloat16*)m.ws.pf_act;
+  return launch_tc<128, EPI_SILU, true>(m, g, m.pf_xn_map, chunk_tiles(a), a, st);
 }
 
 cudaError_t launch_lm_head_tc(Model& m, int T, cudaStream_t st) {

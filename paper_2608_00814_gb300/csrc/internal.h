@@ -17,6 +17,7 @@ constexpr int kTile = 128;          // weight rows per MMA (tcgen05 M)
 constexpr int kLmRows = 256;        // vocabulary rows per work tile of the LM head
 constexpr int kBK = 64;             // reduction elements per pipeline stage (128 bytes of bf16)
 constexpr int kMaxLayers = 128;
+constexpr int kPfTokens = 2048;     // prompt tokens per prefill chunk (bf16 path)
 constexpr int kMaxGridCTAs = 1024;  // upper bound on CTAs of the LM head
 constexpr int kMaxHidden = 8192;    // bf16 models
 constexpr int kMaxInter = 32768;
@@ -35,7 +36,8 @@ struct GemmPlan {
 // One weight GEMM of the bf16 path: up to three matrices (q|k|v, gate|up), each
 // with its own TMA descriptor.
 struct GemmW {
-  CUtensorMap map[3];
+  CUtensorMap map[3];      // boxes of plan.rows weight rows
+  CUtensorMap pf_map[3];   // prefill: boxes of 64 rows
   int n_seg;
   int N, K;     // output rows (gate/up: of one matrix), reduction length
   GemmPlan plan;
@@ -64,6 +66,12 @@ struct Workspace {
   float2* rope;              // (cos, sin) per node and rotary pair [kMaxT][d/2] (bf16 path)
   int32_t* chain_parent;     // [kMaxT]: -1, 0, 1, ... (the chains a prefill runs as trees)
   int32_t* pf_scratch;       // prefill's unused accept outputs: len, bonus, nodes[kMaxT], tokens[kMaxT]
+  // prefill chunks (bf16 path): the buffers above for kPfTokens rows.  act
+  // shares its memory with q and attn, which are dead when it is written.
+  float* pf_x;
+  void *pf_xn, *pf_q, *pf_attn, *pf_act;
+  float* pf_ss;              // [hidden / 128][kPfTokens]
+  float2* pf_rope;           // [kPfTokens][d/2]
 };
 
 // shape + addresses a captured verify graph was recorded with.  The committed
@@ -96,6 +104,9 @@ struct Model {
   std::vector<GemmW> g_qkv, g_o, g_gu, g_down;
   GemmW g_lm;
   CUtensorMap amap_xn[4], amap_attn[4], amap_act[4];  // per N-tile variant 16/32/64/128
+  CUtensorMap pf_xn_map, pf_attn_map, pf_act_map;     // prefill: boxes of 128 rows
+  CUtensorMap pf_qmap_hi, pf_qmap_lo;
+  int fit[9] = {0};               // gemm_fit of 1..8
   CUtensorMap qmap_hi, qmap_lo;   // attention: q rows of one kv head, (d, head in group, kv head, node)
   // attention: the K/V cache maps encoded per layer over the whole capacity
   // (re-encoded only when the cache buffers change)
@@ -146,6 +157,7 @@ cudaError_t set_tree_prep_ctx(Model& m, cudaGraphExec_t ex, cudaGraphNode_t node
                               const int32_t* parent, int T, int ctx);
 cudaError_t launch_embed_norm(Model& m, const int32_t* tokens, int T, cudaStream_t st);
 cudaError_t launch_embed_tc(Model& m, const int32_t* tokens, int T, cudaStream_t st);
+cudaError_t launch_embed_pf(Model& m, const int32_t* tokens, int T, cudaStream_t st);
 cudaError_t launch_final_hidden(Model& m, float* hidden, int T, cudaStream_t st);
 cudaError_t launch_qkv_post(Model& m, int layer, void* kc, void* vc, int T, cudaStream_t st);
 cudaError_t launch_resid_norm(Model& m, const void* gain, float* hidden_out, int T, cudaStream_t st);
@@ -168,7 +180,7 @@ cudaError_t launch_accept_walk(const int32_t* tokens, const int32_t* parent, con
 bool encode_bf16_map(CUtensorMap* map, const void* ptr, int rank, const uint64_t* dims, const uint64_t* strides,
                      const uint32_t* box, bool f16 = false);
 bool encode_act_map(CUtensorMap* map, const void* ptr, int K, int box_rows);
-bool encode_weight_map(CUtensorMap* map, const void* ptr, int rows, int K, int box_rows);
+bool encode_rows_map(CUtensorMap* map, const void* ptr, int rows, int K, int box_rows);
 int bn_index(int T);   // N-tile variant for T tree nodes: 0..3 -> 16/32/64/128
 cudaError_t gemm_setup();
 cudaError_t launch_gemm_qkv(Model& m, int layer, void* kc, void* vc, int T, cudaStream_t st);
@@ -176,9 +188,14 @@ cudaError_t launch_gemm_o(Model& m, int layer, int T, cudaStream_t st);
 cudaError_t launch_gemm_gu(Model& m, int layer, int T, cudaStream_t st);
 cudaError_t launch_gemm_down(Model& m, int layer, int T, cudaStream_t st);
 cudaError_t launch_lm_head_tc(Model& m, int T, cudaStream_t st);
+constexpr int kMaxSplit = 8;                             // CTAs sharing a GEMM tile
+int gemm_fit(int c);                                     // clusters of c CTAs resident at once (after gemm_setup)
 GemmPlan plan_cluster(int N, int K, bool whole_heads);   // after gemm_setup
 GemmPlan plan_rows(int N, int K, int n_sms);
 int norm_chunks(const Model& m, int layer);
+cudaError_t launch_chunk_qkv(Model& m, int layer, void* kc, void* vc, int T, int split, cudaStream_t st);
+cudaError_t launch_chunk_resid(Model& m, int layer, bool down, const void* gain, int T, int split, cudaStream_t st);
+cudaError_t launch_chunk_gu(Model& m, int layer, int T, cudaStream_t st);
 cudaError_t launch_gemm_f32(Model& m, const void* w0, const void* w1, const void* w2, int rows0, int rows1,
                             int rows2, int K, const void* x, int T, cudaStream_t st);
 cudaError_t launch_lm_head_f32(Model& m, int T, cudaStream_t st);
@@ -209,6 +226,16 @@ bool attn_encode_q_maps(Model& m);     // TMA maps of the q buffer (bf16 path), 
 cudaError_t launch_attention(Model& m, int layer, const void* kc, const void* vc, int capacity, int ctx, int T,
                              cudaStream_t st);
 int attn_splits(Model& m, int ctx_hint, int T);
+// causal attention of a prefill chunk of T <= kPfTokens tokens
+cudaError_t launch_attention_pf(Model& m, int layer, const void* kc, const void* vc, int capacity, int ctx, int T,
+                                cudaStream_t st);
+
+// ---- prefill (prefill.cu, bf16 path)
+cudaError_t prefill_setup();
+bool prefill_encode(Model& m);
+cudaError_t prefill_chunk(Model& m, const oos_kv_cache* kv, int ctx, const int32_t* tokens, int T, bool first,
+                          cudaStream_t st);
+cudaError_t prefill_last(Model& m, int T, cudaStream_t st);
 
 }  // namespace oos
 

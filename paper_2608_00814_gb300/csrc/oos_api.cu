@@ -60,6 +60,21 @@ size_t carve_workspace(const oos_model_config& c, int n_sms, uint8_t* base, Work
   w.rope = (float2*)take((size_t)kMaxT * (c.head_dim / 2) * 8);
   w.chain_parent = (int32_t*)take(kMaxT * 4);
   w.pf_scratch = (int32_t*)take((2 + 2 * kMaxT) * 4);
+  if (c.dtype == OOS_DTYPE_BF16) {
+    const size_t P = kPfTokens;
+    w.pf_x = (float*)take(P * H * 4);
+    w.pf_xn = take(2 * P * H * 2);
+    const size_t q_bytes = 2 * P * qd * 2;   // a multiple of 256
+    w.pf_act = take(std::max(2 * q_bytes, 2 * P * I * 2));
+    w.pf_q = w.pf_act;
+    w.pf_attn = base ? (uint8_t*)w.pf_act + q_bytes : nullptr;
+    w.pf_ss = (float*)take(H / 128 * P * 4);
+    w.pf_rope = (float2*)take(P * (c.head_dim / 2) * 8);
+  } else {
+    w.pf_x = w.pf_ss = nullptr;
+    w.pf_xn = w.pf_q = w.pf_attn = w.pf_act = nullptr;
+    w.pf_rope = nullptr;
+  }
   if (ws) *ws = w;
   return align_up(off, 256);
 }
@@ -201,25 +216,37 @@ int enqueue_verify_dev(Model& m, const oos_kv_cache* kv, const int32_t* ctx_dev,
                         nullptr, nullptr, st);
 }
 
-// Prefill: the prompt as chains of at most max_T tokens.  In a chain node j's
-// ancestors are nodes 0..j and its depth is j, so each chunk's tree pass is
-// causal decoding of the chunk after everything before it, and node j's K/V
-// land in their final slot ctx + off + j (no compaction).  Only the last chunk
-// runs the LM head: the argmax of its last node is the greedy next token.
+// Prefill.  bf16 models: chunks of up to kPfTokens tokens through the
+// compute-bound kernels of prefill.cu.  A chunk that fits one tree (and every
+// chunk of an fp32 model) runs through the verify kernels as a chain: node j's
+// ancestors are nodes 0..j and its depth is j, so a tree pass is causal decoding
+// of the chunk after everything before it, and node j's K/V land in their final
+// slot.  Only the prompt's last token runs the LM head: its argmax is the greedy
+// next token.
 static int prefill_impl(Model& m, const oos_kv_cache* kv, int ctx, const int32_t* tokens, int n, int32_t* next_token,
                         cudaStream_t st) {
   const auto& c = m.cfg;
+  const bool tc = c.dtype == OOS_DTYPE_BF16;
   int32_t* sc = m.ws.pf_scratch;
-  for (int off = 0; off < n; off += c.max_T) {
-    const int T = std::min(c.max_T, n - off);
-    const int rc = enqueue_layers(m, kv, ctx + off, nullptr, tokens + off, m.ws.chain_parent, T, nullptr, st);
-    if (rc != OOS_OK) return rc;
-    if (off + T < n) continue;
-    if (c.dtype == OOS_DTYPE_BF16) OOS_TRY(launch_lm_head_tc(m, T, st));
-    else OOS_TRY(launch_lm_head_f32(m, T, st));
-    OOS_TRY(launch_argmax_accept(m, tokens + off, m.ws.chain_parent, T, nullptr, m.lm_grid, sc, sc + 2,
+  int T = 0;
+  for (int off = 0; off < n; off += T) {
+    T = std::min(tc ? kPfTokens : c.max_T, n - off);
+    const bool wide = tc && T > kMaxT;
+    const bool last = off + T == n;
+    if (wide) {
+      OOS_TRY(prefill_chunk(m, kv, ctx + off, tokens + off, T, off == 0, st));
+      if (last) OOS_TRY(prefill_last(m, T, st));
+    } else {
+      const int rc = enqueue_layers(m, kv, ctx + off, nullptr, tokens + off, m.ws.chain_parent, T, nullptr, st);
+      if (rc != OOS_OK) return rc;
+    }
+    if (!last) continue;
+    const int rows = wide ? 1 : T;   // rows the LM head sees, the prompt's last token the last of them
+    if (tc) OOS_TRY(launch_lm_head_tc(m, rows, st));
+    else OOS_TRY(launch_lm_head_f32(m, rows, st));
+    OOS_TRY(launch_argmax_accept(m, tokens + n - rows, m.ws.chain_parent, rows, nullptr, m.lm_grid, sc, sc + 2,
                                  sc + 2 + kMaxT, sc + 1, nullptr, nullptr, nullptr, st));
-    if (next_token) OOS_TRY(cudaMemcpyAsync(next_token, m.ws.argmax + (T - 1), 4, cudaMemcpyDeviceToDevice, st));
+    if (next_token) OOS_TRY(cudaMemcpyAsync(next_token, m.ws.argmax + (rows - 1), 4, cudaMemcpyDeviceToDevice, st));
   }
   return OOS_OK;
 }
@@ -357,7 +384,8 @@ int oos_model_create(const oos_model_config* cfg, const oos_weights* w, void* wo
       rc = OOS_ECUDA;
       break;
     }
-    if (gemm_setup() != cudaSuccess || attn_setup() != cudaSuccess || compact_setup() != cudaSuccess) {
+    if (gemm_setup() != cudaSuccess || attn_setup() != cudaSuccess || compact_setup() != cudaSuccess ||
+        prefill_setup() != cudaSuccess) {
       rc = OOS_ECUDA;
       break;
     }
@@ -367,13 +395,16 @@ int oos_model_create(const oos_model_config* cfg, const oos_weights* w, void* wo
       auto mk = [&](GemmW& g, const void* const* ptrs, const int* rows, int nseg, int K, const GemmPlan& plan) -> bool {
         memset(&g, 0, sizeof(g));
         for (int s = 0; s < nseg; ++s)
-          if (!encode_weight_map(&g.map[s], ptrs[s], rows[s], K, plan.rows)) return false;
+          if (!encode_rows_map(&g.map[s], ptrs[s], rows[s], K, plan.rows) ||
+              !encode_rows_map(&g.pf_map[s], ptrs[s], rows[s], K, 64))
+            return false;
         g.n_seg = nseg;
         g.N = rows[0];
         g.K = K;
         g.plan = plan;
         return plan.grid > 0;
       };
+      for (int s = 1; s <= kMaxSplit; ++s) m->fit[s] = gemm_fit(s);
       const GemmPlan p_qkv = plan_cluster(qd + 2 * kvd, H, true), p_o = plan_cluster(H, qd, false);
       const GemmPlan p_gu = plan_rows(I, H, n_sms), p_down = plan_cluster(H, I, false);
 #ifdef OOS_TIMELINE
@@ -407,7 +438,7 @@ int oos_model_create(const oos_model_config* cfg, const oos_weights* w, void* wo
         ok = encode_act_map(&m->amap_xn[b], m->ws.xn, H, boxes[b]) &&
              encode_act_map(&m->amap_attn[b], m->ws.attn, qd, boxes[b]) &&
              encode_act_map(&m->amap_act[b], m->ws.act, I, boxes[b]);
-      ok = ok && attn_encode_q_maps(*m);
+      ok = ok && attn_encode_q_maps(*m) && prefill_encode(*m);
       if (!ok) {
         rc = OOS_ECUDA;
         break;

@@ -1,0 +1,632 @@
+// Target prefill of the bf16 path: chunks of up to kPfTokens prompt tokens
+// through the decoder, causal attention over the cache and the chunk.
+//
+// A chunk of a thousand tokens has the arithmetic intensity the verify step
+// lacks, so its GEMMs are compute-bound and tiled the ordinary way: 128 tokens in
+// the MMA's M, BN weight rows in N.  The activations keep their two bf16 halves,
+// so every k-step is two MMAs on the same weights.  The tensor core truncates each
+// addition to its accumulator, an error that grows with the chain, so K goes in
+// segments of kPfSeg k-blocks whose sums the epilogue warps add in fp32 registers
+// (one chain over K = 4096 and 12288 added 2e-4 to a K/V error of 5e-4).
+// Persistent blocks, one per SM: one TMA producer thread, one MMA issuer, eight
+// epilogue warps; two accumulators in tensor memory, so a segment is drained, and a
+// tile finished, under the next one's MMAs.
+//
+// With tokens in M a token is one TMEM lane, so a thread holds a token's 128
+// features of a head or residual tile: the q/k norm, the rotary pairs and the
+// RMSNorm sums need no exchange between threads.  The epilogues are those of the
+// verify GEMMs (gemm.cu): bias, q/k norm, RoPE and the cache format; residual add,
+// next norm's gain and sums; SwiGLU.
+#include <string.h>
+
+#include "common.cuh"
+#include "internal.h"
+
+namespace oos {
+
+constexpr int kPfRows = 128;                      // tokens per tile
+constexpr int kPfHalf = kPfRows * kBK * 2;        // bytes of one activation half per stage
+constexpr int kPfEpiWarps = 8;
+constexpr int kPfSeg = 16;                        // k-blocks per accumulator: 128 MMAs
+constexpr int kPfThreads = 128 + 32 * kPfEpiWarps;   // a warp group for the producer and the issuer
+// registers a thread keeps in each role (setmaxnreg): 128 * 56 + 256 * 224 of the
+// 384 * 168 the block is launched with
+constexpr int kPfRegsIssue = 56, kPfRegsEpi = 224;
+static_assert(128 * kPfRegsIssue + 32 * kPfEpiWarps * kPfRegsEpi <= kPfThreads * 168, "register split");
+
+template <int BN>
+struct PfCfg {
+  static constexpr int B_BYTES = BN * kBK * 2;
+  static constexpr int STAGE = 2 * kPfHalf + B_BYTES;
+  static constexpr int S = (227 * 1024 - 2048) / STAGE;
+  static constexpr int SMEM = 2048 + S * STAGE;   // alignment slack + barriers
+  static constexpr int NCOLS = 2 * BN;
+  // warps that finish one tile: all of them (128 columns each) at BN = 256; at
+  // BN = 128 the two groups of four take tiles in turn
+  static constexpr int TILE_WARPS = BN == 256 ? 8 : 4;
+};
+
+enum { PF_QKV = 0, PF_RESID = 1, PF_SILU = 2 };
+
+struct PfArgs {
+  int T;              // tokens of the chunk
+  int kbt;            // k-blocks
+  int m_tiles, n_tiles;
+  int N;              // output features (PF_SILU: intermediate size; PF_QKV: heads * 128)
+  uint32_t* status;
+  const float* ss_in;   // [chunk][kPfTokens]
+  int ss_chunks;
+  float inv_dim, eps;
+  // PF_QKV
+  int nq, nkv, kv_f16;
+  const __nv_bfloat16 *bq, *bk, *bv, *gq, *gk;
+  const float2* rope;   // [kPfTokens][64]
+  __nv_bfloat16 *q_out, *kc, *vc;
+  const int32_t* ctx;
+  // PF_RESID
+  float* x;
+  const __nv_bfloat16* gain;
+  float* ss_out;
+  // PF_RESID, PF_SILU: hi rows, lo rows lo_off elements further
+  __nv_bfloat16* out;
+  size_t lo_off;
+};
+
+// 16 consecutive values as 16-bit words, one 32-byte run
+template <typename H2>
+OOS_DEV void store16(void* dst, const H2 (&h)[8]) {
+  const uint4* s = reinterpret_cast<const uint4*>(h);
+  reinterpret_cast<uint4*>(dst)[0] = s[0];
+  reinterpret_cast<uint4*>(dst)[1] = s[1];
+}
+OOS_DEV void pack16(const float* v, __nv_bfloat162 (&hi)[8], __nv_bfloat162 (&lo)[8]) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    hi[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+    lo[i] = __floats2bfloat162_rn(v[2 * i] - __low2float(hi[i]), v[2 * i + 1] - __high2float(hi[i]));
+  }
+}
+OOS_DEV void pack16(const float* v, __half2 (&hi)[8], __half2 (&lo)[8]) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    hi[i] = __floats2half2_rn(v[2 * i], v[2 * i + 1]);
+    lo[i] = __floats2half2_rn(v[2 * i] - __low2float(hi[i]), v[2 * i + 1] - __high2float(hi[i]));
+  }
+}
+template <typename H2>
+OOS_DEV void store16_hilo(void* hi_dst, void* lo_dst, const float* v) {
+  H2 hi[8], lo[8];
+  pack16(v, hi, lo);
+  store16(hi_dst, hi);
+  store16(lo_dst, lo);
+}
+template <typename H2>
+OOS_DEV void store16_one(void* dst, const float* v) {
+  H2 hi[8], lo[8];
+  pack16(v, hi, lo);
+  store16(dst, hi);
+}
+OOS_DEV void load16(const __nv_bfloat16* p, float (&v)[16]) {
+  uint4 u[2] = {__ldg(reinterpret_cast<const uint4*>(p)), __ldg(reinterpret_cast<const uint4*>(p) + 1)};
+  const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(u);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    v[2 * i] = __low2float(h[i]);
+    v[2 * i + 1] = __high2float(h[i]);
+  }
+}
+
+template <int BN, int EPI>
+__global__ void __launch_bounds__(kPfThreads, 1)
+    k_pf_gemm(const __grid_constant__ CUtensorMap wm0, const __grid_constant__ CUtensorMap wm1,
+              const __grid_constant__ CUtensorMap wm2, const __grid_constant__ CUtensorMap am,
+              const __grid_constant__ PfArgs a) {
+  using C = PfCfg<BN>;
+  constexpr int S = C::S;
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* ring = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  // stage: [activations hi | activations lo | weights]
+  uint64_t* full = reinterpret_cast<uint64_t*>(ring + S * C::STAGE);
+  uint64_t* empty = full + S;
+  uint64_t* accf = empty + S;
+  uint64_t* acce = accf + 2;
+  uint64_t* drain = acce + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  static_assert((2 * S + 5) * 8 + 8 <= 1024, "barrier block");
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int tiles = a.m_tiles * a.n_tiles, G = gridDim.x;
+  const int my_tiles = (int)blockIdx.x < tiles ? (tiles - (int)blockIdx.x + G - 1) / G : 0;
+  const int n_units = my_tiles * a.kbt;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < S; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&accf[b], 1);
+      mbar_init(&acce[b], C::TILE_WARPS);
+    }
+    mbar_init(drain, 1);
+    *abort_flag = 0;
+    mbar_fence_init();
+  }
+  if (warp == 2) tmem_alloc(tmem_slot, C::NCOLS);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+
+  if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kPfRegsIssue));
+    // ------------------------------------------------------------ TMA producer
+    if (warp == 0 && lane == 0) {
+      tma_prefetch_desc(&wm0);
+      tma_prefetch_desc(&am);
+      const uint64_t pol = policy_evict_last();   // every operand is read by many blocks
+      auto load_w = [&](int n, int kb, int stage) {
+        unsigned char* dst = ring + stage * C::STAGE + 2 * kPfHalf;
+#pragma unroll
+        for (int i = 0; i < BN / 64; ++i) {   // boxes of 64 weight rows
+          const CUtensorMap* wm = &wm0;
+          int row = n * BN + i * 64;          // past the last row: zeros
+          if (EPI == PF_SILU) {
+            wm = i < BN / 128 ? &wm0 : &wm1;
+            row = n * (BN / 2) + (i % (BN / 128)) * 64;
+          } else if (EPI == PF_QKV) {
+            int h = n * (BN / 128) + i / 2;
+            if (h >= a.nq + 2 * a.nkv) h = 0;   // an odd head count's last tile: columns nobody reads
+            const int base = h < a.nq ? 0 : h < a.nq + a.nkv ? a.nq : a.nq + a.nkv;
+            wm = h < a.nq ? &wm0 : h < a.nq + a.nkv ? &wm1 : &wm2;
+            row = (h - base) * 128 + (i & 1) * 64;
+          }
+          tma_load_2d(dst + i * 64 * kBK * 2, wm, &full[stage], kb * kBK, row, pol);
+        }
+      };
+      auto load_x = [&](int m, int kb, int stage) {
+        unsigned char* dst = ring + stage * C::STAGE;
+        tma_load_2d(dst, &am, &full[stage], kb * kBK, m * kPfRows, pol);
+        tma_load_2d(dst + kPfHalf, &am, &full[stage], kb * kBK, kPfTokens + m * kPfRows, pol);
+      };
+      // the first stages' weights do not depend on the previous kernel
+      const int n_pre = n_units < S ? n_units : S;
+      int tile = blockIdx.x, kb = 0;
+      for (int j = 0; j < n_pre; ++j) {
+        mbar_arrive_expect_tx(&full[j], C::STAGE);
+        load_w(tile / a.m_tiles, kb, j);
+        if (++kb == a.kbt) { kb = 0; tile += G; }
+      }
+      pdl_wait();
+      pdl_trigger();
+      tile = blockIdx.x;
+      kb = 0;
+      int issued = 0;
+      for (int j = 0; j < n_units; ++j) {
+        const int stage = j % S;
+        if (j >= n_pre) {
+          if (!mbar_wait(&empty[stage], (uint32_t)(j / S - 1) & 1u, abort_flag, a.status)) break;
+          mbar_arrive_expect_tx(&full[stage], C::STAGE);
+          load_w(tile / a.m_tiles, kb, stage);
+        }
+        load_x(tile % a.m_tiles, kb, stage);
+        ++issued;
+        if (++kb == a.kbt) { kb = 0; tile += G; }
+      }
+      // every copy has landed before the block can exit (immediate on the
+      // normal path, where all were consumed)
+      for (int j = issued - S > 0 ? issued - S : 0; j < issued; ++j) {
+        const unsigned long long t0 = globaltimer();
+        while (!mbar_test(smem_addr(&full[j % S]), (uint32_t)((j / S) & 1)) && globaltimer() - t0 < kWaitLimitNs) {
+        }
+      }
+    }
+    // ------------------------------------------------------------ MMA issuer
+    if (warp == 1 && lane == 0) {
+      constexpr uint32_t idesc = idesc_bf16_f32(kPfRows, BN);
+      int j = 0;
+      bool ok = true;
+      uint32_t sg = 0;   // segments handed over; they use the two accumulators in turn
+      for (int it = 0; it < my_tiles && ok; ++it) {
+        for (int kb0 = 0; kb0 < a.kbt && ok; kb0 += kPfSeg, ++sg) {
+          const uint32_t b = sg & 1u;
+          if (!mbar_wait(&acce[b], ((sg >> 1) & 1u) ^ 1u, abort_flag, a.status)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t d = tmem_base + b * BN;
+          const int n = min(kPfSeg, a.kbt - kb0);
+          for (int kb = 0; kb < n; ++kb, ++j) {
+            const int stage = j % S;
+            if (!mbar_wait(&full[stage], (uint32_t)(j / S) & 1u, abort_flag, a.status)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            const uint32_t base = smem_addr(ring + stage * C::STAGE);
+            const uint64_t xh = smem_desc_sw128(base), xl = smem_desc_sw128(base + kPfHalf);
+            const uint64_t w = smem_desc_sw128(base + 2 * kPfHalf);
+#pragma unroll
+            for (int k = 0; k < kBK / 16; ++k) {
+              tc_mma_bf16(d, xh + 2 * k, w + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+              tc_mma_bf16(d, xl + 2 * k, w + 2 * k, idesc, 1u);
+            }
+            tc_commit(&empty[stage]);
+          }
+          if (ok) tc_commit(&accf[b]);
+        }
+      }
+      // all issued MMAs complete before TMEM is released
+      tc_commit(drain);
+      const unsigned long long t0 = globaltimer();
+      while (!mbar_test(smem_addr(drain), 0) && globaltimer() - t0 < kWaitLimitNs) {
+      }
+    }
+    __syncwarp();
+  } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kPfRegsEpi));
+    // ------------------------------------------------------------ epilogue (warps 4..11)
+    pdl_wait();
+    pdl_trigger();
+    const int q = warp & 3, grp = (warp - 4) >> 2;
+    const uint32_t lane_base = tmem_base + ((uint32_t)(q * 32) << 16);
+    const int ctx = EPI == PF_QKV ? *a.ctx : 0;
+    const int segs = (a.kbt + kPfSeg - 1) / kPfSeg;
+    uint32_t sg = 0;
+    for (int it = 0; it < my_tiles; ++it) {
+      if (BN == 128 && (it & 1) != grp) {
+        sg += segs;
+        continue;
+      }
+      const int tile = (int)blockIdx.x + it * G;
+      const int n = tile / a.m_tiles, t = (tile % a.m_tiles) * kPfRows + q * 32 + lane;
+      const bool live = t < a.T;
+      float r = 0.f;
+      if (EPI != PF_RESID && live) {   // the input's RMSNorm factor
+        float s = 0.f;
+#pragma unroll 8
+        for (int c = 0; c < a.ss_chunks; ++c) s += a.ss_in[(size_t)c * kPfTokens + t];
+        r = rsqrtf(s * a.inv_dim + a.eps);
+      }
+      // this thread's 128 sums: a head, 128 features, or 64 gate and 64 up rows
+      float acc[128];
+      bool ok = true;
+      for (int i = 0; i < segs; ++i, ++sg) {
+        const uint32_t b = sg & 1u;
+        ok = __all_sync(0xffffffffu, mbar_wait(&accf[b], (sg >> 1) & 1u, abort_flag, a.status));
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t base = lane_base + b * BN;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const uint32_t col = EPI == PF_SILU ? base + (c < 4 ? 0 : BN / 2) + (BN == 256 ? grp * 64 : 0) + (c & 3) * 16
+                                              : base + (BN == 256 ? grp * 128 : 0) + c * 16;
+          float v[16];
+          tmem_ld16_nowait(col, v);
+          tmem_wait_ld();
+          reg_fence(v);
+#pragma unroll
+          for (int k = 0; k < 16; ++k) acc[c * 16 + k] = i == 0 ? v[k] : acc[c * 16 + k] + v[k];
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&acce[b]);
+      }
+      if (!ok) break;
+      auto finish = [&]() {
+        const int unit = n * (BN / 128) + (BN == 256 ? grp : 0);   // head, or 128-feature block
+        if (EPI == PF_QKV) {
+          if (unit >= a.nq + 2 * a.nkv) return;
+          const int kind = unit < a.nq ? 0 : unit < a.nq + a.nkv ? 1 : 2;
+          const int h = kind == 0 ? unit : kind == 1 ? unit - a.nq : unit - a.nq - a.nkv;
+          const __nv_bfloat16* bias = kind == 0 ? a.bq : kind == 1 ? a.bk : a.bv;
+          const __nv_bfloat16* gn = kind == 0 ? a.gq : kind == 1 ? a.gk : nullptr;
+#pragma unroll
+          for (int c = 0; c < 128; ++c) acc[c] *= r;
+          if (bias) {
+#pragma unroll
+            for (int c = 0; c < 128; c += 16) {
+              float bv[16];
+              load16(bias + h * 128 + c, bv);
+#pragma unroll
+              for (int i = 0; i < 16; ++i) acc[c + i] += bv[i];
+            }
+          }
+          if (gn) {   // per-head RMSNorm
+            float ss[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int c = 0; c < 128; ++c) ss[c & 3] += acc[c] * acc[c];
+            const float rn = rsqrtf(((ss[0] + ss[1]) + (ss[2] + ss[3])) * (1.f / 128.f) + a.eps);
+#pragma unroll
+            for (int c = 0; c < 128; c += 16) {
+              float g[16];
+              load16(gn + c, g);
+#pragma unroll
+              for (int i = 0; i < 16; ++i) acc[c + i] *= rn * g[i];
+            }
+          }
+          if (kind < 2) {   // rotary pairs c and 64 + c
+            const float4* rp = reinterpret_cast<const float4*>(a.rope + (size_t)t * 64);
+#pragma unroll
+            for (int c = 0; c < 64; c += 2) {
+              const float4 cs = __ldg(rp + c / 2);
+              const float p0 = acc[c], p1 = acc[64 + c], q0 = acc[c + 1], q1 = acc[65 + c];
+              acc[c] = p0 * cs.x - p1 * cs.y;
+              acc[64 + c] = p1 * cs.x + p0 * cs.y;
+              acc[c + 1] = q0 * cs.z - q1 * cs.w;
+              acc[65 + c] = q1 * cs.z + q0 * cs.w;
+            }
+          }
+          if (kind == 0) {
+            __nv_bfloat16* dst = a.q_out + ((size_t)t * a.nq + h) * 128;
+            const size_t lo = (size_t)kPfTokens * a.nq * 128;
+#pragma unroll
+            for (int c = 0; c < 128; c += 16) {
+              if (a.kv_f16) store16_hilo<__half2>(dst + c, dst + lo + c, acc + c);
+              else store16_hilo<__nv_bfloat162>(dst + c, dst + lo + c, acc + c);
+            }
+          } else {
+            __nv_bfloat16* dst = (kind == 1 ? a.kc : a.vc) + ((size_t)(ctx + t) * a.nkv + h) * 128;
+#pragma unroll
+            for (int c = 0; c < 128; c += 16) {
+              if (a.kv_f16) store16_one<__half2>(dst + c, acc + c);
+              else store16_one<__nv_bfloat162>(dst + c, acc + c);
+            }
+          }
+        } else if (EPI == PF_RESID) {
+          const int f0 = unit * 128;
+          if (f0 >= a.N) return;
+          float ss = 0.f;
+#pragma unroll
+          for (int c = 0; c < 128; c += 16) {
+            float g[16];
+            float4 xv[4];
+            float4* xp = reinterpret_cast<float4*>(a.x + (size_t)t * a.N + f0 + c);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) xv[i] = xp[i];
+            load16(a.gain + f0 + c, g);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              float* v = acc + c + 4 * i;
+              xv[i].x += v[0];
+              xv[i].y += v[1];
+              xv[i].z += v[2];
+              xv[i].w += v[3];
+              xp[i] = xv[i];
+              ss += xv[i].x * xv[i].x + xv[i].y * xv[i].y + xv[i].z * xv[i].z + xv[i].w * xv[i].w;
+              v[0] = g[4 * i] * xv[i].x;
+              v[1] = g[4 * i + 1] * xv[i].y;
+              v[2] = g[4 * i + 2] * xv[i].z;
+              v[3] = g[4 * i + 3] * xv[i].w;
+            }
+            __nv_bfloat16* y = a.out + (size_t)t * a.N + f0 + c;
+            store16_hilo<__nv_bfloat162>(y, y + a.lo_off, acc + c);
+          }
+          a.ss_out[(size_t)unit * kPfTokens + t] = ss;
+        } else {
+          const int i0 = n * (BN / 2) + (BN == 256 ? grp * 64 : 0);
+          if (i0 >= a.N) return;
+#pragma unroll
+          for (int c = 0; c < 64; c += 16) {
+#pragma unroll
+            for (int i = c; i < c + 16; ++i) {
+              const float gr = acc[i] * r;
+              acc[i] = __fdividef(gr, 1.f + expf(-gr)) * (acc[64 + i] * r);
+            }
+            __nv_bfloat16* y = a.out + (size_t)t * a.N + i0 + c;
+            store16_hilo<__nv_bfloat162>(y, y + a.lo_off, acc + c);
+          }
+        }
+      };
+      if (live) finish();
+      __syncwarp();
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 2) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, C::NCOLS);
+  }
+}
+
+// ------------------------------------------------------------ chunk preparation
+// Validates the chunk's tokens and publishes its committed length.  The first
+// chunk of a prompt clears the status words, later ones only add to them.
+__global__ void __launch_bounds__(1024) k_pf_prep(const int32_t* __restrict__ tokens, int T, int ctx, int first, int vocab,
+                                                  uint32_t* status, int32_t* ctx_out) {
+  pdl_wait();
+  pdl_trigger();
+  bool bad = false;
+  for (int i = threadIdx.x; i < T; i += blockDim.x) bad |= tokens[i] < 0 || tokens[i] >= vocab;
+  const bool any = __syncthreads_or(bad);
+  if (threadIdx.x == 0) {
+    *ctx_out = ctx;
+    *status = (first ? 0u : *status) | (any ? ST_TREE : 0u);
+  }
+  if (first && threadIdx.x >= 1 && threadIdx.x < 8) status[threadIdx.x] = 0u;
+}
+
+// The last token's final-norm input as row 0 of the verify step's buffers, for
+// the LM head: its two halves, and its sum of squares as the first of `chunks`.
+__global__ void __launch_bounds__(256) k_pf_last(const __nv_bfloat16* __restrict__ y, size_t lo_off,
+                                                 const float* __restrict__ ss, int in_chunks, int t, int H,
+                                                 __nv_bfloat16* __restrict__ y_out, float* __restrict__ ss_out,
+                                                 int chunks) {
+  __shared__ float red[32];
+  pdl_wait();
+  pdl_trigger();
+  for (int f = threadIdx.x; f < H; f += blockDim.x) {
+    y_out[f] = y[(size_t)t * H + f];
+    y_out[(size_t)kMaxT * H + f] = y[lo_off + (size_t)t * H + f];
+  }
+  float s = 0.f;
+  for (int c = threadIdx.x; c < in_chunks; c += blockDim.x) s += ss[(size_t)c * kPfTokens + t];
+  s = block_sum(s, red);
+  for (int c = threadIdx.x; c < chunks; c += blockDim.x) ss_out[(size_t)c * kMaxT] = c == 0 ? s : 0.f;
+}
+
+// ------------------------------------------------------------ host side
+template <int BN, int EPI>
+static cudaError_t pf_smem() {
+  return cudaFuncSetAttribute(k_pf_gemm<BN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, PfCfg<BN>::SMEM);
+}
+cudaError_t prefill_setup() {
+  cudaError_t e = pf_smem<128, PF_QKV>();
+  if (e == cudaSuccess) e = pf_smem<128, PF_RESID>();
+  if (e == cudaSuccess) e = pf_smem<128, PF_SILU>();
+  if (e == cudaSuccess) e = pf_smem<256, PF_QKV>();
+  if (e == cudaSuccess) e = pf_smem<256, PF_RESID>();
+  if (e == cudaSuccess) e = pf_smem<256, PF_SILU>();
+  return e;
+}
+
+bool prefill_encode(Model& m) {
+  const auto& c = m.cfg;
+  const int qd = c.n_q_heads * c.head_dim;
+  return encode_rows_map(&m.pf_xn_map, m.ws.pf_xn, 2 * kPfTokens, c.hidden, kPfRows) &&
+         encode_rows_map(&m.pf_attn_map, m.ws.pf_attn, 2 * kPfTokens, qd, kPfRows) &&
+         encode_rows_map(&m.pf_act_map, m.ws.pf_act, 2 * kPfTokens, c.intermediate, kPfRows);
+}
+
+// How one GEMM of a chunk runs: tiles of 128 x 256 or 128 x 128 here, or the
+// verify GEMMs in token tiles of 128, k split over clusters of `split` (0: here).
+struct PfPlan {
+  bool wide;
+  int split;
+};
+
+// Estimates in microseconds, from timings of both kinds: a k-block of a 128 x 256
+// tile takes ~0.6 us and of a 128 x 128 one ~0.45 (operand traffic bounds the
+// narrow one), a k-block of a verify tile (128 tokens x 128 rows) ~0.5; prologue,
+// drain and epilogue ~8 against ~6 plus the sums pulled.  Few tiles and a long K
+// (O and down of small models: 24 tiles for 333 tokens at hidden 1024) go to the
+// clusters, which fill the SMs; anything with a tile for most SMs stays here.
+static PfPlan pf_plan(const Model& m, int rows, int kbt, int T, bool may_split) {
+  const int mt = (T + kPfRows - 1) / kPfRows;
+  auto waves = [](long long tiles, int fit) { return (double)((tiles + fit - 1) / fit); };
+  const double wide = waves((long long)mt * ((rows + 255) / 256), m.num_sms) * kbt * 0.6 + 8;
+  const double narrow = waves((long long)mt * ((rows + 127) / 128), m.num_sms) * kbt * 0.45 + 8;
+  PfPlan p{wide <= narrow, 0};
+  double best = wide <= narrow ? wide : narrow;
+  for (int c = 1; c <= (may_split ? kMaxSplit : 1) && c <= kbt; ++c) {
+    if (m.fit[c] < 1) continue;
+    const double t = waves((long long)mt * ((rows + 127) / 128), m.fit[c]) * ((kbt + c - 1) / c * 0.5 + 6) + 0.2 * c;
+    if (t < best) {
+      best = t;
+      p.split = c;
+    }
+  }
+  return p;
+}
+
+template <int EPI>
+static cudaError_t launch_pf(Model& m, const GemmW& g, const CUtensorMap& am, PfArgs& a, int rows, bool wide,
+                             cudaStream_t st) {
+  // rows: stacked weight rows of the GEMM
+  const auto& c = m.cfg;
+  a.kbt = g.K / kBK;
+  a.m_tiles = (a.T + kPfRows - 1) / kPfRows;
+  a.n_tiles = (rows + (wide ? 255 : 127)) / (wide ? 256 : 128);
+  a.status = m.ws.status;
+  a.ss_in = m.ws.pf_ss;
+  a.ss_chunks = c.hidden / kTile;
+  a.inv_dim = 1.0f / (float)c.hidden;
+  a.eps = c.rms_eps;
+  const CUtensorMap& w1 = g.n_seg > 1 ? g.pf_map[1] : g.pf_map[0];
+  const CUtensorMap& w2 = g.n_seg > 2 ? g.pf_map[2] : g.pf_map[0];
+  const long long tiles = (long long)a.m_tiles * a.n_tiles;
+  const dim3 grid((unsigned)(tiles < m.num_sms ? tiles : m.num_sms));
+  if (wide)
+    return launch(m.pdl, k_pf_gemm<256, EPI>, grid, dim3(kPfThreads), (size_t)PfCfg<256>::SMEM, st, g.pf_map[0], w1, w2,
+                  am, a);
+  return launch(m.pdl, k_pf_gemm<128, EPI>, grid, dim3(kPfThreads), (size_t)PfCfg<128>::SMEM, st, g.pf_map[0], w1, w2,
+                am, a);
+}
+
+static PfArgs pf_args(int T) {
+  PfArgs a;
+  memset(&a, 0, sizeof(a));
+  a.T = T;
+  return a;
+}
+
+static cudaError_t launch_pf_resid(Model& m, int layer, bool down, const void* gain, int T, cudaStream_t st) {
+  const GemmW& g = down ? m.g_down[layer] : m.g_o[layer];
+  const PfPlan p = pf_plan(m, m.cfg.hidden, g.K / kBK, T, true);
+  if (p.split) return launch_chunk_resid(m, layer, down, gain, T, p.split, st);
+  PfArgs a = pf_args(T);
+  a.N = m.cfg.hidden;
+  a.x = m.ws.pf_x;
+  a.gain = (const __nv_bfloat16*)gain;
+  a.out = (__nv_bfloat16*)m.ws.pf_xn;
+  a.lo_off = (size_t)kPfTokens * m.cfg.hidden;
+  a.ss_out = m.ws.pf_ss;
+  return launch_pf<PF_RESID>(m, g, down ? m.pf_act_map : m.pf_attn_map, a, a.N, p.wide, st);
+}
+
+static cudaError_t launch_pf_qkv(Model& m, int layer, void* kc, void* vc, int T, cudaStream_t st) {
+  const auto& c = m.cfg;
+  const oos_layer_weights& L = m.layers[layer];
+  const int rows = (c.n_q_heads + 2 * c.n_kv_heads) * c.head_dim;
+  const PfPlan p = pf_plan(m, rows, c.hidden / kBK, T, true);
+  if (p.split) return launch_chunk_qkv(m, layer, kc, vc, T, p.split, st);
+  PfArgs a = pf_args(T);
+  a.N = rows;
+  a.nq = c.n_q_heads;
+  a.nkv = c.n_kv_heads;
+  a.kv_f16 = c.kv_f16 ? 1 : 0;
+  a.bq = (const __nv_bfloat16*)(c.qkv_bias ? L.b_q : nullptr);
+  a.bk = (const __nv_bfloat16*)(c.qkv_bias ? L.b_k : nullptr);
+  a.bv = (const __nv_bfloat16*)(c.qkv_bias ? L.b_v : nullptr);
+  a.gq = (const __nv_bfloat16*)(c.qk_norm ? L.q_norm : nullptr);
+  a.gk = (const __nv_bfloat16*)(c.qk_norm ? L.k_norm : nullptr);
+  a.rope = m.ws.pf_rope;
+  a.q_out = (__nv_bfloat16*)m.ws.pf_q;
+  a.kc = (__nv_bfloat16*)kc;
+  a.vc = (__nv_bfloat16*)vc;
+  a.ctx = m.ws.ctx;
+  return launch_pf<PF_QKV>(m, m.g_qkv[layer], m.pf_xn_map, a, rows, p.wide, st);
+}
+
+static cudaError_t launch_pf_gu(Model& m, int layer, int T, cudaStream_t st) {
+  const auto& c = m.cfg;
+  const PfPlan p = pf_plan(m, 2 * c.intermediate, c.hidden / kBK, T, false);
+  if (p.split) return launch_chunk_gu(m, layer, T, st);
+  PfArgs a = pf_args(T);
+  a.N = c.intermediate;
+  a.out = (__nv_bfloat16*)m.ws.pf_act;
+  a.lo_off = (size_t)kPfTokens * c.intermediate;
+  return launch_pf<PF_SILU>(m, m.g_gu[layer], m.pf_xn_map, a, 2 * a.N, p.wide, st);
+}
+
+// Every layer of one chunk of T tokens (128 < T <= kPfTokens) at cache position
+// ctx: K/V into slots ctx.., the final norm's input in pf_xn / pf_ss.
+cudaError_t prefill_chunk(Model& m, const oos_kv_cache* kv, int ctx, const int32_t* tokens, int T, bool first,
+                          cudaStream_t st) {
+  const auto& c = m.cfg;
+  cudaError_t e = launch(false, k_pf_prep, dim3(1), dim3(1024), 0, st, tokens, T, ctx, first ? 1 : 0, c.vocab,
+                         m.ws.status, m.ws.ctx);
+  if (e == cudaSuccess) e = launch_embed_pf(m, tokens, T, st);
+  for (int l = 0; l < c.n_layers && e == cudaSuccess; ++l) {
+    const void* gain = l + 1 < c.n_layers ? m.layers[l + 1].attn_norm : m.w.final_norm;
+    e = launch_pf_qkv(m, l, kv->k[l], kv->v[l], T, st);
+    if (e == cudaSuccess) e = launch_attention_pf(m, l, kv->k[l], kv->v[l], kv->capacity, ctx, T, st);
+    if (e == cudaSuccess) e = launch_pf_resid(m, l, false, m.layers[l].mlp_norm, T, st);
+    if (e == cudaSuccess) e = launch_pf_gu(m, l, T, st);
+    if (e == cudaSuccess) e = launch_pf_resid(m, l, true, gain, T, st);
+  }
+  return e;
+}
+
+// the chunk's last token into row 0 of the verify buffers the LM head reads
+cudaError_t prefill_last(Model& m, int T, cudaStream_t st) {
+  const auto& c = m.cfg;
+  return launch(m.pdl, k_pf_last, dim3(1), dim3(256), 0, st, (const __nv_bfloat16*)m.ws.pf_xn,
+                (size_t)kPfTokens * c.hidden, (const float*)m.ws.pf_ss, c.hidden / kTile, T - 1, c.hidden,
+                (__nv_bfloat16*)m.ws.xn, m.ws.ss, norm_chunks(m, c.n_layers));
+}
+
+}  // namespace oos

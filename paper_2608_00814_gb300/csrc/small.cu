@@ -143,11 +143,14 @@ cudaError_t launch_embed_norm(Model& m, const int32_t* tokens, int T, cudaStream
 // rsqrt(mean(x^2) + eps)).
 // Block (t, 0) also fills the step's RoPE table: cos/sin of pos[t] * theta^(-2m/d)
 // for m < d/2, the angle formed and reduced to [-pi, pi] in fp64 once per step
-// (every layer reuses it).
+// (every layer reuses it).  `rows`: token rows the buffers are laid out for (the
+// lo halves lie rows * H elements further, the sums rows apart).  pos: the nodes'
+// positions, or nullptr for consecutive tokens from *ctx (a prefill chunk).
 __global__ void __launch_bounds__(128) k_embed_tc(const int32_t* __restrict__ tokens, const __nv_bfloat16* __restrict__ emb,
                                                   const __nv_bfloat16* __restrict__ gain, int H, int vocab,
-                                                  float* __restrict__ x, __nv_bfloat16* __restrict__ y,
+                                                  float* __restrict__ x, __nv_bfloat16* __restrict__ y, int rows,
                                                   float* __restrict__ ss, const int32_t* __restrict__ pos,
+                                                  const int32_t* __restrict__ ctx,
                                                   const double* __restrict__ inv_freq, int half_d,
                                                   float2* __restrict__ rope) {
   __shared__ float red[32];
@@ -156,7 +159,7 @@ __global__ void __launch_bounds__(128) k_embed_tc(const int32_t* __restrict__ to
   const int t = blockIdx.x, f = blockIdx.y * 128 + threadIdx.x;
   if (blockIdx.y == 0 && threadIdx.x < half_d) {
     const double two_pi = 6.283185307179586476925286766559;
-    const double ang = (double)pos[t] * inv_freq[threadIdx.x];
+    const double ang = (double)(pos ? pos[t] : *ctx + t) * inv_freq[threadIdx.x];
     float sn, cs;
     sincosf((float)(ang - two_pi * rint(ang / two_pi)), &sn, &cs);
     rope[t * half_d + threadIdx.x] = make_float2(cs, sn);
@@ -167,18 +170,25 @@ __global__ void __launch_bounds__(128) k_embed_tc(const int32_t* __restrict__ to
   if (f < H) {
     v = __bfloat162float(emb[(size_t)tok * H + f]);
     x[(size_t)t * H + f] = v;
-    store_act(y, (size_t)t * H + f, (size_t)kMaxT * H, v * __bfloat162float(gain[f]));
+    store_act(y, (size_t)t * H + f, (size_t)rows * H, v * __bfloat162float(gain[f]));
   }
   const float s = block_sum(v * v, red);
-  if (threadIdx.x == 0) ss[(size_t)blockIdx.y * kMaxT + t] = s;
+  if (threadIdx.x == 0) ss[(size_t)blockIdx.y * rows + t] = s;
 }
 
 cudaError_t launch_embed_tc(Model& m, const int32_t* tokens, int T, cudaStream_t st) {
   const auto& c = m.cfg;
   return launch(m.pdl, k_embed_tc, dim3(T, (c.hidden + 127) / 128), dim3(128), 0, st, tokens,
                 (const __nv_bfloat16*)m.w.embed, (const __nv_bfloat16*)m.layers[0].attn_norm, c.hidden, c.vocab,
-                m.ws.x, (__nv_bfloat16*)m.ws.xn, m.ws.ss, (const int32_t*)m.ws.pos, (const double*)m.ws.inv_freq,
-                c.head_dim / 2, m.ws.rope);
+                m.ws.x, (__nv_bfloat16*)m.ws.xn, kMaxT, m.ws.ss, (const int32_t*)m.ws.pos, (const int32_t*)nullptr,
+                (const double*)m.ws.inv_freq, c.head_dim / 2, m.ws.rope);
+}
+cudaError_t launch_embed_pf(Model& m, const int32_t* tokens, int T, cudaStream_t st) {
+  const auto& c = m.cfg;
+  return launch(m.pdl, k_embed_tc, dim3(T, (c.hidden + 127) / 128), dim3(128), 0, st, tokens,
+                (const __nv_bfloat16*)m.w.embed, (const __nv_bfloat16*)m.layers[0].attn_norm, c.hidden, c.vocab,
+                m.ws.pf_x, (__nv_bfloat16*)m.ws.pf_xn, kPfTokens, m.ws.pf_ss, (const int32_t*)nullptr,
+                (const int32_t*)m.ws.ctx, (const double*)m.ws.inv_freq, c.head_dim / 2, m.ws.pf_rope);
 }
 
 // bf16 path, checking output only: the final RMSNorm output in fp32,
