@@ -68,7 +68,14 @@ namespace oos {
 //     the epilogue reads (residual, rotary factors, norm sums) is loaded while
 //     the weights stream.
 //   SILU, ARGMAX: whole-K tiles, dealt round-robin (the weights of the next tile
-//     stream while one is finished).
+//     stream while one is finished).  Above 64 tokens SILU runs in pairs of CTAs
+//     (cta_group::2): two neighbouring tiles share one MMA, each CTA staging its
+//     own weights and one activation half, hi or lo.  A CTA alone would be bound by
+//     its shared memory there: per k-block its MMAs read 128 KB of operands and TMA
+//     writes 56 (96 rows), against ~128 bytes a clock; in pairs 64 and 40.  Gate/up of
+//     the 14336 x 4096 shape at T = 128: last accumulator 57 -> 50 us after the start.
+//     Up to 64 tokens HBM is the bound (5.9 TB/s at 12288 x 4096, T = 64) and a pair's
+//     setup costs more than it gives (8B step 4026 -> 4053 us, 0.6B 1277 -> 1304).
 enum { EPI_QKV = 0, EPI_RESID = 1, EPI_SILU = 2, EPI_ARGMAX = 3 };
 
 // token rows the activation buffers are laid out for; the lo halves follow them
@@ -80,10 +87,6 @@ constexpr int kLdr = CHUNK ? kPfTokens : kMaxT;
 template <int EPI>
 struct EpiOf {
   static constexpr int sub = (EPI == EPI_SILU || EPI == EPI_ARGMAX) ? 2 : 1;
-  // k-segments of a tile with an accumulator each, added in fp32 by the
-  // epilogue: the tensor core truncates every addition to its accumulator, an
-  // error that grows with the chain, so the chains are kept short
-  static constexpr int segs = EPI == EPI_ARGMAX ? 1 : 2;
   static constexpr bool cluster = EPI == EPI_QKV || EPI == EPI_RESID;
 };
 
@@ -141,11 +144,19 @@ struct TcCfg {
   // subtile read from shared memory once); the accumulator then holds the hi
   // products in columns [0, BN) and the lo products in [BN, 2 BN).  Paired
   // when the accumulator buffers then fit the 512 TMEM columns.
-  static constexpr int BUFS = 2;
+  static constexpr bool PAIR = EPI == EPI_SILU && BN == 128;
+  static constexpr int BUFS = PAIR && 2 * kSub * 2 * BN > 512 ? 1 : 2;
   static constexpr bool PAIRED = BUFS * kSub * 2 * BN <= 512;
+  static_assert(!PAIR || PAIRED, "a pair of CTAs splits the hi and lo halves");
   static constexpr int SUB_COLS = PAIRED ? 2 * BN : BN;        // accumulator columns per subtile
   static constexpr int NCOLS = BUFS * kSub * SUB_COLS < 32 ? 32 : BUFS * kSub * SUB_COLS;
-  static int stage_bytes(int rows) { return kSub * rows * kBK * 2 + 2 * B_BYTES; }
+  // k-segments of a tile with an accumulator each, added in fp32 by the
+  // epilogue: the tensor core truncates every addition to its accumulator, an
+  // error that grows with the chain, so the chains are kept short (one segment
+  // where both buffers do not fit: 256 MMAs at K = 4096, hi and lo apart)
+  static constexpr int SEGS = EPI == EPI_ARGMAX ? 1 : BUFS;
+  static constexpr int X_BYTES = PAIR ? B_BYTES : 2 * B_BYTES;   // activations of a stage in this CTA
+  static __host__ __device__ int stage_bytes(int rows) { return kSub * rows * kBK * 2 + X_BYTES; }
   static int stages(int rows) {
     const int s = (kGemmSmemMax - FIXED) / stage_bytes(rows);
     return s > kMaxStages ? kMaxStages : s;
@@ -367,6 +378,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   constexpr int kSub = C::kSub;
   constexpr bool ARGMAX = EPI == EPI_ARGMAX;
   constexpr bool CLUSTER = EpiOf<EPI>::cluster;
+  constexpr bool PAIR = C::PAIR;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   // [barriers | RMSNorm factors | argmax state], then from `ring` on the weight
@@ -388,6 +400,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   unsigned char* ring_x = ring + S * kSub * a_bytes;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // which use of its buffer the n-th accumulator is
+  auto uses = [](uint32_t n) { return C::BUFS > 1 ? n >> 1 : n; };
   if (threadIdx.x == 0) TL_GEMM(0);
 
   // this CTA's work: k-blocks [kb0, kb0 + n_units) of tile `first` (cluster), or
@@ -405,6 +419,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     kb0 = a.kbt * (int)rank / a.split;
     nkb = n_units = a.kbt * ((int)rank + 1) / a.split - kb0;
   } else {
+    if (PAIR) asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
     first = blockIdx.x;
     step = gridDim.x;
     kb0 = 0;
@@ -426,20 +441,27 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&accf[b], 1);
-      mbar_init(&acce[b], kEpiWarps);
+      mbar_init(&acce[b], PAIR ? 2 * kEpiWarps : kEpiWarps);
     }
     mbar_init(drain, 1);
     abort_flag[0] = 0;
     abort_flag[1] = 0;
     mbar_fence_init();
   }
-  if (warp == 2) tmem_alloc(tmem_slot, C::NCOLS);
+  if (warp == 2) {
+    if (PAIR) tmem_alloc_pair(tmem_slot, C::NCOLS);
+    else tmem_alloc(tmem_slot, C::NCOLS);
+  }
   if (ARGMAX && threadIdx.x >= 64) {
     for (int e = threadIdx.x - 64; e < BN; e += kEpiThreads) run[e] = Top2s{-INFINITY, 0x7fffffff, -INFINITY};
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if (PAIR) {   // the other CTA's barriers are set up before anything arrives on them
+    cluster_arrive_release();
+    cluster_wait_acquire();
+  }
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp == 0) {
@@ -449,13 +471,23 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       tma_prefetch_desc(&am);
       const uint64_t pol_w = policy_evict_first();
       const uint64_t pol_a = policy_evict_last();
-      const uint32_t stage_bytes = (uint32_t)(kSub * a_bytes + 2 * C::B_BYTES);
+      const uint32_t stage_bytes = (uint32_t)(kSub * a_bytes + C::X_BYTES);
+      // a pair's copies all complete on rank 0's barriers, which expect both CTAs' bytes
+      const uint32_t full0 = PAIR ? dsmem_addr(full, 0) : 0u;
+      auto load = [&](void* dst, const CUtensorMap* map, int stage, int x, int y, uint64_t pol) {
+        if (PAIR) tma_load_2d_pair(dst, map, full0 + (uint32_t)stage * 8u, x, y, pol);
+        else tma_load_2d(dst, map, &full[stage], x, y, pol);
+      };
+      auto expect = [&](int stage) {
+        if (!PAIR) mbar_arrive_expect_tx(&full[stage], stage_bytes);
+        else if (rank == 0) mbar_arrive_expect_tx(&full[stage], 2 * stage_bytes);
+      };
       // weights of the unit at (tile, kb) into `stage`; rows past the matrix
       // read zeros (TMA out-of-bounds fill)
       auto load_sub = [&](const CUtensorMap* wm, unsigned char* dst, int kb, int row, int stage) {
-        tma_load_2d(dst, wm, &full[stage], kb * kBK, row, pol_w);
+        load(dst, wm, stage, kb * kBK, row, pol_w);
         if (CHUNK && CLUSTER)   // the chunk's boxes are 64 rows high
-          tma_load_2d(dst + 64 * kBK * 2, wm, &full[stage], kb * kBK, row + 64, pol_w);
+          load(dst + 64 * kBK * 2, wm, stage, kb * kBK, row + 64, pol_w);
       };
       auto load_w = [&](int tile, int kb, int stage) {
         unsigned char* dst = ring + stage * kSub * a_bytes;
@@ -473,9 +505,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         }
       };
       auto load_x = [&](int kb, int stage) {
-        unsigned char* dst = ring_x + stage * 2 * C::B_BYTES;
-        tma_load_2d(dst, &am, &full[stage], kb * kBK, tok0, pol_a);                       // hi rows
-        tma_load_2d(dst + C::B_BYTES, &am, &full[stage], kb * kBK, kLdr<CHUNK> + tok0, pol_a);  // lo rows
+        unsigned char* dst = ring_x + stage * C::X_BYTES;
+        if (!PAIR || rank == 0) load(dst, &am, stage, kb * kBK, tok0, pol_a);   // hi rows
+        if (!PAIR || rank == 1)                                                // lo rows
+          load(PAIR ? dst : dst + C::B_BYTES, &am, stage, kb * kBK, kLdr<CHUNK> + tok0, pol_a);
       };
       // weights do not depend on the previous kernel: start streaming them
       // before waiting for it (programmatic dependent launch)
@@ -483,7 +516,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       {
         int tile = first, kb = 0;
         for (int j = 0; j < n_pre; ++j) {
-          mbar_arrive_expect_tx(&full[j], stage_bytes);
+          expect(j);
           load_w(tile, kb0 + kb, j);
           if (++kb == nkb) {
             kb = 0;
@@ -510,7 +543,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       int issued = n_pre;
       for (int j = n_pre; j < n_units; ++j) {
         if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, a.status)) break;
-        mbar_arrive_expect_tx(&full[stage], stage_bytes);
+        expect(stage);
         load_w(tile, kb0 + kb, stage);
         load_x(kb0 + kb, stage);
         advance();
@@ -520,30 +553,42 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
           phase ^= 1u;
         }
       }
-      {
+      if (!PAIR || rank == 0) {
         // every copy this thread issued has landed before the CTA can exit,
-        // whoever gave up (immediate on the normal path, where all were consumed)
+        // whoever gave up (immediate on the normal path, where all were consumed;
+        // after an abort of one CTA of a pair a phase may stay short of the
+        // other's bytes, so the whole wait is bounded, well above a copy's time)
+        const unsigned long long t0 = globaltimer(), most = PAIR ? 10000000ull : kWaitLimitNs;
         for (int j = issued - S > 0 ? issued - S : 0; j < issued; ++j) {
-          const unsigned long long t0 = globaltimer();
-          while (!mbar_test(smem_addr(&full[j % S]), (uint32_t)((j / S) & 1)) && globaltimer() - t0 < kWaitLimitNs) {
+          while (!mbar_test(smem_addr(&full[j % S]), (uint32_t)((j / S) & 1)) && globaltimer() - t0 < most) {
           }
+        }
+      } else if (issued < n_units) {
+        // rank 1 gave up: its last copies complete on rank 0's barriers, which may
+        // never have expected them; they land long before this ends
+        const unsigned long long t0 = globaltimer();
+        while (globaltimer() - t0 < 200000ull) {
         }
       }
     }
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      constexpr uint32_t idesc = idesc_bf16_f32(kTile, C::PAIRED ? 2 * BN : BN);
+    if (lane == 0 && (!PAIR || rank == 0)) {
+      constexpr uint32_t idesc = idesc_bf16_f32(PAIR ? 2 * kTile : kTile, C::PAIRED ? 2 * BN : BN);
+      auto commit = [&](uint64_t* bar) {
+        if (PAIR) tc_commit_pair(bar);
+        else tc_commit(bar);
+      };
       int stage = 0;
       uint32_t phase = 0;
       int acc = 0;
       uint32_t use = 0;   // accumulators handed over so far (two buffers in turn)
       bool ok = true;
-      const int segs = nkb < EpiOf<EPI>::segs ? 1 : EpiOf<EPI>::segs;
+      const int segs = nkb < C::SEGS ? 1 : C::SEGS;
       for (int j = 0; j < n_units && ok; j += nkb) {
         for (int sg = 0; sg < segs && ok; ++sg) {
-          if (!mbar_wait(&acce[acc], ((use >> 1) & 1u) ^ 1u, abort_flag, a.status)) {
+          if (!mbar_wait(&acce[acc], (uses(use) & 1u) ^ 1u, abort_flag, a.status)) {
             ok = false;
             break;
           }
@@ -557,33 +602,33 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             }
             tc_fence_after();
             const uint32_t wbase = smem_addr(ring + stage * kSub * a_bytes);
-            const uint32_t xbase = smem_addr(ring_x + stage * 2 * C::B_BYTES);
+            const uint32_t xbase = smem_addr(ring_x + stage * C::X_BYTES);
             const uint64_t bh = smem_desc_sw128(xbase);
-            const uint64_t bl = smem_desc_sw128(xbase + C::B_BYTES);
 #pragma unroll
             for (int k = 0; k < kBK / 16; ++k) {
 #pragma unroll
               for (int sub = 0; sub < kSub; ++sub) {
                 const uint64_t ad = smem_desc_sw128(wbase + (uint32_t)(sub * a_bytes));
                 const uint32_t d = d0 + (uint32_t)(sub * C::SUB_COLS);
-                tc_mma_bf16(d, ad + 2 * k, bh + 2 * k, idesc, (jj > 0 || k > 0) ? 1u : 0u);
-                if (!C::PAIRED) tc_mma_bf16(d, ad + 2 * k, bl + 2 * k, idesc, 1u);
+                if (PAIR) tc_mma_bf16_pair(d, ad + 2 * k, bh + 2 * k, idesc, (jj > 0 || k > 0) ? 1u : 0u);
+                else tc_mma_bf16(d, ad + 2 * k, bh + 2 * k, idesc, (jj > 0 || k > 0) ? 1u : 0u);
+                if (!C::PAIRED) tc_mma_bf16(d, ad + 2 * k, smem_desc_sw128(xbase + C::B_BYTES) + 2 * k, idesc, 1u);
               }
             }
-            tc_commit(&empty[stage]);
+            commit(&empty[stage]);
             if (++stage == S) {
               stage = 0;
               phase ^= 1u;
             }
           }
           if (!ok) break;
-          tc_commit(&accf[acc]);
+          commit(&accf[acc]);
           ++use;
-          acc ^= 1;
+          if (C::BUFS > 1) acc ^= 1;
         }
       }
       // all issued MMAs complete before TMEM is released
-      tc_commit(drain);
+      commit(drain);
       const unsigned long long t0 = globaltimer();
       while (!mbar_test(smem_addr(drain), 0) && globaltimer() - t0 < kWaitLimitNs) {
       }
@@ -724,8 +769,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   } else if (!ARGMAX && warp >= 2) {
     // Gate and up of one row sit in the same lane, so act is formed in
     // registers.  Tile -1 is a dry run, as above.
-    const bool two = nkb >= 2;
+    const bool two = C::SEGS > 1 && nkb >= 2;
     const bool odd = lane & 1;
+    const uint32_t acce0 = PAIR ? dsmem_addr(acce, 0) : 0u;   // rank 0's, where the issuer waits
     uint32_t use = 0;   // tiles drained
     uint32_t acc0 = 0;  // buffer of the tile's first k-segment (the second's is the other one)
 #pragma unroll 1
@@ -745,7 +791,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         if (it * nkb >= n_units) break;
         const bool ok = two ? mbar_wait(&accf[0], use & 1u, abort_flag, a.status) &&
                                   mbar_wait(&accf[1], use & 1u, abort_flag, a.status)
-                            : mbar_wait(&accf[acc0], (use >> 1) & 1u, abort_flag, a.status);
+                            : mbar_wait(&accf[acc0], uses(use) & 1u, abort_flag, a.status);
         if (!__all_sync(0xffffffffu, ok)) break;
         if (threadIdx.x == 64 && (it + 1) * nkb >= n_units) TL_GEMM(2);
         tc_fence_after();
@@ -794,11 +840,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         tc_fence_before();
         __syncwarp();
         if (lane == 0) {
-          mbar_arrive(&acce[acc0]);
-          if (two) mbar_arrive(&acce[acc0 ^ 1u]);
+          for (uint32_t b = acc0;; b ^= 1u) {
+            if (PAIR) mbar_arrive_remote(acce0 + 8u * b);
+            else mbar_arrive(&acce[b]);
+            if (!two || b != acc0) break;
+          }
         }
         ++use;
-        if (!two) acc0 ^= 1u;
+        if (!two && C::BUFS > 1) acc0 ^= 1u;
       }
     }
   } else if (warp >= 2) {
@@ -869,9 +918,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 0) TL_GEMM(3);
+  if (PAIR) {   // neither CTA leaves while the other's MMAs, copies or arrivals may reach it
+    cluster_arrive_release();
+    cluster_wait_acquire();
+  }
   if (warp == 2) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, C::NCOLS);
+    if (PAIR) tmem_dealloc_pair(tmem_base, C::NCOLS);
+    else tmem_dealloc(tmem_base, C::NCOLS);
   }
 }
 
@@ -1016,11 +1070,13 @@ GemmPlan plan_cluster(int N, int K, bool whole_heads) {
 }
 
 // Whole-K tiles of equal rows that fill the SMs in as few rounds as the MMA's
-// 128 rows allow (gate/up: `rows` of each matrix per tile).
+// 128 rows allow (gate/up: `rows` of each matrix per tile).  The tiles go to pairs
+// of CTAs, so their number is even; the last may lie past the matrix (zeros).
 GemmPlan plan_rows(int N, int K, int n_sms) {
+  n_sms &= ~1;
   const int rounds = (N + kTile * n_sms - 1) / (kTile * n_sms);
   const int rows = ((N + rounds * n_sms - 1) / (rounds * n_sms) + 7) / 8 * 8;
-  const int n_work = (N + rows - 1) / rows;
+  const int n_work = ((N + rows - 1) / rows + 1) & ~1;
   return GemmPlan{rows, n_work, K / kBK, 1, n_work < n_sms ? n_work : n_sms};
 }
 
@@ -1037,9 +1093,9 @@ static cudaError_t launch_tc(Model& m, const GemmW& g, const CUtensorMap& amap, 
   lc.stream = st;
   cudaLaunchAttribute attr[2];
   int n = 0;
-  if (EpiOf<EPI>::cluster) {
+  if (EpiOf<EPI>::cluster || C::PAIR) {
     attr[n].id = cudaLaunchAttributeClusterDimension;
-    attr[n].val.clusterDim.x = a.split;
+    attr[n].val.clusterDim.x = C::PAIR ? 2 : a.split;
     attr[n].val.clusterDim.y = 1;
     attr[n].val.clusterDim.z = 1;
     ++n;
