@@ -154,30 +154,54 @@ OOS_DEV int ordered_select(bool has, int32_t value, int32_t* out, int* s_wcnt, i
   return *s_cnt;
 }
 
-// Insert one lane into the tree (warp 0, all lanes of the warp together): walk
-// down its tokens while the tree has them, then append the rest under the node
-// reached, as far as the node budget goes -- a new node has no children to look
-// for.  Returns whether a node was created.
-OOS_DEV bool hint_insert(int32_t* s_tok, int32_t* s_par, int& T, int max_nodes, const int32_t* lane, int len) {
+// The tree being built: per node its token, parent, depth and path (the 128-bit set
+// of the nodes from the root down to it, itself included).
+struct HintTree {
+  int32_t tok[kMaxT], par[kMaxT], dep[kMaxT];
+  uint32_t path[4][kMaxT];
+};
+
+// Insert one lane into the tree (warp 0, all lanes of the warp together).  The
+// nodes whose token is the lane's at their depth are found for all nodes at once;
+// the lane's longest prefix in the tree ends at the deepest node whose whole path
+// is among them (nodes are distinct per (parent, token), so there is one at most
+// per depth).  The rest of the lane is appended under it, as far as the node
+// budget goes.  Returns whether a node was created.
+OOS_DEV bool hint_insert(HintTree& tr, int& T, int max_nodes, const int32_t* lane, int len) {
   const int lane_id = threadIdx.x & 31;
-  int cur = 0, j = 0;
-  for (; j < len; ++j) {
-    const int t = lane[j];
-    // the child of cur with token t, if any (nodes are distinct per (parent, token))
-    int found = -1;
-    for (int base = 1; base < T && found < 0; base += 32) {
-      const int i = base + lane_id;
-      const unsigned hit = __ballot_sync(0xffffffffu, i < T && s_par[i] == cur && s_tok[i] == t);
-      if (hit) found = base + __ffs(hit) - 1;
-    }
-    if (found < 0) break;
-    cur = found;
+  uint32_t ok[4];
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    const int i = 32 * b + lane_id;
+    const int d = i < T ? tr.dep[i] : 0;
+    ok[b] = __ballot_sync(0xffffffffu, i == 0 || (i < T && d <= len && tr.tok[i] == lane[d - 1]));
   }
+  uint32_t best = 0u;   // depth * 128 + node of the deepest one
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    const int i = 32 * b + lane_id;
+    if (i < T) {
+      bool all = true;
+#pragma unroll
+      for (int w = 0; w < 4; ++w) all = all && (tr.path[w][i] & ~ok[w]) == 0u;
+      if (all) best = max(best, (uint32_t)(tr.dep[i] * kMaxT + i));
+    }
+  }
+  best = __reduce_max_sync(0xffffffffu, best);
+  const int cur = (int)(best % kMaxT), j = (int)(best / kMaxT);
   const int add = min(len - j, max_nodes - T);
   if (add <= 0) return false;
   for (int k = lane_id; k < add; k += 32) {
-    s_tok[T + k] = lane[j + k];
-    s_par[T + k] = k == 0 ? cur : T + k - 1;
+    const int i = T + k;
+    tr.tok[i] = lane[j + k];
+    tr.par[i] = k == 0 ? cur : i - 1;
+    tr.dep[i] = j + k + 1;
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {   // cur's path and the new nodes T .. i
+      const int lo = max(T - 32 * w, 0), hi = min(i - 32 * w, 31);
+      const uint32_t run = hi < lo ? 0u : (0xffffffffu >> (31 - hi)) & (0xffffffffu << lo);
+      tr.path[w][i] = tr.path[w][cur] | run;
+    }
   }
   __syncwarp();
   T += add;
@@ -196,22 +220,43 @@ __global__ void __launch_bounds__(kHintThreads) k_hint_pack(const int32_t* __res
                                                             int max_nodes, const int32_t* __restrict__ prefix_len_dev,
                                                             int pad_to, int32_t* out_tok, int32_t* out_par,
                                                             int32_t* out_T, int32_t* out_info) {
-  __shared__ int32_t s_tok[kMaxT], s_par[kMaxT];
+  __shared__ HintTree tr;
   __shared__ int32_t s_pos[kHintWarps * kHintThreads];   // occurrences in the chunks being visited, in bank order
   __shared__ int32_t s_chunk[kHintFlat];                 // chunks holding an occurrence, in order
   __shared__ int32_t s_span[kHintThreads];               // this round's spans holding an occurrence, in order
   __shared__ int32_t s_lane[kHintWarps][kMaxT];          // the lanes being inserted
+  __shared__ int32_t s_native[kHintWarps][kMaxT];        // the first native lanes
+  __shared__ int s_nlen[kHintWarps];
   __shared__ int s_len[kHintWarps];
   __shared__ int s_wcnt[kHintWarps];
   __shared__ int s_nc, s_ns, s_done;
   const int warp = threadIdx.x >> 5, lane_id = threadIdx.x & 31;
+  // The caller's inputs were written before the match kernel started (it waits for
+  // the kernel before it and lets this one launch only then): what the call needs
+  // of them is loaded while the match kernel runs.
+  auto native_load = [&](int i, int32_t* dst) {   // one native lane, by a warp; returns its length
+    int len = native_len[i];
+    len = len < depth ? len : depth;
+    len = len < native_stride ? len : native_stride;
+    len = len < 0 ? 0 : len;
+    for (int j = lane_id; j < len; j += 32) dst[j] = native[(size_t)i * native_stride + j];
+    return len;
+  };
+  if (warp < n_native) {
+    const int len = native_load(warp, s_native[warp]);
+    if (lane_id == 0) s_nlen[warp] = len;
+  }
+  if (prefix_len_dev) prefix_len = *prefix_len_dev;
+  const int root = prefix[prefix_len - 1];
   pdl_wait();   // the match kernel's results
   pdl_trigger();
-  if (prefix_len_dev) prefix_len = *prefix_len_dev;
   int T = 1, lanes = 0, hint_lanes = 0;       // warp 0's copies are the authoritative ones
   if (threadIdx.x == 0) {
-    s_tok[0] = prefix[prefix_len - 1];
-    s_par[0] = -1;
+    tr.tok[0] = root;
+    tr.par[0] = -1;
+    tr.dep[0] = 0;
+    tr.path[0][0] = 1u;
+    tr.path[1][0] = tr.path[2][0] = tr.path[3][0] = 0u;
     s_done = (max_lanes <= 0 || max_nodes <= 1) ? 1 : 0;
   }
   const int n_chunks = (int)(((long long)N + kHintThreads - 1) / kHintThreads);
@@ -265,7 +310,7 @@ __global__ void __launch_bounds__(kHintThreads) k_hint_pack(const int32_t* __res
         if (warp == 0) {
           for (int u = 0; u < kHintWarps && k + u < total; ++u) {
             if (lanes >= max_lanes || T >= max_nodes) break;
-            if (hint_insert(s_tok, s_par, T, max_nodes, s_lane[u], s_len[u])) {
+            if (hint_insert(tr, T, max_nodes, s_lane[u], s_len[u])) {
               ++lanes;
               ++hint_lanes;
             }
@@ -338,24 +383,21 @@ __global__ void __launch_bounds__(kHintThreads) k_hint_pack(const int32_t* __res
   if (warp == 0) {
     for (int i = 0; i < n_native; ++i) {
       if (lanes >= max_lanes || T >= max_nodes) break;
-      int len = native_len[i];
-      len = len < depth ? len : depth;
-      len = len < native_stride ? len : native_stride;
-      len = len < 0 ? 0 : len;
-      for (int j = lane_id; j < len; j += 32) s_lane[0][j] = native[(size_t)i * native_stride + j];
+      const int32_t* nl = i < kHintWarps ? s_native[i] : s_lane[0];
+      const int len = i < kHintWarps ? s_nlen[i] : native_load(i, s_lane[0]);
       __syncwarp();
-      if (hint_insert(s_tok, s_par, T, max_nodes, s_lane[0], len)) ++lanes;
+      if (hint_insert(tr, T, max_nodes, nl, len)) ++lanes;
       __syncwarp();
     }
     for (int i = lane_id; i < T; i += 32) {
-      out_tok[i] = s_tok[i];
-      out_par[i] = s_par[i];
+      out_tok[i] = tr.tok[i];
+      out_par[i] = tr.par[i];
     }
     // padding up to a fixed node count (the decode loop verifies a fixed T):
     // leaves under the root carrying the root's token; the verifier is told
     // the real node count and never accepts them
     for (int i = T + lane_id; i < pad_to; i += 32) {
-      out_tok[i] = s_tok[0];
+      out_tok[i] = root;
       out_par[i] = 0;
     }
     if (lane_id == 0) {
