@@ -17,7 +17,7 @@ SRC = os.path.join(PKG, "csrc")
 OUT_DIR = os.path.join(PKG, "_lib")
 LIB = os.path.join(OUT_DIR, "liboos.so")
 LIB_TIMELINE = os.path.join(OUT_DIR, "liboos_timeline.so")
-UNITS = ["oos_api.cu", "small.cu", "gemm.cu", "attn.cu", "prefill.cu", "noalloc.cu", "hint.cu", "decode.cu"]
+UNITS = ["oos_api.cu", "small.cu", "gemm.cu", "attn.cu", "prefill.cu", "f32.cu", "noalloc.cu", "hint.cu", "decode.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -40,8 +40,6 @@
 // Prefill runs the same kernel on a chunk of consecutive tokens (CAUSAL): row i
 // attends to every slot up to its own, ctx + i, so a block's keys end at its last
 // row's slot and the mask is a length, not an ancestor set.
-//
-// fp32 path: one block per (node, head), CUDA cores (small models only).
 #include <math.h>
 #include <string.h>
 #include <stdlib.h>
@@ -740,59 +738,6 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
   }
 }
 
-// ------------------------------------------------------------ fp32 path
-__global__ void __launch_bounds__(128) k_attn_f32(const float* __restrict__ q, const float* __restrict__ kc,
-                                                  const float* __restrict__ vc, const unsigned long long* __restrict__ anc,
-                                                  int T, int nq, int nkv, int d, const int32_t* __restrict__ ctx_dev,
-                                                  float scale, float* __restrict__ out) {
-  __shared__ float qs[128];
-  __shared__ float ps[128];
-  __shared__ int kpos[128];
-  __shared__ float red[32];
-  pdl_wait();
-  pdl_trigger();
-  const int ctx = *ctx_dev;
-  const int i = blockIdx.x, h = blockIdx.y, g = h / (nq / nkv), tid = threadIdx.x;
-  if (tid < d) qs[tid] = q[((size_t)i * nq + h) * d + tid];
-  const unsigned long long w0 = anc[2 * i], w1 = anc[2 * i + 1];
-  __syncthreads();
-  float m = -INFINITY, l = 0.f, acc = 0.f;
-  const int n_keys = ctx + T;
-  for (int base = 0; base < n_keys; base += blockDim.x) {
-    const int kk = base + tid;
-    bool valid = kk < n_keys;
-    if (valid && kk >= ctx) {
-      const int j = kk - ctx;
-      valid = ((j < 64 ? (w0 >> j) : (w1 >> (j - 64))) & 1ull) != 0;
-    }
-    float sc = -INFINITY;
-    if (valid) {
-      const float* kr = kc + ((size_t)kk * nkv + g) * d;
-      float dot = 0.f;
-      for (int c = 0; c < d; ++c) dot += qs[c] * kr[c];
-      sc = dot * scale;
-    }
-    const float cmax = block_max(sc, red);
-    const float mn = fmaxf(m, cmax);
-    const float p = valid ? expf(sc - mn) : 0.f;
-    const float corr = (m == -INFINITY) ? 0.f : expf(m - mn);
-    const float psum = block_sum(p, red);
-    l = l * corr + psum;
-    ps[tid] = p;
-    kpos[tid] = kk;
-    __syncthreads();
-    if (tid < d) {
-      acc *= corr;
-      const int nk = min((int)blockDim.x, n_keys - base);
-      for (int k = 0; k < nk; ++k)
-        if (ps[k] != 0.f) acc += ps[k] * vc[((size_t)kpos[k] * nkv + g) * d + tid];
-    }
-    m = mn;
-    __syncthreads();
-  }
-  if (tid < d) out[(size_t)i * nq * d + (size_t)h * d + tid] = acc / l;
-}
-
 int attn_nodes_per_block(int group) { return group >= kAttnRows ? 1 : kAttnRows / group; }
 
 static bool encode_q_maps(const Model& m, const void* q, int nodes, CUtensorMap* hi, CUtensorMap* lo) {
@@ -922,18 +867,13 @@ static cudaError_t launch_attn_tc(Model& m, int layer, const void* kc, const voi
 
 cudaError_t launch_attention(Model& m, int layer, const void* kc, const void* vc, int capacity, int ctx, int T,
                              cudaStream_t st) {
-  const auto& c = m.cfg;
-  if (c.dtype != OOS_DTYPE_BF16) {
-    return launch(m.pdl, k_attn_f32, dim3(T, c.n_q_heads), dim3(128), 0, st, (const float*)m.ws.q, (const float*)kc,
-                  (const float*)vc, (const unsigned long long*)m.ws.anc, T, c.n_q_heads, c.n_kv_heads, c.head_dim,
-                  (const int32_t*)m.ws.ctx, 1.0f / sqrtf((float)c.head_dim), (float*)m.ws.attn);
-  }
+  if (m.cfg.dtype != OOS_DTYPE_BF16) return launch_f32_attention(m, kc, vc, T, st);
   AttnArgs a;
   memset(&a, 0, sizeof(a));
   a.qhi = m.qmap_hi;
   a.qlo = m.qmap_lo;
   a.out = (__nv_bfloat16*)m.ws.attn;
-  a.out_lo_off = (size_t)kMaxT * c.n_q_heads * kAttnD;
+  a.out_lo_off = (size_t)kMaxT * m.cfg.n_q_heads * kAttnD;
   return launch_attn_tc<false>(m, layer, kc, vc, capacity, ctx, T, a, st);
 }
 

@@ -110,6 +110,60 @@ OOS_DEV float block_max(float v, float* red) {
   return s;
 }
 
+// Sums of v[0..N) over the warp.  At each step a lane keeps the half of the values
+// its lane bit selects, so N values cost about 2N shuffles, not 5N; on return
+// v[0..n) hold the sums of elements base..base+n-1.
+template <int N>
+OOS_DEV void warp_sums(float (&v)[N], int& base, int& n) {
+  const int lane = threadIdx.x & 31;
+  base = 0;
+  n = N;
+  int len = N;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    if (len % 2 == 0) {
+      const int h = len / 2;
+      const bool up = lane & o;
+#pragma unroll
+      for (int i = 0; i < N / 2; ++i) {
+        if (i < h) {
+          const float send = up ? v[i] : v[i + h], keep = up ? v[i + h] : v[i];
+          v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+      }
+      if (up) base += h;
+      len = h;
+    } else {
+#pragma unroll
+      for (int i = 0; i < N; ++i)
+        if (i < len) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+    }
+  }
+  n = len;
+}
+
+// ---- running greedy state: largest logit, its (lowest) vocab id, second largest
+// logit counted with multiplicity.  Merging is order independent for finite logits
+// and infinities; a NaN compares false everywhere, so a row whose logits contain
+// NaN gets a layout-dependent result.
+struct Top2 {
+  float v1;
+  int i1;
+  float v2;
+};
+OOS_DEV Top2 top2_merge(Top2 a, Top2 b) {
+  Top2 r;
+  if (a.v1 > b.v1 || (a.v1 == b.v1 && a.i1 <= b.i1)) {
+    r.v1 = a.v1;
+    r.i1 = a.i1;
+  } else {
+    r.v1 = b.v1;
+    r.i1 = b.i1;
+  }
+  r.v2 = fmaxf(fminf(a.v1, b.v1), fmaxf(a.v2, b.v2));
+  return r;
+}
+
 // ---- programmatic dependent launch
 OOS_DEV void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 OOS_DEV void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -10,8 +10,6 @@
 // The layer's elementwise steps run in the GEMM epilogues (see below); the LM
 // head keeps a per-node running (max, argmax, second max) so logits never
 // reach memory.
-//
-// fp32 path: CUDA-core warp-per-row GEMV kernels (small models only).
 #include <string.h>
 
 #include "common.cuh"
@@ -171,24 +169,6 @@ struct TcCfg {
     return FIXED + ring;
   }
 };
-
-struct Top2s {
-  float v1;
-  int i1;
-  float v2;
-};
-OOS_DEV Top2s t2_merge(Top2s a, Top2s b) {
-  Top2s r;
-  if (a.v1 > b.v1 || (a.v1 == b.v1 && a.i1 <= b.i1)) {
-    r.v1 = a.v1;
-    r.i1 = a.i1;
-  } else {
-    r.v1 = b.v1;
-    r.i1 = b.i1;
-  }
-  r.v2 = fmaxf(fminf(a.v1, b.v1), fmaxf(a.v2, b.v2));
-  return r;
-}
 
 OOS_DEV void epi_bar() { asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory"); }
 
@@ -394,8 +374,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   static_assert((2 * kMaxStages + 5) * 8 + 12 <= C::BAR_BYTES, "barrier block");
   float* rms = reinterpret_cast<float*>(smem + C::BAR_BYTES);                                  // [kMaxT]
-  Top2s* red = reinterpret_cast<Top2s*>(smem + C::BAR_BYTES + C::EPI_BYTES);                   // [4][BN]
-  Top2s* run = red + 4 * BN;                                                                   // [BN]
+  Top2* red = reinterpret_cast<Top2*>(smem + C::BAR_BYTES + C::EPI_BYTES);                   // [4][BN]
+  Top2* run = red + 4 * BN;                                                                   // [BN]
   unsigned char* ring = smem + C::HEAD;
   unsigned char* ring_x = ring + S * kSub * a_bytes;
 
@@ -453,7 +433,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     else tmem_alloc(tmem_slot, C::NCOLS);
   }
   if (ARGMAX && threadIdx.x >= 64) {
-    for (int e = threadIdx.x - 64; e < BN; e += kEpiThreads) run[e] = Top2s{-INFINITY, 0x7fffffff, -INFINITY};
+    for (int e = threadIdx.x - 64; e < BN; e += kEpiThreads) run[e] = Top2{-INFINITY, 0x7fffffff, -INFINITY};
   }
   tc_fence_before();
   __syncthreads();
@@ -878,18 +858,18 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
           acc16(col0 + sub * C::SUB_COLS + cc * 16, v);
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
-            Top2s s{f < a.N ? v[i] * rms[cc * 16 + i] : -INFINITY, f, -INFINITY};
+            Top2 s{f < a.N ? v[i] * rms[cc * 16 + i] : -INFINITY, f, -INFINITY};
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
-              Top2s y;
+              Top2 y;
               y.v1 = __shfl_xor_sync(0xffffffffu, s.v1, o);
               y.i1 = __shfl_xor_sync(0xffffffffu, s.i1, o);
               y.v2 = __shfl_xor_sync(0xffffffffu, s.v2, o);
-              s = t2_merge(s, y);
+              s = top2_merge(s, y);
             }
             if (lane == 0) {
-              Top2s* slot = &red[q * BN + cc * 16 + i];
-              *slot = sub == 0 ? s : t2_merge(*slot, s);
+              Top2* slot = &red[q * BN + cc * 16 + i];
+              *slot = sub == 0 ? s : top2_merge(*slot, s);
             }
           }
         }
@@ -899,9 +879,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       if (lane == 0) mbar_arrive(&acce[acc]);
       epi_bar();
       if (e < T) {
-        Top2s r = run[e];
+        Top2 r = run[e];
 #pragma unroll
-        for (int w = 0; w < 4; ++w) r = t2_merge(r, red[w * BN + e]);
+        for (int w = 0; w < 4; ++w) r = top2_merge(r, red[w * BN + e]);
         run[e] = r;
       }
       epi_bar();
@@ -909,7 +889,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       acc ^= 1;
     }
     if (e < T) {
-      const Top2s r = run[e];
+      const Top2 r = run[e];
       a.am_v1[(size_t)blockIdx.x * kMaxT + e] = r.v1;
       a.am_i[(size_t)blockIdx.x * kMaxT + e] = r.i1;
       a.am_v2[(size_t)blockIdx.x * kMaxT + e] = r.v2;
@@ -1245,74 +1225,6 @@ cudaError_t launch_lm_head_tc(Model& m, int T, cudaStream_t st) {
   a.am_i = m.ws.lm_i;
   a.am_v2 = m.ws.lm_v2;
   return dispatch_tc<EPI_ARGMAX>(m, m.g_lm, m.amap_xn, T, a, st);
-}
-
-// ------------------------------------------------------------ fp32 CUDA-core path
-// One warp per output row; part[t][f] = W[f] . x[t] (a single slice).
-__global__ void __launch_bounds__(128) k_gemm_f32(const float* __restrict__ w0, const float* __restrict__ w1,
-                                                  const float* __restrict__ w2, int r0, int r1, int r2, int K,
-                                                  const float* __restrict__ x, int T, float* __restrict__ part) {
-  pdl_wait();
-  pdl_trigger();
-  const int N = r0 + r1 + r2;
-  const int f = blockIdx.x * 4 + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (f < N) {
-    const float* w = f < r0 ? w0 + (size_t)f * K : f < r0 + r1 ? w1 + (size_t)(f - r0) * K : w2 + (size_t)(f - r0 - r1) * K;
-    for (int t = 0; t < T; ++t) {
-      const float* xr = x + (size_t)t * K;
-      float acc = 0.f;
-      for (int k = lane; k < K; k += 32) acc += w[k] * xr[k];
-      acc = warp_sum(acc);
-      if (lane == 0) part[(size_t)t * N + f] = acc;
-    }
-  }
-}
-
-cudaError_t launch_gemm_f32(Model& m, const void* w0, const void* w1, const void* w2, int rows0, int rows1, int rows2,
-                            int K, const void* x, int T, cudaStream_t st) {
-  const int N = rows0 + rows1 + rows2;
-  return launch(m.pdl, k_gemm_f32, dim3((N + 3) / 4), dim3(128), 0, st, (const float*)w0, (const float*)w1,
-                (const float*)w2, rows0, rows1, rows2, K, (const float*)x, T, m.ws.part);
-}
-
-// LM head, fp32: block b scans vocab rows [b*rows, (b+1)*rows); warp w keeps a
-// running top-2 per node over its rows; warps merge in order at the end.
-__global__ void __launch_bounds__(128) k_lm_head_f32(const float* __restrict__ W, int V, int H, int rows_per_block,
-                                                     const float* __restrict__ x, int T, float* am_v1, int32_t* am_i,
-                                                     float* am_v2) {
-  __shared__ Top2s st[4][kMaxT];
-  pdl_wait();
-  pdl_trigger();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int t = lane; t < T; t += 32) st[warp][t] = Top2s{-INFINITY, 0x7fffffff, -INFINITY};
-  const int r_begin = blockIdx.x * rows_per_block;
-  const int r_end = min(V, r_begin + rows_per_block);
-  for (int r = r_begin + warp; r < r_end; r += 4) {
-    const float* w = W + (size_t)r * H;
-    for (int t = 0; t < T; ++t) {
-      const float* xr = x + (size_t)t * H;
-      float acc = 0.f;
-      for (int k = lane; k < H; k += 32) acc += w[k] * xr[k];
-      acc = warp_sum(acc);
-      if (lane == 0) st[warp][t] = t2_merge(st[warp][t], Top2s{acc, r, -INFINITY});
-    }
-  }
-  __syncthreads();
-  for (int t = threadIdx.x; t < T; t += blockDim.x) {
-    Top2s r = st[0][t];
-    for (int w = 1; w < 4; ++w) r = t2_merge(r, st[w][t]);
-    am_v1[(size_t)blockIdx.x * kMaxT + t] = r.v1;
-    am_i[(size_t)blockIdx.x * kMaxT + t] = r.i1;
-    am_v2[(size_t)blockIdx.x * kMaxT + t] = r.v2;
-  }
-}
-
-cudaError_t launch_lm_head_f32(Model& m, int T, cudaStream_t st) {
-  const int V = m.cfg.vocab;
-  const int rows = (V + m.lm_grid - 1) / m.lm_grid;
-  return launch(m.pdl, k_lm_head_f32, dim3(m.lm_grid), dim3(128), 0, st, (const float*)m.w.lm_head, V, m.cfg.hidden,
-                rows, (const float*)m.ws.xn, T, m.ws.lm_v1, m.ws.lm_i, m.ws.lm_v2);
 }
 
 }  // namespace oos

@@ -54,7 +54,6 @@ struct Workspace {
   void* q;                   // [kMaxT][nq][d]
   void* attn;                // attention output [kMaxT][nq*d]
   void* act;                 // SwiGLU activation [kMaxT][I]
-  float* part;               // GEMM outputs before their epilogue kernel (fp32 path)
   float* lm_v1;              // LM-head partial states [kMaxGridCTAs][kMaxT]
   int32_t* lm_i;
   float* lm_v2;
@@ -63,7 +62,7 @@ struct Workspace {
   float* top1;
   float* top2;
   float* ss;                 // sum of x^2 per feature tile [kMaxSsChunks][kMaxT] (bf16 path)
-  float2* rope;              // (cos, sin) per node and rotary pair [kMaxT][d/2] (bf16 path)
+  float2* rope;              // (cos, sin) per node and rotary pair [kMaxT][d/2]
   int32_t* chain_parent;     // [kMaxT]: -1, 0, 1, ... (the chains a prefill runs as trees)
   int32_t* pf_scratch;       // prefill's unused accept outputs: len, bonus, nodes[kMaxT], tokens[kMaxT]
   // prefill chunks (bf16 path): the buffers above for kPfTokens rows.  act
@@ -155,13 +154,9 @@ cudaError_t launch_tree_prep(Model& m, const int32_t* tokens, const int32_t* par
 cudaGraphNode_t find_tree_prep_node(cudaGraph_t g);
 cudaError_t set_tree_prep_ctx(Model& m, cudaGraphExec_t ex, cudaGraphNode_t node, const int32_t* tokens,
                               const int32_t* parent, int T, int ctx);
-cudaError_t launch_embed_norm(Model& m, const int32_t* tokens, int T, cudaStream_t st);
 cudaError_t launch_embed_tc(Model& m, const int32_t* tokens, int T, cudaStream_t st);
 cudaError_t launch_embed_pf(Model& m, const int32_t* tokens, int T, cudaStream_t st);
 cudaError_t launch_final_hidden(Model& m, float* hidden, int T, cudaStream_t st);
-cudaError_t launch_qkv_post(Model& m, int layer, void* kc, void* vc, int T, cudaStream_t st);
-cudaError_t launch_resid_norm(Model& m, const void* gain, float* hidden_out, int T, cudaStream_t st);
-cudaError_t launch_silu_mul(Model& m, int T, cudaStream_t st);
 // n_valid: DEVICE count of real nodes (the rest is padding, never accepted), or nullptr for T
 cudaError_t launch_argmax_accept(Model& m, const int32_t* tokens, const int32_t* parent, int T, const int32_t* n_valid,
                                  int n_parts, int32_t* len, int32_t* nodes, int32_t* toks, int32_t* bonus,
@@ -196,9 +191,16 @@ int norm_chunks(const Model& m, int layer);
 cudaError_t launch_chunk_qkv(Model& m, int layer, void* kc, void* vc, int T, int split, cudaStream_t st);
 cudaError_t launch_chunk_resid(Model& m, int layer, bool down, const void* gain, int T, int split, cudaStream_t st);
 cudaError_t launch_chunk_gu(Model& m, int layer, int T, cudaStream_t st);
-cudaError_t launch_gemm_f32(Model& m, const void* w0, const void* w1, const void* w2, int rows0, int rows1,
-                            int rows2, int K, const void* x, int T, cudaStream_t st);
-cudaError_t launch_lm_head_f32(Model& m, int T, cudaStream_t st);
+
+// ---- fp32 path (f32.cu)
+cudaError_t launch_f32_embed(Model& m, const int32_t* tokens, int T, cudaStream_t st);
+cudaError_t launch_f32_qkv(Model& m, int layer, void* kc, void* vc, int T, cudaStream_t st);
+cudaError_t launch_f32_attention(Model& m, const void* kc, const void* vc, int T, cudaStream_t st);
+cudaError_t launch_f32_o(Model& m, int layer, int T, cudaStream_t st);
+cudaError_t launch_f32_gu(Model& m, int layer, int T, cudaStream_t st);
+cudaError_t launch_f32_down(Model& m, int layer, int T, cudaStream_t st);
+cudaError_t launch_f32_lm_head(Model& m, int T, cudaStream_t st);
+cudaError_t launch_f32_hidden(Model& m, float* hidden, int T, cudaStream_t st);
 
 // ---- verify step with the committed length and the count of real nodes in
 // device memory (oos_api.cu): tokens/parent hold T nodes of which *n_valid are

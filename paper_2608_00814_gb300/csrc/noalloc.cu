@@ -16,46 +16,26 @@ constexpr int kStaticBlocks = 512;   // vocabulary blocks per call (grid size)
 constexpr int kStaticMaxT = 128;     // rows of `hidden` per call
 constexpr int kStaticThreads = 256;
 
-struct StaticTop2 {
-  float v1;
-  int i1;
-  float v2;
-};
-
 // Shared by every call on a device: [block][row] partial top-2 states, then the
 // arrival counter (zero at load; the last block of a call sets it back to zero).
 struct StaticScratch {
-  StaticTop2 part[kStaticBlocks][kStaticMaxT];
+  Top2 part[kStaticBlocks][kStaticMaxT];
   int arrived;
 };
 static __device__ __align__(256) StaticScratch g_argmax_scratch;
-
-// Merge of two running top-2 states.  Order independent for finite logits (and
-// infinities); a NaN logit compares false everywhere, so rows whose logits
-// contain NaN get a layout-dependent result.
-OOS_DEV StaticTop2 st_merge(StaticTop2 a, StaticTop2 b) {
-  StaticTop2 r;
-  if (a.v1 > b.v1 || (a.v1 == b.v1 && a.i1 <= b.i1)) {
-    r.v1 = a.v1;
-    r.i1 = a.i1;
-  } else {
-    r.v1 = b.v1;
-    r.i1 = b.i1;
-  }
-  r.v2 = fmaxf(fminf(a.v1, b.v1), fmaxf(a.v2, b.v2));
-  return r;
-}
 
 // A task is `R` vocabulary rows by `TT` hidden rows, one warp.  The lanes split
 // the hidden dimension (VEC consecutive elements each in turn), so that every
 // logit is 32 short fp32 chains added as a tree; the R x TT products of the
 // loaded elements are formed in registers.
 //
-// What bounds it is FMA issue from about 8 hidden rows on, below that the weight
-// stream: per VEC elements a lane loads R + 2 TT 16-byte words for R * TT * VEC
-// FMAs.  R = 8 (bf16) or 4 (fp32) and TT <= 8 keep the sums and the loaded weights
-// in registers.  The warps of a block take the token groups of a row group side by side, so a row group
-// comes from HBM once and from L1 after that.
+// What bounds it is the weight stream for a few hidden rows (T = 1: 230 us for the
+// 1.24 GB of 151936 x 4096 bf16) and, from about 6 on, FMA issue behind loads of
+// hidden rows that L1 does not hold: per VEC elements a lane loads R + 2 TT 16-byte
+// words for R * TT * VEC FMAs.  R = 8 (bf16) or 4 (fp32) and TT <= 8 keep the sums
+// and the loaded weights in registers.  The warps of a block take the token groups
+// of a row group side by side, so a row group comes from HBM once and from L1 after
+// that.  17 rows: 9051 us with one FMA per load, 765 now (303 of FMAs).
 template <typename E>
 struct StaticRows {
   static constexpr int v = sizeof(E) == 2 ? 8 : 4;
@@ -94,38 +74,6 @@ struct StaticVec<E, 1> {
   OOS_DEV float get(int) const { return v; }
 };
 
-// Sums of v[0..N) over the warp.  At each step a lane keeps the half of the
-// values its lane bit selects, so N values cost about 2N shuffles, not 5N; on
-// return v[0..n) hold the sums of elements base..base+n-1.
-template <int N>
-OOS_DEV void warp_sums(float (&v)[N], int& base, int& n) {
-  const int lane = threadIdx.x & 31;
-  base = 0;
-  n = N;
-  int len = N;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    if (len % 2 == 0) {
-      const int h = len / 2;
-      const bool up = lane & o;
-#pragma unroll
-      for (int i = 0; i < N / 2; ++i) {
-        if (i < h) {
-          const float send = up ? v[i] : v[i + h], keep = up ? v[i + h] : v[i];
-          v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-        }
-      }
-      if (up) base += h;
-      len = h;
-    } else {
-#pragma unroll
-      for (int i = 0; i < N; ++i)
-        if (i < len) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
-    }
-  }
-  n = len;
-}
-
 // Block b scans vocabulary rows [b*rows, (b+1)*rows) in tasks (row group, token
 // group), one warp each; every logit updates that warp's running top-2.  The
 // last block to finish merges all blocks' states, in block order.
@@ -134,11 +82,11 @@ __global__ void __launch_bounds__(kStaticThreads, static_blocks_per_sm(TT))
     k_lm_argmax_static(const E* __restrict__ W, int V, int H, int rows_per_block, const float* __restrict__ hidden, int T,
                        StaticScratch* sc, int32_t* out_argmax, float* out_top1, float* out_top2) {
   constexpr int R = StaticRows<E>::v, WARPS = kStaticThreads / 32;
-  __shared__ StaticTop2 st[WARPS][kStaticMaxT];
+  __shared__ Top2 st[WARPS][kStaticMaxT];
   __shared__ float lg[WARPS][R * TT];
   __shared__ int s_last;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int t = lane; t < T; t += 32) st[warp][t] = StaticTop2{-INFINITY, 0x7fffffff, -INFINITY};
+  for (int t = lane; t < T; t += 32) st[warp][t] = Top2{-INFINITY, 0x7fffffff, -INFINITY};
   __syncwarp();
   const int r_begin = blockIdx.x * rows_per_block;
   const int r_end = min(V, r_begin + rows_per_block);
@@ -177,16 +125,16 @@ __global__ void __launch_bounds__(kStaticThreads, static_blocks_per_sm(TT))
       if (i < n) lg[warp][base + i] = acc[i];
     __syncwarp();
     if (lane < nt) {
-      StaticTop2 s = st[warp][t0 + lane];
-      for (int r = 0; r < nr; ++r) s = st_merge(s, StaticTop2{lg[warp][r * TT + lane], r0 + r, -INFINITY});
+      Top2 s = st[warp][t0 + lane];
+      for (int r = 0; r < nr; ++r) s = top2_merge(s, Top2{lg[warp][r * TT + lane], r0 + r, -INFINITY});
       st[warp][t0 + lane] = s;
     }
     __syncwarp();
   }
   __syncthreads();
   for (int t = threadIdx.x; t < T; t += blockDim.x) {
-    StaticTop2 r = st[0][t];
-    for (int w = 1; w < WARPS; ++w) r = st_merge(r, st[w][t]);
+    Top2 r = st[0][t];
+    for (int w = 1; w < WARPS; ++w) r = top2_merge(r, st[w][t]);
     sc->part[blockIdx.x][t] = r;
   }
   __threadfence();
@@ -199,10 +147,10 @@ __global__ void __launch_bounds__(kStaticThreads, static_blocks_per_sm(TT))
   if (!s_last) return;
   __threadfence();
   for (int t = threadIdx.x; t < T; t += blockDim.x) {
-    StaticTop2 r{-INFINITY, 0x7fffffff, -INFINITY};
+    Top2 r{-INFINITY, 0x7fffffff, -INFINITY};
     for (int b = 0; b < (int)gridDim.x; ++b) {
-      const StaticTop2 p{__ldcg(&sc->part[b][t].v1), __ldcg(&sc->part[b][t].i1), __ldcg(&sc->part[b][t].v2)};
-      r = st_merge(r, p);
+      const Top2 p{__ldcg(&sc->part[b][t].v1), __ldcg(&sc->part[b][t].i1), __ldcg(&sc->part[b][t].v2)};
+      r = top2_merge(r, p);
     }
     out_argmax[t] = r.i1;
     out_top1[t] = r.v1;

@@ -33,7 +33,6 @@ size_t carve_workspace(const oos_model_config& c, int n_sms, uint8_t* base, Work
   };
   const size_t es = c.dtype == OOS_DTYPE_BF16 ? 2 : 4;
   const size_t H = c.hidden, I = c.intermediate, qd = (size_t)c.n_q_heads * c.head_dim;
-  const size_t kvd = (size_t)c.n_kv_heads * c.head_dim;
   Workspace w;
   w.status = (uint32_t*)take(256);
   w.ctx = (int32_t*)take(256);
@@ -46,8 +45,6 @@ size_t carve_workspace(const oos_model_config& c, int n_sms, uint8_t* base, Work
   w.q = take(halves * kMaxT * qd * es);
   w.attn = take(halves * kMaxT * qd * es);
   w.act = take(halves * kMaxT * I * es);
-  const size_t Nq = qd + 2 * kvd;
-  w.part = (float*)take(c.dtype == OOS_DTYPE_BF16 ? 0 : (size_t)kMaxT * std::max(std::max(Nq, H), 2 * I) * 4);
   const size_t lm = (size_t)kMaxGridCTAs * kMaxT;
   w.lm_v1 = (float*)take(lm * 4);
   w.lm_i = (int32_t*)take(lm * 4);
@@ -155,37 +152,19 @@ static unsigned long long kv_hash(const oos_kv_cache* kv) {
 // committed length ctx comes from the host, or from device memory when ctx_dev
 // is not null (then any value up to the cache capacity is allowed).
 static int enqueue_layers(Model& m, const oos_kv_cache* kv, int ctx, const int32_t* ctx_dev, const int32_t* tokens,
-                          const int32_t* parent, int T, float* hidden, cudaStream_t st) {
+                          const int32_t* parent, int T, cudaStream_t st) {
   const auto& c = m.cfg;
-  const int L = c.n_layers;
-  const int qd = c.n_q_heads * c.head_dim, kvd = c.n_kv_heads * c.head_dim;
   const int ctx_hint = ctx_dev ? kv->capacity - T : ctx;   // sizes the attention's key splits
+  const bool tc = c.dtype == OOS_DTYPE_BF16;
   OOS_TRY(launch_tree_prep(m, tokens, parent, T, ctx, ctx_dev, st));
-  if (c.dtype == OOS_DTYPE_BF16) OOS_TRY(launch_embed_tc(m, tokens, T, st));
-  else OOS_TRY(launch_embed_norm(m, tokens, T, st));
-  for (int l = 0; l < L; ++l) {
-    const oos_layer_weights& W = m.layers[l];
-    const void* next_gain = (l + 1 < L) ? m.layers[l + 1].attn_norm : m.w.final_norm;
-    float* hid = (l + 1 < L) ? nullptr : hidden;
-    if (c.dtype == OOS_DTYPE_BF16) {
-      // five kernels per layer; every elementwise step runs in a GEMM epilogue
-      OOS_TRY(launch_gemm_qkv(m, l, kv->k[l], kv->v[l], T, st));
-      OOS_TRY(launch_attention(m, l, kv->k[l], kv->v[l], kv->capacity, ctx_hint, T, st));
-      OOS_TRY(launch_gemm_o(m, l, T, st));
-      OOS_TRY(launch_gemm_gu(m, l, T, st));
-      OOS_TRY(launch_gemm_down(m, l, T, st));
-    } else {
-      OOS_TRY(launch_gemm_f32(m, W.w_q, W.w_k, W.w_v, qd, kvd, kvd, c.hidden, m.ws.xn, T, st));
-      OOS_TRY(launch_qkv_post(m, l, kv->k[l], kv->v[l], T, st));
-      OOS_TRY(launch_attention(m, l, kv->k[l], kv->v[l], kv->capacity, ctx_hint, T, st));
-      OOS_TRY(launch_gemm_f32(m, W.w_o, nullptr, nullptr, c.hidden, 0, 0, qd, m.ws.attn, T, st));
-      OOS_TRY(launch_resid_norm(m, W.mlp_norm, nullptr, T, st));
-      OOS_TRY(launch_gemm_f32(m, W.w_gate, W.w_up, nullptr, c.intermediate, c.intermediate, 0, c.hidden, m.ws.xn, T,
-                              st));
-      OOS_TRY(launch_silu_mul(m, T, st));
-      OOS_TRY(launch_gemm_f32(m, W.w_down, nullptr, nullptr, c.hidden, 0, 0, c.intermediate, m.ws.act, T, st));
-      OOS_TRY(launch_resid_norm(m, next_gain, hid, T, st));
-    }
+  OOS_TRY(tc ? launch_embed_tc(m, tokens, T, st) : launch_f32_embed(m, tokens, T, st));
+  // five kernels per layer; every elementwise step runs in a projection
+  for (int l = 0; l < c.n_layers; ++l) {
+    OOS_TRY(tc ? launch_gemm_qkv(m, l, kv->k[l], kv->v[l], T, st) : launch_f32_qkv(m, l, kv->k[l], kv->v[l], T, st));
+    OOS_TRY(launch_attention(m, l, kv->k[l], kv->v[l], kv->capacity, ctx_hint, T, st));
+    OOS_TRY(tc ? launch_gemm_o(m, l, T, st) : launch_f32_o(m, l, T, st));
+    OOS_TRY(tc ? launch_gemm_gu(m, l, T, st) : launch_f32_gu(m, l, T, st));
+    OOS_TRY(tc ? launch_gemm_down(m, l, T, st) : launch_f32_down(m, l, T, st));
   }
   return OOS_OK;
 }
@@ -196,13 +175,14 @@ static int enqueue_verify(Model& m, const oos_kv_cache* kv, int ctx, const int32
                           int32_t* toks, int32_t* bonus, float* hidden, int32_t* dbg_arg, float* dbg_t1,
                           float* dbg_t2, cudaStream_t st) {
   const auto& c = m.cfg;
-  const int rc = enqueue_layers(m, kv, ctx, ctx_dev, tokens, parent, T, hidden, st);
+  const int rc = enqueue_layers(m, kv, ctx, ctx_dev, tokens, parent, T, st);
   if (rc != OOS_OK) return rc;
   if (c.dtype == OOS_DTYPE_BF16) {
     if (hidden) OOS_TRY(launch_final_hidden(m, hidden, T, st));
     OOS_TRY(launch_lm_head_tc(m, T, st));
   } else {
-    OOS_TRY(launch_lm_head_f32(m, T, st));
+    if (hidden) OOS_TRY(launch_f32_hidden(m, hidden, T, st));
+    OOS_TRY(launch_f32_lm_head(m, T, st));
   }
   OOS_TRY(launch_argmax_accept(m, tokens, parent, T, n_valid, m.lm_grid, len, nodes, toks, bonus, dbg_arg, dbg_t1,
                                dbg_t2, st));
@@ -237,13 +217,13 @@ static int prefill_impl(Model& m, const oos_kv_cache* kv, int ctx, const int32_t
       OOS_TRY(prefill_chunk(m, kv, ctx + off, tokens + off, T, off == 0, st));
       if (last) OOS_TRY(prefill_last(m, T, st));
     } else {
-      const int rc = enqueue_layers(m, kv, ctx + off, nullptr, tokens + off, m.ws.chain_parent, T, nullptr, st);
+      const int rc = enqueue_layers(m, kv, ctx + off, nullptr, tokens + off, m.ws.chain_parent, T, st);
       if (rc != OOS_OK) return rc;
     }
     if (!last) continue;
     const int rows = wide ? 1 : T;   // rows the LM head sees, the prompt's last token the last of them
     if (tc) OOS_TRY(launch_lm_head_tc(m, rows, st));
-    else OOS_TRY(launch_lm_head_f32(m, rows, st));
+    else OOS_TRY(launch_f32_lm_head(m, rows, st));
     OOS_TRY(launch_argmax_accept(m, tokens + n - rows, m.ws.chain_parent, rows, nullptr, m.lm_grid, sc, sc + 2,
                                  sc + 2 + kMaxT, sc + 1, nullptr, nullptr, nullptr, st));
     if (next_token) OOS_TRY(cudaMemcpyAsync(next_token, m.ws.argmax + (rows - 1), 4, cudaMemcpyDeviceToDevice, st));
@@ -524,10 +504,8 @@ int oos_launch_stage(oos_model* m, int32_t layer, int32_t stage, int32_t T, void
   if (!m || T < 1 || T > m->cfg.max_T || stage < OOS_STAGE_QKV || stage > OOS_STAGE_LM_HEAD) return OOS_EINVAL;
   if (stage != OOS_STAGE_LM_HEAD && (layer < 0 || layer >= m->cfg.n_layers)) return OOS_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
-  const auto& c = m->cfg;
-  const int qd = c.n_q_heads * c.head_dim, kvd = c.n_kv_heads * c.head_dim;
   cudaError_t e;
-  if (c.dtype == OOS_DTYPE_BF16) {
+  if (m->cfg.dtype == OOS_DTYPE_BF16) {
     switch (stage) {
       case OOS_STAGE_QKV: return OOS_EINVAL;   // its epilogue writes the KV cache
       case OOS_STAGE_O: e = launch_gemm_o(*m, layer, T, st); break;
@@ -536,18 +514,12 @@ int oos_launch_stage(oos_model* m, int32_t layer, int32_t stage, int32_t T, void
       default: e = launch_lm_head_tc(*m, T, st); break;
     }
   } else {
-    const oos_layer_weights& W = m->layers[stage == OOS_STAGE_LM_HEAD ? 0 : layer];
     switch (stage) {
-      case OOS_STAGE_QKV: e = launch_gemm_f32(*m, W.w_q, W.w_k, W.w_v, qd, kvd, kvd, c.hidden, m->ws.xn, T, st); break;
-      case OOS_STAGE_O: e = launch_gemm_f32(*m, W.w_o, nullptr, nullptr, c.hidden, 0, 0, qd, m->ws.attn, T, st); break;
-      case OOS_STAGE_GATE_UP:
-        e = launch_gemm_f32(*m, W.w_gate, W.w_up, nullptr, c.intermediate, c.intermediate, 0, c.hidden, m->ws.xn, T,
-                            st);
-        break;
-      case OOS_STAGE_DOWN:
-        e = launch_gemm_f32(*m, W.w_down, nullptr, nullptr, c.hidden, 0, 0, c.intermediate, m->ws.act, T, st);
-        break;
-      default: e = launch_lm_head_f32(*m, T, st); break;
+      case OOS_STAGE_QKV: e = launch_f32_qkv(*m, layer, nullptr, nullptr, T, st); break;   // leaves the KV cache alone
+      case OOS_STAGE_O: e = launch_f32_o(*m, layer, T, st); break;
+      case OOS_STAGE_GATE_UP: e = launch_f32_gu(*m, layer, T, st); break;
+      case OOS_STAGE_DOWN: e = launch_f32_down(*m, layer, T, st); break;
+      default: e = launch_f32_lm_head(*m, T, st); break;
     }
   }
   return e == cudaSuccess ? OOS_OK : OOS_ECUDA;

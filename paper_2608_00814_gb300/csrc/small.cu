@@ -1,5 +1,4 @@
-// Small kernels of the verify step: tree preparation, embedding, the GEMM
-// reduce-epilogues (q/k/v with RoPE, residual + RMSNorm, SwiGLU), the argmax
+// Small kernels of the verify step: tree preparation, embedding, the argmax
 // merge with the greedy-acceptance walk, and KV compaction.
 #include <math.h>
 
@@ -106,37 +105,7 @@ cudaError_t set_tree_prep_ctx(Model& m, cudaGraphExec_t ex, cudaGraphNode_t node
   return cudaGraphExecKernelNodeSetParams(ex, node, &p);
 }
 
-// ============================================================ embedding + first RMSNorm
-// x[t] = E[token_t] (fp32 residual); xn[t] = x * rsqrt(mean(x^2) + eps) * g.
-template <typename E>
-__global__ void __launch_bounds__(256) k_embed_norm(const int32_t* __restrict__ tokens, const E* __restrict__ emb,
-                                                    const E* __restrict__ gain, int H, int vocab, float eps,
-                                                    float* __restrict__ x, E* __restrict__ xn) {
-  __shared__ float red[32];
-  pdl_wait();
-  pdl_trigger();
-  const int t = blockIdx.x;
-  int tok = tokens[t];
-  tok = tok < 0 ? 0 : (tok >= vocab ? vocab - 1 : tok);   // invalid trees are flagged by tree_prep
-  const E* row = emb + (size_t)tok * H;
-  float ss = 0.f;
-  for (int f = threadIdx.x; f < H; f += blockDim.x) {
-    const float v = to_f32(row[f]);
-    x[(size_t)t * H + f] = v;
-    ss += v * v;
-  }
-  ss = block_sum(ss, red);
-  const float r = rsqrtf(ss / (float)H + eps);
-  for (int f = threadIdx.x; f < H; f += blockDim.x)
-    store_act(xn, (size_t)t * H + f, (size_t)kMaxT * H, x[(size_t)t * H + f] * r * to_f32(gain[f]));
-}
-
-cudaError_t launch_embed_norm(Model& m, const int32_t* tokens, int T, cudaStream_t st) {
-  const auto& c = m.cfg;
-  return launch(m.pdl, k_embed_norm<float>, dim3(T), dim3(256), 0, st, tokens, (const float*)m.w.embed,
-                (const float*)m.layers[0].attn_norm, c.hidden, c.vocab, c.rms_eps, m.ws.x, (float*)m.ws.xn);
-}
-
+// ============================================================ embedding
 // bf16 path: the first RMSNorm is folded into the QKV GEMM.  Block (t, chunk)
 // writes x = E[token] (fp32 residual), y = g (.) x (hi/lo bf16 GEMM input) and
 // the chunk's sum of x^2 (the GEMM epilogue turns the chunk sums into
@@ -212,174 +181,7 @@ cudaError_t launch_final_hidden(Model& m, float* hidden, int T, cudaStream_t st)
                 norm_chunks(m, c.n_layers), (const __nv_bfloat16*)m.w.final_norm, c.hidden, c.rms_eps, hidden);
 }
 
-// ============================================================ q/k/v epilogue
-// One block per (node t, head slot hs in [0, nq + 2 nkv)); thread j owns the
-// rotate-half pair (j, j + d/2).  q/k: optional per-head RMSNorm, then RoPE at
-// pos[t]; q goes to the query buffer, k and v to cache slot ctx + t.
-struct QkvPostArgs {
-  const float* part;
-  int N, nq, nkv, d;
-  const void* bq;
-  const void* bk;
-  const void* bv;
-  const void* gq;
-  const void* gk;
-  float eps;
-  const int32_t* pos;
-  const double* inv_freq;
-  void* q;
-  void* kc;
-  void* vc;
-  const int32_t* ctx;   // committed length of the step (device)
-};
-
-template <typename E>
-__global__ void k_qkv_post(QkvPostArgs a) {
-  __shared__ float red[32];
-  pdl_wait();
-  pdl_trigger();
-  const int t = blockIdx.x, hs = blockIdx.y, j = threadIdx.x, half = a.d / 2;
-  const int f0 = hs * a.d + j, f1 = f0 + half;
-  float v0 = a.part[(size_t)t * a.N + f0];
-  float v1 = a.part[(size_t)t * a.N + f1];
-  int kind, h;  // 0 = q, 1 = k, 2 = v
-  if (hs < a.nq) { kind = 0; h = hs; }
-  else if (hs < a.nq + a.nkv) { kind = 1; h = hs - a.nq; }
-  else { kind = 2; h = hs - a.nq - a.nkv; }
-  const E* bias = (const E*)(kind == 0 ? a.bq : kind == 1 ? a.bk : a.bv);
-  if (bias) {
-    v0 += to_f32(bias[h * a.d + j]);
-    v1 += to_f32(bias[h * a.d + j + half]);
-  }
-  if (kind < 2) {
-    const E* g = (const E*)(kind == 0 ? a.gq : a.gk);
-    if (g) {
-      const float ss = block_sum(v0 * v0 + v1 * v1, red);
-      const float r = rsqrtf(ss / (float)a.d + a.eps);
-      v0 = v0 * r * to_f32(g[j]);
-      v1 = v1 * r * to_f32(g[j + half]);
-    }
-    // angle = pos * theta^(-2j/d), reduced to [-pi, pi] before the fp32 sincos
-    const double ang = (double)a.pos[t] * a.inv_freq[j];
-    const double two_pi = 6.283185307179586476925286766559;
-    const float red_ang = (float)(ang - two_pi * rint(ang / two_pi));
-    float s, c;
-    sincosf(red_ang, &s, &c);
-    const float o0 = v0 * c - v1 * s;
-    const float o1 = v1 * c + v0 * s;
-    v0 = o0;
-    v1 = o1;
-  }
-  E* dst;
-  if (kind == 0) dst = (E*)a.q + ((size_t)t * a.nq + h) * a.d;
-  else dst = (E*)(kind == 1 ? a.kc : a.vc) + ((size_t)(*a.ctx + t) * a.nkv + h) * a.d;
-  dst[j] = from_f32<E>(v0);
-  dst[j + half] = from_f32<E>(v1);
-}
-
-cudaError_t launch_qkv_post(Model& m, int layer, void* kc, void* vc, int T, cudaStream_t st) {
-  const auto& c = m.cfg;
-  const auto& L = m.layers[layer];
-  QkvPostArgs a;
-  a.part = m.ws.part;
-  a.nq = c.n_q_heads;
-  a.nkv = c.n_kv_heads;
-  a.d = c.head_dim;
-  a.N = (c.n_q_heads + 2 * c.n_kv_heads) * c.head_dim;
-  a.bq = c.qkv_bias ? L.b_q : nullptr;
-  a.bk = c.qkv_bias ? L.b_k : nullptr;
-  a.bv = c.qkv_bias ? L.b_v : nullptr;
-  a.gq = c.qk_norm ? L.q_norm : nullptr;
-  a.gk = c.qk_norm ? L.k_norm : nullptr;
-  a.eps = c.rms_eps;
-  a.pos = m.ws.pos;
-  a.inv_freq = m.ws.inv_freq;
-  a.q = m.ws.q;
-  a.kc = kc;
-  a.vc = vc;
-  a.ctx = m.ws.ctx;
-  dim3 grid(T, c.n_q_heads + 2 * c.n_kv_heads);
-  return launch(m.pdl, k_qkv_post<float>, grid, dim3(c.head_dim / 2), 0, st, a);
-}
-
-// ============================================================ residual add + RMSNorm
-// x[t] += sum of partial slices (O-projection or down-projection output);
-// xn[t] = RMSNorm(x[t]) * gain (input of the next GEMM).  For the final norm
-// the fp32 normalised row is also written to hidden_out (when given).
-template <typename E>
-__global__ void __launch_bounds__(256) k_resid_norm(const float* __restrict__ part, int H,
-                                                    const E* __restrict__ gain, float eps, float* __restrict__ x,
-                                                    E* __restrict__ xn, float* __restrict__ hidden_out) {
-  __shared__ float red[32];
-  pdl_wait();
-  pdl_trigger();
-  const int t = blockIdx.x;
-  float* xr = x + (size_t)t * H;
-  float ss = 0.f;
-  for (int f = threadIdx.x; f < H; f += blockDim.x) {
-    const float v = xr[f] + part[(size_t)t * H + f];
-    xr[f] = v;
-    ss += v * v;
-  }
-  ss = block_sum(ss, red);
-  const float r = rsqrtf(ss / (float)H + eps);
-  for (int f = threadIdx.x; f < H; f += blockDim.x) {
-    const float y = xr[f] * r * to_f32(gain[f]);
-    store_act(xn, (size_t)t * H + f, (size_t)kMaxT * H, y);
-    if (hidden_out) hidden_out[(size_t)t * H + f] = y;
-  }
-}
-
-cudaError_t launch_resid_norm(Model& m, const void* gain, float* hidden_out, int T, cudaStream_t st) {
-  const auto& c = m.cfg;
-  return launch(m.pdl, k_resid_norm<float>, dim3(T), dim3(256), 0, st, (const float*)m.ws.part, c.hidden,
-                (const float*)gain, c.rms_eps, m.ws.x, (float*)m.ws.xn, hidden_out);
-}
-
-// ============================================================ SwiGLU
-// act[t][i] = silu(gate) * up, gate/up = rows i and I + i of the stacked GEMM.
-template <typename E>
-__global__ void __launch_bounds__(256) k_silu_mul(const float* __restrict__ part, int I,
-                                                  E* __restrict__ act) {
-  pdl_wait();
-  pdl_trigger();
-  const int t = blockIdx.y;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < I) {
-    const float g = part[(size_t)t * 2 * I + i];
-    const float u = part[(size_t)t * 2 * I + I + i];
-    store_act(act, (size_t)t * I + i, (size_t)kMaxT * I, g / (1.f + expf(-g)) * u);
-  }
-}
-
-cudaError_t launch_silu_mul(Model& m, int T, cudaStream_t st) {
-  const auto& c = m.cfg;
-  dim3 grid((c.intermediate + 255) / 256, T);
-  return launch(m.pdl, k_silu_mul<float>, grid, dim3(256), 0, st, (const float*)m.ws.part, c.intermediate,
-                (float*)m.ws.act);
-}
-
 // ============================================================ argmax merge + acceptance walk
-// Running greedy state: largest logit, its (lowest) vocab id, second largest
-// logit counted with multiplicity.
-struct Top2 {
-  float v1;
-  int i1;
-  float v2;
-};
-OOS_DEV Top2 top2_merge(Top2 a, Top2 b) {
-  Top2 r;
-  if (a.v1 > b.v1 || (a.v1 == b.v1 && a.i1 <= b.i1)) {
-    r.v1 = a.v1;
-    r.i1 = a.i1;
-  } else {
-    r.v1 = b.v1;
-    r.i1 = b.i1;
-  }
-  r.v2 = fmaxf(fminf(a.v1, b.v1), fmaxf(a.v2, b.v2));
-  return r;
-}
-
 // Greedy longest-prefix acceptance (Eq. 1; "Verify and commit") by one warp.
 // ok(0) = 1; ok(i) = ok(parent) and token_i == argmax(parent).  The committed
 // path ends at the deepest ok node (lowest id on ties); bonus = its argmax.
