@@ -16,9 +16,11 @@
 //   - S = q K^T on the tensor cores into TMEM, N = 128 keys, q as hi + lo
 //     bf16 halves (two MMA chains), the A operand straight from the shared
 //     memory TMA staged it in;
-//   - softmax, one thread per query row: the row's S from TMEM, the valid-key
-//     mask (cache keys, then the node's ancestors), exp2, and P (bf16 pairs)
-//     written back over the first 64 columns of the same S buffer;
+//   - softmax, two threads per query row, 64 keys each (one warp per SM quarter
+//     left the exponentials waiting on their own latency): the row's S from TMEM,
+//     the valid-key mask (cache keys, then the node's ancestors), the two halves'
+//     maxima exchanged through shared memory, exp2, and P (bf16 pairs) written back
+//     to TMEM;
 //   - O += P V on the tensor cores (P the A operand from TMEM, V in the
 //     MN-major layout TMA writes, [key][d]).
 // Two threads issue the MMAs (S, and P.V) so neither waits behind the other's
@@ -26,9 +28,8 @@
 // maximum moves only when a tile exceeds it by more than 2^8 (O is rescaled
 // in TMEM then).
 // Merge: each block stages its unnormalised O rows and (max, sum) in its own
-// shared memory, and one thread copies each owner's rows into that owner's
-// shared memory (bulk copies that complete on the owner's barrier, no round
-// trips); the owner adds the splits by log-sum-exp in split order
+// shared memory over the K/V ring; after a cluster barrier a warp per owned row
+// pulls it from every split, adds the splits by log-sum-exp in split order
 // (deterministic) and writes the hi/lo bf16 GEMM input.
 //
 // The slot range is read through tensor maps over the cache's whole capacity,
@@ -51,9 +52,8 @@
 // of the last attention launch, the globaltimer at entry (0), at the end of the
 // loader's dependency wait (1), when q has landed (2), at the start and end of
 // the softmax of tiles 0..5 (3 + 2t, 4 + 2t), when all MMAs are done (15), when
-// the merge rows are staged (21), past the cluster barrier (22), when this
-// block's rows have been copied out (16) and its own rows received (17), and at
-// exit (18); slots 19 and 20 hold the block's tile count and the split count.
+// the merge rows are staged (21), past the cluster barrier (22) and at exit (18);
+// slots 19 and 20 hold the block's tile count and the split count.
 #ifdef OOS_TIMELINE
 namespace oos {
 __device__ unsigned long long g_tl_attn[2048][24];
@@ -90,29 +90,32 @@ constexpr int kTileBytes = 2 * kDBlock;                   // 32 KB
 constexpr int kOffK = 0;                                  // [kKvStages]
 constexpr int kOffV = kOffK + kKvStages * kTileBytes;     // [kKvStages]
 constexpr int kMaxSplits = 16;
-constexpr int kRecvRows = kAttnRows + kMaxSplits;         // >= splits * ceil(rows / splits)
 // a merge row: the unnormalised O row (128 fp32), then (max, sum), padded to 16 bytes
 constexpr int kMergeLd = kAttnD + 4;                      // floats
 constexpr int kMergeRowBytes = kMergeLd * 4;              // 528
 constexpr int kOffStage = kOffK;                          // merge: this block's rows, staged over the K/V ring
-constexpr int kOffRecv = kOffV + kKvStages * kTileBytes;  // merge: rows copied in by the splits [slot][kMergeLd]
-constexpr int kOffWgt = kOffRecv + kRecvRows * kMergeRowBytes;   // merge weights [owned row][split]
-constexpr int kOffBar = kOffWgt + kAttnRows * kMaxSplits * 4;
+constexpr int kOffQ = kOffV + kKvStages * kTileBytes;     // q hi and lo, two 64-wide d blocks of 128 rows each
+constexpr int kOffMax = kOffQ + 4 * kAttnRows * 128;      // [tile parity][key half][row] softmax exchange
+constexpr int kOffBar = kOffMax + 4 * kAttnRows * 4;
 static_assert(kAttnRows * kMergeRowBytes <= kKvStages * 2 * kTileBytes, "merge staging");
-static_assert(4 * kAttnRows * 128 <= kRecvRows * kMergeRowBytes, "q staging in the receive buffer");
-static_assert((kOffRecv & 1023) == 0, "swizzled q staging is 1024-aligned");
+static_assert((kOffQ & 1023) == 0, "swizzled q staging is 1024-aligned");
 constexpr int kAttnSmem = kOffBar + 256 + 1024;           // + barriers + alignment slack
-constexpr int kAttnThreads = 224;                         // 7 warps, roles below
+constexpr int kAttnThreads = 384;                         // 12 warps, roles below
+constexpr int kSoftWarp0 = 4;                             // softmax warps 4..11
 static_assert(kAttnSmem <= 227 * 1024, "shared memory per block");
 static_assert(kMaxSplits <= 16, "cluster size");
-// TMEM columns (lane = query row): S[2] fp32 scores of a tile (P, bf16 pairs,
-// overwrites the first 64 columns of its S buffer), O fp32.  Prefill keeps an O of
+// TMEM columns (lane = query row): S[2] fp32 scores of a tile, O fp32, P[2] bf16
+// pairs.  With P apart from S the next S MMAs into a buffer wait only until its
+// scores are in registers, not for the P.V product (8 k cached positions, T = 128:
+// a tile every 1.2 us, 1.35 before).  Prefill keeps an O of
 // the even and one of the odd tiles: its blocks go through every key unsplit, the
 // tensor core truncates each addition to an accumulator, and two chains half as
 // long are closer to the sum (K/V error 5.3e-4 -> 5.2e-4 over 2048 tokens; the
-// verify step's chains are short, and reading a second O cost it 1 %)
+// verify step's chains are short, and reading a second O cost it 1 %); P then
+// overwrites the first 64 columns of its S buffer
 constexpr int kTmS = 0;                            // [2] x 128
 constexpr int kTmO = 2 * kAttnKeys;                // [2] x 128
+constexpr int kTmP = kTmO + kAttnD;                // verify: [2] x 64
 constexpr int kAttnTmemCols = 512;                 // allocation unit: a power of two
 static_assert(kTmO + 2 * kAttnD <= kAttnTmemCols, "TMEM columns");
 
@@ -194,23 +197,27 @@ OOS_DEV void tmem_wait_ld_regs(float (&v)[N]) {
 #pragma unroll
   for (int i = 0; i < N; ++i) asm volatile("" : "+f"(v[i]));
 }
-// all 128 columns of one lane row starting at taddr
-OOS_DEV void tmem_ld128(uint32_t taddr, float (&v)[128]) {
-#pragma unroll
-  for (int c = 0; c < 4; ++c) tmem_ld32_nowait(taddr + c * 32, v + c * 32);
+// 64 columns of one lane row starting at taddr
+OOS_DEV void tmem_ld64(uint32_t taddr, float (&v)[64]) {
+  tmem_ld32_nowait(taddr, v);
+  tmem_ld32_nowait(taddr + 32, v + 32);
   tmem_wait_ld_regs(v);
 }
-// bulk copy shared::cta -> shared::cluster of another block, completing bytes on
-// that block's mbarrier (both remote addresses from mapa)
-OOS_DEV void bulk_copy_to_peer(uint32_t dst, const void* src, uint32_t bytes, uint32_t remote_bar) {
-  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   dst),
-               "r"(smem_addr(src)), "r"(bytes), "r"(remote_bar)
+OOS_DEV float4 ld_cluster4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(addr)
                : "memory");
+  return v;
 }
-OOS_DEV void bulk_commit_and_wait_read() {
-  asm volatile("cp.async.bulk.commit_group;\n\tcp.async.bulk.wait_group.read 0;" ::: "memory");
+OOS_DEV float2 ld_cluster2(uint32_t addr) {
+  float2 v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
+  return v;
 }
+// the 64 threads of the two softmax warps that share 32 query rows
+OOS_DEV void row_pair_bar(int q4) { asm volatile("bar.sync %0, 64;" ::"r"(1 + q4) : "memory"); }
 
 // 128-bit masks as (lo: bits 0..63, hi: bits 64..127)
 OOS_DEV void shr128(unsigned long long lo, unsigned long long hi, int s, unsigned long long& rlo,
@@ -228,9 +235,14 @@ OOS_DEV void shl128(unsigned long long lo, unsigned long long hi, int s, unsigne
   else { rhi = (hi << s) | (lo >> (64 - s)); rlo = lo << s; }
 }
 
+template <int N>
+struct Int {
+  static constexpr int value = N;
+};
+
 // sites of the bounded waits (recorded on the status word when one expires)
 enum { AW_KEMPTY = 21, AW_VEMPTY, AW_QFULL, AW_KFULL, AW_SFREE, AW_PFULL, AW_VFULL, AW_SFULL, AW_PV_RESCALE,
-       AW_VZERO };
+       AW_VZERO, AW_PFREE };
 OOS_DEV bool attn_wait(uint64_t* bar, uint32_t parity, volatile int* abort, uint32_t* status, uint32_t site, int ti) {
   if (mbar_wait(bar, parity, abort, status)) return true;
   if (*(volatile uint32_t*)(status + 1) == 0u && (*(volatile uint32_t*)status & ST_TIMEOUT))
@@ -244,10 +256,11 @@ OOS_DEV void drain_wait(uint64_t* bar, uint32_t parity) {
   }
 }
 
-// Block roles: warp 0 lane 0 loads K and V tiles (TMA into the swizzled
-// layouts); warp 1 lane 0 issues the S MMAs, warp 6 lane 0 the P.V MMAs;
-// warps 2..5 run the softmax (thread = query row = TMEM lane); all warps take
-// part in the merge.
+// Block roles: warp 0 lane 0 loads K tiles and q, warp 3 lane 0 V tiles (TMA into
+// the swizzled layouts; apart, so that a K tile does not queue behind a V tile whose
+// stage is still in use); warp 1 lane 0 issues the S MMAs, warp 2 lane 0 the P.V MMAs;
+// warps 4..11 run the softmax (lane = query row = TMEM lane, warps 4..7 on the
+// first 64 keys of a tile, 8..11 on the others); all warps take part in the merge.
 // F16: the KV cache (and q) are IEEE binary16 -- every product runs in f16;
 // otherwise bf16.  CAUSAL: a prefill chunk.
 template <bool F16, bool CAUSAL>
@@ -260,14 +273,15 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
   uint64_t* vfull = bar + 4;      // [2] TMA transaction bytes
   uint64_t* vempty = bar + 6;     // [2] P.V MMAs of the stage's tile done
   uint64_t* sfull = bar + 8;      // [2] S MMAs done
-  uint64_t* pfull = bar + 10;     // [2] 4 softmax warps: P written
+  uint64_t* pfull = bar + 10;     // [2] 8 softmax warps: P written
   uint64_t* pvdone = bar + 12;    // [2] P.V MMAs done (S/P buffer free, O current)
   uint64_t* odone = bar + 15;     // both MMA issuers done
-  uint64_t* recv_full = bar + 16; // merge: every split's rows for this block copied in (transaction bytes)
   uint64_t* qfull = bar + 17;     // q tile landed (transaction bytes)
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar + 18);
+  uint64_t* sread = bar + 18;     // [2] 8 softmax warps: S in registers (verify)
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar + 20);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  static_assert(18 * 8 + 8 <= 256, "barrier block");
+  static_assert(20 * 8 + 8 <= 256, "barrier block");
+  constexpr bool P_APART = !CAUSAL;
 
   if (threadIdx.x == 0) TL_ATTN(0);
   const int T = a.T, nq = a.nq, G = a.group, npc = a.npc, S = a.splits;
@@ -289,12 +303,6 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
   const int n_all = (n_keys + kAttnKeys - 1) / kAttnKeys;   // tiles over the block's keys, slots [0, n_keys)
   const int t0 = (int)((long long)split * n_all / S);
   const int n_tiles = (int)((long long)(split + 1) * n_all / S) - t0;
-  // merge: rows [0, vrows) are dealt to the S blocks of the cluster, block j
-  // owning rows [vrows j / S, vrows (j+1) / S)
-  const int n_max = (vrows + S - 1) / S;
-  const int lr0_mine = (int)((long long)vrows * split / S);
-  const int n_mine = (int)((long long)vrows * (split + 1) / S) - lr0_mine;
-
   if (threadIdx.x == 0) {
     for (int s = 0; s < 2; ++s) {
       mbar_init(&kfull[s], 1);
@@ -302,14 +310,12 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
       mbar_init(&vfull[s], 1);
       mbar_init(&vempty[s], 1);
       mbar_init(&sfull[s], 1);
-      mbar_init(&pfull[s], 4);
+      mbar_init(&pfull[s], 8);
+      mbar_init(&sread[s], 8);
       mbar_init(&pvdone[s], 1);
     }
     mbar_init(odone, 2);
-    mbar_init(recv_full, 1);
     mbar_init(qfull, 1);
-    // every split copies its rows of this block in: S * n_mine merge rows
-    mbar_arrive_expect_tx(recv_full, (uint32_t)(S * n_mine * kMergeRowBytes));
     *abort_flag = 0;
     mbar_fence_init();
   }
@@ -317,73 +323,57 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  // Another block may copy into this block's receive buffer only once the
-  // block runs, its receive barrier is armed and the S MMAs no longer read the
-  // q tile staged in that buffer: every thread arrives on the cluster barrier
-  // when it is past that point (the softmax threads after the last tile's S,
-  // the others now), and every block waits for the whole cluster before its
-  // merge copies.
-  if (warp < 2 || warp > 5) cluster_arrive_release();
   const uint32_t tmem = *tmem_slot;
   const uint32_t tmem_o = tmem + kTmO;
 
-  if (warp == 0) {
-    // ------------------------------------------------------------ loader (one thread, TMA)
+  if (warp == 0 || warp == 3) {
+    // ------------------------------------------------------------ loaders (one thread each, TMA)
     if (lane == 0) {
-      tma_prefetch_desc(&a.kmap);
-      tma_prefetch_desc(&a.vmap);
+      const bool v = warp == 3;
+      const CUtensorMap* map = v ? &a.vmap : &a.kmap;
+      uint64_t* full = v ? vfull : kfull;
+      uint64_t* empty = v ? vempty : kempty;
+      tma_prefetch_desc(map);
       const uint64_t pol_kv = policy_evict_first();
-      auto load = [&](int ti, bool v) {   // K or V tile: two 64-wide d blocks of 128 slots
+      auto load = [&](int ti) {   // two 64-wide d blocks of 128 slots
         const int st = ti & 1;
         const int key0 = (t0 + ti) * kAttnKeys;
-        uint64_t* full = v ? &vfull[st] : &kfull[st];
         unsigned char* dst = sm + (v ? kOffV : kOffK) + st * kTileBytes;
-        mbar_arrive_expect_tx(full, kTileBytes);
-        tma_load_3d(dst, v ? &a.vmap : &a.kmap, full, 0, g, key0, pol_kv);
-        tma_load_3d(dst + kDBlock, v ? &a.vmap : &a.kmap, full, 64, g, key0, pol_kv);
+        mbar_arrive_expect_tx(&full[st], kTileBytes);
+        tma_load_3d(dst, map, &full[st], 0, g, key0, pol_kv);
+        tma_load_3d(dst + kDBlock, map, &full[st], 64, g, key0, pol_kv);
       };
       // tiles of committed slots only do not depend on the producing kernel:
       // the first stages are fetched before waiting for it
-      int nk = 0, nv = 0;   // K and V tiles issued
-      while (nk < n_tiles && nk < kKvStages && (t0 + nk + 1) * kAttnKeys <= ctx) {
-        load(nk, false);
-        load(nk, true);
-        ++nk;
-        ++nv;
-      }
+      int n = 0;   // tiles issued
+      while (n < n_tiles && n < kKvStages && (t0 + n + 1) * kAttnKeys <= ctx) load(n++);
       pdl_wait();
       pdl_trigger();
-      TL_ATTN(1);
-      // q rows of the block's nodes, hi and lo halves, two 64-wide d blocks
-      // each, staged in the (still unused) receive buffer
-      tma_prefetch_desc(&a.qhi);
-      tma_prefetch_desc(&a.qlo);
-      {
+      if (!v) {
+        TL_ATTN(1);
+        // q rows of the block's nodes, hi and lo halves, two 64-wide d blocks each
+        tma_prefetch_desc(&a.qhi);
+        tma_prefetch_desc(&a.qlo);
         const uint64_t pol_q = policy_evict_last();
-        unsigned char* qs = sm + kOffRecv;
+        unsigned char* qs = sm + kOffQ;
         mbar_arrive_expect_tx(qfull, (uint32_t)(4 * rows * 128));
         tma_load_4d(qs, &a.qhi, qfull, 0, 0, g, node0, pol_q);
         tma_load_4d(qs + kAttnRows * 128, &a.qhi, qfull, 64, 0, g, node0, pol_q);
         tma_load_4d(qs + 2 * kAttnRows * 128, &a.qlo, qfull, 0, 0, g, node0, pol_q);
         tma_load_4d(qs + 3 * kAttnRows * 128, &a.qlo, qfull, 64, 0, g, node0, pol_q);
       }
-      for (int ti = nk; ti < n_tiles; ++ti) {
-        const int st = ti & 1;
-        const uint32_t use = (uint32_t)(ti >> 1);
-        if (!attn_wait(&kempty[st], (use & 1u) ^ 1u, abort_flag, status, AW_KEMPTY, ti)) break;
-        load(ti, false);
-        ++nk;
-        if (!attn_wait(&vempty[st], (use & 1u) ^ 1u, abort_flag, status, AW_VEMPTY, ti)) break;
-        load(ti, true);
-        ++nv;
+      for (int ti = n; ti < n_tiles; ++ti) {
+        if (!attn_wait(&empty[ti & 1], ((uint32_t)(ti >> 1) & 1u) ^ 1u, abort_flag, status, v ? AW_VEMPTY : AW_KEMPTY, ti))
+          break;
+        load(ti);
+        ++n;
       }
       // every copy this thread issued has landed before the block can exit,
       // whoever gave up (immediate on the normal path, where all were consumed)
-      for (int ti = nk > 2 ? nk - 2 : 0; ti < nk; ++ti) drain_wait(&kfull[ti & 1], (uint32_t)(ti >> 1) & 1u);
-      for (int ti = nv > 2 ? nv - 2 : 0; ti < nv; ++ti) drain_wait(&vfull[ti & 1], (uint32_t)(ti >> 1) & 1u);
-      drain_wait(qfull, 0);
+      for (int ti = n > 2 ? n - 2 : 0; ti < n; ++ti) drain_wait(&full[ti & 1], (uint32_t)(ti >> 1) & 1u);
+      if (!v) drain_wait(qfull, 0);
     }
-  } else if (warp == 1 || warp == 6) {
+  } else if (warp == 1 || warp == 2) {
     // ------------------------------------------------------------ MMA issuers
     // Operands reach the tensor cores through the async proxy only: q, K and
     // V by TMA, P from threads that wait for their TMEM stores before they
@@ -399,13 +389,14 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
       // q as staged by TMA: [hi d0, hi d1, lo d0, lo d1], each 128 rows x 128
       // bytes in the swizzled K-major layout (rows of padding nodes hold
       // whatever the q buffer holds; every row of S, P and O is its own)
-      const uint64_t qdesc0 = smem_desc_sw128(smem_addr(sm + kOffRecv));
+      const uint64_t qdesc0 = smem_desc_sw128(smem_addr(sm + kOffQ));
       for (int ti = 0; ti < n_tiles && ok; ++ti) {
         const int b = ti & 1;
         const uint32_t use = (uint32_t)(ti >> 1);
-        // S buffer b holds P of tile ti - 2 until that tile's P.V is done
+        // S buffer b holds tile ti - 2's scores until they are read, or its P until
+        // that tile's P.V is done
         if (!attn_wait(&kfull[b], use & 1u, abort_flag, status, AW_KFULL, ti) ||
-            !attn_wait(&pvdone[b], (use & 1u) ^ 1u, abort_flag, status, AW_SFREE, ti))
+            !attn_wait(P_APART ? &sread[b] : &pvdone[b], (use & 1u) ^ 1u, abort_flag, status, AW_SFREE, ti))
           break;
         tc_fence_after();
         const uint64_t kd0 = kdesc0 + (uint64_t)((b * kTileBytes) >> 4);
@@ -425,7 +416,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
         tc_commit(&sfull[b]);
       }
       tc_commit(odone);
-    } else if (lane == 0 && warp == 6) {
+    } else if (lane == 0 && warp == 2) {
       constexpr uint32_t idesc_pv =
           (F16 ? idesc_f16_f32(kAttnRows, kAttnD) : idesc_bf16_f32(kAttnRows, kAttnD)) | (1u << 16);   // B (V) MN-major
       // V tile: d blocks of 64 (kDBlock apart) along N, 16 keys (2 KB) per MMA along K
@@ -437,7 +428,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
             !attn_wait(&vfull[b], use & 1u, abort_flag, status, AW_VFULL, ti))
           break;
         tc_fence_after();
-        const uint32_t pt = tmem + kTmS + b * kAttnKeys;   // P: 8 columns = 16 keys per MMA
+        // P: 8 columns = 16 keys per MMA
+        const uint32_t pt = tmem + (P_APART ? kTmP + b * 64 : kTmS + b * kAttnKeys);
         const uint64_t vd = vdesc0 + (uint64_t)((b * kTileBytes) >> 4);
 #pragma unroll
         for (int kk = 0; kk < kAttnKeys / 16; ++kk)
@@ -450,16 +442,21 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
     }
   }
 
-  // ------------------------------------------------------------ softmax (warps 2..5)
-  float m_used = -INFINITY, l_sum = 0.f;
+  // ------------------------------------------------------------ softmax (warps 4..11)
+  float m_used = -INFINITY, l_sum = 0.f;            // l_sum: of this thread's keys
   const int q4 = warp & 3;
+  const int hf = warp >= kSoftWarp0 + 4 ? 1 : 0;    // key half
   const int lrow = q4 * 32 + lane;                  // local row = TMEM lane
   const uint32_t lane_off = (uint32_t)(q4 * 32) << 16;
-  if (warp >= 2 && warp <= 5) {
+  float* s_max = reinterpret_cast<float*>(sm + kOffMax);
+  if (warp >= kSoftWarp0) {
     const bool real = lrow < vrows;
     const int node = real ? node0 + lrow / G : node0;
     unsigned long long anc0 = 0ull, anc1 = 0ull;
     bool waited = false;
+    // A wait that gives up ends the warp's work, but it still meets the warp that
+    // shares its rows at the barrier of every tile.
+    bool dead = false;
     // Iteration -1 is a dry pass of the tile body, run before the dependency
     // wait while the block has nothing else to do: it brings the body's code
     // into the SM's instruction caches (the step's other kernels have evicted
@@ -481,19 +478,19 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
       const int tt = dry ? 0 : ti;
       const int b = tt & 1;
       const uint32_t use = (uint32_t)(tt >> 1);
-      if (!dry) {
+      if (!dry && !dead) {
         // every wait's outcome is made warp-uniform: the .sync.aligned TMEM
         // accesses and __syncwarp below need the whole warp on one path
-        if (!__all_sync(0xffffffffu, attn_wait(&sfull[b], use & 1u, abort_flag, status, AW_SFULL, ti))) break;
+        dead = !__all_sync(0xffffffffu, attn_wait(&sfull[b], use & 1u, abort_flag, status, AW_SFULL, ti));
         tc_fence_after();
       }
       const int key0 = dry ? ctx : (t0 + ti) * kAttnKeys;
-      if (!dry && warp == 2 && lane == 0 && ti < 6) TL_ATTN(3 + 2 * ti);
-      // valid keys of this row in the tile: committed slots, then the tree
+      if (!dry && warp == kSoftWarp0 && lane == 0 && ti < 6) TL_ATTN(3 + 2 * ti);
+      // valid keys of this row in the tile's half: committed slots, then the tree
       // slots of the node's ancestors (slot ctx + j for ancestor j); slots at
       // or past ctx + T are never ancestors (the dry pass takes the masked path)
       const bool full_tile = !dry && key0 + kAttnKeys <= ctx + (CAUSAL ? node0 + 1 : 0);   // tile-uniform
-      unsigned long long mlo = ~0ull, mhi = ~0ull;
+      unsigned long long mask = ~0ull;
       if (!full_tile) {
         // leading valid slots: the committed ones (< 128), or those up to the row's own
         const int c = CAUSAL ? max(0, min(kAttnKeys, ctx + node + 1 - key0)) : max(0, ctx - key0);
@@ -504,43 +501,55 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
         }
         const unsigned long long clo = c >= 64 ? ~0ull : (c == 0 ? 0ull : (~0ull >> (64 - c)));
         const unsigned long long chi = c <= 64 ? 0ull : (~0ull >> (128 - c));
-        mlo = clo | tlo;
-        mhi = chi | thi;
+        mask = hf ? chi | thi : clo | tlo;
       }
-      // the row's 128 scores, masked keys at -inf
-      float sv[kAttnKeys];
-      tmem_ld128(tmem + lane_off + kTmS + b * kAttnKeys, sv);
+      // the row's 64 scores, masked keys at -inf
+      float sv[64];
+      tmem_ld64(tmem + lane_off + kTmS + b * kAttnKeys + hf * 64, sv);
+      if (P_APART && !dry && !dead) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sread[b]);
+      }
       if (!full_tile) {
 #pragma unroll
-        for (int i = 0; i < kAttnKeys; ++i)
-          if (!((((i < 64) ? mlo : mhi) >> (i & 63)) & 1ull)) sv[i] = -INFINITY;
+        for (int i = 0; i < 64; ++i)
+          if (!((mask >> i) & 1ull)) sv[i] = -INFINITY;
       }
       float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-      for (int i = 0; i < kAttnKeys; ++i) mx[i & 3] = fmaxf(mx[i & 3], sv[i]);
-      const float tmax = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * scale_log2;   // scale > 0
+      for (int i = 0; i < 64; ++i) mx[i & 3] = fmaxf(mx[i & 3], sv[i]);
+      float tmax = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+      // the row's maximum over both halves; past the barrier both have also read S,
+      // whose columns P overwrites where they are not apart
+      float* sx = s_max + b * 2 * kAttnRows + lrow;
+      sx[hf * kAttnRows] = tmax;
+      row_pair_bar(q4);
+      tmax = fmaxf(tmax, sx[(hf ^ 1) * kAttnRows]) * scale_log2;   // scale > 0
+      if (dead) continue;
       // move the running maximum only when this tile exceeds it by 2^8 (a
-      // lane that moves its maximum rescales its O row; the whole warp takes
-      // part in the TMEM accesses, lanes that keep theirs scale by 1)
+      // lane that moves its maximum rescales its half of the O row; the whole warp
+      // takes part in the TMEM accesses, lanes that keep theirs scale by 1)
       const bool move = !dry && tmax > m_used + 8.f;
       const bool rescale = move && m_used != -INFINITY;
       if (__any_sync(0xffffffffu, rescale)) {
         // O holds P.V of tiles < ti: wait for the last of them, then rescale
         const int pb = (ti - 1) & 1;
-        if (!__all_sync(0xffffffffu, attn_wait(&pvdone[pb], (uint32_t)((ti - 1) >> 1) & 1u, abort_flag, status,
-                                               AW_PV_RESCALE, ti)))
-          break;
+        dead = !__all_sync(0xffffffffu, attn_wait(&pvdone[pb], (uint32_t)((ti - 1) >> 1) & 1u, abort_flag, status,
+                                                  AW_PV_RESCALE, ti));
+        if (dead) continue;
         tc_fence_after();
         const float f = rescale ? exp2f(m_used - tmax) : 1.f;
 #pragma unroll 1
-        for (int c = 0; c < (CAUSAL ? 2 : 1) * kAttnD / 32; ++c) {   // 32 columns at a time: the scores stay in registers
+        for (int c = 0; c < (CAUSAL ? 4 : 2); ++c) {   // 32 columns at a time: the scores stay in registers
+          const uint32_t col = tmem_o + lane_off + (c >> 1) * kAttnD + hf * 64 + (c & 1) * 32;
           float ov[32];
-          tmem_ld32_nowait(tmem_o + lane_off + c * 32, ov);
+          tmem_ld32_nowait(col, ov);
           tmem_wait_ld_regs(ov);
 #pragma unroll
           for (int i = 0; i < 32; ++i) ov[i] *= f;
-          tmem_st16u(tmem_o + lane_off + c * 32, reinterpret_cast<const uint32_t*>(ov));
-          tmem_st16u(tmem_o + lane_off + c * 32 + 16, reinterpret_cast<const uint32_t*>(ov + 16));
+          tmem_st16u(col, reinterpret_cast<const uint32_t*>(ov));
+          tmem_st16u(col + 16, reinterpret_cast<const uint32_t*>(ov + 16));
           tmem_wait_st();
         }
         l_sum *= f;
@@ -548,12 +557,12 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
       if (move) m_used = tmax;
       // p = 2^(s * scale - m): one FMA and one ex2 per score; a masked score
       // (-inf) gives 0, and a row with nothing valid yet (m = -inf) gives 0
-      uint32_t pk[kAttnKeys / 2];
+      uint32_t pk[32];
       float ps[4] = {0.f, 0.f, 0.f, 0.f};
       const bool live = dry || m_used != -INFINITY;
       const float neg_m = (live && !dry) ? -m_used : 0.f;
 #pragma unroll
-      for (int i = 0; i < kAttnKeys; i += 2) {
+      for (int i = 0; i < 64; i += 2) {
         const float p0 = live ? ex2_approx(fmaf(sv[i], scale_log2, neg_m)) : 0.f;
         const float p1 = live ? ex2_approx(fmaf(sv[i + 1], scale_log2, neg_m)) : 0.f;
         // P in the operand format of V; the sum uses the rounded weights that P.V multiplies
@@ -569,48 +578,48 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
       }
       if (dry) {   // the weights count as used, so that the dry pass computes them
 #pragma unroll
-        for (int i = 0; i < kAttnKeys / 2; ++i) asm volatile("" ::"r"(pk[i]));
+        for (int i = 0; i < 32; ++i) asm volatile("" ::"r"(pk[i]));
         asm volatile("" ::"f"(ps[0]), "f"(ps[1]), "f"(ps[2]), "f"(ps[3]));
         continue;
       }
       l_sum += (ps[0] + ps[1]) + (ps[2] + ps[3]);
       // slots at or past ctx + T in this tile hold whatever the cache holds
-      // there: zero their V rows (P is 0 for them, but 0 * NaN is not 0)
+      // there: zero their V rows (P is 0 for them, but 0 * NaN is not 0), each
+      // half of the warps one 64-wide d block
       const int n_ok = ctx + T - key0;                   // tile-uniform
       if (n_ok < kAttnKeys) {
-        if (!__all_sync(0xffffffffu, attn_wait(&vfull[b], use & 1u, abort_flag, status, AW_VZERO, ti))) break;
+        dead = !__all_sync(0xffffffffu, attn_wait(&vfull[b], use & 1u, abort_flag, status, AW_VZERO, ti));
+        if (dead) continue;
         if (lrow >= n_ok) {
-          unsigned char* vt = sm + kOffV + b * kTileBytes + lrow * 128;
+          unsigned char* vt = sm + kOffV + b * kTileBytes + hf * kDBlock + lrow * 128;
 #pragma unroll
-          for (int c = 0; c < 8; ++c) {
-            *reinterpret_cast<uint4*>(vt + c * 16) = make_uint4(0, 0, 0, 0);
-            *reinterpret_cast<uint4*>(vt + kDBlock + c * 16) = make_uint4(0, 0, 0, 0);
-          }
+          for (int c = 0; c < 8; ++c) *reinterpret_cast<uint4*>(vt + c * 16) = make_uint4(0, 0, 0, 0);
           fence_async_smem();
         }
       }
-      // P over the first 64 columns of S buffer b (S of this tile is read)
+      if (P_APART && ti >= 2) {   // tile ti - 2's P.V has read this P buffer
+        dead = !__all_sync(0xffffffffu, attn_wait(&pvdone[b], (use & 1u) ^ 1u, abort_flag, status, AW_PFREE, ti));
+        if (dead) continue;
+        tc_fence_after();
+      }
 #pragma unroll
-      for (int part = 0; part < 4; ++part) tmem_st16u(tmem + lane_off + kTmS + b * kAttnKeys + part * 16, pk + part * 16);
+      for (int part = 0; part < 2; ++part)
+        tmem_st16u(tmem + lane_off + (P_APART ? kTmP + b * 64 : kTmS + b * kAttnKeys) + hf * 32 + part * 16, pk + part * 16);
       tmem_wait_st();
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&pfull[b]);
-      if (warp == 2 && lane == 0 && ti < 6) TL_ATTN(4 + 2 * ti);
+      if (warp == kSoftWarp0 && lane == 0 && ti < 6) TL_ATTN(4 + 2 * ti);
     }
     if (!waited) {   // no tile: the dependency wait is still owed
       pdl_wait();
       pdl_trigger();
     }
-    // the S MMAs are done with the staged q (every S this thread waited for);
-    // after an abort an S MMA may still read it while a peer's merge rows
-    // arrive -- the step has failed then, and only values are affected
-    cluster_arrive_release();
     // every role is done with the rings and TMEM once all MMAs have completed;
     // both issuers always commit this barrier, and TMEM must not be released
     // under a running MMA, so the wait is not cut short by the handle's limit
     drain_wait(odone, 0);
-    if (warp == 2 && lane == 0) TL_ATTN(15);
+    if (warp == kSoftWarp0 && lane == 0) TL_ATTN(15);
   }
   tc_fence_before();
   __syncthreads();
@@ -618,23 +627,20 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
 
   // ------------------------------------------------------------ merge
   // Each block stages its O row, max and sum of every real row in its own
-  // shared memory (over the K/V ring, idle now), and one thread copies each
-  // owner's rows into slots split * n_max .. of that owner's receive buffer
-  // (bulk copies, completing on the owner's receive barrier).  The owner then
-  // adds the S splits of its rows by log-sum-exp, in split order.
+  // shared memory (over the K/V ring, idle now).  Rows [0, vrows) are dealt to the S
+  // blocks of the cluster; past the cluster barrier a warp takes an owned row at a
+  // time, pulls it from every split and adds the splits by log-sum-exp, in order.
   float* stage = reinterpret_cast<float*>(sm + kOffStage);   // [row][kMergeLd]
-  const float* recv = reinterpret_cast<const float*>(sm + kOffRecv);
-  float* wgt = reinterpret_cast<float*>(sm + kOffWgt);
   const bool have_o = n_tiles > 0 && !*abort_flag;   // block-uniform after the barrier
-  if (warp >= 2 && warp <= 5) {
-    float ov[kAttnD];
+  if (warp >= kSoftWarp0) {
+    float ov[64];
     if (have_o) {
-      tmem_ld128(tmem_o + lane_off, ov);
+      tmem_ld64(tmem_o + lane_off + hf * 64, ov);
       if (CAUSAL && n_tiles > 1) {
+        float o1[32];
 #pragma unroll
-        for (int c = 0; c < kAttnD / 32; ++c) {
-          float o1[32];
-          tmem_ld32_nowait(tmem_o + kAttnD + lane_off + c * 32, o1);
+        for (int c = 0; c < 2; ++c) {
+          tmem_ld32_nowait(tmem_o + kAttnD + lane_off + hf * 64 + c * 32, o1);
           tmem_wait_ld_regs(o1);
 #pragma unroll
           for (int i = 0; i < 32; ++i) ov[c * 32 + i] += o1[i];
@@ -642,90 +648,95 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
       }
     } else {
 #pragma unroll
-      for (int i = 0; i < kAttnD; ++i) ov[i] = 0.f;
+      for (int i = 0; i < 64; ++i) ov[i] = 0.f;
     }
+    if (hf) s_max[lrow] = l_sum;
     if (lrow < vrows) {
-      float* row = stage + (size_t)lrow * kMergeLd;
+      float* row = stage + (size_t)lrow * kMergeLd + hf * 64;
 #pragma unroll
-      for (int i = 0; i < kAttnD; i += 4) *reinterpret_cast<float4*>(row + i) = make_float4(ov[i], ov[i + 1], ov[i + 2], ov[i + 3]);
-      *reinterpret_cast<float4*>(row + kAttnD) = make_float4(have_o ? m_used : -INFINITY, have_o ? l_sum : 0.f, 0.f, 0.f);
-      fence_async_smem();   // the rows are read by the bulk-copy engine
+      for (int i = 0; i < 64; i += 4) *reinterpret_cast<float4*>(row + i) = make_float4(ov[i], ov[i + 1], ov[i + 2], ov[i + 3]);
+    }
+    row_pair_bar(q4);
+    if (!hf && lrow < vrows) {
+      const float l = l_sum + s_max[lrow];
+      *reinterpret_cast<float2*>(stage + (size_t)lrow * kMergeLd + kAttnD) =
+          make_float2(have_o ? m_used : -INFINITY, have_o ? l : 0.f);
     }
   }
-  __syncthreads();
-  if (threadIdx.x == 0) TL_ATTN(21);
-  cluster_wait_acquire();   // every block of the cluster runs and has armed its receive barrier
-  if (threadIdx.x == 0) TL_ATTN(22);
-  if (threadIdx.x == 0) {
-    for (int j = 0; j < S; ++j) {
-      const int r0 = (int)((long long)vrows * j / S), r1 = (int)((long long)vrows * (j + 1) / S);
-      if (r1 > r0)
-        bulk_copy_to_peer(dsmem_addr(sm + kOffRecv + (size_t)split * n_max * kMergeRowBytes, (uint32_t)j),
-                          stage + (size_t)r0 * kMergeLd, (uint32_t)((r1 - r0) * kMergeRowBytes),
-                          dsmem_addr(recv_full, (uint32_t)j));
-    }
-    bulk_commit_and_wait_read();   // the staged rows have been read before this block moves on
-  }
-  if (threadIdx.x == 0) TL_ATTN(16);
-  // this block's rows from every split.  Every block copies its rows even
-  // after an abort, so this wait ends; it is not cut short by the handle's
-  // limit, because the block must not exit while copies into it are in flight.
-  drain_wait(recv_full, 0);
-  if (threadIdx.x == 0) TL_ATTN(17);
+  if (threadIdx.x == 128) TL_ATTN(21);
+  // Every thread of the cluster arrives twice, whatever happened before: its
+  // block's rows are staged, and it has pulled (a stage must outlive its readers).
+  cluster_arrive_release();
+  __syncwarp();
+  cluster_wait_acquire();
+  if (threadIdx.x == 128) TL_ATTN(22);
   {
-    // split weights of every owned row: 2^(m_s - M) / sum_s 2^(m_s - M) l_s
-    // (every split's value of a row is loaded before any is used: the loops
-    // run over the largest split count, guarded, so they unroll)
-    if (threadIdx.x < n_mine) {
-      const int i = threadIdx.x;
-      float ms[kMaxSplits], ls[kMaxSplits];
-      float M = -INFINITY;
+    // A warp takes KR owned rows at a time, so that about 16 pulls of a lane are in
+    // flight whatever the split count (one row at a time: 4.4 us from the barrier to
+    // the exit of 6 splits).
+    const int lr0 = (int)((long long)vrows * split / S);
+    const int n_mine = (int)((long long)vrows * (split + 1) / S) - lr0;
+    constexpr int kWarps = kAttnThreads / 32;
+    auto merge = [&](auto kr, auto sm_max) {
+      constexpr int KR = decltype(kr)::value, SM = decltype(sm_max)::value;
+      bool arrived = false;
+      for (int i0 = warp; i0 < n_mine || !arrived; i0 += KR * kWarps) {
+        float2 ml[KR];
+        float4 v[KR][SM];
 #pragma unroll
-      for (int s2 = 0; s2 < kMaxSplits; ++s2) {
-        if (s2 < S) {
-          const float2 ml = *reinterpret_cast<const float2*>(recv + (size_t)(s2 * n_max + i) * kMergeLd + kAttnD);
-          ms[s2] = ml.x;
-          ls[s2] = ml.y;
-          M = fmaxf(M, ml.x);
+        for (int k = 0; k < KR; ++k) {
+          const int i = i0 + k * kWarps;
+          const bool on = i < n_mine;
+          const uint32_t off = (uint32_t)((lr0 + (on ? i : 0)) * kMergeRowBytes);
+          // lane s: (max, sum) of split s; then every split's four values of this lane
+          ml[k] = make_float2(-INFINITY, 0.f);
+          if (on && lane < S) ml[k] = ld_cluster2(dsmem_addr(stage, (uint32_t)lane) + off + kAttnD * 4);
+#pragma unroll
+          for (int s = 0; s < SM; ++s)
+            v[k][s] = on && s < S ? ld_cluster4(dsmem_addr(stage, (uint32_t)s) + off + (uint32_t)lane * 16u)
+                                  : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        float4 acc[KR];
+#pragma unroll
+        for (int k = 0; k < KR; ++k) {
+          const float M = warp_max(ml[k].x);
+          const float w = ml[k].x == -INFINITY ? 0.f : exp2f(ml[k].x - M);
+          const float den = warp_sum(w * ml[k].y);
+          const float wn = den > 0.f ? w / den : 0.f;
+          acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int s = 0; s < SM; ++s) {
+            const float ws = __shfl_sync(0xffffffffu, wn, s);   // 0 past the splits
+            acc[k].x += ws * v[k][s].x;
+            acc[k].y += ws * v[k][s].y;
+            acc[k].z += ws * v[k][s].z;
+            acc[k].w += ws * v[k][s].w;
+          }
+        }
+        if (i0 + KR * kWarps >= n_mine) {   // the last pull: the barrier need not await the stores
+#pragma unroll
+          for (int k = 0; k < KR; ++k) asm volatile("" ::"f"(acc[k].x), "f"(acc[k].y), "f"(acc[k].z), "f"(acc[k].w) : "memory");
+          cluster_arrive_relaxed();
+          arrived = true;
+        }
+#pragma unroll
+        for (int k = 0; k < KR; ++k) {
+          const int i = i0 + k * kWarps;
+          if (i < n_mine) {
+            const int lr = lr0 + i;
+            const size_t grow = (size_t)(node0 + lr / G) * nq + g * G + lr % G;
+            store_act4(a.out, grow * kAttnD + 4 * lane, a.out_lo_off, acc[k]);
+          }
         }
       }
-      float den = 0.f, w[kMaxSplits];
-#pragma unroll
-      for (int s2 = 0; s2 < kMaxSplits; ++s2) {
-        if (s2 < S) {
-          w[s2] = ms[s2] == -INFINITY ? 0.f : exp2f(ms[s2] - M);
-          den += w[s2] * ls[s2];
-        }
-      }
-      const float inv = den > 0.f ? 1.f / den : 0.f;
-#pragma unroll
-      for (int s2 = 0; s2 < kMaxSplits; ++s2)
-        if (s2 < S) wgt[i * kMaxSplits + s2] = w[s2] * inv;
-    }
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < n_mine * (kAttnD / 4); idx += blockDim.x) {
-      const int i = idx / (kAttnD / 4), d4 = (idx % (kAttnD / 4)) * 4;
-      float4 v[kMaxSplits];
-#pragma unroll
-      for (int s2 = 0; s2 < kMaxSplits; ++s2)
-        if (s2 < S) v[s2] = *reinterpret_cast<const float4*>(recv + (size_t)(s2 * n_max + i) * kMergeLd + d4);
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int s2 = 0; s2 < kMaxSplits; ++s2) {
-        if (s2 < S) {
-          const float ws = wgt[i * kMaxSplits + s2];
-          acc.x += ws * v[s2].x;
-          acc.y += ws * v[s2].y;
-          acc.z += ws * v[s2].z;
-          acc.w += ws * v[s2].w;
-        }
-      }
-      const int lr = lr0_mine + i;
-      const size_t grow = (size_t)(node0 + lr / G) * nq + g * G + lr % G;
-      store_act4(a.out, grow * kAttnD + d4, a.out_lo_off, acc);
-    }
+    };
+    if (S <= 5) merge(Int<3>{}, Int<5>{});
+    else if (S <= 8) merge(Int<2>{}, Int<8>{});
+    else merge(Int<1>{}, Int<kMaxSplits>{});
   }
-  if (threadIdx.x == 0) {
+  __syncwarp();
+  cluster_wait_acquire();
+  if (threadIdx.x == 128) {
     TL_ATTN(18);
     TL_ATTN_VAL(19, n_tiles);
     TL_ATTN_VAL(20, S);

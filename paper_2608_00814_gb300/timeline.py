@@ -121,7 +121,7 @@ def main():
         for t in range(6):
             names += [(3 + 2 * t, "softmax tile %d start" % t), (4 + 2 * t, "softmax tile %d end" % t)]
         names += [(15, "all MMAs done"), (21, "merge rows staged"), (22, "cluster barrier passed"),
-                  (16, "rows copied out"), (17, "own rows received"), (18, "exit")]
+                  (18, "exit")]
         print("last attention launch: %d blocks, %d splits, %d-%d tiles per block (us from the first entry, "
               "median over blocks [max])" % (len(b), b[0, 20], b[:, 19].min(), b[:, 19].max()))
         for e, label in names:
