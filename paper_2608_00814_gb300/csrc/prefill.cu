@@ -40,10 +40,15 @@ struct PfCfg {
   static constexpr int STAGE = 2 * kPfHalf + B_BYTES;
   static constexpr int S = (227 * 1024 - 2048) / STAGE;
   static constexpr int SMEM = 2048 + S * STAGE;   // alignment slack + barriers
-  static constexpr int NCOLS = 2 * BN;
-  // warps that finish one tile: all of them (128 columns each) at BN = 256; at
-  // BN = 128 the two groups of four take tiles in turn
-  static constexpr int TILE_WARPS = BN == 256 ? 8 : 4;
+  static constexpr int NCOLS = 512;
+  // Warps that finish one tile: all of them (128 columns each) at BN = 256; at BN =
+  // 128 the two groups of four take tiles in turn.  A tile's segments alternate
+  // between two accumulators of the group that drains them, so that a warp sees
+  // every phase of the barriers it waits on: BN = 256 has one such pair, BN = 128 two.
+  static constexpr int GROUPS = BN == 256 ? 1 : 2;
+  static constexpr int TILE_WARPS = kPfEpiWarps / GROUPS;
+  static constexpr int ACCS = 2 * GROUPS;
+  static_assert(ACCS * BN <= NCOLS, "accumulators");
 };
 
 enum { PF_QKV = 0, PF_RESID = 1, PF_SILU = 2 };
@@ -129,11 +134,11 @@ __global__ void __launch_bounds__(kPfThreads, 1)
   uint64_t* full = reinterpret_cast<uint64_t*>(ring + S * C::STAGE);
   uint64_t* empty = full + S;
   uint64_t* accf = empty + S;
-  uint64_t* acce = accf + 2;
-  uint64_t* drain = acce + 2;
+  uint64_t* acce = accf + C::ACCS;
+  uint64_t* drain = acce + C::ACCS;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  static_assert((2 * S + 5) * 8 + 8 <= 1024, "barrier block");
+  static_assert((2 * S + 2 * C::ACCS + 1) * 8 + 8 <= 1024, "barrier block");
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tiles = a.m_tiles * a.n_tiles, G = gridDim.x;
@@ -145,7 +150,7 @@ __global__ void __launch_bounds__(kPfThreads, 1)
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
-    for (int b = 0; b < 2; ++b) {
+    for (int b = 0; b < C::ACCS; ++b) {
       mbar_init(&accf[b], 1);
       mbar_init(&acce[b], C::TILE_WARPS);
     }
@@ -227,10 +232,12 @@ __global__ void __launch_bounds__(kPfThreads, 1)
       constexpr uint32_t idesc = idesc_bf16_f32(kPfRows, BN);
       int j = 0;
       bool ok = true;
-      uint32_t sg = 0;   // segments handed over; they use the two accumulators in turn
+      uint32_t handed[2] = {0u, 0u};   // segments handed to each group of epilogue warps
       for (int it = 0; it < my_tiles && ok; ++it) {
-        for (int kb0 = 0; kb0 < a.kbt && ok; kb0 += kPfSeg, ++sg) {
-          const uint32_t b = sg & 1u;
+        const uint32_t grp = it % C::GROUPS;
+        for (int kb0 = 0; kb0 < a.kbt && ok; kb0 += kPfSeg) {
+          const uint32_t sg = grp ? handed[1]++ : handed[0]++;
+          const uint32_t b = 2 * grp + (sg & 1u);
           if (!mbar_wait(&acce[b], ((sg >> 1) & 1u) ^ 1u, abort_flag, a.status)) {
             ok = false;
             break;
@@ -274,12 +281,8 @@ __global__ void __launch_bounds__(kPfThreads, 1)
     const uint32_t lane_base = tmem_base + ((uint32_t)(q * 32) << 16);
     const int ctx = EPI == PF_QKV ? *a.ctx : 0;
     const int segs = (a.kbt + kPfSeg - 1) / kPfSeg;
-    uint32_t sg = 0;
-    for (int it = 0; it < my_tiles; ++it) {
-      if (BN == 128 && (it & 1) != grp) {
-        sg += segs;
-        continue;
-      }
+    uint32_t sg = 0;   // segments this warp's group has drained
+    for (int it = C::GROUPS > 1 ? grp : 0; it < my_tiles; it += C::GROUPS) {
       const int tile = (int)blockIdx.x + it * G;
       const int n = tile / a.m_tiles, t = (tile % a.m_tiles) * kPfRows + q * 32 + lane;
       const bool live = t < a.T;
@@ -294,7 +297,7 @@ __global__ void __launch_bounds__(kPfThreads, 1)
       float acc[128];
       bool ok = true;
       for (int i = 0; i < segs; ++i, ++sg) {
-        const uint32_t b = sg & 1u;
+        const uint32_t b = (C::GROUPS > 1 ? 2 * grp : 0) + (sg & 1u);
         ok = __all_sync(0xffffffffu, mbar_wait(&accf[b], (sg >> 1) & 1u, abort_flag, a.status));
         if (!ok) break;
         tc_fence_after();

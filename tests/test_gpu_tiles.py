@@ -84,6 +84,7 @@ def test_prefill_reports_a_bad_token_of_any_chunk():
 @pytest.mark.parametrize("hidden,inter,n", [
     (1280, 3072, 2048),   # 128 x 256 tiles
     (2432, 1024, 300),    # 128 x 128 tiles; ragged last token tile
+    (2432, 1152, 2048),   # O and down in two 128 x 128 tiles a block, each of two k segments
 ])
 def test_prefill_wide_tiles(hidden, inter, n):
     """Sizes that take the compute-bound tiles in every GEMM, one layer."""
