@@ -583,6 +583,13 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
         continue;
       }
       l_sum += (ps[0] + ps[1]) + (ps[2] + ps[3]);
+      // Tile ti - 2's P.V has read this P buffer and this V buffer.  Waited for before
+      // the V wait below, whose parity alone would also match a phase two back.
+      if (P_APART && ti >= 2) {
+        dead = !__all_sync(0xffffffffu, attn_wait(&pvdone[b], (use & 1u) ^ 1u, abort_flag, status, AW_PFREE, ti));
+        if (dead) continue;
+        tc_fence_after();
+      }
       // slots at or past ctx + T in this tile hold whatever the cache holds
       // there: zero their V rows (P is 0 for them, but 0 * NaN is not 0), each
       // half of the warps one 64-wide d block
@@ -596,11 +603,6 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
           for (int c = 0; c < 8; ++c) *reinterpret_cast<uint4*>(vt + c * 16) = make_uint4(0, 0, 0, 0);
           fence_async_smem();
         }
-      }
-      if (P_APART && ti >= 2) {   // tile ti - 2's P.V has read this P buffer
-        dead = !__all_sync(0xffffffffu, attn_wait(&pvdone[b], (use & 1u) ^ 1u, abort_flag, status, AW_PFREE, ti));
-        if (dead) continue;
-        tc_fence_after();
       }
 #pragma unroll
       for (int part = 0; part < 2; ++part)

@@ -39,6 +39,25 @@ def test_gemm_tile_edges(hidden, inter, nq, nkv):
         check_compaction(model, kv, case.ctx_len, g)
 
 
+@pytest.mark.parametrize("kv", ["", "f16"])
+@pytest.mark.parametrize("T", [1, 100, 128])
+def test_attention_ragged_end_of_long_ranges(T, kv):
+    """Three and more key tiles a block, the last one cut by ctx + T: slots past it
+    hold NaN and add nothing, and the tiles before it keep their values."""
+    ctx = 2500
+    over = dict(hidden=256, intermediate=256, n_q_heads=16, n_kv_heads=8, n_layers=2, vocab=700,
+                init_std=1.0 / 16, cache_dtype=kv)
+    case = build_case("mini-bf16", 7, T=T, plant=0, ctx_len=ctx, cfg_overrides=over, gain_std=0.1, prefill=False)
+    model, _ = gpu_model(case)
+    cache = gpu_cache(case, ctx + T + 128)
+    for l in range(case.cfg.n_layers):
+        cache.k[l][ctx:] = float("nan")
+        cache.v[l][ctx:] = float("nan")
+    r = oracle.verify_tree(case.view, case.cache_k64, case.cache_v64, ctx, case.tokens, case.parent)
+    for _ in range(3):
+        check_case(case, run(model, cache, ctx, case.tokens, case.parent), r)
+
+
 @pytest.mark.parametrize("hidden,inter,nq,nkv,kv,ctx,n", [
     (256, 512, 4, 2, "", 0, 129),          # the smallest chunk, one token into the second tile
     (256, 512, 4, 2, "", 131, 2049),       # a whole chunk, then one token through the verify kernels
