@@ -2,13 +2,18 @@
 // through the decoder, causal attention over the cache and the chunk.
 //
 // A chunk of a thousand tokens has the arithmetic intensity the verify step
-// lacks, so its GEMMs are compute-bound and tiled the ordinary way: 128 tokens in
-// the MMA's M, BN weight rows in N.  The activations keep their two bf16 halves,
+// lacks, so its GEMMs are compute-bound and tiled the ordinary way: tokens in the
+// MMA's M, 256 weight rows in N.  The activations keep their two bf16 halves,
 // so every k-step is two MMAs on the same weights.  The tensor core truncates each
 // addition to its accumulator, an error that grows with the chain, so K goes in
 // segments of kPfSeg k-blocks whose sums the epilogue warps add in fp32 registers
 // (one chain over K = 4096 and 12288 added 2e-4 to a K/V error of 5e-4).
-// Persistent blocks, one per SM: one TMA producer thread, one MMA issuer, eight
+// A tile goes to a pair of CTAs (cta_group::2): 256 tokens, each CTA staging its 128
+// and half the weight rows.  A CTA alone would stage 64 KB per k-block and read 96 KB
+// of MMA operands in the 1024 clocks of its MMAs, more than its shared memory and its
+// share of L2 give; in a pair 48 and 64 (four layers of the 8B shape, 2048 tokens:
+// 5138 us in single CTAs, 4666 in pairs).
+// Persistent pairs, one CTA per SM: one TMA producer thread, one MMA issuer, eight
 // epilogue warps; two accumulators in tensor memory, so a segment is drained, and a
 // tile finished, under the next one's MMAs.
 //
@@ -34,29 +39,18 @@ constexpr int kPfThreads = 128 + 32 * kPfEpiWarps;   // a warp group for the pro
 constexpr int kPfRegsIssue = 56, kPfRegsEpi = 224;
 static_assert(128 * kPfRegsIssue + 32 * kPfEpiWarps * kPfRegsEpi <= kPfThreads * 168, "register split");
 
-template <int BN>
-struct PfCfg {
-  static constexpr int B_BYTES = BN * kBK * 2;
-  static constexpr int STAGE = 2 * kPfHalf + B_BYTES;
-  static constexpr int S = (227 * 1024 - 2048) / STAGE;
-  static constexpr int SMEM = 2048 + S * STAGE;   // alignment slack + barriers
-  static constexpr int NCOLS = 512;
-  // Warps that finish one tile: all of them (128 columns each) at BN = 256; at BN =
-  // 128 the two groups of four take tiles in turn.  A tile's segments alternate
-  // between two accumulators of the group that drains them, so that a warp sees
-  // every phase of the barriers it waits on: BN = 256 has one such pair, BN = 128 two.
-  static constexpr int GROUPS = BN == 256 ? 1 : 2;
-  static constexpr int TILE_WARPS = kPfEpiWarps / GROUPS;
-  static constexpr int ACCS = 2 * GROUPS;
-  static_assert(ACCS * BN <= NCOLS, "accumulators");
-};
+constexpr int kPfCols = 256;                      // weight rows per tile
+constexpr int kPfStage = 2 * kPfHalf + kPfCols / 2 * kBK * 2;   // a CTA's activations and half the weight rows
+constexpr int kPfStages = (227 * 1024 - 2048) / kPfStage;
+constexpr int kPfSmem = 2048 + kPfStages * kPfStage;   // alignment slack + barriers
+constexpr int kPfTmem = 512;                      // two accumulators
 
 enum { PF_QKV = 0, PF_RESID = 1, PF_SILU = 2 };
 
 struct PfArgs {
   int T;              // tokens of the chunk
   int kbt;            // k-blocks
-  int m_tiles, n_tiles;
+  int m_tiles, n_tiles;   // token tiles (of 256 for a pair), weight tiles
   int N;              // output features (PF_SILU: intermediate size; PF_QKV: heads * 128)
   uint32_t* status;
   const float* ss_in;   // [chunk][kPfTokens]
@@ -121,28 +115,30 @@ OOS_DEV void load16(const __nv_bfloat16* p, float (&v)[16]) {
   }
 }
 
-template <int BN, int EPI>
+template <int EPI>
 __global__ void __launch_bounds__(kPfThreads, 1)
     k_pf_gemm(const __grid_constant__ CUtensorMap wm0, const __grid_constant__ CUtensorMap wm1,
               const __grid_constant__ CUtensorMap wm2, const __grid_constant__ CUtensorMap am,
               const __grid_constant__ PfArgs a) {
-  using C = PfCfg<BN>;
-  constexpr int S = C::S;
+  constexpr int S = kPfStages;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* ring = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   // stage: [activations hi | activations lo | weights]
-  uint64_t* full = reinterpret_cast<uint64_t*>(ring + S * C::STAGE);
+  uint64_t* full = reinterpret_cast<uint64_t*>(ring + S * kPfStage);
   uint64_t* empty = full + S;
   uint64_t* accf = empty + S;
-  uint64_t* acce = accf + C::ACCS;
-  uint64_t* drain = acce + C::ACCS;
+  uint64_t* acce = accf + 2;
+  uint64_t* drain = acce + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  static_assert((2 * S + 2 * C::ACCS + 1) * 8 + 8 <= 1024, "barrier block");
+  static_assert((2 * S + 5) * 8 + 8 <= 1024, "barrier block");
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int tiles = a.m_tiles * a.n_tiles, G = gridDim.x;
-  const int my_tiles = (int)blockIdx.x < tiles ? (tiles - (int)blockIdx.x + G - 1) / G : 0;
+  // a pair works on one tile, each CTA (rank) on 128 of its tokens
+  const int rank = blockIdx.x & 1, me = blockIdx.x >> 1, G = gridDim.x >> 1;
+  const int tiles = a.m_tiles * a.n_tiles;
+  const int my_tiles = me < tiles ? (tiles - me + G - 1) / G : 0;
+  auto m_of = [&](int tile) { return tile % a.m_tiles * 2 + rank; };   // 128-token tile
   const int n_units = my_tiles * a.kbt;
 
   if (threadIdx.x == 0) {
@@ -150,18 +146,21 @@ __global__ void __launch_bounds__(kPfThreads, 1)
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
-    for (int b = 0; b < C::ACCS; ++b) {
+    for (int b = 0; b < 2; ++b) {
       mbar_init(&accf[b], 1);
-      mbar_init(&acce[b], C::TILE_WARPS);
+      mbar_init(&acce[b], 2 * kPfEpiWarps);
     }
     mbar_init(drain, 1);
     *abort_flag = 0;
     mbar_fence_init();
   }
-  if (warp == 2) tmem_alloc(tmem_slot, C::NCOLS);
+  if (warp == 2) tmem_alloc_pair(tmem_slot, kPfTmem);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  // the other CTA's barriers are set up before anything arrives on them
+  cluster_arrive_release();
+  cluster_wait_acquire();
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp < 4) {
@@ -171,79 +170,92 @@ __global__ void __launch_bounds__(kPfThreads, 1)
       tma_prefetch_desc(&wm0);
       tma_prefetch_desc(&am);
       const uint64_t pol = policy_evict_last();   // every operand is read by many blocks
+      // a pair's copies all complete on rank 0's barriers, which expect both CTAs' bytes
+      const uint32_t full0 = dsmem_addr(full, 0);
+      auto load = [&](void* dst, const CUtensorMap* map, int stage, int x, int y) {
+        tma_load_2d_pair(dst, map, full0 + (uint32_t)stage * 8u, x, y, pol);
+      };
+      auto expect = [&](int stage) {
+        if (rank == 0) mbar_arrive_expect_tx(&full[stage], 2 * kPfStage);
+      };
       auto load_w = [&](int n, int kb, int stage) {
-        unsigned char* dst = ring + stage * C::STAGE + 2 * kPfHalf;
+        unsigned char* dst = ring + stage * kPfStage + 2 * kPfHalf;
 #pragma unroll
-        for (int i = 0; i < BN / 64; ++i) {   // boxes of 64 weight rows
+        for (int j = 0; j < kPfCols / 128; ++j) {   // boxes of 64 weight rows
+          const int i = rank * (kPfCols / 128) + j;
           const CUtensorMap* wm = &wm0;
-          int row = n * BN + i * 64;          // past the last row: zeros
+          int row = n * kPfCols + i * 64;          // past the last row: zeros
           if (EPI == PF_SILU) {
-            wm = i < BN / 128 ? &wm0 : &wm1;
-            row = n * (BN / 2) + (i % (BN / 128)) * 64;
+            wm = i < 2 ? &wm0 : &wm1;
+            row = n * (kPfCols / 2) + (i & 1) * 64;
           } else if (EPI == PF_QKV) {
-            int h = n * (BN / 128) + i / 2;
+            int h = n * 2 + i / 2;
             if (h >= a.nq + 2 * a.nkv) h = 0;   // an odd head count's last tile: columns nobody reads
             const int base = h < a.nq ? 0 : h < a.nq + a.nkv ? a.nq : a.nq + a.nkv;
             wm = h < a.nq ? &wm0 : h < a.nq + a.nkv ? &wm1 : &wm2;
             row = (h - base) * 128 + (i & 1) * 64;
           }
-          tma_load_2d(dst + i * 64 * kBK * 2, wm, &full[stage], kb * kBK, row, pol);
+          load(dst + j * 64 * kBK * 2, wm, stage, kb * kBK, row);
         }
       };
       auto load_x = [&](int m, int kb, int stage) {
-        unsigned char* dst = ring + stage * C::STAGE;
-        tma_load_2d(dst, &am, &full[stage], kb * kBK, m * kPfRows, pol);
-        tma_load_2d(dst + kPfHalf, &am, &full[stage], kb * kBK, kPfTokens + m * kPfRows, pol);
+        unsigned char* dst = ring + stage * kPfStage;
+        load(dst, &am, stage, kb * kBK, m * kPfRows);
+        load(dst + kPfHalf, &am, stage, kb * kBK, kPfTokens + m * kPfRows);
       };
       // the first stages' weights do not depend on the previous kernel
       const int n_pre = n_units < S ? n_units : S;
-      int tile = blockIdx.x, kb = 0;
+      int tile = me, kb = 0;
       for (int j = 0; j < n_pre; ++j) {
-        mbar_arrive_expect_tx(&full[j], C::STAGE);
+        expect(j);
         load_w(tile / a.m_tiles, kb, j);
         if (++kb == a.kbt) { kb = 0; tile += G; }
       }
       pdl_wait();
       pdl_trigger();
-      tile = blockIdx.x;
+      tile = me;
       kb = 0;
       int issued = 0;
       for (int j = 0; j < n_units; ++j) {
         const int stage = j % S;
         if (j >= n_pre) {
           if (!mbar_wait(&empty[stage], (uint32_t)(j / S - 1) & 1u, abort_flag, a.status)) break;
-          mbar_arrive_expect_tx(&full[stage], C::STAGE);
+          expect(stage);
           load_w(tile / a.m_tiles, kb, stage);
         }
-        load_x(tile % a.m_tiles, kb, stage);
+        load_x(m_of(tile), kb, stage);
         ++issued;
         if (++kb == a.kbt) { kb = 0; tile += G; }
       }
-      // every copy has landed before the block can exit (immediate on the
-      // normal path, where all were consumed)
-      for (int j = issued - S > 0 ? issued - S : 0; j < issued; ++j) {
-        const unsigned long long t0 = globaltimer();
-        while (!mbar_test(smem_addr(&full[j % S]), (uint32_t)((j / S) & 1)) && globaltimer() - t0 < kWaitLimitNs) {
+      // every copy has landed before the block can exit (immediate on the normal
+      // path, where all were consumed; after an abort of one CTA of a pair a phase
+      // may stay short of the other's bytes, so the whole wait is bounded)
+      const unsigned long long t0 = globaltimer(), most = 10000000ull;
+      if (rank == 0) {
+        for (int j = issued - S > 0 ? issued - S : 0; j < issued; ++j) {
+          while (!mbar_test(smem_addr(&full[j % S]), (uint32_t)((j / S) & 1)) && globaltimer() - t0 < most) {
+          }
+        }
+      } else if (issued < n_units) {   // rank 1 gave up: its last copies land long before this ends
+        while (globaltimer() - t0 < 200000ull) {
         }
       }
     }
     // ------------------------------------------------------------ MMA issuer
-    if (warp == 1 && lane == 0) {
-      constexpr uint32_t idesc = idesc_bf16_f32(kPfRows, BN);
+    if (warp == 1 && lane == 0 && rank == 0) {
+      constexpr uint32_t idesc = idesc_bf16_f32(2 * kPfRows, kPfCols);
       int j = 0;
       bool ok = true;
-      uint32_t handed[2] = {0u, 0u};   // segments handed to each group of epilogue warps
+      uint32_t sg = 0;   // segments handed over; they use the two accumulators in turn
       for (int it = 0; it < my_tiles && ok; ++it) {
-        const uint32_t grp = it % C::GROUPS;
-        for (int kb0 = 0; kb0 < a.kbt && ok; kb0 += kPfSeg) {
-          const uint32_t sg = grp ? handed[1]++ : handed[0]++;
-          const uint32_t b = 2 * grp + (sg & 1u);
+        for (int kb0 = 0; kb0 < a.kbt && ok; kb0 += kPfSeg, ++sg) {
+          const uint32_t b = sg & 1u;
           if (!mbar_wait(&acce[b], ((sg >> 1) & 1u) ^ 1u, abort_flag, a.status)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t d = tmem_base + b * BN;
+          const uint32_t d = tmem_base + b * kPfCols;
           const int n = min(kPfSeg, a.kbt - kb0);
           for (int kb = 0; kb < n; ++kb, ++j) {
             const int stage = j % S;
@@ -252,21 +264,21 @@ __global__ void __launch_bounds__(kPfThreads, 1)
               break;
             }
             tc_fence_after();
-            const uint32_t base = smem_addr(ring + stage * C::STAGE);
+            const uint32_t base = smem_addr(ring + stage * kPfStage);
             const uint64_t xh = smem_desc_sw128(base), xl = smem_desc_sw128(base + kPfHalf);
             const uint64_t w = smem_desc_sw128(base + 2 * kPfHalf);
 #pragma unroll
             for (int k = 0; k < kBK / 16; ++k) {
-              tc_mma_bf16(d, xh + 2 * k, w + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
-              tc_mma_bf16(d, xl + 2 * k, w + 2 * k, idesc, 1u);
+              tc_mma_bf16_pair(d, xh + 2 * k, w + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+              tc_mma_bf16_pair(d, xl + 2 * k, w + 2 * k, idesc, 1u);
             }
-            tc_commit(&empty[stage]);
+            tc_commit_pair(&empty[stage]);
           }
-          if (ok) tc_commit(&accf[b]);
+          if (ok) tc_commit_pair(&accf[b]);
         }
       }
       // all issued MMAs complete before TMEM is released
-      tc_commit(drain);
+      tc_commit_pair(drain);
       const unsigned long long t0 = globaltimer();
       while (!mbar_test(smem_addr(drain), 0) && globaltimer() - t0 < kWaitLimitNs) {
       }
@@ -280,11 +292,12 @@ __global__ void __launch_bounds__(kPfThreads, 1)
     const int q = warp & 3, grp = (warp - 4) >> 2;
     const uint32_t lane_base = tmem_base + ((uint32_t)(q * 32) << 16);
     const int ctx = EPI == PF_QKV ? *a.ctx : 0;
+    const uint32_t acce0 = dsmem_addr(acce, 0);   // rank 0's, where the issuer waits
     const int segs = (a.kbt + kPfSeg - 1) / kPfSeg;
-    uint32_t sg = 0;   // segments this warp's group has drained
-    for (int it = C::GROUPS > 1 ? grp : 0; it < my_tiles; it += C::GROUPS) {
-      const int tile = (int)blockIdx.x + it * G;
-      const int n = tile / a.m_tiles, t = (tile % a.m_tiles) * kPfRows + q * 32 + lane;
+    uint32_t sg = 0;
+    for (int it = 0; it < my_tiles; ++it) {
+      const int tile = me + it * G;
+      const int n = tile / a.m_tiles, t = m_of(tile) * kPfRows + q * 32 + lane;
       const bool live = t < a.T;
       float r = 0.f;
       if (EPI != PF_RESID && live) {   // the input's RMSNorm factor
@@ -297,15 +310,15 @@ __global__ void __launch_bounds__(kPfThreads, 1)
       float acc[128];
       bool ok = true;
       for (int i = 0; i < segs; ++i, ++sg) {
-        const uint32_t b = (C::GROUPS > 1 ? 2 * grp : 0) + (sg & 1u);
+        const uint32_t b = sg & 1u;
         ok = __all_sync(0xffffffffu, mbar_wait(&accf[b], (sg >> 1) & 1u, abort_flag, a.status));
         if (!ok) break;
         tc_fence_after();
-        const uint32_t base = lane_base + b * BN;
+        const uint32_t base = lane_base + b * kPfCols;
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
-          const uint32_t col = EPI == PF_SILU ? base + (c < 4 ? 0 : BN / 2) + (BN == 256 ? grp * 64 : 0) + (c & 3) * 16
-                                              : base + (BN == 256 ? grp * 128 : 0) + c * 16;
+          const uint32_t col = EPI == PF_SILU ? base + (c < 4 ? 0 : kPfCols / 2) + grp * 64 + (c & 3) * 16
+                                              : base + grp * 128 + c * 16;
           float v[16];
           tmem_ld16_nowait(col, v);
           tmem_wait_ld();
@@ -315,11 +328,11 @@ __global__ void __launch_bounds__(kPfThreads, 1)
         }
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&acce[b]);
+        if (lane == 0) mbar_arrive_remote(acce0 + 8u * b);
       }
       if (!ok) break;
       auto finish = [&]() {
-        const int unit = n * (BN / 128) + (BN == 256 ? grp : 0);   // head, or 128-feature block
+        const int unit = n * 2 + grp;   // head, or 128-feature block
         if (EPI == PF_QKV) {
           if (unit >= a.nq + 2 * a.nkv) return;
           const int kind = unit < a.nq ? 0 : unit < a.nq + a.nkv ? 1 : 2;
@@ -409,7 +422,7 @@ __global__ void __launch_bounds__(kPfThreads, 1)
           }
           a.ss_out[(size_t)unit * kPfTokens + t] = ss;
         } else {
-          const int i0 = n * (BN / 2) + (BN == 256 ? grp * 64 : 0);
+          const int i0 = n * (kPfCols / 2) + grp * 64;
           if (i0 >= a.N) return;
 #pragma unroll
           for (int c = 0; c < 64; c += 16) {
@@ -429,9 +442,12 @@ __global__ void __launch_bounds__(kPfThreads, 1)
   }
   tc_fence_before();
   __syncthreads();
+  // neither CTA leaves while the other's MMAs, copies or arrivals may reach it
+  cluster_arrive_release();
+  cluster_wait_acquire();
   if (warp == 2) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, C::NCOLS);
+    tmem_dealloc_pair(tmem_base, kPfTmem);
   }
 }
 
@@ -472,18 +488,14 @@ __global__ void __launch_bounds__(256) k_pf_last(const __nv_bfloat16* __restrict
 }
 
 // ------------------------------------------------------------ host side
-template <int BN, int EPI>
+template <int EPI>
 static cudaError_t pf_smem() {
-  return cudaFuncSetAttribute(k_pf_gemm<BN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, PfCfg<BN>::SMEM);
+  return cudaFuncSetAttribute(k_pf_gemm<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPfSmem);
 }
 cudaError_t prefill_setup() {
-  cudaError_t e = pf_smem<128, PF_QKV>();
-  if (e == cudaSuccess) e = pf_smem<128, PF_RESID>();
-  if (e == cudaSuccess) e = pf_smem<128, PF_SILU>();
-  if (e == cudaSuccess) e = pf_smem<256, PF_QKV>();
-  if (e == cudaSuccess) e = pf_smem<256, PF_RESID>();
-  if (e == cudaSuccess) e = pf_smem<256, PF_SILU>();
-  return e;
+  cudaError_t e = pf_smem<PF_QKV>();
+  if (e == cudaSuccess) e = pf_smem<PF_RESID>();
+  return e == cudaSuccess ? pf_smem<PF_SILU>() : e;
 }
 
 bool prefill_encode(Model& m) {
@@ -494,45 +506,44 @@ bool prefill_encode(Model& m) {
          encode_rows_map(&m.pf_act_map, m.ws.pf_act, 2 * kPfTokens, c.intermediate, kPfRows);
 }
 
-// How one GEMM of a chunk runs: tiles of 128 x 256 or 128 x 128 here, or the
-// verify GEMMs in token tiles of 128, k split over clusters of `split` (0: here).
-struct PfPlan {
-  bool wide;
-  int split;
-};
-
-// Estimates in microseconds, from timings of both kinds: a k-block of a 128 x 256
-// tile takes ~0.6 us and of a 128 x 128 one ~0.45 (operand traffic bounds the
-// narrow one), a k-block of a verify tile (128 tokens x 128 rows) ~0.5; prologue,
-// drain and epilogue ~8 against ~6 plus the sums pulled.  Few tiles and a long K
-// (O and down of small models: 24 tiles for 333 tokens at hidden 1024) go to the
-// clusters, which fill the SMs; anything with a tile for most SMs stays here.
-static PfPlan pf_plan(const Model& m, int rows, int kbt, int T, bool may_split) {
+// How one GEMM of a chunk runs: 0 as pairs' tiles of 256 tokens x 256 weight rows
+// here, c >= 1 as the verify GEMM's tiles of 128 x 128, k split over clusters of c
+// (gate/up: unsplit, in pairs of its own).
+//
+// Estimates in microseconds of work in line, one wave after the other: a k-block of
+// a pair's tile takes 0.53 and a tile's turnover 10, a k-block of a verify tile 0.4 and
+// its turnover 8.5, each rank of a cluster 0.9 for the sums it pulls; the residual's
+// tiles cost 24 more here (64 or fewer pairs hide neither the first loads nor the
+// rows of x they read and write), gate/up's 5.  Set against timings of each choice
+// in turn at 8 chunk lengths of 136..2048 tokens in 4 shapes (hidden 1024..5120): the
+// choice was the fastest or within 4 us of it in 125 of 128, and within 14 in all.
+// Both ways, one layer's down GEMM: 512 tokens of the 8B shape 24 us less in verify
+// tiles, 1024 tokens 25 us less in pairs.
+static int pf_split(const Model& m, int rows, int kbt, int T, int epi) {
   const int mt = (T + kPfRows - 1) / kPfRows;
   auto waves = [](long long tiles, int fit) { return (double)((tiles + fit - 1) / fit); };
-  const double wide = waves((long long)mt * ((rows + 255) / 256), m.num_sms) * kbt * 0.6 + 8;
-  const double narrow = waves((long long)mt * ((rows + 127) / 128), m.num_sms) * kbt * 0.45 + 8;
-  PfPlan p{wide <= narrow, 0};
-  double best = wide <= narrow ? wide : narrow;
-  for (int c = 1; c <= (may_split ? kMaxSplit : 1) && c <= kbt; ++c) {
+  const long long tiles = (long long)mt * ((rows + 127) / 128);
+  double best = waves((long long)((mt + 1) / 2) * ((rows + kPfCols - 1) / kPfCols), m.num_sms / 2) * (kbt * 0.53 + 10) +
+                (epi == PF_RESID ? 24 : epi == PF_SILU ? 5 : 0);
+  int split = 0;
+  for (int c = 1; c <= (epi == PF_SILU ? 1 : kMaxSplit) && c <= kbt; ++c) {
     if (m.fit[c] < 1) continue;
-    const double t = waves((long long)mt * ((rows + 127) / 128), m.fit[c]) * ((kbt + c - 1) / c * 0.5 + 6) + 0.2 * c;
+    const double t = waves(tiles, m.fit[c]) * ((kbt + c - 1) / c * 0.4 + 8.5) + 0.9 * c;
     if (t < best) {
       best = t;
-      p.split = c;
+      split = c;
     }
   }
-  return p;
+  return split;
 }
 
 template <int EPI>
-static cudaError_t launch_pf(Model& m, const GemmW& g, const CUtensorMap& am, PfArgs& a, int rows, bool wide,
-                             cudaStream_t st) {
+static cudaError_t launch_pf(Model& m, const GemmW& g, const CUtensorMap& am, PfArgs& a, int rows, cudaStream_t st) {
   // rows: stacked weight rows of the GEMM
   const auto& c = m.cfg;
   a.kbt = g.K / kBK;
-  a.m_tiles = (a.T + kPfRows - 1) / kPfRows;
-  a.n_tiles = (rows + (wide ? 255 : 127)) / (wide ? 256 : 128);
+  a.m_tiles = (a.T + 2 * kPfRows - 1) / (2 * kPfRows);
+  a.n_tiles = (rows + kPfCols - 1) / kPfCols;
   a.status = m.ws.status;
   a.ss_in = m.ws.pf_ss;
   a.ss_chunks = c.hidden / kTile;
@@ -541,12 +552,22 @@ static cudaError_t launch_pf(Model& m, const GemmW& g, const CUtensorMap& am, Pf
   const CUtensorMap& w1 = g.n_seg > 1 ? g.pf_map[1] : g.pf_map[0];
   const CUtensorMap& w2 = g.n_seg > 2 ? g.pf_map[2] : g.pf_map[0];
   const long long tiles = (long long)a.m_tiles * a.n_tiles;
-  const dim3 grid((unsigned)(tiles < m.num_sms ? tiles : m.num_sms));
-  if (wide)
-    return launch(m.pdl, k_pf_gemm<256, EPI>, grid, dim3(kPfThreads), (size_t)PfCfg<256>::SMEM, st, g.pf_map[0], w1, w2,
-                  am, a);
-  return launch(m.pdl, k_pf_gemm<128, EPI>, grid, dim3(kPfThreads), (size_t)PfCfg<128>::SMEM, st, g.pf_map[0], w1, w2,
-                am, a);
+  const int pairs = (int)(tiles < m.num_sms / 2 ? tiles : m.num_sms / 2);
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3(2 * pairs);
+  lc.blockDim = dim3(kPfThreads);
+  lc.dynamicSmemBytes = (size_t)kPfSmem;
+  lc.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = attr;
+  lc.numAttrs = m.pdl ? 2 : 1;
+  return cudaLaunchKernelEx(&lc, k_pf_gemm<EPI>, g.pf_map[0], w1, w2, am, a);
 }
 
 static PfArgs pf_args(int T) {
@@ -558,8 +579,8 @@ static PfArgs pf_args(int T) {
 
 static cudaError_t launch_pf_resid(Model& m, int layer, bool down, const void* gain, int T, cudaStream_t st) {
   const GemmW& g = down ? m.g_down[layer] : m.g_o[layer];
-  const PfPlan p = pf_plan(m, m.cfg.hidden, g.K / kBK, T, true);
-  if (p.split) return launch_chunk_resid(m, layer, down, gain, T, p.split, st);
+  const int split = pf_split(m, m.cfg.hidden, g.K / kBK, T, PF_RESID);
+  if (split) return launch_chunk_resid(m, layer, down, gain, T, split, st);
   PfArgs a = pf_args(T);
   a.N = m.cfg.hidden;
   a.x = m.ws.pf_x;
@@ -567,15 +588,15 @@ static cudaError_t launch_pf_resid(Model& m, int layer, bool down, const void* g
   a.out = (__nv_bfloat16*)m.ws.pf_xn;
   a.lo_off = (size_t)kPfTokens * m.cfg.hidden;
   a.ss_out = m.ws.pf_ss;
-  return launch_pf<PF_RESID>(m, g, down ? m.pf_act_map : m.pf_attn_map, a, a.N, p.wide, st);
+  return launch_pf<PF_RESID>(m, g, down ? m.pf_act_map : m.pf_attn_map, a, a.N, st);
 }
 
 static cudaError_t launch_pf_qkv(Model& m, int layer, void* kc, void* vc, int T, cudaStream_t st) {
   const auto& c = m.cfg;
   const oos_layer_weights& L = m.layers[layer];
   const int rows = (c.n_q_heads + 2 * c.n_kv_heads) * c.head_dim;
-  const PfPlan p = pf_plan(m, rows, c.hidden / kBK, T, true);
-  if (p.split) return launch_chunk_qkv(m, layer, kc, vc, T, p.split, st);
+  const int split = pf_split(m, rows, c.hidden / kBK, T, PF_QKV);
+  if (split) return launch_chunk_qkv(m, layer, kc, vc, T, split, st);
   PfArgs a = pf_args(T);
   a.N = rows;
   a.nq = c.n_q_heads;
@@ -591,18 +612,17 @@ static cudaError_t launch_pf_qkv(Model& m, int layer, void* kc, void* vc, int T,
   a.kc = (__nv_bfloat16*)kc;
   a.vc = (__nv_bfloat16*)vc;
   a.ctx = m.ws.ctx;
-  return launch_pf<PF_QKV>(m, m.g_qkv[layer], m.pf_xn_map, a, rows, p.wide, st);
+  return launch_pf<PF_QKV>(m, m.g_qkv[layer], m.pf_xn_map, a, rows, st);
 }
 
 static cudaError_t launch_pf_gu(Model& m, int layer, int T, cudaStream_t st) {
   const auto& c = m.cfg;
-  const PfPlan p = pf_plan(m, 2 * c.intermediate, c.hidden / kBK, T, false);
-  if (p.split) return launch_chunk_gu(m, layer, T, st);
+  if (pf_split(m, 2 * c.intermediate, c.hidden / kBK, T, PF_SILU)) return launch_chunk_gu(m, layer, T, st);
   PfArgs a = pf_args(T);
   a.N = c.intermediate;
   a.out = (__nv_bfloat16*)m.ws.pf_act;
   a.lo_off = (size_t)kPfTokens * c.intermediate;
-  return launch_pf<PF_SILU>(m, m.g_gu[layer], m.pf_xn_map, a, 2 * a.N, p.wide, st);
+  return launch_pf<PF_SILU>(m, m.g_gu[layer], m.pf_xn_map, a, 2 * a.N, st);
 }
 
 // Every layer of one chunk of T tokens (128 < T <= kPfTokens) at cache position

@@ -101,12 +101,13 @@ def test_prefill_reports_a_bad_token_of_any_chunk():
 
 
 @pytest.mark.parametrize("hidden,inter,n", [
-    (1280, 3072, 2048),   # 128 x 256 tiles
-    (2432, 1024, 300),    # 128 x 128 tiles; ragged last token tile
-    (2432, 1152, 2048),   # O and down in two 128 x 128 tiles a block, each of two k segments
+    (1280, 3072, 2048),   # QKV and gate/up: 256 x 256 tiles, more than one a pair
+    (2432, 1024, 300),    # every GEMM in 128 x 128 tiles; ragged last token tile
+    (2432, 1152, 2048),   # O and down: two 128 x 128 tiles a block
+    (2432, 4096, 1700),   # down: 256 x 256 tiles, the last cut by the matrix and the prompt
 ])
 def test_prefill_wide_tiles(hidden, inter, n):
-    """Sizes that take the compute-bound tiles in every GEMM, one layer."""
+    """Sizes on both sides of the choice of tiles, one layer."""
     over = dict(hidden=hidden, intermediate=inter, n_q_heads=16, n_kv_heads=8, n_layers=1, vocab=700,
                 init_std=1.0 / hidden ** 0.5)
     case = build_case("mini-bf16", 6, T=4, plant=0, ctx_len=0, cfg_overrides=over, gain_std=0.1, prefill=False)
