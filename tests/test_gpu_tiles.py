@@ -1,6 +1,7 @@
-"""bf16 kernels at the edges of their tiles, against the CPU checker: weight
-matrices that the GEMM tiles (rows cut to the SM count, k split over a cluster)
-do not divide evenly, and trees at the edges of the token tiles; prompts at the edges of the prefill chunks."""
+"""Kernels at the edges of their tiles, against the CPU checker: weight matrices
+that the GEMM tiles (rows cut to the SM count, k split over a cluster) do not
+divide evenly, and trees at the edges of the token tiles; prompts at the edges of
+the prefill chunks; fp32 rows that do not divide into fours."""
 
 import numpy as np
 import pytest
@@ -56,6 +57,23 @@ def test_attention_ragged_end_of_long_ranges(T, kv):
     r = oracle.verify_tree(case.view, case.cache_k64, case.cache_v64, ctx, case.tokens, case.parent)
     for _ in range(3):
         check_case(case, run(model, cache, ctx, case.tokens, case.parent), r)
+
+
+@pytest.mark.parametrize("hidden,inter,nq,nkv,d", [
+    (66, 130, 4, 2, 18),    # no row of any weight on a 16-byte boundary
+    (64, 131, 3, 1, 6),     # down and O a value at a time, QKV and gate/up in fours
+    (70, 128, 5, 5, 2),     # the reverse; the smallest head
+])
+def test_f32_rows_not_in_fours(hidden, inter, nq, nkv, d):
+    over = dict(hidden=hidden, intermediate=inter, n_q_heads=nq, n_kv_heads=nkv, head_dim=d, vocab=501)
+    for T in (1, 7, 64):
+        case = build_case("tiny", 9, T=T, plant=0, ctx_len=T, cfg_overrides=over, gain_std=0.1, prefill=False)
+        model, _ = gpu_model(case)
+        kv = gpu_cache(case, case.ctx_len + T)
+        g = run(model, kv, case.ctx_len, case.tokens, case.parent)
+        r = oracle.verify_tree(case.view, case.cache_k64, case.cache_v64, case.ctx_len, case.tokens, case.parent)
+        check_case(case, g, r)
+        check_compaction(model, kv, case.ctx_len, g)
 
 
 @pytest.mark.parametrize("hidden,inter,nq,nkv,kv,ctx,n", [
