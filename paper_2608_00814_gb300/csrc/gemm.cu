@@ -856,21 +856,32 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
           if (cc * 16 >= T) break;
           float v[16];
           acc16(col0 + sub * C::SUB_COLS + cc * 16, v);
+          // Top 2 over the warp's 32 rows, the 16 tokens folded over the lanes: each
+          // exchange halves the tokens a lane still holds, 16 merges.  With every lane
+          // reducing every token (80) the epilogue of the last tile, and at T = 128 that
+          // of every tile, was what the weights waited for: 151936 x 4096 at T = 1 / 64
+          // 182.7 / 193.2 -> 177.4 / 182.5 us, 128256 x 4096 at T = 128 234 -> 205.
+          Top2 s[16];
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            Top2 s{f < a.N ? v[i] * rms[cc * 16 + i] : -INFINITY, f, -INFINITY};
+          for (int i = 0; i < 16; ++i) s[i] = Top2{f < a.N ? v[i] * rms[cc * 16 + i] : -INFINITY, f, -INFINITY};
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
+          for (int o = 16; o > 0; o >>= 1) {
+            const bool up = lane & o;
+            const int n = o / 2;   // tokens kept (0: the last one, by both lanes)
+#pragma unroll
+            for (int i = 0; i < (n ? n : 1); ++i) {
+              const Top2 give = n && !up ? s[i + n] : s[i];
+              const Top2 keep = n && up ? s[i + n] : s[i];
               Top2 y;
-              y.v1 = __shfl_xor_sync(0xffffffffu, s.v1, o);
-              y.i1 = __shfl_xor_sync(0xffffffffu, s.i1, o);
-              y.v2 = __shfl_xor_sync(0xffffffffu, s.v2, o);
-              s = top2_merge(s, y);
+              y.v1 = __shfl_xor_sync(0xffffffffu, give.v1, o);
+              y.i1 = __shfl_xor_sync(0xffffffffu, give.i1, o);
+              y.v2 = __shfl_xor_sync(0xffffffffu, give.v2, o);
+              s[i] = top2_merge(keep, y);
             }
-            if (lane == 0) {
-              Top2* slot = &red[q * BN + cc * 16 + i];
-              *slot = sub == 0 ? s : top2_merge(*slot, s);
-            }
+          }
+          if (!(lane & 1)) {
+            Top2* slot = &red[q * BN + cc * 16 + lane / 2];
+            *slot = sub == 0 ? s[0] : top2_merge(*slot, s[0]);
           }
         }
       }
