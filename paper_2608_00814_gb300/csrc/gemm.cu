@@ -56,8 +56,7 @@ namespace oos {
 //
 // Work split.  Every matrix is cut into tiles of `rows` weight rows (a multiple
 // of 8 up to the MMA's 128; the accumulator lanes past it hold sums of whatever
-// follows in shared memory and are never read), chosen so that the tiles fill
-// the SMs about once (make_plan):
+// follows in shared memory and are never read), see plan_cluster and plan_rows:
 //   QKV, RESID: a thread-block cluster of `split` CTAs shares a tile, each CTA
 //     one k-range of it.  Each stages its fp32 sums in its own shared memory
 //     (over the ring, idle by then); after a cluster barrier CTA i pulls every
@@ -1035,10 +1034,15 @@ int gemm_fit(int c) {
 }
 
 // Tile rows and k-split of a QKV (rows fixed at one head) or RESID GEMM: of the
-// splits whose clusters fit the GPU, the one whose CTAs move the fewest bytes
-// in sequence, weights and activations (for 64 nodes) together, with a charge
-// per split for the sums it pulls and one per extra wave for a second prologue
-// and epilogue (~8 us at ~80 KB/us).
+// splits whose clusters fit the GPU, the one whose CTAs move the fewest bytes in
+// sequence, weights and activations (for 64 nodes) together, with a charge per
+// split for the sums it pulls and one per extra wave for a second prologue and
+// epilogue (~8 us at ~80 KB/us).  Tiles are cut below the MMA's 128 rows only when
+// every cluster that fits then has one of at least kMinCut: a CTA stages the whole
+// activation slice however few its rows.  O and down of the 0.6B shape as 32 rows x 4
+// splits and 48 x 6 took 2.8 / 2.5 / 2.1 / 8.5 us more per layer at T = 1 / 32 / 64 / 128
+// than as 128 x 8; 4096 rows as 120 x 4 take 0.7 us less than as 128 x 4 (T = 64).
+constexpr int kMinCut = 112;   // 7/8 of the MMA's rows
 GemmPlan plan_cluster(int N, int K, bool whole_heads) {
   GemmPlan best = {};
   long long best_cost = -1;
@@ -1046,8 +1050,8 @@ GemmPlan plan_cluster(int N, int K, bool whole_heads) {
   for (int c = 1; c <= kMaxSplit && c <= kbt; ++c) {
     const int fit = gemm_fit(c);
     if (fit < 1) continue;
-    int rows = kTile;
-    if (!whole_heads && N < kTile * fit) rows = ((N + fit - 1) / fit + 7) / 8 * 8;
+    const int even = ((N + fit - 1) / fit + 7) / 8 * 8;   // rows that give every cluster a tile
+    const int rows = !whole_heads && even >= kMinCut && even < kTile ? even : kTile;
     const int n_work = (N + rows - 1) / rows;
     const long long waves = (n_work + fit - 1) / fit;
     const long long cost = waves * ((kbt + c - 1) / c) * (rows * 128 + 16384) + (long long)c * 16384 +
@@ -1060,13 +1064,21 @@ GemmPlan plan_cluster(int N, int K, bool whole_heads) {
   return best;
 }
 
-// Whole-K tiles of equal rows that fill the SMs in as few rounds as the MMA's
-// 128 rows allow (gate/up: `rows` of each matrix per tile).  The tiles go to pairs
-// of CTAs, so their number is even; the last may lie past the matrix (zeros).
+// Whole-K tiles (gate/up: `rows` of each matrix per tile), an even number, since they
+// go to pairs of CTAs; the last may lie past the matrix (zeros).  Tiles of 128 rows
+// where one round of them takes up to half the SMs (a short stream: the fewer CTAs
+// stage the activations, and the next kernel's CTAs start on the SMs left) or at least
+// 7 in 10 (enough to draw the full bandwidth).  Else tiles of equal rows that fill
+// the SMs in as few rounds as 128 rows allow.  Per layer, 128 rows against the even
+// cut at T = 1 / 32 / 64 / 128: 3072 rows (24 tiles against 128) -1.3 / -2.8 / -5.0 /
+// -10.8 us, 9728 (76, 152) -1.0 / -1.8 / -2.2 / -1.6, 14336 (112, 150) 0 / -2.6 / -1.0 /
+// -1.3; between the lines, 12288 (96, 140), +1.6 / +1.0 / -0.2 / -1.3.
 GemmPlan plan_rows(int N, int K, int n_sms) {
   n_sms &= ~1;
-  const int rounds = (N + kTile * n_sms - 1) / (kTile * n_sms);
-  const int rows = ((N + rounds * n_sms - 1) / (rounds * n_sms) + 7) / 8 * 8;
+  const int rounds = (N + kTile * n_sms - 1) / (kTile * n_sms), full = (N + kTile - 1) / kTile;
+  int rows = kTile;
+  if (rounds > 1 || (2 * full > n_sms && 10 * full < 7 * n_sms))
+    rows = ((N + rounds * n_sms - 1) / (rounds * n_sms) + 7) / 8 * 8;
   const int n_work = ((N + rows - 1) / rows + 1) & ~1;
   return GemmPlan{rows, n_work, K / kBK, 1, n_work < n_sms ? n_work : n_sms};
 }

@@ -18,9 +18,11 @@ if not torch.cuda.is_available():
 import oracle  # noqa: E402
 from paper_2608_00814_gb300 import binding as B  # noqa: E402
 
-# hidden, intermediate, q heads, kv heads: the smallest matrices there are; a
-# last residual tile cut by the matrix end, and 3, 5 and 4 query heads a kv head
-SHAPES = [(128, 128, 1, 1), (384, 640, 3, 1), (640, 1152, 5, 1), (1152, 384, 8, 2)]
+# hidden, intermediate, q heads, kv heads: the smallest matrices there are; 3, 5 and
+# 4 query heads a kv head; gate/up tiles cut so that every SM has one (80 rows); residual
+# tiles cut so that every cluster has one (120 rows, the last one shorter)
+SHAPES = [(128, 128, 1, 1), (384, 640, 3, 1), (640, 1152, 5, 1), (1152, 384, 8, 2), (128, 11520, 1, 1),
+          (4096, 512, 2, 1)]
 
 
 @pytest.mark.parametrize("hidden,inter,nq,nkv", SHAPES)
