@@ -715,10 +715,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
             acc[k].w += ws * v[k][s].w;
           }
         }
-        if (i0 + KR * kWarps >= n_mine) {   // the last pull: the barrier need not await the stores
-#pragma unroll
-          for (int k = 0; k < KR; ++k) asm volatile("" ::"f"(acc[k].x), "f"(acc[k].y), "f"(acc[k].z), "f"(acc[k].w) : "memory");
-          cluster_arrive_relaxed();
+        if (i0 + KR * kWarps >= n_mine) {   // the last pull: the barrier need not await this round's stores
+          cluster_arrive_release();
           arrived = true;
         }
 #pragma unroll

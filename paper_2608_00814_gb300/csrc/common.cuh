@@ -172,12 +172,11 @@ OOS_DEV void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::
 OOS_DEV uint32_t smem_addr(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
 
 // ---- thread-block clusters
-// not .aligned: the threads of a warp may arrive at different points
+// not .aligned: the threads of a warp may arrive at different points.  Every arrival
+// releases: only that orders the thread's earlier accesses, its reads of a peer's
+// shared memory included, before what the peer does past the barrier (such as leaving).
 OOS_DEV void cluster_arrive_release() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 OOS_DEV void cluster_wait_acquire() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-// arrival that orders nothing but the thread's own completed reads: it does not
-// wait for stores in flight
-OOS_DEV void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); }
 // address of the same shared-memory location in block `rank` of the cluster
 OOS_DEV uint32_t dsmem_addr(const void* p, uint32_t rank) {
   uint32_t r;

@@ -728,11 +728,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       for (int s = 0; s < kMaxSplit; ++s) peer[s] = dsmem_addr(stage, dry ? rank : (uint32_t)(s < a.split ? s : 0));
       float4 acc[kFinRows];
       pull_rows(acc, peer, a.split, t0, te, ew, live);
-      if (!dry && t0 + kFinPass >= te) {   // the last pull: before the stores, which the barrier need not await
-#pragma unroll
-        for (int k = 0; k < kFinRows; ++k) asm volatile("" ::"f"(acc[k].x), "f"(acc[k].y), "f"(acc[k].z), "f"(acc[k].w) : "memory");
-        cluster_arrive_relaxed();
-      }
+      // the last pull: before this pass's stores, which the barrier then need not await
+      if (!dry && t0 + kFinPass >= te) cluster_arrive_release();
       if (EPI == EPI_RESID) resid_finish<CHUNK>(a, rr, acc, g4, tile, f, live, have, tok0, t0, te, ew);
       else qkv_finish<CHUNK>(a, qr, acc, b4, norm, g4, kind, h, ctx, rms, have, tok0, t0, te, ew);
     }
