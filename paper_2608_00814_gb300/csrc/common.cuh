@@ -77,6 +77,20 @@ OOS_DEV void store_act4_h(__half* p, size_t i, size_t lo_off, float4 v) {
   *reinterpret_cast<uint2*>(p + i + lo_off) = *reinterpret_cast<const uint2*>(lo);
 }
 
+// g / (1 + e^-g), as exact as with the division operator (at most 4.2 and 0.8 rms units of
+// 2^-24 of the value, the exponential's error; the same at 2.5e8 values of -88.7 .. 80), which
+// waits for a branch per value: the quotient of __fdividef, within 2 ulp, and one step
+// of iterative refinement.  The scale keeps the denominator below the 2^126 that
+// __fdividef takes; an infinite one, or g, gives what the operator gives.
+OOS_DEV float silu(float g) {
+  const float d = 1.f + expf(-g);
+  const float s = d > 1e37f ? 0.25f : 1.f;
+  const float n = g * s, e = d * s;
+  const float q = __fdividef(n, e);
+  const float c = __fdividef(fmaf(-q, e, n), e);
+  return fabsf(c) < INFINITY ? q + c : q;
+}
+
 // ---- block reductions (deterministic order)
 OOS_DEV float warp_sum(float v) {
 #pragma unroll

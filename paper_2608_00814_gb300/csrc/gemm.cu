@@ -793,8 +793,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
           const float r = rms[cc * 16 + i];
-          const float gr = g[i] * r;
-          u[i] = __fdividef(gr, 1.f + expf(-gr)) * (u[i] * r);   // 2 ulp; exp's infinity gives 0
+          u[i] = silu(g[i] * r) * (u[i] * r);
         }
         // lane pairs swap tokens so that a store covers two neighbouring features
 #pragma unroll

@@ -427,10 +427,7 @@ __global__ void __launch_bounds__(kPfThreads, 1)
 #pragma unroll
           for (int c = 0; c < 64; c += 16) {
 #pragma unroll
-            for (int i = c; i < c + 16; ++i) {
-              const float gr = acc[i] * r;
-              acc[i] = __fdividef(gr, 1.f + expf(-gr)) * (acc[64 + i] * r);
-            }
+            for (int i = c; i < c + 16; ++i) acc[i] = silu(acc[i] * r) * (acc[64 + i] * r);
             __nv_bfloat16* y = a.out + (size_t)t * a.N + i0 + c;
             store16_hilo<__nv_bfloat162>(y, y + a.lo_off, acc + c);
           }

@@ -1,0 +1,69 @@
+"""Precision of the fused kernels: SwiGLU over the whole range of the gate."""
+
+import dataclasses
+
+import numpy as np
+import pytest
+import torch
+
+from gpu_util import gpu_cache
+from synth.configs import workload
+from synth.device import upload_model
+from synth.model import SynthModel
+
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():
+    pytest.skip("needs a GPU", allow_module_level=True)
+
+from paper_2608_00814_gb300 import binding as B  # noqa: E402
+
+# gate pre-activations, each exact in bf16 over 128; the up values (powers of two) bring
+# silu(gate) * up to about 1
+GATES = [-88.5, -88.0, -87.5, -86.0, -60.0, -20.0, -4.0, -0.5, 0.0, 0.75, 3.0, 20.0, 80.0]
+
+
+@pytest.mark.parametrize("hidden,inter,T,n", [
+    (128, 128, 1, 0), (128, 128, 64, 0), (128, 128, 128, 0),   # each form of the verify GEMM
+    (128, 128, 0, 130), (1280, 3072, 0, 2048),                 # a prefill chunk in token tiles, and in pairs' tiles
+])
+def test_swiglu_over_the_range_of_the_gate(hidden, inter, T, n):
+    """One decoder layer whose MLP adds silu(g_f) u_f to feature f, and a second one
+    whose V rows show the result.  e^-g is near the largest float for the lowest g,
+    where a division that flushes a large denominator would give 0."""
+    cfg = dataclasses.replace(workload("mini-bf16").model, hidden=hidden, intermediate=inter, n_q_heads=1,
+                              n_kv_heads=1, n_layers=2, vocab=300, qk_norm=False)
+    w = upload_model(SynthModel(cfg, 0))
+    gate = np.array([GATES[f % len(GATES)] for f in range(128)])
+    silu = gate / (1 + np.exp(-gate))
+    up = np.where(silu == 0, 1.0, 2.0 ** np.round(-np.log2(np.abs(silu) + (silu == 0))))
+    w["embed"].fill_(1.0)
+    L = w["layers"][0]
+    for t in [L["w_o"], L["w_gate"], L["w_up"], L["w_down"], w["layers"][1]["w_v"]]:
+        t.zero_()
+    for t in [L["mlp_norm"], w["layers"][1]["attn_norm"]]:
+        t.fill_(1.0)
+    L["w_gate"][:128, :128] = torch.as_tensor(gate / 128)[:, None].to(torch.bfloat16).cuda()
+    L["w_up"][:128, :128] = torch.as_tensor(up / 128)[:, None].to(torch.bfloat16).cuda()
+    idx = torch.arange(128, device="cuda")
+    L["w_down"][idx, idx] = 1.0
+    w["layers"][1]["w_v"][idx, idx] = 1.0
+    model = B.OosModel(cfg, w)
+    case = dataclasses.make_dataclass("C", ["cfg", "cache_native"])(cfg, [(np.zeros((0, 1, 128), np.uint16),) * 2] * 2)
+    m = T or n
+    cache = gpu_cache(case, m)
+    tok = torch.zeros(m, dtype=torch.int32, device="cuda")
+    if T:
+        B.tree_verify(model, cache, 0, tok, torch.arange(T, dtype=torch.int32, device="cuda") - 1)
+    else:
+        B.oos_prefill(model, cache, 0, tok, n, None)
+    torch.cuda.synchronize()
+    assert B.oos_last_status(model) == B.OOS_OK
+    r = 1 / np.sqrt(1 + cfg.rms_eps)
+    x = np.ones(hidden)
+    x[:128] += gate * r / (1 + np.exp(-gate * r)) * up * r
+    want = x / np.sqrt((x * x).mean() + cfg.rms_eps)
+    got = cache.v[1][:, 0].double().cpu().numpy()
+    # bf16 V rows, half a step 2^-9; e^-g turns an fp32 step of g <= 88 into 88 * 2^-23
+    assert np.abs(got - want[:128]).max() <= 2.0 ** -8 * np.abs(want).max()
+    assert (np.abs(got - want[:128]) <= 2.0 ** -8 * np.abs(want[:128]) + 1e-6).all()
