@@ -47,8 +47,8 @@ namespace oos {
 //   EPI_ARGMAX: LM head -- logits scaled by the final RMSNorm factor and folded
 //               into a per-node running top-2.
 // A prefill chunk too small for the tiles of prefill.cu runs through the same
-// kernels in token tiles of 128 (CHUNK): the token tiles of a weight tile are
-// separate clusters (or CTAs).
+// kernels in token tiles (CHUNK) of 128, or 64 for gate/up: the token tiles of a
+// weight tile are separate clusters (or CTAs).
 //
 // RMSNorm is split across kernels by linearity: a producer stores y = g (.) x
 // and sum(x^2) per feature tile; the consumer GEMM computes W.y and multiplies
@@ -92,6 +92,7 @@ struct GemmArgs {
   int rows;           // weight rows per subtile
   int n_work, kbt;    // work tiles, k-blocks per tile
   int split;          // CTAs sharing a tile (cluster size)
+  int chain;          // prefill chunks: most k-blocks an accumulator collects (see k_chain)
   int stages;         // ring depth
   int N;              // output rows (features / vocab; intermediate rows for EPI_SILU)
   int T;              // valid columns (tree nodes; all token tiles together)
@@ -152,6 +153,8 @@ struct TcCfg {
   // error that grows with the chain, so the chains are kept short (one segment
   // where both buffers do not fit: 256 MMAs at K = 4096, hi and lo apart)
   static constexpr int SEGS = EPI == EPI_ARGMAX ? 1 : BUFS;
+  // 16-token column chunks of an epilogue warp (`half`, `half` + 2, ...)
+  static constexpr int CHUNKS = BN >= 32 ? BN / 32 : 1;
   static constexpr int X_BYTES = PAIR ? B_BYTES : 2 * B_BYTES;   // activations of a stage in this CTA
   static __host__ __device__ int stage_bytes(int rows) { return kSub * rows * kBK * 2 + X_BYTES; }
   static int stages(int rows) {
@@ -218,18 +221,20 @@ constexpr int kFinRows = 4;
 constexpr int kFinPass = kFinRows * kEpiWarps;
 
 // acc[k] = sum over the cluster's CTAs, in rank order, of their staged row of
-// token t0 + w + 8k (peer[s]: shared-memory address of CTA s's stage)
+// token t0 + w + 8k (peer[s]: shared-memory address of CTA s's stage), SB CTAs' rows
+// in flight
+template <int SB>
 OOS_DEV void pull_rows(float4 (&acc)[kFinRows], const uint32_t (&peer)[kMaxSplit], int split, int t0, int te, int w,
                        bool live) {
   const uint32_t off = (uint32_t)(threadIdx.x & 31) * 16;
 #pragma unroll
   for (int k = 0; k < kFinRows; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-  for (int s0 = 0; s0 < kMaxSplit; s0 += 4) {
+  for (int s0 = 0; s0 < kMaxSplit; s0 += SB) {
     if (s0 >= split) break;
-    float4 v[4][kFinRows];
+    float4 v[SB][kFinRows];
 #pragma unroll
-    for (int s = 0; s < 4; ++s)
+    for (int s = 0; s < SB; ++s)
 #pragma unroll
       for (int k = 0; k < kFinRows; ++k) {
         const int t = t0 + w + kEpiWarps * k;
@@ -237,7 +242,7 @@ OOS_DEV void pull_rows(float4 (&acc)[kFinRows], const uint32_t (&peer)[kMaxSplit
                                                      : make_float4(0.f, 0.f, 0.f, 0.f);
       }
 #pragma unroll
-    for (int s = 0; s < 4; ++s)
+    for (int s = 0; s < SB; ++s)
 #pragma unroll
       for (int k = 0; k < kFinRows; ++k) acc[k] = f4_add(acc[k], v[s][k]);
   }
@@ -392,7 +397,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     first = blockIdx.x / a.split;
     step = 0;
     if (CHUNK) {
-      tok0 = first / a.n_work * kTile;
+      tok0 = first / a.n_work * BN;
       first %= a.n_work;
     }
     kb0 = a.kbt * (int)rank / a.split;
@@ -404,14 +409,17 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     kb0 = 0;
     nkb = a.kbt;
     if (CHUNK) {   // one tile per CTA
-      tok0 = first / a.n_work * kTile;
+      tok0 = first / a.n_work * BN;
       first %= a.n_work;
       n_units = a.kbt;
     } else {
       n_units = first < a.n_work ? (a.n_work - first + step - 1) / step * a.kbt : 0;
     }
   }
-  const int T = CHUNK ? min(a.T - tok0, kMaxT) : a.T;   // tokens of this CTA's tiles
+  const int T = CHUNK ? min(a.T - tok0, BN) : a.T;   // tokens of this CTA's tiles
+  // k-segments of a tile: as many as it has accumulators, or, in a prefill chunk, as
+  // the longest chain makes, the accumulators taken in turn
+  const int segs = CHUNK ? (nkb + a.chain - 1) / a.chain : nkb < C::SEGS ? 1 : C::SEGS;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
@@ -465,7 +473,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       // read zeros (TMA out-of-bounds fill)
       auto load_sub = [&](const CUtensorMap* wm, unsigned char* dst, int kb, int row, int stage) {
         load(dst, wm, stage, kb * kBK, row, pol_w);
-        if (CHUNK && CLUSTER)   // the chunk's boxes are 64 rows high
+        if (CHUNK)   // the chunk's boxes are 64 rows high
           load(dst + 64 * kBK * 2, wm, stage, kb * kBK, row + 64, pol_w);
       };
       auto load_w = [&](int tile, int kb, int stage) {
@@ -564,7 +572,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       int acc = 0;
       uint32_t use = 0;   // accumulators handed over so far (two buffers in turn)
       bool ok = true;
-      const int segs = nkb < C::SEGS ? 1 : C::SEGS;
       for (int j = 0; j < n_units && ok; j += nkb) {
         for (int sg = 0; sg < segs && ok; ++sg) {
           if (!mbar_wait(&acce[acc], (uses(use) & 1u) ^ 1u, abort_flag, a.status)) {
@@ -637,13 +644,50 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     }
   };
 
+  // Prefill chunks: the k-segments before the last, added up in registers while the
+  // MMAs of the next run: part[c][sub] is chunk c of this warp.  `use` counts the
+  // accumulators taken.  False when a wait gave up.
+  auto take_early = [&](float (&part)[C::CHUNKS][kSub][16], uint32_t& use) {
+    for (int sg = 0; sg + 1 < segs; ++sg, ++use) {
+      const uint32_t b = use & 1u;
+      if (!__all_sync(0xffffffffu, mbar_wait(&accf[b], uses(use) & 1u, abort_flag, a.status))) return false;
+      tc_fence_after();
+#pragma unroll
+      for (int c = 0; c < C::CHUNKS; ++c) {
+        const int cc = half + 2 * c;
+        if (cc * 16 >= T) continue;   // warp-uniform
+#pragma unroll
+        for (int sub = 0; sub < kSub; ++sub) {
+          float v[16];
+          acc16(b * (uint32_t)(kSub * C::SUB_COLS) + (uint32_t)(sub * C::SUB_COLS + cc * 16), v);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) part[c][sub][i] = sg == 0 ? v[i] : part[c][sub][i] + v[i];
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&acce[b]);
+    }
+    return true;
+  };
+  // chunk 0 of the sums leaves and the others move up: a window over registers in a
+  // loop that is not unrolled
+  auto next_chunk = [&](float (&part)[C::CHUNKS][kSub][16]) {
+#pragma unroll
+    for (int c = 0; c + 1 < C::CHUNKS; ++c)
+#pragma unroll
+      for (int sub = 0; sub < kSub; ++sub)
+#pragma unroll
+        for (int i = 0; i < 16; ++i) part[c][sub][i] = part[c + 1][sub][i];
+  };
+
   if (CLUSTER && warp >= 2) {
     const int tile = first;
     // tokens [tb, te) are finished here
     const int tb = T * (int)rank / a.split, te = T * ((int)rank + 1) / a.split;
     const int f = EPI == EPI_RESID ? tile * a.rows + 4 * lane : 4 * lane;
     const bool live = 4 * lane < a.rows && (EPI != EPI_RESID || f < a.N);
-    const bool two = nkb >= 2;   // one accumulator per k-segment
+    const bool two = nkb >= 2;   // one accumulator per k-segment, both read at the end
     int kind = 0, h = 0, ctx = 0;
     bool norm = false, have = false;
     float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f), g4 = make_float4(1.f, 1.f, 1.f, 1.f);
@@ -662,13 +706,65 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       if (gn) g4 = bf16x4(gn + f);
       norm = gn != nullptr;
     }
+    if (CHUNK) {
+      pdl_wait();
+      pdl_trigger();
+      uint32_t use = 0;
+      float part[C::CHUNKS][kSub][16];
+      have = take_early(part, use);
+      if (EPI == EPI_QKV) {
+        ctx = *a.ctx;
+        input_rms<CHUNK>(a, rms, tok0, tb, te, ew);
+      }
+      have = have && mbar_wait(&accf[use & 1u], uses(use) & 1u, abort_flag, a.status);
+      have = __all_sync(0xffffffffu, have);
+      tc_fence_after();
+      // every MMA has read its operands: the ring is free for the sums
+#pragma unroll 1
+      for (int cc = half; cc < BN / 16; cc += 2) {
+        if (cc * 16 >= T) break;
+        float v[16];
+        acc16((use & 1u) * (uint32_t)C::SUB_COLS + (uint32_t)(cc * 16), v);
+        if (segs > 1) {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) v[i] += part[0][0][i];
+          next_chunk(part);
+        }
+        if (have && row < a.rows) {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) stage[(cc * 16 + i) * kTile + row] = v[i];
+        }
+      }
+      auto load = [&](int t0) {   // what a finishing pass reads
+        if (EPI == EPI_RESID) resid_load<CHUNK>(a, rr, f, live, tok0, t0, te, ew);
+        else qkv_load<CHUNK>(a, qr, kind, tok0, t0, te, ew);
+      };
+      load(tb);
+      cluster_arrive_release();   // twice, as below
+      __syncwarp();
+      cluster_wait_acquire();
+      uint32_t peer[kMaxSplit];
+#pragma unroll
+      for (int s = 0; s < kMaxSplit; ++s) peer[s] = dsmem_addr(stage, (uint32_t)(s < a.split ? s : 0));
+#pragma unroll 1
+      for (int t0 = tb;; t0 += kFinPass) {
+        const bool last = t0 + kFinPass >= te;
+        float4 acc[kFinRows];
+        pull_rows<2>(acc, peer, a.split, t0, te, ew, live);
+        if (last) cluster_arrive_release();
+        if (EPI == EPI_RESID) resid_finish<CHUNK>(a, rr, acc, g4, tile, f, live, have, tok0, t0, te, ew);
+        else qkv_finish<CHUNK>(a, qr, acc, b4, norm, g4, kind, h, ctx, rms, have, tok0, t0, te, ew);
+        if (last) break;
+        load(t0 + kFinPass);
+      }
+    }
     // Pass -1 is a dry run of the whole epilogue before the dependency wait:
     // no wait, barrier or store, values discarded.  The epilogue runs once per
     // launch, and the step's other kernels have evicted its code from the SM's
     // instruction caches since the previous layer; this fetches it while the
     // warps have nothing else to do.
 #pragma unroll 1
-    for (int pass = -1;; ++pass) {
+    for (int pass = -1; !CHUNK; ++pass) {
       asm volatile("" : "+r"(pass));   // one copy of the body for every pass
       const bool dry = pass < 0;
       const int t0 = dry ? tb : tb + pass * kFinPass;
@@ -727,7 +823,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 #pragma unroll
       for (int s = 0; s < kMaxSplit; ++s) peer[s] = dsmem_addr(stage, dry ? rank : (uint32_t)(s < a.split ? s : 0));
       float4 acc[kFinRows];
-      pull_rows(acc, peer, a.split, t0, te, ew, live);
+      pull_rows<4>(acc, peer, a.split, t0, te, ew, live);
       // the last pull: before this pass's stores, which the barrier then need not await
       if (!dry && t0 + kFinPass >= te) cluster_arrive_release();
       if (EPI == EPI_RESID) resid_finish<CHUNK>(a, rr, acc, g4, tile, f, live, have, tok0, t0, te, ew);
@@ -745,13 +841,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   } else if (!ARGMAX && warp >= 2) {
     // Gate and up of one row sit in the same lane, so act is formed in
     // registers.  Tile -1 is a dry run, as above.
-    const bool two = C::SEGS > 1 && nkb >= 2;
+    const bool two = !CHUNK && C::SEGS > 1 && nkb >= 2;
     const bool odd = lane & 1;
     const uint32_t acce0 = PAIR ? dsmem_addr(acce, 0) : 0u;   // rank 0's, where the issuer waits
     uint32_t use = 0;   // tiles drained
     uint32_t acc0 = 0;  // buffer of the tile's first k-segment (the second's is the other one)
 #pragma unroll 1
-    for (int it = -1;; ++it) {
+    for (int it = CHUNK ? 0 : -1;; ++it) {
       asm volatile("" : "+r"(it));
       const bool dry = it < 0;
       const int tile = first + (dry ? 0 : it) * step;
@@ -763,7 +859,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         input_rms<CHUNK>(a, rms, tok0, 0, T, ew);
         epi_bar();
       }
-      if (!dry) {
+      float part[C::CHUNKS][kSub][16];
+      if (CHUNK && !dry) {   // one tile a CTA
+        if (it > 0 || !take_early(part, use) ||
+            !__all_sync(0xffffffffu, mbar_wait(&accf[use & 1u], uses(use) & 1u, abort_flag, a.status)))
+          break;
+        tc_fence_after();
+        acc0 = use & 1u;
+      } else if (!dry) {
         if (it * nkb >= n_units) break;
         const bool ok = two ? mbar_wait(&accf[0], use & 1u, abort_flag, a.status) &&
                                   mbar_wait(&accf[1], use & 1u, abort_flag, a.status)
@@ -781,6 +884,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         float g[16], u[16];
         acc16(col0 + cc * 16, g);
         acc16(col0 + C::SUB_COLS + cc * 16, u);
+        if (CHUNK && !dry && segs > 1) {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            g[i] += part[0][0][i];
+            u[i] += part[0][kSub - 1][i];
+          }
+          next_chunk(part);
+        }
         if (two) {
           float v[16];
           acc16(col1 + cc * 16, v);
@@ -811,7 +922,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
           }
         }
       }
-      if (!dry) {
+      if (!dry && !CHUNK) {
         tc_fence_before();
         __syncwarp();
         if (lane == 0) {
@@ -999,7 +1110,7 @@ cudaError_t gemm_setup() {
   if (e == cudaSuccess) e = set_smem_all<128>();
   if (e == cudaSuccess) e = set_smem<128, EPI_QKV, true>();
   if (e == cudaSuccess) e = set_smem<128, EPI_RESID, true>();
-  if (e == cudaSuccess) e = set_smem<128, EPI_SILU, true>();
+  if (e == cudaSuccess) e = set_smem<64, EPI_SILU, true>();
   return e;
 }
 
@@ -1027,6 +1138,21 @@ int gemm_fit(int c) {
   }
   if (c > 1) n -= (c & 1) ? (n + 11) / 12 : 1;
   return n;
+}
+
+// k-blocks that one accumulator of a prefill chunk may collect.  The tensor core
+// truncates every addition to its accumulator, an error that grows with the chain of
+// MMAs, so K goes in chains no longer than the pieces that an even deal of the matrix's
+// k-blocks over the SMs would cut (8B shape: q/k/v 15, O 11, down 33, gate/up 24; 0.6B:
+// two each), added in fp32 registers.  A small matrix has short chains, which its
+// latency mostly hides.  Four MMAs a k-block where the hi and lo products have columns
+// of their own.  Error of the first layer's V (mostly bf16 values rounded the other
+// way) of 2048 tokens with the 0.6B / 8B shape: 1.1e-4 / 1.0e-4 in chains of 128 MMAs,
+// 2.4e-5 / 7.2e-5 so.  One layer of the 0.6B shape, 333 tokens: 77 -> 86 us.
+int k_chain(int rows, int K, int n_sms) {
+  const int tiles = (rows + kTile - 1) / kTile, kbt = K / kBK;
+  const int kb = tiles * kbt / (tiles + n_sms);
+  return kb < 2 ? 2 : kb;
 }
 
 // Tile rows and k-split of a QKV (rows fixed at one head) or RESID GEMM: of the
@@ -1129,6 +1255,7 @@ static GemmArgs base_args(Model& m, const GemmW& g, int T, int slot) {
   a.n_work = g.plan.n_work;
   a.kbt = g.plan.kbt;
   a.split = g.plan.split;
+  a.chain = g.chain;
   a.N = g.N;
   a.T = T;
   a.tl_slot = slot;
@@ -1201,40 +1328,41 @@ cudaError_t launch_gemm_gu(Model& m, int layer, int T, cudaStream_t st) {
   return dispatch_tc<EPI_SILU>(m, m.g_gu[layer], m.amap_xn, T, a, st);
 }
 
-// ---- a prefill chunk in token tiles of 128 (prefill.cu chooses between these
-// and its own tiles): 128 weight rows a tile (64 of gate and up), buffers of
-// kPfTokens rows, norm sums per 128 features as prefill.cu writes them
-static void chunk_args(Model& m, GemmArgs& a, int rows, int n_work, int split) {
-  a.rows = rows;
+// ---- a prefill chunk in token tiles (prefill.cu chooses between these and its own
+// tiles): 128 weight rows a tile, buffers of kPfTokens rows, norm sums per 128
+// features as prefill.cu writes them
+static void chunk_args(Model& m, GemmArgs& a, int n_work, int split) {
+  a.rows = kTile;
   a.n_work = n_work;
   a.split = split;
   a.ss_in = m.ws.pf_ss;
   a.ss_chunks = m.cfg.hidden / kTile;
 }
-static int chunk_tiles(const GemmArgs& a) { return a.n_work * ((a.T + kTile - 1) / kTile); }
+static int chunk_tiles(const GemmArgs& a, int tokens) { return a.n_work * ((a.T + tokens - 1) / tokens); }
 cudaError_t launch_chunk_qkv(Model& m, int layer, void* kc, void* vc, int T, int split, cudaStream_t st) {
   GemmArgs a = qkv_args(m, layer, kc, vc, T);
-  chunk_args(m, a, kTile, m.cfg.n_q_heads + 2 * m.cfg.n_kv_heads, split);
+  chunk_args(m, a, m.cfg.n_q_heads + 2 * m.cfg.n_kv_heads, split);
   a.rope = m.ws.pf_rope;
   a.q_out = (__nv_bfloat16*)m.ws.pf_q;
-  return launch_tc<128, EPI_QKV, true>(m, m.g_qkv[layer], m.pf_xn_map, chunk_tiles(a) * split, a, st);
+  return launch_tc<128, EPI_QKV, true>(m, m.g_qkv[layer], m.pf_xn_map, chunk_tiles(a, 128) * split, a, st);
 }
 cudaError_t launch_chunk_resid(Model& m, int layer, bool down, const void* gain, int T, int split, cudaStream_t st) {
   const GemmW& g = down ? m.g_down[layer] : m.g_o[layer];
   GemmArgs a = base_args(m, g, T, layer * 4 + (down ? 3 : 1));
-  chunk_args(m, a, kTile, g.N / kTile, split);
+  chunk_args(m, a, g.N / kTile, split);
   a.x = m.ws.pf_x;
   a.gain = (const __nv_bfloat16*)gain;
   a.y_out = (__nv_bfloat16*)m.ws.pf_xn;
   a.ss_out = m.ws.pf_ss;
-  return launch_tc<128, EPI_RESID, true>(m, g, down ? m.pf_act_map : m.pf_attn_map, chunk_tiles(a) * split, a, st);
+  return launch_tc<128, EPI_RESID, true>(m, g, down ? m.pf_act_map : m.pf_attn_map, chunk_tiles(a, 128) * split, a, st);
 }
+// 64 tokens a tile: the registers hold the segments' sums of gate and up
 cudaError_t launch_chunk_gu(Model& m, int layer, int T, cudaStream_t st) {
   const GemmW& g = m.g_gu[layer];
   GemmArgs a = base_args(m, g, T, layer * 4 + 2);
-  chunk_args(m, a, 64, g.N / 64, 1);
+  chunk_args(m, a, g.N / kTile, 1);
   a.act_out = (__nv_bfloat16*)m.ws.pf_act;
-  return launch_tc<128, EPI_SILU, true>(m, g, m.pf_xn_map, chunk_tiles(a), a, st);
+  return launch_tc<64, EPI_SILU, true>(m, g, m.pf_xn64_map, chunk_tiles(a, 64), a, st);
 }
 
 cudaError_t launch_lm_head_tc(Model& m, int T, cudaStream_t st) {

@@ -40,6 +40,7 @@ struct GemmW {
   CUtensorMap pf_map[3];   // prefill: boxes of 64 rows
   int n_seg;
   int N, K;     // output rows (gate/up: of one matrix), reduction length
+  int chain;    // k_chain of the stacked matrix
   GemmPlan plan;
 };
 
@@ -104,6 +105,7 @@ struct Model {
   GemmW g_lm;
   CUtensorMap amap_xn[4], amap_attn[4], amap_act[4];  // per N-tile variant 16/32/64/128
   CUtensorMap pf_xn_map, pf_attn_map, pf_act_map;     // prefill: boxes of 128 rows
+  CUtensorMap pf_xn64_map;                            // of 64
   CUtensorMap pf_qmap_hi, pf_qmap_lo;
   int fit[9] = {0};               // gemm_fit of 1..8
   CUtensorMap qmap_hi, qmap_lo;   // attention: q rows of one kv head, (d, head in group, kv head, node)
@@ -144,6 +146,14 @@ inline cudaError_t launch(bool pdl, void (*kernel)(KArgs...), dim3 grid, dim3 bl
   lc.attrs = attr;
   lc.numAttrs = pdl ? 1 : 0;
   return cudaLaunchKernelEx(&lc, kernel, std::forward<Args>(args)...);
+}
+
+// A kernel that splits its registers between warps (setmaxnreg) waits forever for a
+// share that its launch did not bring: an error unless it was compiled for `regs`.
+inline cudaError_t check_launch_regs(const void* kernel, int regs) {
+  cudaFuncAttributes a;
+  const cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+  return e != cudaSuccess ? e : a.numRegs >= regs ? cudaSuccess : cudaErrorInvalidConfiguration;
 }
 
 // ---- small kernels (small.cu)
@@ -187,6 +197,7 @@ constexpr int kMaxSplit = 8;                             // CTAs sharing a GEMM 
 int gemm_fit(int c);                                     // clusters of c CTAs resident at once (after gemm_setup)
 GemmPlan plan_cluster(int N, int K, bool whole_heads);   // after gemm_setup
 GemmPlan plan_rows(int N, int K, int n_sms);
+int k_chain(int rows, int K, int n_sms);
 int norm_chunks(const Model& m, int layer);
 cudaError_t launch_chunk_qkv(Model& m, int layer, void* kc, void* vc, int T, int split, cudaStream_t st);
 cudaError_t launch_chunk_resid(Model& m, int layer, bool down, const void* gain, int T, int split, cudaStream_t st);

@@ -382,6 +382,8 @@ int oos_model_create(const oos_model_config* cfg, const oos_weights* w, void* wo
         g.N = rows[0];
         g.K = K;
         g.plan = plan;
+        // gate/up: a tile of each matrix shares the k-blocks
+        g.chain = k_chain(nseg == 3 ? rows[0] + rows[1] + rows[2] : rows[0], K, n_sms);
         return plan.grid > 0;
       };
       for (int s = 1; s <= kMaxSplit; ++s) m->fit[s] = gemm_fit(s);

@@ -6,8 +6,10 @@
 // MMA's M, 256 weight rows in N.  The activations keep their two bf16 halves,
 // so every k-step is two MMAs on the same weights.  The tensor core truncates each
 // addition to its accumulator, an error that grows with the chain, so K goes in
-// segments of kPfSeg k-blocks whose sums the epilogue warps add in fp32 registers
-// (one chain over K = 4096 and 12288 added 2e-4 to a K/V error of 5e-4).
+// segments whose sums the epilogue warps add in fp32 registers, as long as k_chain
+// (gemm.cu) has them.  A segment costs 0.6 us: four layers of the 8B shape, 2048
+// tokens, take 4714 us in segments of 16 k-blocks (128 MMAs) and 4802 so (64 MMAs for
+// q/k/v, 48 for O).
 // A tile goes to a pair of CTAs (cta_group::2): 256 tokens, each CTA staging its 128
 // and half the weight rows.  A CTA alone would stage 64 KB per k-block and read 96 KB
 // of MMA operands in the 1024 clocks of its MMAs, more than its shared memory and its
@@ -32,12 +34,11 @@ namespace oos {
 constexpr int kPfRows = 128;                      // tokens per tile
 constexpr int kPfHalf = kPfRows * kBK * 2;        // bytes of one activation half per stage
 constexpr int kPfEpiWarps = 8;
-constexpr int kPfSeg = 16;                        // k-blocks per accumulator: 128 MMAs
 constexpr int kPfThreads = 128 + 32 * kPfEpiWarps;   // a warp group for the producer and the issuer
 // registers a thread keeps in each role (setmaxnreg): 128 * 56 + 256 * 224 of the
 // 384 * 168 the block is launched with
-constexpr int kPfRegsIssue = 56, kPfRegsEpi = 224;
-static_assert(128 * kPfRegsIssue + 32 * kPfEpiWarps * kPfRegsEpi <= kPfThreads * 168, "register split");
+constexpr int kPfRegsIssue = 56, kPfRegsEpi = 224, kPfRegsLaunch = 168;
+static_assert(128 * kPfRegsIssue + 32 * kPfEpiWarps * kPfRegsEpi <= kPfThreads * kPfRegsLaunch, "register split");
 
 constexpr int kPfCols = 256;                      // weight rows per tile
 constexpr int kPfStage = 2 * kPfHalf + kPfCols / 2 * kBK * 2;   // a CTA's activations and half the weight rows
@@ -50,6 +51,7 @@ enum { PF_QKV = 0, PF_RESID = 1, PF_SILU = 2 };
 struct PfArgs {
   int T;              // tokens of the chunk
   int kbt;            // k-blocks
+  int segs;           // segments of them, an accumulator each
   int m_tiles, n_tiles;   // token tiles (of 256 for a pair), weight tiles
   int N;              // output features (PF_SILU: intermediate size; PF_QKV: heads * 128)
   uint32_t* status;
@@ -248,7 +250,7 @@ __global__ void __launch_bounds__(kPfThreads, 1)
       bool ok = true;
       uint32_t sg = 0;   // segments handed over; they use the two accumulators in turn
       for (int it = 0; it < my_tiles && ok; ++it) {
-        for (int kb0 = 0; kb0 < a.kbt && ok; kb0 += kPfSeg, ++sg) {
+        for (int i = 0; i < a.segs && ok; ++i, ++sg) {
           const uint32_t b = sg & 1u;
           if (!mbar_wait(&acce[b], ((sg >> 1) & 1u) ^ 1u, abort_flag, a.status)) {
             ok = false;
@@ -256,7 +258,7 @@ __global__ void __launch_bounds__(kPfThreads, 1)
           }
           tc_fence_after();
           const uint32_t d = tmem_base + b * kPfCols;
-          const int n = min(kPfSeg, a.kbt - kb0);
+          const int n = a.kbt * (i + 1) / a.segs - a.kbt * i / a.segs;
           for (int kb = 0; kb < n; ++kb, ++j) {
             const int stage = j % S;
             if (!mbar_wait(&full[stage], (uint32_t)(j / S) & 1u, abort_flag, a.status)) {
@@ -267,11 +269,12 @@ __global__ void __launch_bounds__(kPfThreads, 1)
             const uint32_t base = smem_addr(ring + stage * kPfStage);
             const uint64_t xh = smem_desc_sw128(base), xl = smem_desc_sw128(base + kPfHalf);
             const uint64_t w = smem_desc_sw128(base + 2 * kPfHalf);
+            // lo first: the accumulator is small then, and so is what an addition truncates
 #pragma unroll
-            for (int k = 0; k < kBK / 16; ++k) {
-              tc_mma_bf16_pair(d, xh + 2 * k, w + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
-              tc_mma_bf16_pair(d, xl + 2 * k, w + 2 * k, idesc, 1u);
-            }
+            for (int k = 0; k < kBK / 16; ++k)
+              tc_mma_bf16_pair(d, xl + 2 * k, w + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+#pragma unroll
+            for (int k = 0; k < kBK / 16; ++k) tc_mma_bf16_pair(d, xh + 2 * k, w + 2 * k, idesc, 1u);
             tc_commit_pair(&empty[stage]);
           }
           if (ok) tc_commit_pair(&accf[b]);
@@ -293,7 +296,6 @@ __global__ void __launch_bounds__(kPfThreads, 1)
     const uint32_t lane_base = tmem_base + ((uint32_t)(q * 32) << 16);
     const int ctx = EPI == PF_QKV ? *a.ctx : 0;
     const uint32_t acce0 = dsmem_addr(acce, 0);   // rank 0's, where the issuer waits
-    const int segs = (a.kbt + kPfSeg - 1) / kPfSeg;
     uint32_t sg = 0;
     for (int it = 0; it < my_tiles; ++it) {
       const int tile = me + it * G;
@@ -309,7 +311,7 @@ __global__ void __launch_bounds__(kPfThreads, 1)
       // this thread's 128 sums: a head, 128 features, or 64 gate and 64 up rows
       float acc[128];
       bool ok = true;
-      for (int i = 0; i < segs; ++i, ++sg) {
+      for (int i = 0; i < a.segs; ++i, ++sg) {
         const uint32_t b = sg & 1u;
         ok = __all_sync(0xffffffffu, mbar_wait(&accf[b], (sg >> 1) & 1u, abort_flag, a.status));
         if (!ok) break;
@@ -487,7 +489,8 @@ __global__ void __launch_bounds__(256) k_pf_last(const __nv_bfloat16* __restrict
 // ------------------------------------------------------------ host side
 template <int EPI>
 static cudaError_t pf_smem() {
-  return cudaFuncSetAttribute(k_pf_gemm<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPfSmem);
+  const cudaError_t e = cudaFuncSetAttribute(k_pf_gemm<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPfSmem);
+  return e == cudaSuccess ? check_launch_regs((const void*)k_pf_gemm<EPI>, kPfRegsLaunch) : e;
 }
 cudaError_t prefill_setup() {
   cudaError_t e = pf_smem<PF_QKV>();
@@ -499,28 +502,40 @@ bool prefill_encode(Model& m) {
   const auto& c = m.cfg;
   const int qd = c.n_q_heads * c.head_dim;
   return encode_rows_map(&m.pf_xn_map, m.ws.pf_xn, 2 * kPfTokens, c.hidden, kPfRows) &&
+         encode_rows_map(&m.pf_xn64_map, m.ws.pf_xn, 2 * kPfTokens, c.hidden, 64) &&
          encode_rows_map(&m.pf_attn_map, m.ws.pf_attn, 2 * kPfTokens, qd, kPfRows) &&
          encode_rows_map(&m.pf_act_map, m.ws.pf_act, 2 * kPfTokens, c.intermediate, kPfRows);
 }
 
+// Segments of a GEMM in pairs' tiles: their hi and lo products share an accumulator,
+// eight MMAs a k-block, so the k-blocks are half of k_chain's.  Not gate/up's: the MLP's
+// share of the next layer's K/V error shows no difference (hidden 1024 .. 5120).
+static int pf_segs(const GemmW& g, int epi) {
+  const int kbt = g.K / kBK, chain = epi == PF_SILU ? g.chain : (g.chain + 1) / 2;
+  return (kbt + chain - 1) / chain;
+}
+
 // How one GEMM of a chunk runs: 0 as pairs' tiles of 256 tokens x 256 weight rows
 // here, c >= 1 as the verify GEMM's tiles of 128 x 128, k split over clusters of c
-// (gate/up: unsplit, in pairs of its own).
+// (gate/up: unsplit, 64 tokens x 128 rows of each).
 //
 // Estimates in microseconds of work in line, one wave after the other: a k-block of
-// a pair's tile takes 0.53 and a tile's turnover 10, a k-block of a verify tile 0.4 and
-// its turnover 8.5, each rank of a cluster 0.9 for the sums it pulls; the residual's
-// tiles cost 24 more here (64 or fewer pairs hide neither the first loads nor the
-// rows of x they read and write), gate/up's 5.  Set against timings of each choice
-// in turn at 8 chunk lengths of 136..2048 tokens in 4 shapes (hidden 1024..5120): the
-// choice was the fastest or within 4 us of it in 125 of 128, and within 14 in all.
-// Both ways, one layer's down GEMM: 512 tokens of the 8B shape 24 us less in verify
-// tiles, 1024 tokens 25 us less in pairs.
-static int pf_split(const Model& m, int rows, int kbt, int T, int epi) {
+// a pair's tile takes 0.5, a segment 0.6 and a tile's turnover 10, a k-block of a
+// verify tile 0.4 and its turnover 8.5, each rank of a cluster 0.9 for the sums it
+// pulls; the residual's tiles cost 24 more here (64 or fewer pairs hide neither the
+// first loads nor the rows of x they read and write), gate/up's 5.  Against timings of
+// each choice in turn at 8 chunk lengths of 136..2048 tokens in 6 shapes (hidden
+// 256..5120), the choice is the fastest or within 4 us of it in 180 of 192, and within
+// 10 in all.  Both ways, one layer's down GEMM: 512 tokens of the 8B shape 45 us less
+// in verify tiles, 2048 tokens of the 2048 x 6144 shape 6 us less in pairs.
+static int pf_split(const Model& m, const GemmW& g, int rows, int T, int epi) {
+  const int kbt = g.K / kBK;
   const int mt = (T + kPfRows - 1) / kPfRows;
   auto waves = [](long long tiles, int fit) { return (double)((tiles + fit - 1) / fit); };
-  const long long tiles = (long long)mt * ((rows + 127) / 128);
-  double best = waves((long long)((mt + 1) / 2) * ((rows + kPfCols - 1) / kPfCols), m.num_sms / 2) * (kbt * 0.53 + 10) +
+  const long long tiles = epi == PF_SILU ? (long long)((T + 63) / 64) * ((rows + 255) / 256)
+                                         : (long long)mt * ((rows + 127) / 128);
+  double best = waves((long long)((mt + 1) / 2) * ((rows + kPfCols - 1) / kPfCols), m.num_sms / 2) *
+                    (kbt * 0.5 + pf_segs(g, epi) * 0.6 + 10) +
                 (epi == PF_RESID ? 24 : epi == PF_SILU ? 5 : 0);
   int split = 0;
   for (int c = 1; c <= (epi == PF_SILU ? 1 : kMaxSplit) && c <= kbt; ++c) {
@@ -539,6 +554,7 @@ static cudaError_t launch_pf(Model& m, const GemmW& g, const CUtensorMap& am, Pf
   // rows: stacked weight rows of the GEMM
   const auto& c = m.cfg;
   a.kbt = g.K / kBK;
+  a.segs = pf_segs(g, EPI);
   a.m_tiles = (a.T + 2 * kPfRows - 1) / (2 * kPfRows);
   a.n_tiles = (rows + kPfCols - 1) / kPfCols;
   a.status = m.ws.status;
@@ -576,7 +592,7 @@ static PfArgs pf_args(int T) {
 
 static cudaError_t launch_pf_resid(Model& m, int layer, bool down, const void* gain, int T, cudaStream_t st) {
   const GemmW& g = down ? m.g_down[layer] : m.g_o[layer];
-  const int split = pf_split(m, m.cfg.hidden, g.K / kBK, T, PF_RESID);
+  const int split = pf_split(m, g, m.cfg.hidden, T, PF_RESID);
   if (split) return launch_chunk_resid(m, layer, down, gain, T, split, st);
   PfArgs a = pf_args(T);
   a.N = m.cfg.hidden;
@@ -592,7 +608,7 @@ static cudaError_t launch_pf_qkv(Model& m, int layer, void* kc, void* vc, int T,
   const auto& c = m.cfg;
   const oos_layer_weights& L = m.layers[layer];
   const int rows = (c.n_q_heads + 2 * c.n_kv_heads) * c.head_dim;
-  const int split = pf_split(m, rows, c.hidden / kBK, T, PF_QKV);
+  const int split = pf_split(m, m.g_qkv[layer], rows, T, PF_QKV);
   if (split) return launch_chunk_qkv(m, layer, kc, vc, T, split, st);
   PfArgs a = pf_args(T);
   a.N = rows;
@@ -614,7 +630,7 @@ static cudaError_t launch_pf_qkv(Model& m, int layer, void* kc, void* vc, int T,
 
 static cudaError_t launch_pf_gu(Model& m, int layer, int T, cudaStream_t st) {
   const auto& c = m.cfg;
-  if (pf_split(m, 2 * c.intermediate, c.hidden / kBK, T, PF_SILU)) return launch_chunk_gu(m, layer, T, st);
+  if (pf_split(m, m.g_gu[layer], 2 * c.intermediate, T, PF_SILU)) return launch_chunk_gu(m, layer, T, st);
   PfArgs a = pf_args(T);
   a.N = c.intermediate;
   a.out = (__nv_bfloat16*)m.ws.pf_act;

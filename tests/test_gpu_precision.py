@@ -1,4 +1,5 @@
-"""Precision of the fused kernels: SwiGLU over the whole range of the gate."""
+"""Precision of the fused kernels: SwiGLU over the whole range of the gate; a prefill
+chunk against the same prompt in trees."""
 
 import dataclasses
 
@@ -6,7 +7,9 @@ import numpy as np
 import pytest
 import torch
 
-from gpu_util import gpu_cache
+import oracle
+from cases import build_case
+from gpu_util import gpu_cache, gpu_model, to_f64
 from synth.configs import workload
 from synth.device import upload_model
 from synth.model import SynthModel
@@ -67,3 +70,41 @@ def test_swiglu_over_the_range_of_the_gate(hidden, inter, T, n):
     # bf16 V rows, half a step 2^-9; e^-g turns an fp32 step of g <= 88 into 88 * 2^-23
     assert np.abs(got - want[:128]).max() <= 2.0 ** -8 * np.abs(want).max()
     assert (np.abs(got - want[:128]) <= 2.0 ** -8 * np.abs(want[:128]) + 1e-6).all()
+
+
+def _kv_error(case, cut, n):
+    """2-norm errors, relative, of K and V of every layer after prompts of `cut` tokens."""
+    model, _ = gpu_model(case)
+    cache = gpu_cache(case, n)
+    prompt = np.random.default_rng(n).integers(0, case.cfg.vocab, size=n).astype(np.int32)
+    tok = torch.as_tensor(prompt, device="cuda")
+    for at in range(0, n, cut):
+        m = min(cut, n - at)
+        B.oos_prefill(model, cache, at, tok[at:at + m], m, None)
+    torch.cuda.synchronize()
+    assert B.oos_last_status(model) == B.OOS_OK
+    r = oracle.verify_tree(case.view, case.cache_k64, case.cache_v64, 0, prompt, np.arange(n) - 1)
+    out = []
+    for l in range(case.cfg.n_layers):
+        e = s = 0.0
+        for got, want in ((cache.k[l], r["tree_k"][l]), (cache.v[l], r["tree_v"][l])):
+            e += ((to_f64(case.cfg, got) - want) ** 2).sum()
+            s += (want ** 2).sum()
+        out.append((e / s) ** 0.5)
+    return out
+
+
+@pytest.mark.parametrize("hidden,inter,n", [
+    (1024, 1024, 400),    # q/k/v in token tiles of 128
+    (1024, 1024, 900),    # in pairs' tiles
+])
+def test_prefill_chunk_is_as_exact_as_chains_of_trees(hidden, inter, n):
+    """A chunk's first K/V are one projection of the embedding, so their error is that of
+    its accumulators (and of 16-bit values that it rounds the other way).  In trees of
+    128 tokens the chains are 8 MMAs; in chunks they are as long, in pairs with the lo
+    products among them: twice the truncations, and so at most twice the error.  Chains
+    of 32 and 128 MMAs gave 2.4 and 6.2 times the error."""
+    over = dict(hidden=hidden, intermediate=inter, n_q_heads=16, n_kv_heads=8, n_layers=1, vocab=700,
+                init_std=1.0 / hidden ** 0.5)
+    case = build_case("mini-bf16", 8, T=4, plant=0, ctx_len=0, cfg_overrides=over, gain_std=0.1, prefill=False)
+    assert _kv_error(case, n, n)[0] <= 2 * _kv_error(case, 128, n)[0]
