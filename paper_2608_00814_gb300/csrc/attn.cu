@@ -102,19 +102,28 @@ static_assert((kOffQ & 1023) == 0, "swizzled q staging is 1024-aligned");
 constexpr int kAttnSmem = kOffBar + 256 + 1024;           // + barriers + alignment slack
 constexpr int kAttnThreads = 384;                         // 12 warps, roles below
 constexpr int kSoftWarp0 = 4;                             // softmax warps 4..11
+// prefill: registers a thread keeps in the loaders' and issuers' warps and in the
+// softmax warps (setmaxnreg), of the 384 * 168 the block is launched with
+constexpr int kPfRegsIo = 56, kPfRegsSoft = 224, kPfRegsLaunch = 168;
+static_assert(128 * kPfRegsIo + (kAttnThreads - 128) * kPfRegsSoft <= kAttnThreads * kPfRegsLaunch, "register split");
 static_assert(kAttnSmem <= 227 * 1024, "shared memory per block");
 static_assert(kMaxSplits <= 16, "cluster size");
 // TMEM columns (lane = query row): S[2] fp32 scores of a tile, O fp32, P[2] bf16
 // pairs.  With P apart from S the next S MMAs into a buffer wait only until its
 // scores are in registers, not for the P.V product (8 k cached positions, T = 128:
-// a tile every 1.2 us, 1.35 before).  Prefill keeps an O of
-// the even and one of the odd tiles: its blocks go through every key unsplit, the
-// tensor core truncates each addition to an accumulator, and two chains half as
-// long are closer to the sum (K/V error 5.3e-4 -> 5.2e-4 over 2048 tokens; the
-// verify step's chains are short, and reading a second O cost it 1 %); P then
-// overwrites the first 64 columns of its S buffer
+// a tile every 1.2 us, 1.35 before).  In prefill P overwrites the first 64 columns of
+// its S buffer, and there are two O, of the even and the odd tiles.
+//
+// Prefill's blocks go through every key unsplit or nearly.  Under one running maximum
+// only its own key's weight is exact in 16 bits, and the tensor core truncates every
+// addition to an O that collects all tiles: the K/V of the layers above were up to
+// 15 % (FP16 cache) and 12 % (bf16) further from the exact ones than with trees of 128
+// tokens, whose keys are cut over up to 16 splits, each with a maximum and an O of its own.
+// So every tile has its own maximum and its own P.V, and the softmax threads add the
+// tiles' O up in registers, scaled, in fp32: errors 0 .. 25 % below the trees' in seven
+// shapes, for 101 -> 114 us (2048 tokens, 8B shape) and 21 -> 23 us (0.6B, 333).
 constexpr int kTmS = 0;                            // [2] x 128
-constexpr int kTmO = 2 * kAttnKeys;                // [2] x 128
+constexpr int kTmO = 2 * kAttnKeys;                // verify: 128, prefill: [2] x 128
 constexpr int kTmP = kTmO + kAttnD;                // verify: [2] x 64
 constexpr int kAttnTmemCols = 512;                 // allocation unit: a power of two
 static_assert(kTmO + 2 * kAttnD <= kAttnTmemCols, "TMEM columns");
@@ -260,7 +269,8 @@ OOS_DEV void drain_wait(uint64_t* bar, uint32_t parity) {
 // the swizzled layouts; apart, so that a K tile does not queue behind a V tile whose
 // stage is still in use); warp 1 lane 0 issues the S MMAs, warp 2 lane 0 the P.V MMAs;
 // warps 4..11 run the softmax (lane = query row = TMEM lane, warps 4..7 on the
-// first 64 keys of a tile, 8..11 on the others); all warps take part in the merge.
+// first 64 keys of a tile, 8..11 on the others); all warps take part in the merge
+// (prefill: the softmax warps, the others having given up their registers).
 // F16: the KV cache (and q) are IEEE binary16 -- every product runs in f16;
 // otherwise bf16.  CAUSAL: a prefill chunk.
 template <bool F16, bool CAUSAL>
@@ -326,130 +336,249 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
   const uint32_t tmem = *tmem_slot;
   const uint32_t tmem_o = tmem + kTmO;
 
-  if (warp == 0 || warp == 3) {
-    // ------------------------------------------------------------ loaders (one thread each, TMA)
-    if (lane == 0) {
-      const bool v = warp == 3;
-      const CUtensorMap* map = v ? &a.vmap : &a.kmap;
-      uint64_t* full = v ? vfull : kfull;
-      uint64_t* empty = v ? vempty : kempty;
-      tma_prefetch_desc(map);
-      const uint64_t pol_kv = policy_evict_first();
-      auto load = [&](int ti) {   // two 64-wide d blocks of 128 slots
-        const int st = ti & 1;
-        const int key0 = (t0 + ti) * kAttnKeys;
-        unsigned char* dst = sm + (v ? kOffV : kOffK) + st * kTileBytes;
-        mbar_arrive_expect_tx(&full[st], kTileBytes);
-        tma_load_3d(dst, map, &full[st], 0, g, key0, pol_kv);
-        tma_load_3d(dst + kDBlock, map, &full[st], 64, g, key0, pol_kv);
-      };
-      // tiles of committed slots only do not depend on the producing kernel:
-      // the first stages are fetched before waiting for it
-      int n = 0;   // tiles issued
-      while (n < n_tiles && n < kKvStages && (t0 + n + 1) * kAttnKeys <= ctx) load(n++);
-      pdl_wait();
-      pdl_trigger();
-      if (!v) {
-        TL_ATTN(1);
-        // q rows of the block's nodes, hi and lo halves, two 64-wide d blocks each
-        tma_prefetch_desc(&a.qhi);
-        tma_prefetch_desc(&a.qlo);
-        const uint64_t pol_q = policy_evict_last();
-        unsigned char* qs = sm + kOffQ;
-        mbar_arrive_expect_tx(qfull, (uint32_t)(4 * rows * 128));
-        tma_load_4d(qs, &a.qhi, qfull, 0, 0, g, node0, pol_q);
-        tma_load_4d(qs + kAttnRows * 128, &a.qhi, qfull, 64, 0, g, node0, pol_q);
-        tma_load_4d(qs + 2 * kAttnRows * 128, &a.qlo, qfull, 0, 0, g, node0, pol_q);
-        tma_load_4d(qs + 3 * kAttnRows * 128, &a.qlo, qfull, 64, 0, g, node0, pol_q);
-      }
-      for (int ti = n; ti < n_tiles; ++ti) {
-        if (!attn_wait(&empty[ti & 1], ((uint32_t)(ti >> 1) & 1u) ^ 1u, abort_flag, status, v ? AW_VEMPTY : AW_KEMPTY, ti))
-          break;
-        load(ti);
-        ++n;
-      }
-      // every copy this thread issued has landed before the block can exit,
-      // whoever gave up (immediate on the normal path, where all were consumed)
-      for (int ti = n > 2 ? n - 2 : 0; ti < n; ++ti) drain_wait(&full[ti & 1], (uint32_t)(ti >> 1) & 1u);
-      if (!v) drain_wait(qfull, 0);
-    }
-  } else if (warp == 1 || warp == 2) {
-    // ------------------------------------------------------------ MMA issuers
-    // Operands reach the tensor cores through the async proxy only: q, K and
-    // V by TMA, P from threads that wait for their TMEM stores before they
-    // arrive, the zeroed V rows fenced by the threads that wrote them.
-    // Descriptors: the start address is the low field (16-byte units), so a
-    // byte offset o inside an operand region is added as o >> 4.
-    if (lane == 0 && warp == 1) {
-      constexpr uint32_t idesc_s = F16 ? idesc_f16_f32(kAttnRows, kAttnKeys) : idesc_bf16_f32(kAttnRows, kAttnKeys);
-      bool ok = attn_wait(qfull, 0, abort_flag, status, AW_QFULL, 0);
-      TL_ATTN(2);
-      tc_fence_after();
-      const uint64_t kdesc0 = smem_desc_sw128(smem_addr(sm + kOffK));
-      // q as staged by TMA: [hi d0, hi d1, lo d0, lo d1], each 128 rows x 128
-      // bytes in the swizzled K-major layout (rows of padding nodes hold
-      // whatever the q buffer holds; every row of S, P and O is its own)
-      const uint64_t qdesc0 = smem_desc_sw128(smem_addr(sm + kOffQ));
-      for (int ti = 0; ti < n_tiles && ok; ++ti) {
-        const int b = ti & 1;
-        const uint32_t use = (uint32_t)(ti >> 1);
-        // S buffer b holds tile ti - 2's scores until they are read, or its P until
-        // that tile's P.V is done
-        if (!attn_wait(&kfull[b], use & 1u, abort_flag, status, AW_KFULL, ti) ||
-            !attn_wait(P_APART ? &sread[b] : &pvdone[b], (use & 1u) ^ 1u, abort_flag, status, AW_SFREE, ti))
-          break;
-        tc_fence_after();
-        const uint64_t kd0 = kdesc0 + (uint64_t)((b * kTileBytes) >> 4);
-        const uint32_t d = tmem + kTmS + b * kAttnKeys;
-        // S = q_hi K^T + q_lo K^T over the 128 head dims: q and K both from
-        // their two 64-wide d blocks (32 bytes of d per MMA)
+  // every role is done with the rings and TMEM past this
+  auto block_done = [&]() {
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+  };
+  float* stage = reinterpret_cast<float*>(sm + kOffStage);   // [row][kMergeLd]
+
+  // ------------------------------------------------------------ merge
+  // Each block stages its O row, max and sum of every real row in its own
+  // shared memory (over the K/V ring, idle by then).  Rows [0, vrows) are dealt to the S
+  // blocks of the cluster; past the cluster barrier a warp takes an owned row at a
+  // time, pulls it from every split and adds the splits by log-sum-exp, in order.
+  // Every thread of the cluster arrives twice, whatever happened before: its
+  // block's rows are staged, and it has pulled (a stage must outlive its readers).
+  auto finish = [&]() {
+    if (threadIdx.x == 128) TL_ATTN(21);
+    cluster_arrive_release();
+    __syncwarp();
+    cluster_wait_acquire();
+    if (threadIdx.x == 128) TL_ATTN(22);
+    {
+      // A warp takes KR owned rows at a time, so that about 16 pulls of a lane are in
+      // flight whatever the split count (one row at a time: 4.4 us from the barrier to
+      // the exit of 6 splits).
+      const int lr0 = (int)((long long)vrows * split / S);
+      const int n_mine = (int)((long long)vrows * (split + 1) / S) - lr0;
+      constexpr int kWarp0 = CAUSAL ? kSoftWarp0 : 0, kWarps = kAttnThreads / 32 - kWarp0;
+      auto merge = [&](auto kr, auto sm_max) {
+        constexpr int KR = decltype(kr)::value, SM = decltype(sm_max)::value;
+        bool arrived = false;
+        for (int i0 = warp - kWarp0; i0 < n_mine || !arrived; i0 += KR * kWarps) {
+          float2 ml[KR];
+          float4 v[KR][SM];
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
+          for (int k = 0; k < KR; ++k) {
+            const int i = i0 + k * kWarps;
+            const bool on = i < n_mine;
+            const uint32_t off = (uint32_t)((lr0 + (on ? i : 0)) * kMergeRowBytes);
+            // lane s: (max, sum) of split s; then every split's four values of this lane
+            ml[k] = make_float2(-INFINITY, 0.f);
+            if (on && lane < S) ml[k] = ld_cluster2(dsmem_addr(stage, (uint32_t)lane) + off + kAttnD * 4);
 #pragma unroll
-          for (int k = 0; k < kAttnD / 16; ++k) {
-            const uint64_t kd = kd0 + (uint64_t)(((k >> 2) * kDBlock) >> 4) + 2 * (k & 3);
-            const uint64_t qd = qdesc0 + (uint64_t)(((2 * half + (k >> 2)) * (kAttnRows * 128)) >> 4) + 2 * (k & 3);
-            tc_mma_bf16(d, qd, kd, idesc_s, (half > 0 || k > 0) ? 1u : 0u);
+            for (int s = 0; s < SM; ++s)
+              v[k][s] = on && s < S ? ld_cluster4(dsmem_addr(stage, (uint32_t)s) + off + (uint32_t)lane * 16u)
+                                    : make_float4(0.f, 0.f, 0.f, 0.f);
+          }
+          float4 acc[KR];
+#pragma unroll
+          for (int k = 0; k < KR; ++k) {
+            const float M = warp_max(ml[k].x);
+            const float w = ml[k].x == -INFINITY ? 0.f : exp2f(ml[k].x - M);
+            const float den = warp_sum(w * ml[k].y);
+            const float wn = den > 0.f ? w / den : 0.f;
+            acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int s = 0; s < SM; ++s) {
+              const float ws = __shfl_sync(0xffffffffu, wn, s);   // 0 past the splits
+              acc[k].x += ws * v[k][s].x;
+              acc[k].y += ws * v[k][s].y;
+              acc[k].z += ws * v[k][s].z;
+              acc[k].w += ws * v[k][s].w;
+            }
+          }
+          if (i0 + KR * kWarps >= n_mine) {   // the last pull: the barrier need not await this round's stores
+            cluster_arrive_release();
+            arrived = true;
+          }
+#pragma unroll
+          for (int k = 0; k < KR; ++k) {
+            const int i = i0 + k * kWarps;
+            if (i < n_mine) {
+              const int lr = lr0 + i;
+              const size_t grow = (size_t)(node0 + lr / G) * nq + g * G + lr % G;
+              store_act4(a.out, grow * kAttnD + 4 * lane, a.out_lo_off, acc[k]);
+            }
           }
         }
-        tc_commit(&kempty[b]);
-        tc_commit(&sfull[b]);
-      }
-      tc_commit(odone);
-    } else if (lane == 0 && warp == 2) {
-      constexpr uint32_t idesc_pv =
-          (F16 ? idesc_f16_f32(kAttnRows, kAttnD) : idesc_bf16_f32(kAttnRows, kAttnD)) | (1u << 16);   // B (V) MN-major
-      // V tile: d blocks of 64 (kDBlock apart) along N, 16 keys (2 KB) per MMA along K
-      const uint64_t vdesc0 = smem_desc_sw128_mn(smem_addr(sm + kOffV), kDBlock);
-      for (int ti = 0; ti < n_tiles; ++ti) {
-        const int b = ti & 1;
-        const uint32_t use = (uint32_t)(ti >> 1);
-        if (!attn_wait(&pfull[b], use & 1u, abort_flag, status, AW_PFULL, ti) ||
-            !attn_wait(&vfull[b], use & 1u, abort_flag, status, AW_VFULL, ti))
-          break;
-        tc_fence_after();
-        // P: 8 columns = 16 keys per MMA
-        const uint32_t pt = tmem + (P_APART ? kTmP + b * 64 : kTmS + b * kAttnKeys);
-        const uint64_t vd = vdesc0 + (uint64_t)((b * kTileBytes) >> 4);
-#pragma unroll
-        for (int kk = 0; kk < kAttnKeys / 16; ++kk)
-          tc_mma_bf16_ts(tmem_o + (CAUSAL ? b * kAttnD : 0), pt + 8 * kk, vd + (uint64_t)((kk * 16 * 128) >> 4), idesc_pv,
-                         (ti > (CAUSAL ? 1 : 0) || kk > 0) ? 1u : 0u);
-        tc_commit(&pvdone[b]);
-        tc_commit(&vempty[b]);
-      }
-      tc_commit(odone);
+      };
+      if (S <= 5) merge(Int<3>{}, Int<5>{});
+      else if (S <= 8) merge(Int<2>{}, Int<8>{});
+      else merge(Int<1>{}, Int<kMaxSplits>{});
     }
-  }
+  };
 
-  // ------------------------------------------------------------ softmax (warps 4..11)
-  float m_used = -INFINITY, l_sum = 0.f;            // l_sum: of this thread's keys
-  const int q4 = warp & 3;
-  const int hf = warp >= kSoftWarp0 + 4 ? 1 : 0;    // key half
-  const int lrow = q4 * 32 + lane;                  // local row = TMEM lane
-  const uint32_t lane_off = (uint32_t)(q4 * 32) << 16;
-  float* s_max = reinterpret_cast<float*>(sm + kOffMax);
-  if (warp >= kSoftWarp0) {
+  if (warp < kSoftWarp0) {
+    if constexpr (CAUSAL) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kPfRegsIo));
+    if (warp == 0 || warp == 3) {
+      // ------------------------------------------------------------ loaders (one thread each, TMA)
+      if (lane == 0) {
+        const bool v = warp == 3;
+        const CUtensorMap* map = v ? &a.vmap : &a.kmap;
+        uint64_t* full = v ? vfull : kfull;
+        uint64_t* empty = v ? vempty : kempty;
+        tma_prefetch_desc(map);
+        const uint64_t pol_kv = policy_evict_first();
+        auto load = [&](int ti) {   // two 64-wide d blocks of 128 slots
+          const int st = ti & 1;
+          const int key0 = (t0 + ti) * kAttnKeys;
+          unsigned char* dst = sm + (v ? kOffV : kOffK) + st * kTileBytes;
+          mbar_arrive_expect_tx(&full[st], kTileBytes);
+          tma_load_3d(dst, map, &full[st], 0, g, key0, pol_kv);
+          tma_load_3d(dst + kDBlock, map, &full[st], 64, g, key0, pol_kv);
+        };
+        // tiles of committed slots only do not depend on the producing kernel:
+        // the first stages are fetched before waiting for it
+        int n = 0;   // tiles issued
+        while (n < n_tiles && n < kKvStages && (t0 + n + 1) * kAttnKeys <= ctx) load(n++);
+        pdl_wait();
+        pdl_trigger();
+        if (!v) {
+          TL_ATTN(1);
+          // q rows of the block's nodes, hi and lo halves, two 64-wide d blocks each
+          tma_prefetch_desc(&a.qhi);
+          tma_prefetch_desc(&a.qlo);
+          const uint64_t pol_q = policy_evict_last();
+          unsigned char* qs = sm + kOffQ;
+          mbar_arrive_expect_tx(qfull, (uint32_t)(4 * rows * 128));
+          tma_load_4d(qs, &a.qhi, qfull, 0, 0, g, node0, pol_q);
+          tma_load_4d(qs + kAttnRows * 128, &a.qhi, qfull, 64, 0, g, node0, pol_q);
+          tma_load_4d(qs + 2 * kAttnRows * 128, &a.qlo, qfull, 0, 0, g, node0, pol_q);
+          tma_load_4d(qs + 3 * kAttnRows * 128, &a.qlo, qfull, 64, 0, g, node0, pol_q);
+        }
+        for (int ti = n; ti < n_tiles; ++ti) {
+          if (!attn_wait(&empty[ti & 1], ((uint32_t)(ti >> 1) & 1u) ^ 1u, abort_flag, status, v ? AW_VEMPTY : AW_KEMPTY, ti))
+            break;
+          load(ti);
+          ++n;
+        }
+        // every copy this thread issued has landed before the block can exit,
+        // whoever gave up (immediate on the normal path, where all were consumed)
+        for (int ti = n > 2 ? n - 2 : 0; ti < n; ++ti) drain_wait(&full[ti & 1], (uint32_t)(ti >> 1) & 1u);
+        if (!v) drain_wait(qfull, 0);
+      }
+    } else if (warp == 1 || warp == 2) {
+      // ------------------------------------------------------------ MMA issuers
+      // Operands reach the tensor cores through the async proxy only: q, K and
+      // V by TMA, P from threads that wait for their TMEM stores before they
+      // arrive, the zeroed V rows fenced by the threads that wrote them.
+      // Descriptors: the start address is the low field (16-byte units), so a
+      // byte offset o inside an operand region is added as o >> 4.
+      if (lane == 0 && warp == 1) {
+        constexpr uint32_t idesc_s = F16 ? idesc_f16_f32(kAttnRows, kAttnKeys) : idesc_bf16_f32(kAttnRows, kAttnKeys);
+        bool ok = attn_wait(qfull, 0, abort_flag, status, AW_QFULL, 0);
+        TL_ATTN(2);
+        tc_fence_after();
+        const uint64_t kdesc0 = smem_desc_sw128(smem_addr(sm + kOffK));
+        // q as staged by TMA: [hi d0, hi d1, lo d0, lo d1], each 128 rows x 128
+        // bytes in the swizzled K-major layout (rows of padding nodes hold
+        // whatever the q buffer holds; every row of S, P and O is its own)
+        const uint64_t qdesc0 = smem_desc_sw128(smem_addr(sm + kOffQ));
+        for (int ti = 0; ti < n_tiles && ok; ++ti) {
+          const int b = ti & 1;
+          const uint32_t use = (uint32_t)(ti >> 1);
+          // S buffer b holds tile ti - 2's scores until they are read, or its P until
+          // that tile's P.V is done
+          if (!attn_wait(&kfull[b], use & 1u, abort_flag, status, AW_KFULL, ti) ||
+              !attn_wait(P_APART ? &sread[b] : &pvdone[b], (use & 1u) ^ 1u, abort_flag, status, AW_SFREE, ti))
+            break;
+          tc_fence_after();
+          const uint64_t kd0 = kdesc0 + (uint64_t)((b * kTileBytes) >> 4);
+          const uint32_t d = tmem + kTmS + b * kAttnKeys;
+          // S = q_hi K^T + q_lo K^T over the 128 head dims: q and K both from
+          // their two 64-wide d blocks (32 bytes of d per MMA)
+#pragma unroll
+          for (int half = 0; half < 2; ++half) {
+#pragma unroll
+            for (int k = 0; k < kAttnD / 16; ++k) {
+              const uint64_t kd = kd0 + (uint64_t)(((k >> 2) * kDBlock) >> 4) + 2 * (k & 3);
+              const uint64_t qd = qdesc0 + (uint64_t)(((2 * half + (k >> 2)) * (kAttnRows * 128)) >> 4) + 2 * (k & 3);
+              tc_mma_bf16(d, qd, kd, idesc_s, (half > 0 || k > 0) ? 1u : 0u);
+            }
+          }
+          tc_commit(&kempty[b]);
+          tc_commit(&sfull[b]);
+        }
+        tc_commit(odone);
+      } else if (lane == 0 && warp == 2) {
+        constexpr uint32_t idesc_pv =
+            (F16 ? idesc_f16_f32(kAttnRows, kAttnD) : idesc_bf16_f32(kAttnRows, kAttnD)) | (1u << 16);   // B (V) MN-major
+        // V tile: d blocks of 64 (kDBlock apart) along N, 16 keys (2 KB) per MMA along K
+        const uint64_t vdesc0 = smem_desc_sw128_mn(smem_addr(sm + kOffV), kDBlock);
+        for (int ti = 0; ti < n_tiles; ++ti) {
+          const int b = ti & 1;
+          const uint32_t use = (uint32_t)(ti >> 1);
+          if (!attn_wait(&pfull[b], use & 1u, abort_flag, status, AW_PFULL, ti) ||
+              !attn_wait(&vfull[b], use & 1u, abort_flag, status, AW_VFULL, ti))
+            break;
+          tc_fence_after();
+          // P: 8 columns = 16 keys per MMA
+          const uint32_t pt = tmem + (P_APART ? kTmP + b * 64 : kTmS + b * kAttnKeys);
+          const uint64_t vd = vdesc0 + (uint64_t)((b * kTileBytes) >> 4);
+#pragma unroll
+          for (int kk = 0; kk < kAttnKeys / 16; ++kk)
+            tc_mma_bf16_ts(tmem_o + (CAUSAL ? b * kAttnD : 0), pt + 8 * kk, vd + (uint64_t)((kk * 16 * 128) >> 4),
+                           idesc_pv, (kk > 0 || (!CAUSAL && ti > 0)) ? 1u : 0u);
+          tc_commit(&pvdone[b]);
+          tc_commit(&vempty[b]);
+        }
+        tc_commit(odone);
+      }
+    }
+    block_done();
+    if (CAUSAL) {   // their registers are given up: the softmax warps merge
+      cluster_arrive_release();
+      __syncwarp();
+      cluster_wait_acquire();
+      cluster_arrive_release();
+    }
+  } else {
+    if constexpr (CAUSAL) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kPfRegsSoft));   // half an O row each
+    // ------------------------------------------------------------ softmax (warps 4..11)
+    float m_used = -INFINITY, l_sum = 0.f;            // l_sum: of this thread's keys
+    const int q4 = warp & 3;
+    const int hf = warp >= kSoftWarp0 + 4 ? 1 : 0;    // key half
+    const int lrow = q4 * 32 + lane;                  // local row = TMEM lane
+    const uint32_t lane_off = (uint32_t)(q4 * 32) << 16;
+    float* s_max = reinterpret_cast<float*>(sm + kOffMax);
+    // Prefill: this thread's half of its O row, of the tiles taken so far, and the
+    // maximum it is scaled by (m_used: the last tile's own).
+    float o_sum[CAUSAL ? 64 : 1], m_sum = -INFINITY;
+#pragma unroll
+    for (int i = 0; i < (CAUSAL ? 64 : 1); ++i) o_sum[i] = 0.f;
+    // tile t, complete by now, whose maximum is m and whose weights sum to l (of this
+    // thread's keys)
+    auto take_o = [&](int t, float m, float l) {
+      if constexpr (CAUSAL) {
+        const float to = fmaxf(m_sum, m);
+        const float fo = m_sum == -INFINITY ? 0.f : exp2f(m_sum - to), ft = m == -INFINITY ? 0.f : exp2f(m - to);
+        m_sum = to;
+        l_sum = l_sum * fo + l * ft;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          float ov[32];
+          tmem_ld32_nowait(tmem_o + lane_off + (t & 1) * kAttnD + hf * 64 + c * 32, ov);
+          tmem_wait_ld_regs(ov);
+#pragma unroll
+          for (int i = 0; i < 32; ++i) o_sum[c * 32 + i] = fmaf(ov[i], ft, o_sum[c * 32 + i] * fo);
+        }
+      }
+    };
+    float l_tile = 0.f, m_prev = -INFINITY, l_prev = 0.f;   // prefill: of the tile at hand, and the one before it
     const bool real = lrow < vrows;
     const int node = real ? node0 + lrow / G : node0;
     unsigned long long anc0 = 0ull, anc1 = 0ull;
@@ -530,9 +659,10 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
       // move the running maximum only when this tile exceeds it by 2^8 (a
       // lane that moves its maximum rescales its half of the O row; the whole warp
       // takes part in the TMEM accesses, lanes that keep theirs scale by 1)
-      const bool move = !dry && tmax > m_used + 8.f;
-      const bool rescale = move && m_used != -INFINITY;
-      if (__any_sync(0xffffffffu, rescale)) {
+      // (prefill: every tile its own maximum)
+      const bool move = CAUSAL ? !dry : !dry && tmax > m_used + 8.f;
+      const bool rescale = !CAUSAL && move && m_used != -INFINITY;
+      if (!CAUSAL && __any_sync(0xffffffffu, rescale)) {
         // O holds P.V of tiles < ti: wait for the last of them, then rescale
         const int pb = (ti - 1) & 1;
         dead = !__all_sync(0xffffffffu, attn_wait(&pvdone[pb], (uint32_t)((ti - 1) >> 1) & 1u, abort_flag, status,
@@ -541,8 +671,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
         tc_fence_after();
         const float f = rescale ? exp2f(m_used - tmax) : 1.f;
 #pragma unroll 1
-        for (int c = 0; c < (CAUSAL ? 4 : 2); ++c) {   // 32 columns at a time: the scores stay in registers
-          const uint32_t col = tmem_o + lane_off + (c >> 1) * kAttnD + hf * 64 + (c & 1) * 32;
+        for (int c = 0; c < 2; ++c) {   // 32 columns at a time: the scores stay in registers
+          const uint32_t col = tmem_o + lane_off + hf * 64 + c * 32;
           float ov[32];
           tmem_ld32_nowait(col, ov);
           tmem_wait_ld_regs(ov);
@@ -582,7 +712,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
         asm volatile("" ::"f"(ps[0]), "f"(ps[1]), "f"(ps[2]), "f"(ps[3]));
         continue;
       }
-      l_sum += (ps[0] + ps[1]) + (ps[2] + ps[3]);
+      if (CAUSAL) l_tile = (ps[0] + ps[1]) + (ps[2] + ps[3]);
+      else l_sum += (ps[0] + ps[1]) + (ps[2] + ps[3]);
       // Tile ti - 2's P.V has read this P buffer and this V buffer.  Waited for before
       // the V wait below, whose parity alone would also match a phase two back.
       if (P_APART && ti >= 2) {
@@ -612,6 +743,18 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
       __syncwarp();
       if (lane == 0) mbar_arrive(&pfull[b]);
       if (warp == kSoftWarp0 && lane == 0 && ti < 6) TL_ATTN(4 + 2 * ti);
+      if (CAUSAL) {   // the tile before, whose O columns tile ti + 1 takes (it waits for these threads' P)
+        if (ti > 0) {
+          dead = !__all_sync(0xffffffffu, attn_wait(&pvdone[b ^ 1], (uint32_t)((ti - 1) >> 1) & 1u, abort_flag, status,
+                                                    AW_PFREE, ti));
+          if (dead) continue;
+          tc_fence_after();
+          take_o(ti - 1, m_prev, l_prev);
+          tc_fence_before();
+        }
+        m_prev = m_used;
+        l_prev = l_tile;
+      }
     }
     if (!waited) {   // no tile: the dependency wait is still owed
       pdl_wait();
@@ -622,32 +765,16 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
     // under a running MMA, so the wait is not cut short by the handle's limit
     drain_wait(odone, 0);
     if (warp == kSoftWarp0 && lane == 0) TL_ATTN(15);
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-
-  // ------------------------------------------------------------ merge
-  // Each block stages its O row, max and sum of every real row in its own
-  // shared memory (over the K/V ring, idle now).  Rows [0, vrows) are dealt to the S
-  // blocks of the cluster; past the cluster barrier a warp takes an owned row at a
-  // time, pulls it from every split and adds the splits by log-sum-exp, in order.
-  float* stage = reinterpret_cast<float*>(sm + kOffStage);   // [row][kMergeLd]
-  const bool have_o = n_tiles > 0 && !*abort_flag;   // block-uniform after the barrier
-  if (warp >= kSoftWarp0) {
+    block_done();
+    const bool have_o = n_tiles > 0 && !*abort_flag;   // block-uniform after the barrier
     float ov[64];
-    if (have_o) {
+    if (have_o && CAUSAL) {
+      take_o(n_tiles - 1, m_prev, l_prev);
+      m_used = m_sum;
+#pragma unroll
+      for (int i = 0; i < 64; ++i) ov[i] = o_sum[CAUSAL ? i : 0];
+    } else if (have_o) {
       tmem_ld64(tmem_o + lane_off + hf * 64, ov);
-      if (CAUSAL && n_tiles > 1) {
-        float o1[32];
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          tmem_ld32_nowait(tmem_o + kAttnD + lane_off + hf * 64 + c * 32, o1);
-          tmem_wait_ld_regs(o1);
-#pragma unroll
-          for (int i = 0; i < 32; ++i) ov[c * 32 + i] += o1[i];
-        }
-      }
     } else {
 #pragma unroll
       for (int i = 0; i < 64; ++i) ov[i] = 0.f;
@@ -664,76 +791,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_attn_tc(const __grid_consta
       *reinterpret_cast<float2*>(stage + (size_t)lrow * kMergeLd + kAttnD) =
           make_float2(have_o ? m_used : -INFINITY, have_o ? l : 0.f);
     }
+    if (CAUSAL) finish();
   }
-  if (threadIdx.x == 128) TL_ATTN(21);
-  // Every thread of the cluster arrives twice, whatever happened before: its
-  // block's rows are staged, and it has pulled (a stage must outlive its readers).
-  cluster_arrive_release();
-  __syncwarp();
-  cluster_wait_acquire();
-  if (threadIdx.x == 128) TL_ATTN(22);
-  {
-    // A warp takes KR owned rows at a time, so that about 16 pulls of a lane are in
-    // flight whatever the split count (one row at a time: 4.4 us from the barrier to
-    // the exit of 6 splits).
-    const int lr0 = (int)((long long)vrows * split / S);
-    const int n_mine = (int)((long long)vrows * (split + 1) / S) - lr0;
-    constexpr int kWarps = kAttnThreads / 32;
-    auto merge = [&](auto kr, auto sm_max) {
-      constexpr int KR = decltype(kr)::value, SM = decltype(sm_max)::value;
-      bool arrived = false;
-      for (int i0 = warp; i0 < n_mine || !arrived; i0 += KR * kWarps) {
-        float2 ml[KR];
-        float4 v[KR][SM];
-#pragma unroll
-        for (int k = 0; k < KR; ++k) {
-          const int i = i0 + k * kWarps;
-          const bool on = i < n_mine;
-          const uint32_t off = (uint32_t)((lr0 + (on ? i : 0)) * kMergeRowBytes);
-          // lane s: (max, sum) of split s; then every split's four values of this lane
-          ml[k] = make_float2(-INFINITY, 0.f);
-          if (on && lane < S) ml[k] = ld_cluster2(dsmem_addr(stage, (uint32_t)lane) + off + kAttnD * 4);
-#pragma unroll
-          for (int s = 0; s < SM; ++s)
-            v[k][s] = on && s < S ? ld_cluster4(dsmem_addr(stage, (uint32_t)s) + off + (uint32_t)lane * 16u)
-                                  : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        float4 acc[KR];
-#pragma unroll
-        for (int k = 0; k < KR; ++k) {
-          const float M = warp_max(ml[k].x);
-          const float w = ml[k].x == -INFINITY ? 0.f : exp2f(ml[k].x - M);
-          const float den = warp_sum(w * ml[k].y);
-          const float wn = den > 0.f ? w / den : 0.f;
-          acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-          for (int s = 0; s < SM; ++s) {
-            const float ws = __shfl_sync(0xffffffffu, wn, s);   // 0 past the splits
-            acc[k].x += ws * v[k][s].x;
-            acc[k].y += ws * v[k][s].y;
-            acc[k].z += ws * v[k][s].z;
-            acc[k].w += ws * v[k][s].w;
-          }
-        }
-        if (i0 + KR * kWarps >= n_mine) {   // the last pull: the barrier need not await this round's stores
-          cluster_arrive_release();
-          arrived = true;
-        }
-#pragma unroll
-        for (int k = 0; k < KR; ++k) {
-          const int i = i0 + k * kWarps;
-          if (i < n_mine) {
-            const int lr = lr0 + i;
-            const size_t grow = (size_t)(node0 + lr / G) * nq + g * G + lr % G;
-            store_act4(a.out, grow * kAttnD + 4 * lane, a.out_lo_off, acc[k]);
-          }
-        }
-      }
-    };
-    if (S <= 5) merge(Int<3>{}, Int<5>{});
-    else if (S <= 8) merge(Int<2>{}, Int<8>{});
-    else merge(Int<1>{}, Int<kMaxSplits>{});
-  }
+  if (!CAUSAL) finish();
   __syncwarp();
   cluster_wait_acquire();
   if (threadIdx.x == 128) {
@@ -797,7 +857,8 @@ static cudaError_t attn_setup_one() {
   cudaError_t e = cudaFuncSetAttribute(k_attn_tc<F16, CAUSAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttnSmem);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_attn_tc<F16, CAUSAL>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  return e;
+  // the register split must not ask for more than the block is launched with
+  return e == cudaSuccess && CAUSAL ? check_launch_regs((const void*)k_attn_tc<F16, CAUSAL>, kPfRegsLaunch) : e;
 }
 
 cudaError_t attn_setup() {
