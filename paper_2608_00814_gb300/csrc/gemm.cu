@@ -48,7 +48,8 @@ namespace oos {
 //               into a per-node running top-2.
 // A prefill chunk too small for the tiles of prefill.cu runs through the same
 // kernels in token tiles (CHUNK) of 128, or 64 for gate/up: the token tiles of a
-// weight tile are separate clusters (or CTAs).
+// weight tile are separate clusters (or CTAs).  So does gate/up of a narrow model's
+// tree of more than 64 nodes.
 //
 // RMSNorm is split across kernels by linearity: a producer stores y = g (.) x
 // and sum(x^2) per feature tile; the consumer GEMM computes W.y and multiplies
@@ -73,11 +74,8 @@ namespace oos {
 //     the 14336 x 4096 shape at T = 128: last accumulator 57 -> 50 us after the start.
 //     Up to 64 tokens HBM is the bound (5.9 TB/s at 12288 x 4096, T = 64) and a pair's
 //     setup costs more than it gives (8B step 4026 -> 4053 us, 0.6B 1277 -> 1304).
+//     A narrow model's gate/up goes in tiles of 64 tokens instead (launch_gemm_gu).
 enum { EPI_QKV = 0, EPI_RESID = 1, EPI_SILU = 2, EPI_ARGMAX = 3 };
-
-// token rows the activation buffers are laid out for; the lo halves follow them
-template <bool CHUNK>
-constexpr int kLdr = CHUNK ? kPfTokens : kMaxT;
 
 // A work tile is SUB weight subtiles that share every staged activation slice:
 // gate and up rows, or 2 x 128 rows of the LM head.
@@ -92,10 +90,11 @@ struct GemmArgs {
   int rows;           // weight rows per subtile
   int n_work, kbt;    // work tiles, k-blocks per tile
   int split;          // CTAs sharing a tile (cluster size)
-  int chain;          // prefill chunks: most k-blocks an accumulator collects (see k_chain)
+  int chain;          // CHUNK: most k-blocks an accumulator collects (see k_chain)
   int stages;         // ring depth
   int N;              // output rows (features / vocab; intermediate rows for EPI_SILU)
   int T;              // valid columns (tree nodes; all token tiles together)
+  int ldr;            // CHUNK: token rows the activation buffers are laid out for (else kMaxT)
   int tl_slot;        // timeline slot (layer * 4 + kind)
   uint32_t* status;
   // RMSNorm scale of the GEMM input (EPI_QKV, EPI_SILU, EPI_ARGMAX)
@@ -121,6 +120,10 @@ struct GemmArgs {
   int32_t* am_i;
   float* am_v2;
 };
+
+// token rows of the activation buffers; the lo halves follow them
+template <bool CHUNK>
+OOS_DEV int ldr(const GemmArgs& a) { return CHUNK ? a.ldr : kMaxT; }
 
 constexpr int kEpiWarps = 8;
 constexpr int kEpiThreads = kEpiWarps * 32;
@@ -201,7 +204,7 @@ OOS_DEV void input_rms(const GemmArgs& a, float* rms, int tok0, int tb, int te, 
     for (int c = l; c < a.ss_chunks; c += 32) {
 #pragma unroll
       for (int k = 0; k < 4; ++k)
-        if (t0 + k < te) s[k] += __ldcg(a.ss_in + (size_t)c * kLdr<CHUNK> + tok0 + t0 + k);
+        if (t0 + k < te) s[k] += __ldcg(a.ss_in + (size_t)c * ldr<CHUNK>(a) + tok0 + t0 + k);
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) s[k] = warp_sum(s[k]);
@@ -273,11 +276,11 @@ OOS_DEV void resid_finish(const GemmArgs& a, const ResidRows& r, const float4 (&
     const float4 xv = f4_add(r.x[k], acc[k]);
     if (live && st) {
       *reinterpret_cast<float4*>(a.x + (size_t)(tok0 + t) * a.N + f) = xv;
-      store_act4(a.y_out, (size_t)(tok0 + t) * a.N + f, (size_t)kLdr<CHUNK> * a.N,
+      store_act4(a.y_out, (size_t)(tok0 + t) * a.N + f, (size_t)ldr<CHUNK>(a) * a.N,
                  make_float4(g.x * xv.x, g.y * xv.y, g.z * xv.z, g.w * xv.w));
     }
     const float sq = warp_sum(live ? xv.x * xv.x + xv.y * xv.y + xv.z * xv.z + xv.w * xv.w : 0.f);
-    if (l == 0 && st) a.ss_out[(size_t)tile * kLdr<CHUNK> + tok0 + t] = sq;
+    if (l == 0 && st) a.ss_out[(size_t)tile * ldr<CHUNK>(a) + tok0 + t] = sq;
   }
 }
 
@@ -331,7 +334,7 @@ OOS_DEV void qkv_finish(const GemmArgs& a, const QkvRows& r, const float4 (&acc)
     if (!st) {
       asm volatile("" ::"f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]));
     } else if (kind == 0) {   // q as hi/lo halves in the cache's 16-bit format: the attention product sees ~16-bit q
-      const size_t qi = ((size_t)(tok0 + t) * a.nq + h) * kTile + 4 * l, lo_off = (size_t)kLdr<CHUNK> * a.nq * kTile;
+      const size_t qi = ((size_t)(tok0 + t) * a.nq + h) * kTile + 4 * l, lo_off = (size_t)ldr<CHUNK>(a) * a.nq * kTile;
       if (a.kv_f16) store_act4_h(reinterpret_cast<__half*>(a.q_out), qi, lo_off, make_float4(v[0], v[1], v[2], v[3]));
       else store_act4(a.q_out, qi, lo_off, make_float4(v[0], v[1], v[2], v[3]));
     } else {           // K/V in the cache's format (bf16, or binary16)
@@ -417,8 +420,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     }
   }
   const int T = CHUNK ? min(a.T - tok0, BN) : a.T;   // tokens of this CTA's tiles
-  // k-segments of a tile: as many as it has accumulators, or, in a prefill chunk, as
-  // the longest chain makes, the accumulators taken in turn
+  // k-segments of a tile: as many as it has accumulators, or (CHUNK) as the longest
+  // chain makes, the accumulators taken in turn
   const int segs = CHUNK ? (nkb + a.chain - 1) / a.chain : nkb < C::SEGS ? 1 : C::SEGS;
 
   if (threadIdx.x == 0) {
@@ -495,7 +498,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         unsigned char* dst = ring_x + stage * C::X_BYTES;
         if (!PAIR || rank == 0) load(dst, &am, stage, kb * kBK, tok0, pol_a);   // hi rows
         if (!PAIR || rank == 1)                                                // lo rows
-          load(PAIR ? dst : dst + C::B_BYTES, &am, stage, kb * kBK, kLdr<CHUNK> + tok0, pol_a);
+          load(PAIR ? dst : dst + C::B_BYTES, &am, stage, kb * kBK, ldr<CHUNK>(a) + tok0, pol_a);
       };
       // weights do not depend on the previous kernel: start streaming them
       // before waiting for it (programmatic dependent launch)
@@ -644,7 +647,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     }
   };
 
-  // Prefill chunks: the k-segments before the last, added up in registers while the
+  // CHUNK: the k-segments before the last, added up in registers while the
   // MMAs of the next run: part[c][sub] is chunk c of this warp.  `use` counts the
   // accumulators taken.  False when a wait gave up.
   auto take_early = [&](float (&part)[C::CHUNKS][kSub][16], uint32_t& use) {
@@ -918,7 +921,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
           if (live && t < T) {
             __nv_bfloat16* dst = a.act_out + (size_t)(tok0 + t) * a.N + fi;
             *reinterpret_cast<__nv_bfloat162*>(dst) = hi;
-            *reinterpret_cast<__nv_bfloat162*>(dst + (size_t)kLdr<CHUNK> * a.N) = lo;
+            *reinterpret_cast<__nv_bfloat162*>(dst + (size_t)ldr<CHUNK>(a) * a.N) = lo;
           }
         }
       }
@@ -1140,7 +1143,7 @@ int gemm_fit(int c) {
   return n;
 }
 
-// k-blocks that one accumulator of a prefill chunk may collect.  The tensor core
+// k-blocks that one accumulator may collect where K goes in segments (CHUNK, prefill.cu).  The tensor core
 // truncates every addition to its accumulator, an error that grows with the chain of
 // MMAs, so K goes in chains no longer than the pieces that an even deal of the matrix's
 // k-blocks over the SMs would cut (8B shape: q/k/v 15, O 11, down 33, gate/up 24; 0.6B:
@@ -1325,6 +1328,18 @@ cudaError_t launch_gemm_gu(Model& m, int layer, int T, cudaStream_t st) {
   GemmArgs a = base_args(m, m.g_gu[layer], T, layer * 4 + 2);
   a.ss_chunks = m.g_o[layer].plan.n_work;
   a.act_out = (__nv_bfloat16*)m.ws.act;
+  // Above 64 tokens, where tiles of 64 tokens x 128 rows fit the SMs at once: chains of
+  // k_chain, where a pair's single accumulator collects all of K (an MLP's error, its
+  // attention off: 2048 x 6144 6.3e-6, of which 5.6e-6 so; trees of 64 5.7e-6), and
+  // twice the CTAs (a layer at T = 65 / 128: 9728 rows 92.0 -> 90.1 / 107.2 -> 101.4 us,
+  // 6144 69.3 -> 67.2 / 82.4 -> 79.9, 3072 52.7 -> 54.3 / 64.1 -> 64.4).
+  const int tiles = a.N / kTile;
+  if (T > 64 && 2 * tiles <= m.num_sms) {
+    a.rows = kTile;
+    a.n_work = tiles;
+    a.ldr = kMaxT;
+    return launch_tc<64, EPI_SILU, true>(m, m.g_gu[layer], m.amap_xn[2], 2 * tiles, a, st);
+  }
   return dispatch_tc<EPI_SILU>(m, m.g_gu[layer], m.amap_xn, T, a, st);
 }
 
@@ -1335,6 +1350,7 @@ static void chunk_args(Model& m, GemmArgs& a, int n_work, int split) {
   a.rows = kTile;
   a.n_work = n_work;
   a.split = split;
+  a.ldr = kPfTokens;
   a.ss_in = m.ws.pf_ss;
   a.ss_chunks = m.cfg.hidden / kTile;
 }

@@ -121,3 +121,34 @@ def test_prefill_attention_is_as_exact_as_that_of_trees(kv):
     case = build_case("mini-bf16", 8, T=4, plant=0, ctx_len=0, cfg_overrides=over, gain_std=0.1, prefill=False)
     n = 900
     assert _kv_error(case, n, n)[1] <= 1.02 * _kv_error(case, 128, n)[1]
+
+
+def test_mlp_of_wide_trees_is_as_exact_as_of_narrow_ones():
+    """One layer whose attention adds nothing: a row's error is that of its MLP, the
+    same for a token in a tree of 64 nodes and in one of 128, which takes other
+    kernels.  With all of K in one accumulator it was 1.1 times as large there."""
+    cfg = dataclasses.replace(workload("mini-bf16").model, hidden=2048, intermediate=6144, n_q_heads=16, n_kv_heads=8,
+                              n_layers=1, vocab=700, init_std=0.02)
+    w = upload_model(SynthModel(cfg, 3))
+    w["layers"][0]["w_o"].zero_()
+    w["layers"][0]["w_down"].mul_(4)
+    model = B.OosModel(cfg, w)
+    case = dataclasses.make_dataclass("C", ["cfg", "cache_native"])(cfg, [(np.zeros((0, 8, 128), np.uint16),) * 2])
+    tok = torch.arange(128, dtype=torch.int32, device="cuda") * 5
+    par = torch.zeros(128, dtype=torch.int32, device="cuda")
+    par[0] = -1
+
+    def norm(x, g):
+        return x * torch.rsqrt((x * x).mean(-1, keepdim=True) + cfg.rms_eps) * g.cpu().double()
+
+    L = w["layers"][0]
+    x = w["embed"][tok[:64].long()].cpu().double()
+    h = norm(x, L["mlp_norm"])
+    g, u = h @ L["w_gate"].cpu().double().T, h @ L["w_up"].cpu().double().T
+    want = norm(x + (g * torch.sigmoid(g) * u) @ L["w_down"].cpu().double().T, w["final_norm"])
+
+    def err(T):
+        o = B.tree_verify(model, gpu_cache(case, T), 0, tok[:T], par[:T], debug=True)
+        return float((o.final_hidden[:64].cpu().double() - want).norm() / want.norm())
+
+    assert err(128) <= 1.02 * err(64)
