@@ -371,8 +371,8 @@ int oos_lm_head_argmax_static(int32_t dtype, int32_t vocab, int32_t hidden_dim, 
  * call; synchronises `stream`. */
 int oos_set_wait_limit(oos_model* m, uint64_t limit_ns, void* stream);
 
-/* Synchronise `stream` and return the device status of the last verify on
- * this handle: OOS_OK, OOS_ETREE or OOS_ETIMEOUT (or OOS_ECUDA). */
+/* Synchronise `stream` and return the device status of the last verify or
+ * prefill (every token of its prompt) on this handle: OOS_OK, OOS_ETREE or OOS_ETIMEOUT (or OOS_ECUDA). */
 int oos_last_status(oos_model* m, void* stream);
 
 /* Static description of a status code. */

@@ -157,9 +157,10 @@ inline cudaError_t check_launch_regs(const void* kernel, int regs) {
 }
 
 // ---- small kernels (small.cu)
-// ctx from the host, or from device memory when ctx_dev is not null
+// ctx from the host, or from device memory when ctx_dev is not null; first: the call's
+// status words are cleared, else kept
 cudaError_t launch_tree_prep(Model& m, const int32_t* tokens, const int32_t* parent, int T, int ctx,
-                             const int32_t* ctx_dev, cudaStream_t st);
+                             const int32_t* ctx_dev, bool first, cudaStream_t st);
 // the tree-prep kernel node of a captured graph, and a new committed length for it
 cudaGraphNode_t find_tree_prep_node(cudaGraph_t g);
 cudaError_t set_tree_prep_ctx(Model& m, cudaGraphExec_t ex, cudaGraphNode_t node, const int32_t* tokens,

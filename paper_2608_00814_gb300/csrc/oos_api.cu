@@ -150,13 +150,14 @@ static unsigned long long kv_hash(const oos_kv_cache* kv) {
 // tree prep, embedding and every decoder layer of a tree on stream st: the
 // K/V of the T nodes land in slots ctx.., the final-norm input in ws.x.  The
 // committed length ctx comes from the host, or from device memory when ctx_dev
-// is not null (then any value up to the cache capacity is allowed).
+// is not null (then any value up to the cache capacity is allowed).  first: not a
+// later chunk of a prompt.
 static int enqueue_layers(Model& m, const oos_kv_cache* kv, int ctx, const int32_t* ctx_dev, const int32_t* tokens,
-                          const int32_t* parent, int T, cudaStream_t st) {
+                          const int32_t* parent, int T, bool first, cudaStream_t st) {
   const auto& c = m.cfg;
   const int ctx_hint = ctx_dev ? kv->capacity - T : ctx;   // sizes the attention's key splits
   const bool tc = c.dtype == OOS_DTYPE_BF16;
-  OOS_TRY(launch_tree_prep(m, tokens, parent, T, ctx, ctx_dev, st));
+  OOS_TRY(launch_tree_prep(m, tokens, parent, T, ctx, ctx_dev, first, st));
   OOS_TRY(tc ? launch_embed_tc(m, tokens, T, st) : launch_f32_embed(m, tokens, T, st));
   // five kernels per layer; every elementwise step runs in a projection
   for (int l = 0; l < c.n_layers; ++l) {
@@ -175,7 +176,7 @@ static int enqueue_verify(Model& m, const oos_kv_cache* kv, int ctx, const int32
                           int32_t* toks, int32_t* bonus, float* hidden, int32_t* dbg_arg, float* dbg_t1,
                           float* dbg_t2, cudaStream_t st) {
   const auto& c = m.cfg;
-  const int rc = enqueue_layers(m, kv, ctx, ctx_dev, tokens, parent, T, st);
+  const int rc = enqueue_layers(m, kv, ctx, ctx_dev, tokens, parent, T, true, st);
   if (rc != OOS_OK) return rc;
   if (c.dtype == OOS_DTYPE_BF16) {
     if (hidden) OOS_TRY(launch_final_hidden(m, hidden, T, st));
@@ -217,7 +218,7 @@ static int prefill_impl(Model& m, const oos_kv_cache* kv, int ctx, const int32_t
       OOS_TRY(prefill_chunk(m, kv, ctx + off, tokens + off, T, off == 0, st));
       if (last) OOS_TRY(prefill_last(m, T, st));
     } else {
-      const int rc = enqueue_layers(m, kv, ctx + off, nullptr, tokens + off, m.ws.chain_parent, T, st);
+      const int rc = enqueue_layers(m, kv, ctx + off, nullptr, tokens + off, m.ws.chain_parent, T, off == 0, st);
       if (rc != OOS_OK) return rc;
     }
     if (!last) continue;

@@ -15,10 +15,12 @@ namespace oos {
 // RoPE position is ctx + depth(i).  Ancestor sets are 128-bit masks.
 // ctx: the committed length, from the host (ctx_in == nullptr) or from device
 // memory; written to ctx_out, where every later kernel of the step reads it.
+// first: the call starts here; a later tree of a prompt adds to the status words that
+// the chunks before it left.
 __global__ void __launch_bounds__(kMaxT) k_tree_prep(const int32_t* __restrict__ tokens,
                                                      const int32_t* __restrict__ parent, int T, int ctx,
                                                      const int32_t* __restrict__ ctx_in, int32_t* ctx_out,
-                                                     int vocab, uint32_t* status, int32_t* depth_out,
+                                                     int first, int vocab, uint32_t* status, int32_t* depth_out,
                                                      int32_t* pos_out, unsigned long long* anc_out) {
   __shared__ int s_parent[kMaxT];
   __shared__ int s_bad;
@@ -37,8 +39,8 @@ __global__ void __launch_bounds__(kMaxT) k_tree_prep(const int32_t* __restrict__
     if (!ok) atomicOr(&s_bad, 1);
   }
   __syncthreads();
-  if (i == 0) *status = s_bad ? ST_TREE : 0u;
-  if (i >= 1 && i < 8) status[i] = 0u;   // where a pipeline wait gave up (see common.cuh)
+  if (i == 0) *status = (first ? 0u : *status) | (s_bad ? ST_TREE : 0u);
+  if (first && i >= 1 && i < 8) status[i] = 0u;   // where a pipeline wait gave up (see common.cuh)
   if (i < T) {
     int d = 0;
     unsigned long long lo = 0, hi = 0;
@@ -65,9 +67,9 @@ __global__ void __launch_bounds__(kMaxT) k_tree_prep(const int32_t* __restrict__
 // complete: later kernels may read cache positions < ctx, and ctx itself,
 // before their own dependency wait.
 cudaError_t launch_tree_prep(Model& m, const int32_t* tokens, const int32_t* parent, int T, int ctx,
-                             const int32_t* ctx_dev, cudaStream_t st) {
+                             const int32_t* ctx_dev, bool first, cudaStream_t st) {
   return launch(false, k_tree_prep, dim3(1), dim3(kMaxT), 0, st, tokens, parent, T, ctx, ctx_dev, m.ws.ctx,
-                m.cfg.vocab, m.ws.status, m.ws.depth, m.ws.pos, m.ws.anc);
+                first ? 1 : 0, m.cfg.vocab, m.ws.status, m.ws.depth, m.ws.pos, m.ws.anc);
 }
 
 cudaGraphNode_t find_tree_prep_node(cudaGraph_t g) {
@@ -90,12 +92,13 @@ cudaError_t set_tree_prep_ctx(Model& m, cudaGraphExec_t ex, cudaGraphNode_t node
                               const int32_t* parent, int T, int ctx) {
   const int32_t* ctx_in = nullptr;
   int32_t* ctx_out = m.ws.ctx;
+  int first = 1;
   int vocab = m.cfg.vocab;
   uint32_t* status = m.ws.status;
   int32_t* depth = m.ws.depth;
   int32_t* pos = m.ws.pos;
   unsigned long long* anc = m.ws.anc;
-  void* args[] = {&tokens, &parent, &T, &ctx, &ctx_in, &ctx_out, &vocab, &status, &depth, &pos, &anc};
+  void* args[] = {&tokens, &parent, &T, &ctx, &ctx_in, &ctx_out, &first, &vocab, &status, &depth, &pos, &anc};
   cudaKernelNodeParams p = {};
   p.func = (void*)k_tree_prep;
   p.gridDim = dim3(1);
