@@ -107,8 +107,10 @@ OOS_DEV void store16_one(void* dst, const float* v) {
   pack16(v, hi, lo);
   store16(dst, hi);
 }
+// norm gains and biases: 8 bytes at a time, the alignment the verify GEMMs ask of them too
 OOS_DEV void load16(const __nv_bfloat16* p, float (&v)[16]) {
-  uint4 u[2] = {__ldg(reinterpret_cast<const uint4*>(p)), __ldg(reinterpret_cast<const uint4*>(p) + 1)};
+  const uint2* q = reinterpret_cast<const uint2*>(p);
+  const uint2 u[4] = {__ldg(q), __ldg(q + 1), __ldg(q + 2), __ldg(q + 3)};
   const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(u);
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
