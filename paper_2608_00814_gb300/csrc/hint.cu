@@ -10,12 +10,16 @@
 // bank order, cut at the lane depth or before an EOS; a lane counts towards
 // the budget only when it creates a node.
 //
-// k_hint_match: for every bank position the longest n whose suffix ends there (0
-// when nothing, or EOS, follows); a warp per 256-position chunk.  What it cannot
-// do without is reading the bank once, so it compares every token with y's last
-// one and looks at a position's neighbours only where that matches; the match
-// lengths (one byte each) are written only for chunks that hold one, the chunk
-// maximum always.
+// k_hint_match: for every 256-position chunk of the bank the longest n whose suffix
+// ends in it (0 when none does before a token that is not EOS) and the set of the
+// positions where it ends; a warp per chunk.  What it cannot do without is reading the
+// bank once, so it compares every token with y's last one and goes on only where
+// that matches.  y's last token may be a common one, in every chunk: the sets are formed
+// by warp votes from the tokens in registers, and only the set of the chunk's own
+// maximum is written (32 bytes; the call's maximum is all that packing asks for).  A
+// bank of 64 M tokens of which 0 / 1 / 5 / 50 % are y's last one takes 56 / 99 / 108 / 126
+// us; with a loop per matching position and a byte per position it took 55 / 111 / 150 /
+// 261.
 // k_hint_pack: one block finds the chunks that hold an occurrence, in bank
 // order -- from the chunk maxima themselves in a bank of up to kHintFlat chunks,
 // through maxima of 256-chunk spans in a larger one -- gathers the occurrences of
@@ -37,15 +41,78 @@ constexpr int kHintWarps = kHintThreads / 32;
 constexpr int kHintFlat = kHintThreads * 16;
 constexpr int kHintUnroll = 4;      // chunks a warp has in flight
 
+// Sets of positions of a chunk: bit l of word [h][k] is position 128 h + 4 l + k, the
+// k-th token of lane l's h-th load.
+struct HintSet {
+  uint32_t w[2][4];
+  OOS_DEV bool any() const {
+    return ((w[0][0] | w[0][1] | w[0][2] | w[0][3]) | (w[1][0] | w[1][1] | w[1][2] | w[1][3])) != 0u;
+  }
+};
+// where the tokens equal t
+OOS_DEV HintSet hint_eq(const int4 (&v)[2], int t) {
+  HintSet s;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    s.w[h][0] = __ballot_sync(0xffffffffu, v[h].x == t);
+    s.w[h][1] = __ballot_sync(0xffffffffu, v[h].y == t);
+    s.w[h][2] = __ballot_sync(0xffffffffu, v[h].z == t);
+    s.w[h][3] = __ballot_sync(0xffffffffu, v[h].w == t);
+  }
+  return s;
+}
+// m without the positions whose J-th token before them is not t.  o: for the 8 tokens
+// ahead of the chunk, in bits 30 and 31 of word k, whether they are t.
+template <int J>
+OOS_DEV HintSet hint_step(const HintSet& m, const int4 (&v)[2], const uint32_t (&o)[4], int t) {
+  const HintSet e = hint_eq(v, t);
+  HintSet r;
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      constexpr int L = 8;   // k - J + L > 0
+      const int at = (k - J + L) & 3, lanes = (L - (k - J + L) + 3) / 4;   // token of the lane that many below
+      const uint32_t x = lanes == 0 ? e.w[h][at] : __funnelshift_l(h ? e.w[0][at] : o[at], e.w[h][at], lanes);
+      r.w[h][k] = m.w[h][k] & x;
+    }
+  return r;
+}
+// The longest suffix: m holds the positions where J tokens match, at least one.  The
+// tokens ahead of the chunk (`ahead`, nullptr where the bank starts) are loaded only
+// where the step would find one if they all matched.
+template <int J>
+OOS_DEV int hint_longest(HintSet& m, const int4 (&v)[2], const int32_t* ahead, const int* suf, int nmax) {
+  if constexpr (J < kHintMaxN) {
+    if (J < nmax) {
+      const uint32_t all[4] = {~0u, ~0u, ~0u, ~0u};
+      HintSet r = hint_step<J>(m, v, all, suf[J]);
+      if (r.any()) {
+        const int lane = threadIdx.x & 31;
+        uint32_t o[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          o[k] = __ballot_sync(0xffffffffu, ahead && lane >= 30 && ahead[(lane - 30) * 4 + k] == suf[J]);
+        r = hint_step<J>(m, v, o, suf[J]);
+        if (r.any()) {
+          m = r;
+          return hint_longest<J + 1>(m, v, ahead, suf, nmax);
+        }
+      }
+    }
+  }
+  return J;
+}
+
 // prefix_len_dev: the prefix length in device memory (the decode loop's
 // committed length), or nullptr to use prefix_len.  Lane l of a chunk's warp holds
 // positions 4l .. 4l+3 of both 128-position halves, so that a 16-byte load of the
 // warp is one contiguous run.  vec: the bank address is 16-byte aligned.
 // smax, best: nullptr in a bank of up to kHintFlat chunks.
-__global__ void __launch_bounds__(kHintThreads) k_hint_match(const int32_t* __restrict__ bank, int N, int eos,
+__global__ void __launch_bounds__(kHintThreads, 3) k_hint_match(const int32_t* __restrict__ bank, int N, int eos,
                                                              const int32_t* __restrict__ prefix, int prefix_len,
                                                              const int32_t* __restrict__ prefix_len_dev, int vec,
-                                                             uint8_t* __restrict__ mlen, uint8_t* __restrict__ cmax,
+                                                             uint32_t* __restrict__ sets, uint8_t* __restrict__ cmax,
                                                              int* __restrict__ smax, int* __restrict__ best) {
   __shared__ int suf[kHintMaxN];
   pdl_wait();   // the committed tokens and their count may come from the previous kernel
@@ -62,8 +129,6 @@ __global__ void __launch_bounds__(kHintThreads) k_hint_match(const int32_t* __re
   int wbest = 0;
   for (long long c0 = (long long)blockIdx.x * kHintWarps + (threadIdx.x >> 5); c0 < n_chunks;
        c0 += n_warps * kHintUnroll) {
-    // bit i: the lane's token i equals y's last one (positions past the bank never do)
-    uint32_t hits[kHintUnroll];
     int4 v[kHintUnroll][2];
 #pragma unroll
     for (int u = 0; u < kHintUnroll; ++u) {
@@ -74,52 +139,60 @@ __global__ void __launch_bounds__(kHintThreads) k_hint_match(const int32_t* __re
         v[u][1] = __ldcs(src + 32);
       }
     }
+    uint32_t some = 0u;       // chunks that hold y's last token
 #pragma unroll
     for (int u = 0; u < kHintUnroll; ++u) {
-      const long long c = c0 + u * n_warps;
-      hits[u] = 0u;
-      if (vec && (c + 1) * kHintThreads <= N) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-          hits[u] |= ((v[u][h].x == last ? 1u : 0u) | (v[u][h].y == last ? 2u : 0u) | (v[u][h].z == last ? 4u : 0u) |
-                      (v[u][h].w == last ? 8u : 0u))
-                     << (4 * h);
-      } else {
+      const long long c = c0 + u * n_warps, p0 = c * kHintThreads;
+      if (!vec || p0 + kHintThreads > N) {
+        int t[8];   // past the bank: EOS, as if that followed its last token
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-          const long long p = c * kHintThreads + (i >> 2) * 128 + lane * 4 + (i & 3);
-          if (p < N && bank[p] == last) hits[u] |= 1u << i;
+          const long long p = p0 + (i >> 2) * 128 + lane * 4 + (i & 3);
+          t[i] = p < N ? bank[p] : eos;
         }
+        v[u][0] = make_int4(t[0], t[1], t[2], t[3]);
+        v[u][1] = make_int4(t[4], t[5], t[6], t[7]);
       }
+      bool hit = false;
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        hit = hit || v[u][h].x == last || v[u][h].y == last || v[u][h].z == last || v[u][h].w == last;
+      if (c < n_chunks && __any_sync(0xffffffffu, hit)) some |= 1u << u;
     }
-#pragma unroll 1
+#pragma unroll
     for (int u = 0; u < kHintUnroll; ++u) {
       const long long c = c0 + u * n_warps;
       if (c >= n_chunks) break;
-      uint32_t h = hits[0];   // a rotating window: no indexed registers
-#pragma unroll
-      for (int k = 0; k + 1 < kHintUnroll; ++k) hits[k] = hits[k + 1];
       int lmax = 0;
-      if (__any_sync(0xffffffffu, h != 0u)) {
-        uint32_t packed[2] = {0u, 0u};
-        while (h) {
-          const int i = __ffs(h) - 1;
-          h &= h - 1;
-          const long long p = c * kHintThreads + (i >> 2) * 128 + lane * 4 + (i & 3);
-          // the next bank token must exist and not be EOS
-          if (p + 1 >= N || bank[p + 1] == eos) continue;
-          int m = 1;
-          while (m < nmax && p - m >= 0 && bank[p - m] == suf[m]) ++m;
-          if (i < 4) packed[0] |= (uint32_t)m << (8 * i);
-          else packed[1] |= (uint32_t)m << (8 * (i - 4));
-          lmax = m > lmax ? m : lmax;
-        }
+      if (some >> u & 1u) {
+        HintSet m = hint_eq(v[u], last);
+        // a match counts unless EOS, or nothing, follows: the set of the next tokens' EOS
+        const HintSet f = hint_eq(v[u], eos);
+        bool after = false;   // after the chunk's last position, asked for only where that one matches
+        if (m.w[1][3] >> 31) after = (c + 1) * kHintThreads >= N || bank[(c + 1) * kHintThreads] == eos;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) lmax = max(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
-        if (lmax > 0) {
-          uint32_t* dst = reinterpret_cast<uint32_t*>(mlen + c * kHintThreads) + lane;
-          dst[0] = packed[0];
-          dst[32] = packed[1];
+        for (int h = 0; h < 2; ++h) {
+#pragma unroll
+          for (int k = 0; k < 3; ++k) m.w[h][k] &= ~f.w[h][k + 1];
+          m.w[h][3] &= ~__funnelshift_r(f.w[h][0], h ? (after ? 1u : 0u) : f.w[1][0], 1);
+        }
+        // a token past the bank is not one of it
+        const long long left = N - c * kHintThreads;
+        if (left < kHintThreads) {
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const int n = ((int)left - 128 * h - k + 3) / 4;   // lanes whose k-th token is
+              m.w[h][k] &= n <= 0 ? 0u : n >= 32 ? ~0u : (1u << n) - 1u;
+            }
+        }
+        if (m.any()) {
+          lmax = hint_longest<1>(m, v[u], c > 0 ? bank + c * kHintThreads - 8 : nullptr, suf, nmax);
+          uint32_t mine = m.w[0][0];
+#pragma unroll
+          for (int i = 1; i < 8; ++i) mine = lane == i ? m.w[i >> 2][i & 3] : mine;
+          if (lane < 8) sets[c * 8 + lane] = mine;
         }
       }
       if (lane == 0) {
@@ -210,7 +283,7 @@ OOS_DEV bool hint_insert(HintTree& tr, int& T, int max_nodes, const int32_t* lan
 
 __global__ void __launch_bounds__(kHintThreads) k_hint_pack(const int32_t* __restrict__ bank, int N, int eos,
                                                             const int32_t* __restrict__ prefix, int prefix_len,
-                                                            const uint8_t* __restrict__ mlen,
+                                                            const uint32_t* __restrict__ sets,
                                                             const uint8_t* __restrict__ cmax,
                                                             const int* __restrict__ smax,
                                                             const int* __restrict__ best,
@@ -261,17 +334,19 @@ __global__ void __launch_bounds__(kHintThreads) k_hint_pack(const int32_t* __res
   }
   const int n_chunks = (int)(((long long)N + kHintThreads - 1) / kHintThreads);
 
-  // the lanes of the occurrences (match length >= n) in the nc chunks of s_chunk
-  auto visit = [&](int nc, int n) {
+  // the lanes of the occurrences in the nc chunks of s_chunk
+  auto visit = [&](int nc) {
     for (int ci = 0; ci < nc && !s_done; ci += kHintWarps) {
       // one chunk per warp, 8 positions per lane
       const int c = ci + warp < nc ? s_chunk[ci + warp] : -1;
-      uint2 m = make_uint2(0u, 0u);
-      if (c >= 0) m = reinterpret_cast<const uint2*>(mlen + (size_t)c * kHintThreads)[lane_id];
+      uint4 m = make_uint4(0u, 0u, 0u, 0u);
+      if (c >= 0) m = reinterpret_cast<const uint4*>(sets + (size_t)c * 8)[lane_id >> 4];
       uint32_t hit = 0u;
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
-        if ((int)(((i < 4 ? m.x : m.y) >> (8 * (i & 3))) & 255u) >= n) hit |= 1u << i;
+      for (int i = 0; i < 8; ++i) {
+        const uint32_t w = (i & 3) == 0 ? m.x : (i & 3) == 1 ? m.y : (i & 3) == 2 ? m.z : m.w;
+        hit |= (w >> (2 * (lane_id & 15) + (i >> 2)) & 1u) << i;
+      }
       const int mine = c >= 0 ? __popc(hit) : 0;
       int upto = mine;   // hits of lanes 0 .. lane_id
 #pragma unroll
@@ -362,7 +437,7 @@ __global__ void __launch_bounds__(kHintThreads) k_hint_pack(const int32_t* __res
       for (int i = 0; i < 16; ++i)
         if (mx[i] >= n) s_chunk[off++] = b0 + i;
       __syncthreads();
-      visit(nc, n);
+      visit(nc);
     }
   } else {
     n = *best;
@@ -374,7 +449,7 @@ __global__ void __launch_bounds__(kHintThreads) k_hint_pack(const int32_t* __res
       for (int si = 0; si < ns && !s_done; ++si) {
         const int c = s_span[si] * kHintThreads + threadIdx.x;
         const int nc = ordered_select(c < n_chunks && cmax[c] >= n, c, s_chunk, s_wcnt, &s_nc);
-        visit(nc, n);
+        visit(nc);
       }
     }
   }
@@ -410,7 +485,8 @@ __global__ void __launch_bounds__(kHintThreads) k_hint_pack(const int32_t* __res
 }
 
 // Workspace: the call's n (best) and the span maxima first, so that one
-// zeroing copy covers both; then one match byte per position and the chunk maxima.
+// zeroing copy covers both; then the chunks' sets (32 bytes each; a byte per position is
+// reserved) and the chunk maxima.
 static size_t hint_head_bytes(size_t spans) { return (4 + spans * 4 + 255) / 256 * 256; }
 
 size_t hint_workspace_bytes(long long bank_len) {
@@ -428,8 +504,8 @@ cudaError_t launch_hint_tree(const int32_t* bank, int N, int eos, const int32_t*
   const long long n_spans = (n_chunks + kHintThreads - 1) / kHintThreads;
   int* best = (int*)ws;
   int* smax = best + 1;
-  uint8_t* mlen = (uint8_t*)ws + hint_head_bytes((size_t)n_spans);
-  uint8_t* cmax = mlen + n_chunks * kHintThreads;
+  uint32_t* sets = (uint32_t*)((uint8_t*)ws + hint_head_bytes((size_t)n_spans));
+  uint8_t* cmax = (uint8_t*)sets + n_chunks * kHintThreads;
   cudaError_t e = cudaSuccess;
   if (n_chunks <= kHintFlat) {
     best = smax = nullptr;
@@ -447,10 +523,10 @@ cudaError_t launch_hint_tree(const int32_t* bank, int N, int eos, const int32_t*
   // the packing block launches while the match kernel runs (programmatic
   // dependent launch) and waits for it before reading its results
   e = launch(true, k_hint_match, dim3(grid), dim3(kHintThreads), 0, st, bank, N, eos, prefix, prefix_len,
-             prefix_len_dev, vec, mlen, cmax, smax, best);
+             prefix_len_dev, vec, sets, cmax, smax, best);
   if (e != cudaSuccess) return e;
   return launch(true, k_hint_pack, dim3(1), dim3(kHintThreads), 0, st, bank, N, eos, prefix, prefix_len,
-                (const uint8_t*)mlen, (const uint8_t*)cmax, (const int*)smax, (const int*)best, native, native_len,
+                (const uint32_t*)sets, (const uint8_t*)cmax, (const int*)smax, (const int*)best, native, native_len,
                 n_native, native_stride, max_lanes, depth, max_nodes, prefix_len_dev, pad_to, out_tok, out_par, out_T,
                 out_info);
 }
