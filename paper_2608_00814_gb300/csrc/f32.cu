@@ -3,8 +3,11 @@
 // A step of such a model is bound by launch and load latency, not by bytes (6 MB
 // for the 2-layer, 256-wide decoder), so the kernels are few -- five per layer, the
 // elementwise steps in the projections -- and every one forms all the dot products
-// it can from one round of loads: a warp takes R weight rows and 8 tokens at a
-// time, the lanes split the reduction, and the 8 R sums are reduced together.
+// it can from one round of loads: a warp takes R weight rows and TOK tokens at a
+// time, the lanes split the reduction, and the R TOK sums are reduced together.
+// TOK is 8, or 4, 2 or 1 for a tree that has no more nodes: a wide model's weights
+// would otherwise wait for arithmetic that nobody reads (2 layers of the
+// 2048-wide shape at T = 1 / 2 / 8: 671 / 624 / 370 us with 8 always, 208 / 239 / 322 so).
 // RMSNorm needs no kernel of its own: a projection reads the whole input rows, so
 // it sums their squares alongside and scales its products by the row's factor.
 // The 2-layer decoder's step (T = 8, 128 cached positions): 176 us with a kernel
@@ -16,7 +19,7 @@
 
 namespace oos {
 
-constexpr int kF32Tok = 8;        // tokens a warp takes at a time
+constexpr int kF32Tok = 8;        // most tokens a warp takes at a time
 constexpr int kF32Warps = 4;      // warps per block, but for the q/k/v projection
 
 // V consecutive floats (V = 4: from a 16-byte boundary)
@@ -36,31 +39,35 @@ struct F32Vec {
   }
 };
 
-// Number of values a call of f32_dots leaves in buf: R rows x 8 tokens, then the 8
-// sums of squares when NORM.
-template <int R, bool NORM>
-constexpr int kDots = R * kF32Tok + (NORM ? kF32Tok : 0);
+// Number of values a call of f32_dots leaves in buf: R rows x TOK tokens, then the
+// TOK sums of squares when NORM.
+template <int R, bool NORM, int TOK>
+constexpr int kDots = R * TOK + (NORM ? TOK : 0);
 
-// buf[r * 8 + t] = w[r] . (gain (.) x[t]), buf[R * 8 + t] = |x[t]|^2, by one warp.
-// x: nt <= 8 rows of K floats; plain loads, since the previous kernel wrote them.
-template <int R, int V, bool NORM>
-OOS_DEV void f32_dots(const float* const (&w)[R], const float* x, const float* __restrict__ gain, int K, int nt,
-                      float* buf) {
+// buf[r * TOK + t] = w[r] . (gain (.) x[t]), buf[R * TOK + t] = |x[t]|^2, by one warp.
+// x: nt <= TOK rows of K floats, FULL: TOK of them; plain loads, since the previous
+// kernel wrote them.
+template <int R, int V, bool NORM, int TOK, bool FULL>
+OOS_DEV void f32_dots_of(const float* const (&w)[R], const float* x, const float* __restrict__ gain, int K, int nt,
+                         float* buf) {
   const int lane = threadIdx.x & 31;
-  float acc[kDots<R, NORM>];
+  float acc[kDots<R, NORM, TOK>];
 #pragma unroll
-  for (int i = 0; i < kDots<R, NORM>; ++i) acc[i] = 0.f;
-#pragma unroll 2
+  for (int i = 0; i < kDots<R, NORM, TOK>; ++i) acc[i] = 0.f;
+#pragma unroll(TOK <= 2 ? 16 / (TOK * V) : 2)
   for (int k = lane * V; k < K; k += 32 * V) {
     F32Vec<V> wv[R], g;
 #pragma unroll
     for (int r = 0; r < R; ++r) wv[r].load(w[r] + k);
     if (NORM) g.load(gain + k);
 #pragma unroll
-    for (int t = 0; t < kF32Tok; ++t) {
-      const float* p = x + (size_t)min(t, nt - 1) * K + k;
+    for (int t = 0; t < TOK; ++t) {
+      const float* p = x + (size_t)t * K + k;
       float xv[V];
-      if (V == 4) {
+      if (!FULL && t >= nt) {
+#pragma unroll
+        for (int c = 0; c < V; ++c) xv[c] = 0.f;
+      } else if (V == 4) {
         const float4 u = __ldcg(reinterpret_cast<const float4*>(p));
         xv[0] = u.x;
         xv[V > 1 ? 1 : 0] = u.y;
@@ -73,17 +80,24 @@ OOS_DEV void f32_dots(const float* const (&w)[R], const float* x, const float* _
       for (int c = 0; c < V; ++c) {
         const float xg = NORM ? xv[c] * g.v[c] : xv[c];
 #pragma unroll
-        for (int r = 0; r < R; ++r) acc[r * kF32Tok + t] = fmaf(wv[r].v[c], xg, acc[r * kF32Tok + t]);
-        if (NORM) acc[R * kF32Tok + t] = fmaf(xv[c], xv[c], acc[R * kF32Tok + t]);
+        for (int r = 0; r < R; ++r) acc[r * TOK + t] = fmaf(wv[r].v[c], xg, acc[r * TOK + t]);
+        if (NORM) acc[R * TOK + t] = fmaf(xv[c], xv[c], acc[R * TOK + t]);
       }
     }
   }
   int base, n;
   warp_sums(acc, base, n);
 #pragma unroll
-  for (int i = 0; i < kDots<R, NORM>; ++i)
+  for (int i = 0; i < kDots<R, NORM, TOK>; ++i)
     if (i < n) buf[base + i] = acc[i];
   __syncwarp();
+}
+
+template <int R, int V, bool NORM, int TOK>
+OOS_DEV void f32_dots(const float* const (&w)[R], const float* x, const float* __restrict__ gain, int K, int nt,
+                      float* buf) {
+  if (nt == TOK) f32_dots_of<R, V, NORM, TOK, true>(w, x, gain, K, nt, buf);
+  else f32_dots_of<R, V, NORM, TOK, false>(w, x, gain, K, nt, buf);
 }
 
 // ------------------------------------------------------------ embedding, rotary table
@@ -109,7 +123,7 @@ __global__ void __launch_bounds__(256) k_f32_embed(const int32_t* __restrict__ t
 }
 
 // ------------------------------------------------------------ q/k/v
-// Block (head slot, token group): the d rows of one q, k or v head for 8 tokens,
+// Block (head slot, token group): the d rows of one q, k or v head for TOK tokens,
 // kQkvWarps warps of 4 rows at a time; then a warp per token: bias, q/k RMSNorm,
 // RoPE; q to the query buffer, k and v to cache slots *ctx + t (skipped when the
 // cache pointers are null).
@@ -124,14 +138,14 @@ struct F32QkvArgs {
   float eps;
 };
 
-template <int V>
+template <int V, int TOK>
 __global__ void __launch_bounds__(32 * kQkvWarps) k_f32_qkv(F32QkvArgs a) {
-  __shared__ float s_out[kF32Tok][128];
-  __shared__ float s_buf[kQkvWarps][kDots<4, true>];
+  __shared__ float s_out[TOK][128];
+  __shared__ float s_buf[kQkvWarps][kDots<4, true, TOK>];
   pdl_wait();
   pdl_trigger();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int hs = blockIdx.x, t0 = blockIdx.y * kF32Tok, nt = min(kF32Tok, a.T - t0);
+  const int hs = blockIdx.x, t0 = blockIdx.y * TOK, nt = min(TOK, a.T - t0);
   const int kind = hs < a.nq ? 0 : hs < a.nq + a.nkv ? 1 : 2;
   const int h = kind == 0 ? hs : kind == 1 ? hs - a.nq : hs - a.nq - a.nkv;
   const float* W = (kind == 0 ? a.wq : kind == 1 ? a.wk : a.wv) + (size_t)h * a.d * a.H;
@@ -139,11 +153,11 @@ __global__ void __launch_bounds__(32 * kQkvWarps) k_f32_qkv(F32QkvArgs a) {
     const float* w[4];
 #pragma unroll
     for (int r = 0; r < 4; ++r) w[r] = W + (size_t)min(r0 + r, a.d - 1) * a.H;
-    f32_dots<4, V, true>(w, a.x + (size_t)t0 * a.H, a.gain, a.H, nt, s_buf[warp]);
+    f32_dots<4, V, true, TOK>(w, a.x + (size_t)t0 * a.H, a.gain, a.H, nt, s_buf[warp]);
     // lane = (row, token)
-    const int r = lane >> 3, t = lane & 7;
-    if (r0 + r < a.d)
-      s_out[t][r0 + r] = s_buf[warp][lane] * rsqrtf(s_buf[warp][4 * kF32Tok + t] / (float)a.H + a.eps);
+    const int r = lane / TOK, t = lane % TOK;
+    if (r < 4 && r0 + r < a.d)
+      s_out[t][r0 + r] = s_buf[warp][lane] * rsqrtf(s_buf[warp][4 * TOK + t] / (float)a.H + a.eps);
     __syncwarp();
   }
   __syncthreads();
@@ -269,40 +283,40 @@ __global__ void __launch_bounds__(kF32Keys) k_f32_attn(const float* __restrict__
 }
 
 // ------------------------------------------------------------ O and down: x[t][f] += W[f] . in[t]
-// a warp per output row and 8 tokens
-template <int V>
+// a warp per output row and TOK tokens
+template <int V, int TOK>
 __global__ void __launch_bounds__(32 * kF32Warps) k_f32_resid(const float* __restrict__ W, int N, int K, const float* in,
                                                               int T, float* x) {
-  __shared__ float s_buf[kF32Warps][kDots<1, false>];
+  __shared__ float s_buf[kF32Warps][kDots<1, false, TOK>];
   pdl_wait();
   pdl_trigger();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int f = blockIdx.x * kF32Warps + warp, t0 = blockIdx.y * kF32Tok, nt = min(kF32Tok, T - t0);
+  const int f = blockIdx.x * kF32Warps + warp, t0 = blockIdx.y * TOK, nt = min(TOK, T - t0);
   if (f >= N) return;
   const float* w[1] = {W + (size_t)f * K};
   const float old = lane < nt ? __ldcg(x + (size_t)(t0 + lane) * N + f) : 0.f;
-  f32_dots<1, V, false>(w, in + (size_t)t0 * K, nullptr, K, nt, s_buf[warp]);
+  f32_dots<1, V, false, TOK>(w, in + (size_t)t0 * K, nullptr, K, nt, s_buf[warp]);
   if (lane < nt) x[(size_t)(t0 + lane) * N + f] = old + s_buf[warp][lane];
 }
 
 // ------------------------------------------------------------ gate/up: act = silu(gate) * up
-// a warp per intermediate row (its gate and its up row) and 8 tokens
-template <int V>
+// a warp per intermediate row (its gate and its up row) and TOK tokens
+template <int V, int TOK>
 __global__ void __launch_bounds__(32 * kF32Warps) k_f32_gu(const float* __restrict__ Wg, const float* __restrict__ Wu, int I,
                                                            int K, const float* x, const float* __restrict__ gain, float eps,
                                                            int T, float* __restrict__ act) {
-  __shared__ float s_buf[kF32Warps][kDots<2, true>];
+  __shared__ float s_buf[kF32Warps][kDots<2, true, TOK>];
   pdl_wait();
   pdl_trigger();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i = blockIdx.x * kF32Warps + warp, t0 = blockIdx.y * kF32Tok, nt = min(kF32Tok, T - t0);
+  const int i = blockIdx.x * kF32Warps + warp, t0 = blockIdx.y * TOK, nt = min(TOK, T - t0);
   if (i >= I) return;
   const float* w[2] = {Wg + (size_t)i * K, Wu + (size_t)i * K};
   float* b = s_buf[warp];
-  f32_dots<2, V, true>(w, x + (size_t)t0 * K, gain, K, nt, b);
+  f32_dots<2, V, true, TOK>(w, x + (size_t)t0 * K, gain, K, nt, b);
   if (lane < nt) {
-    const float r = rsqrtf(b[2 * kF32Tok + lane] / (float)K + eps);
-    const float g = b[lane] * r, u = b[kF32Tok + lane] * r;
+    const float r = rsqrtf(b[2 * TOK + lane] / (float)K + eps);
+    const float g = b[lane] * r, u = b[TOK + lane] * r;
     act[(size_t)(t0 + lane) * I + i] = g / (1.f + expf(-g)) * u;
   }
 }
@@ -310,13 +324,13 @@ __global__ void __launch_bounds__(32 * kF32Warps) k_f32_gu(const float* __restri
 // ------------------------------------------------------------ LM head
 // Block b scans vocabulary rows [b*rows, (b+1)*rows), four rows of a warp at a time;
 // each warp keeps a running top-2 per node, merged at the end.
-template <int V>
+template <int V, int TOK>
 __global__ void __launch_bounds__(32 * kF32Warps) k_f32_lm_head(const float* __restrict__ W, int vocab, int H,
                                                                 int rows_per_block, const float* x,
                                                                 const float* __restrict__ gain, float eps, int T,
                                                                 float* am_v1, int32_t* am_i, float* am_v2) {
   __shared__ Top2 st[kF32Warps][kMaxT];
-  __shared__ float s_buf[kF32Warps][kDots<4, true>];
+  __shared__ float s_buf[kF32Warps][kDots<4, true, TOK>];
   pdl_wait();
   pdl_trigger();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -329,14 +343,14 @@ __global__ void __launch_bounds__(32 * kF32Warps) k_f32_lm_head(const float* __r
     const float* w[4];
 #pragma unroll
     for (int r = 0; r < 4; ++r) w[r] = W + (size_t)min(r0 + r, r_end - 1) * H;
-    for (int t0 = 0; t0 < T; t0 += kF32Tok) {
-      const int nt = min(kF32Tok, T - t0);
-      f32_dots<4, V, true>(w, x + (size_t)t0 * H, gain, H, nt, b);
+    for (int t0 = 0; t0 < T; t0 += TOK) {
+      const int nt = min(TOK, T - t0);
+      f32_dots<4, V, true, TOK>(w, x + (size_t)t0 * H, gain, H, nt, b);
       if (lane < nt) {
-        const float rt = rsqrtf(b[4 * kF32Tok + lane] / (float)H + eps);
+        const float rt = rsqrtf(b[4 * TOK + lane] / (float)H + eps);
         Top2 s = st[warp][t0 + lane];
         for (int r = 0; r < 4 && r0 + r < r_end; ++r)
-          s = top2_merge(s, Top2{b[r * kF32Tok + lane] * rt, r0 + r, -INFINITY});
+          s = top2_merge(s, Top2{b[r * TOK + lane] * rt, r0 + r, -INFINITY});
         st[warp][t0 + lane] = s;
       }
       __syncwarp();
@@ -372,7 +386,22 @@ static const float* fp(const void* p) { return (const float*)p; }
 static bool rows16(int K, const void* a, const void* b = nullptr, const void* c = nullptr, const void* d = nullptr) {
   return K % 4 == 0 && (((uintptr_t)a | (uintptr_t)b | (uintptr_t)c | (uintptr_t)d) & 15) == 0;
 }
-static int tok_groups(int T) { return (T + kF32Tok - 1) / kF32Tok; }
+template <int N>
+struct Tok {
+  static constexpr int value = N;
+};
+// f(tokens a warp takes) for a tree of T nodes
+template <typename F>
+static cudaError_t by_tokens(int T, F f) {
+  if (T == 1) return f(Tok<1>{});
+  if (T == 2) return f(Tok<2>{});
+  return T <= 4 ? f(Tok<4>{}) : f(Tok<kF32Tok>{});
+}
+// f(floats a load, tokens a warp takes)
+template <typename F>
+static cudaError_t by_form(bool rows_16, int T, F f) {
+  return by_tokens(T, [&](auto tok) { return rows_16 ? f(Tok<4>{}, tok) : f(Tok<1>{}, tok); });
+}
 
 cudaError_t launch_f32_embed(Model& m, const int32_t* tokens, int T, cudaStream_t st) {
   const auto& c = m.cfg;
@@ -405,10 +434,11 @@ cudaError_t launch_f32_qkv(Model& m, int layer, void* kc, void* vc, int T, cudaS
   a.d = c.head_dim;
   a.T = T;
   a.eps = c.rms_eps;
-  const dim3 grid(c.n_q_heads + 2 * c.n_kv_heads, tok_groups(T));
-  if (rows16(c.hidden, L.w_q, L.w_k, L.w_v, L.attn_norm))
-    return launch(m.pdl, k_f32_qkv<4>, grid, dim3(32 * kQkvWarps), 0, st, a);
-  return launch(m.pdl, k_f32_qkv<1>, grid, dim3(32 * kQkvWarps), 0, st, a);
+  return by_form(rows16(c.hidden, L.w_q, L.w_k, L.w_v, L.attn_norm), T, [&](auto v, auto tok) {
+    constexpr int V = decltype(v)::value, TOK = decltype(tok)::value;
+    return launch(m.pdl, k_f32_qkv<V, TOK>, dim3(c.n_q_heads + 2 * c.n_kv_heads, (T + TOK - 1) / TOK),
+                  dim3(32 * kQkvWarps), 0, st, a);
+  });
 }
 
 cudaError_t launch_f32_attention(Model& m, const void* kc, const void* vc, int T, cudaStream_t st) {
@@ -421,9 +451,11 @@ cudaError_t launch_f32_attention(Model& m, const void* kc, const void* vc, int T
 
 static cudaError_t launch_f32_resid(Model& m, const void* W, int K, const void* in, int T, cudaStream_t st) {
   const int H = m.cfg.hidden;
-  const dim3 grid((H + kF32Warps - 1) / kF32Warps, tok_groups(T));
-  if (rows16(K, W)) return launch(m.pdl, k_f32_resid<4>, grid, dim3(32 * kF32Warps), 0, st, fp(W), H, K, fp(in), T, m.ws.x);
-  return launch(m.pdl, k_f32_resid<1>, grid, dim3(32 * kF32Warps), 0, st, fp(W), H, K, fp(in), T, m.ws.x);
+  return by_form(rows16(K, W), T, [&](auto v, auto tok) {
+    constexpr int V = decltype(v)::value, TOK = decltype(tok)::value;
+    return launch(m.pdl, k_f32_resid<V, TOK>, dim3((H + kF32Warps - 1) / kF32Warps, (T + TOK - 1) / TOK),
+                  dim3(32 * kF32Warps), 0, st, fp(W), H, K, fp(in), T, m.ws.x);
+  });
 }
 cudaError_t launch_f32_o(Model& m, int layer, int T, cudaStream_t st) {
   return launch_f32_resid(m, m.layers[layer].w_o, m.cfg.n_q_heads * m.cfg.head_dim, m.ws.attn, T, st);
@@ -435,22 +467,23 @@ cudaError_t launch_f32_down(Model& m, int layer, int T, cudaStream_t st) {
 cudaError_t launch_f32_gu(Model& m, int layer, int T, cudaStream_t st) {
   const auto& c = m.cfg;
   const oos_layer_weights& L = m.layers[layer];
-  const dim3 grid((c.intermediate + kF32Warps - 1) / kF32Warps, tok_groups(T));
-  if (rows16(c.hidden, L.w_gate, L.w_up, L.mlp_norm))
-    return launch(m.pdl, k_f32_gu<4>, grid, dim3(32 * kF32Warps), 0, st, fp(L.w_gate), fp(L.w_up), c.intermediate, c.hidden,
-                  (const float*)m.ws.x, fp(L.mlp_norm), c.rms_eps, T, (float*)m.ws.act);
-  return launch(m.pdl, k_f32_gu<1>, grid, dim3(32 * kF32Warps), 0, st, fp(L.w_gate), fp(L.w_up), c.intermediate, c.hidden,
-                (const float*)m.ws.x, fp(L.mlp_norm), c.rms_eps, T, (float*)m.ws.act);
+  return by_form(rows16(c.hidden, L.w_gate, L.w_up, L.mlp_norm), T, [&](auto v, auto tok) {
+    constexpr int V = decltype(v)::value, TOK = decltype(tok)::value;
+    return launch(m.pdl, k_f32_gu<V, TOK>, dim3((c.intermediate + kF32Warps - 1) / kF32Warps, (T + TOK - 1) / TOK),
+                  dim3(32 * kF32Warps), 0, st, fp(L.w_gate), fp(L.w_up), c.intermediate, c.hidden, (const float*)m.ws.x,
+                  fp(L.mlp_norm), c.rms_eps, T, (float*)m.ws.act);
+  });
 }
 
 cudaError_t launch_f32_lm_head(Model& m, int T, cudaStream_t st) {
   const auto& c = m.cfg;
   const int rows = (c.vocab + m.lm_grid - 1) / m.lm_grid;
-  if (rows16(c.hidden, m.w.lm_head, m.w.final_norm))
-    return launch(m.pdl, k_f32_lm_head<4>, dim3(m.lm_grid), dim3(32 * kF32Warps), 0, st, fp(m.w.lm_head), c.vocab, c.hidden,
-                  rows, (const float*)m.ws.x, fp(m.w.final_norm), c.rms_eps, T, m.ws.lm_v1, m.ws.lm_i, m.ws.lm_v2);
-  return launch(m.pdl, k_f32_lm_head<1>, dim3(m.lm_grid), dim3(32 * kF32Warps), 0, st, fp(m.w.lm_head), c.vocab, c.hidden,
-                rows, (const float*)m.ws.x, fp(m.w.final_norm), c.rms_eps, T, m.ws.lm_v1, m.ws.lm_i, m.ws.lm_v2);
+  return by_form(rows16(c.hidden, m.w.lm_head, m.w.final_norm), T, [&](auto v, auto tok) {
+    constexpr int V = decltype(v)::value, TOK = decltype(tok)::value;
+    return launch(m.pdl, k_f32_lm_head<V, TOK>, dim3(m.lm_grid), dim3(32 * kF32Warps), 0, st, fp(m.w.lm_head), c.vocab,
+                  c.hidden, rows, (const float*)m.ws.x, fp(m.w.final_norm), c.rms_eps, T, m.ws.lm_v1, m.ws.lm_i,
+                  m.ws.lm_v2);
+  });
 }
 
 cudaError_t launch_f32_hidden(Model& m, float* hidden, int T, cudaStream_t st) {

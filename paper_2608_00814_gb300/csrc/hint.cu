@@ -78,30 +78,38 @@ OOS_DEV HintSet hint_step(const HintSet& m, const int4 (&v)[2], const uint32_t (
     }
   return r;
 }
-// The longest suffix: m holds the positions where J tokens match, at least one.  The
-// tokens ahead of the chunk (`ahead`, nullptr where the bank starts) are loaded only
-// where the step would find one if they all matched.
+// The longest suffix from J tokens on: m holds the positions where J match, at least
+// one.  before: the 8 tokens ahead of the chunk in lanes 30 and 31 (`is`: where there are).
 template <int J>
-OOS_DEV int hint_longest(HintSet& m, const int4 (&v)[2], const int32_t* ahead, const int* suf, int nmax) {
+OOS_DEV int hint_longer(HintSet& m, const int4 (&v)[2], int4 before, bool is, const int* suf, int nmax) {
   if constexpr (J < kHintMaxN) {
     if (J < nmax) {
-      const uint32_t all[4] = {~0u, ~0u, ~0u, ~0u};
-      HintSet r = hint_step<J>(m, v, all, suf[J]);
+      const int t = suf[J];
+      const uint32_t o[4] = {__ballot_sync(0xffffffffu, is && before.x == t), __ballot_sync(0xffffffffu, is && before.y == t),
+                             __ballot_sync(0xffffffffu, is && before.z == t), __ballot_sync(0xffffffffu, is && before.w == t)};
+      const HintSet r = hint_step<J>(m, v, o, t);
       if (r.any()) {
-        const int lane = threadIdx.x & 31;
-        uint32_t o[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          o[k] = __ballot_sync(0xffffffffu, ahead && lane >= 30 && ahead[(lane - 30) * 4 + k] == suf[J]);
-        r = hint_step<J>(m, v, o, suf[J]);
-        if (r.any()) {
-          m = r;
-          return hint_longest<J + 1>(m, v, ahead, suf, nmax);
-        }
+        m = r;
+        return hint_longer<J + 1>(m, v, before, is, suf, nmax);
       }
     }
   }
   return J;
+}
+// From one token on; the tokens ahead of the chunk (`ahead`, nullptr where the bank
+// starts) are loaded only where two would match if they did.
+OOS_DEV int hint_longest(HintSet& m, const int4 (&v)[2], const int32_t* ahead, const int* suf, int nmax) {
+  if (nmax < 2) return 1;
+  const uint32_t all[4] = {~0u, ~0u, ~0u, ~0u};
+  if (!hint_step<1>(m, v, all, suf[1]).any()) return 1;
+  const int lane = threadIdx.x & 31;
+  const bool is = ahead && lane >= 30;
+  int4 before = make_int4(0, 0, 0, 0);
+  if (is) {
+    const int32_t* p = ahead + (lane - 30) * 4;
+    before = make_int4(p[0], p[1], p[2], p[3]);
+  }
+  return hint_longer<1>(m, v, before, is, suf, nmax);
 }
 
 // prefix_len_dev: the prefix length in device memory (the decode loop's
@@ -188,7 +196,7 @@ __global__ void __launch_bounds__(kHintThreads, 3) k_hint_match(const int32_t* _
             }
         }
         if (m.any()) {
-          lmax = hint_longest<1>(m, v[u], c > 0 ? bank + c * kHintThreads - 8 : nullptr, suf, nmax);
+          lmax = hint_longest(m, v[u], c > 0 ? bank + c * kHintThreads - 8 : nullptr, suf, nmax);
           uint32_t mine = m.w[0][0];
 #pragma unroll
           for (int i = 1; i < 8; ++i) mine = lane == i ? m.w[i >> 2][i & 3] : mine;
