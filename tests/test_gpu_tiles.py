@@ -144,3 +144,17 @@ def test_prefill_wide_tiles(hidden, inter, n):
     # the layer's own output is seen through the greedy token of the last position
     if r["top1"][-1] - r["top2"][-1] > 0.05:
         assert int(nxt.item()) == int(r["argmax"][-1])
+
+
+@pytest.mark.parametrize("hidden,inter,nq,nkv,d", [(512, 1536, 8, 4, 64), (514, 1538, 3, 1, 6)])
+def test_f32_trees_of_few_nodes(hidden, inter, nq, nkv, d):
+    """Every number of tokens that a warp takes at a time, full and in part."""
+    over = dict(hidden=hidden, intermediate=inter, n_q_heads=nq, n_kv_heads=nkv, head_dim=d, vocab=501)
+    for T in (1, 2, 3, 4, 5, 8, 9):
+        case = build_case("tiny", 9, T=T, plant=0, ctx_len=3, cfg_overrides=over, gain_std=0.1, prefill=False)
+        model, _ = gpu_model(case)
+        kv = gpu_cache(case, case.ctx_len + T)
+        g = run(model, kv, case.ctx_len, case.tokens, case.parent)
+        r = oracle.verify_tree(case.view, case.cache_k64, case.cache_v64, case.ctx_len, case.tokens, case.parent)
+        check_case(case, g, r)
+        check_compaction(model, kv, case.ctx_len, g)
