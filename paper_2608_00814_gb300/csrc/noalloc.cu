@@ -6,6 +6,7 @@
 // entry point needs no workspace: its per-block partial results live in a
 // fixed file-scope device array that every call shares.
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "internal.h"
@@ -89,7 +90,7 @@ __global__ void __launch_bounds__(kStaticThreads, static_blocks_per_sm(TT))
   for (int t = lane; t < T; t += 32) st[warp][t] = Top2{-INFINITY, 0x7fffffff, -INFINITY};
   __syncwarp();
   const int r_begin = blockIdx.x * rows_per_block;
-  const int r_end = min(V, r_begin + rows_per_block);
+  const int r_end = V - r_begin > rows_per_block ? r_begin + rows_per_block : V;
   const int groups = (T + TT - 1) / TT;
   const int tasks = r_begin < r_end ? (r_end - r_begin + R - 1) / R * groups : 0;
   const int chunks = H / VEC;
@@ -101,17 +102,18 @@ __global__ void __launch_bounds__(kStaticThreads, static_blocks_per_sm(TT))
     const E* w0 = W + (size_t)r0 * H;
     const float* h0 = hidden + (size_t)t0 * H;
     const int nr = min(R, r_end - r0), nt = min(TT, T - t0);   // rows past the end repeat the last one
-    // element offsets from the group's first rows: 32 bits, and kept as indexes,
-    // so that they do not take the registers of R + TT pointers
+    // element offsets from the group's first rows: 32 bits (launch_static), and kept as
+    // indexes, so that they do not take the registers of R + TT pointers
+    using Off = std::conditional_t<VEC == 1, size_t, uint32_t>;
 #pragma unroll 1
     for (int c = lane; c < chunks; c += 32) {
       StaticVec<E, VEC> w[R];
 #pragma unroll
-      for (int r = 0; r < R; ++r) w[r].load(w0 + ((uint32_t)min(r, nr - 1) * (uint32_t)H + (uint32_t)(c * VEC)));
+      for (int r = 0; r < R; ++r) w[r].load(w0 + ((Off)min(r, nr - 1) * (Off)H + (Off)(c * VEC)));
 #pragma unroll
       for (int t = 0; t < TT; ++t) {
         StaticVec<float, VEC> h;
-        h.load(h0 + ((uint32_t)min(t, nt - 1) * (uint32_t)H + (uint32_t)(c * VEC)));
+        h.load(h0 + ((Off)min(t, nt - 1) * (Off)H + (Off)(c * VEC)));
 #pragma unroll
         for (int r = 0; r < R; ++r)
 #pragma unroll
@@ -214,9 +216,9 @@ static bool launch_static_tt(const StaticCall& c) {
 template <typename E>
 static bool launch_static(const StaticCall& c) {
   // 16-byte loads where every row of both matrices starts on a 16-byte
-  // boundary; any other shape or address goes element by element.  (Offsets
-  // within a row group are 32-bit: 8 rows of up to 2^29 elements.)
-  if (c.H % 8 == 0 && (((uintptr_t)c.w | (uintptr_t)c.hidden) & 15) == 0) {
+  // boundary and a row group's offsets fit 32 bits (8 rows of up to 2^29 elements);
+  // any other shape or address goes element by element, in 64 bits.
+  if (c.H % 8 == 0 && c.H <= 1 << 29 && (((uintptr_t)c.w | (uintptr_t)c.hidden) & 15) == 0) {
     const int groups = (c.T + 7) / 8, tt = (c.T + groups - 1) / groups;   // the fewest groups, evenly filled
     if (tt <= 1) return launch_static_tt<E, 1, 8>(c);
     if (tt <= 2) return launch_static_tt<E, 2, 8>(c);
