@@ -659,6 +659,19 @@ cudaError_t prefill_chunk(Model& m, const oos_kv_cache* kv, int ctx, const int32
   return e;
 }
 
+// pf_split of one GEMM of a chunk of T tokens: what the tests of the tiles ask, so that
+// they know which ones they reach
+static int pf_choice(const Model& m, int layer, int stage, int T) {
+  const auto& c = m.cfg;
+  switch (stage) {
+    case OOS_STAGE_QKV:
+      return pf_split(m, m.g_qkv[layer], (c.n_q_heads + 2 * c.n_kv_heads) * c.head_dim, T, PF_QKV);
+    case OOS_STAGE_O: return pf_split(m, m.g_o[layer], c.hidden, T, PF_RESID);
+    case OOS_STAGE_GATE_UP: return pf_split(m, m.g_gu[layer], 2 * c.intermediate, T, PF_SILU);
+    default: return pf_split(m, m.g_down[layer], c.hidden, T, PF_RESID);
+  }
+}
+
 // the chunk's last token into row 0 of the verify buffers the LM head reads
 cudaError_t prefill_last(Model& m, int T, cudaStream_t st) {
   const auto& c = m.cfg;
@@ -668,3 +681,12 @@ cudaError_t prefill_last(Model& m, int T, cudaStream_t st) {
 }
 
 }  // namespace oos
+
+// not part of the C ABI: 0 pairs' tiles, c >= 1 the verify GEMM's in clusters of c, -1
+// no chunk of T tokens or no such GEMM
+extern "C" int oos_prefill_tiles(const oos_model* m, int32_t layer, int32_t stage, int32_t T) {
+  if (!m || m->cfg.dtype != OOS_DTYPE_BF16 || layer < 0 || layer >= m->cfg.n_layers || T <= oos::kMaxT ||
+      T > oos::kPfTokens || stage < OOS_STAGE_QKV || stage > OOS_STAGE_DOWN)
+    return -1;
+  return oos::pf_choice(*m, layer, stage, T);
+}
