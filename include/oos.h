@@ -362,17 +362,18 @@ int oos_lm_head_argmax_static(int32_t dtype, int32_t vocab, int32_t hidden_dim, 
                               float* out_top2, void* stream);
 
 /* Limit, in nanoseconds, of every pipeline wait inside this handle's kernels
- * (a TMA or tensor-core stage, a split-K partner, an attention split): a wait
- * that runs out sets OOS_ETIMEOUT in the status word, the kernel drains its
- * own copies and MMAs, frees its tensor memory and returns, and the rest of
- * the step returns early.  0 or a value above the default restores the
- * default of 2 s.  Meant for tests and diagnostics of the failure path (the
- * paper has no counterpart).  Applies to work enqueued on `stream` after the
- * call; synchronises `stream`. */
+ * (a TMA or tensor-core stage, the other CTA of a pair): a wait that runs out
+ * sets OOS_ETIMEOUT in the status word, the kernel drains its own copies and
+ * MMAs, frees its tensor memory and returns, and the rest of the step returns
+ * early.  0 or a value above the default restores the default of 2 s.  Meant
+ * for tests and diagnostics of the failure path (the paper has no
+ * counterpart).  Applies to work enqueued on `stream` after the call;
+ * synchronises `stream`. */
 int oos_set_wait_limit(oos_model* m, uint64_t limit_ns, void* stream);
 
 /* Synchronise `stream` and return the device status of the last verify or
- * prefill (every token of its prompt) on this handle: OOS_OK, OOS_ETREE or OOS_ETIMEOUT (or OOS_ECUDA). */
+ * prefill (all of its prompt) on this handle: OOS_OK, OOS_ETREE or
+ * OOS_ETIMEOUT (or OOS_ECUDA). */
 int oos_last_status(oos_model* m, void* stream);
 
 /* Static description of a status code. */

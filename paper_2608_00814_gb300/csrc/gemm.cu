@@ -72,7 +72,7 @@ namespace oos {
 //     its shared memory there: per k-block its MMAs read 128 KB of operands and TMA
 //     writes 56 (96 rows), against ~128 bytes a clock; in pairs 64 and 40.  Gate/up of
 //     the 14336 x 4096 shape at T = 128: last accumulator 57 -> 50 us after the start.
-//     Up to 64 tokens HBM is the bound (5.9 TB/s at 12288 x 4096, T = 64) and a pair's
+//     Up to 64 tokens HBM is the bound (5.2 TB/s at 12288 x 4096, T = 64) and a pair's
 //     setup costs more than it gives (8B step 4026 -> 4053 us, 0.6B 1277 -> 1304).
 //     A narrow model's gate/up goes in tiles of 64 tokens instead (launch_gemm_gu).
 enum { EPI_QKV = 0, EPI_RESID = 1, EPI_SILU = 2, EPI_ARGMAX = 3 };

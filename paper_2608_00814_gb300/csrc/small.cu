@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(1024) k_argmax_accept(const float* __restrict_
   // One SM's loads bound this kernel, so a warp reads 32 neighbouring nodes of a CTA's
   // states at a time, its share of the CTAs; then a warp per node merges the shares.
   // A lane per CTA instead fetched 32 bytes for every 4 it used: the Llama step at T =
-  // 128 took 17 us more (5064 against 5046), the 0.6B one at T = 32 1 us.
+  // 128 took 18 us more (5064 against 5046), the 0.6B one at T = 32 1 us.
   const int groups = (T + 31) / 32, shares = nw / groups;
   const int share = warp / groups, node = warp % groups * 32 + lane;
   if (share < shares && node < T) {

@@ -82,7 +82,7 @@ def test_f32_rows_not_in_fours(hidden, inter, nq, nkv, d):
     (256, 512, 4, 2, "", 0, 129),          # the smallest chunk, one token into the second tile
     (256, 512, 4, 2, "", 131, 2049),       # a whole chunk, then one token through the verify kernels
     (256, 512, 4, 2, "f16", 0, 2048 + 130),   # two chunks
-    (384, 640, 3, 1, "", 5, 256),          # an odd number of heads; columns past the matrices
+    (384, 640, 3, 1, "", 5, 256),          # an odd number of heads
     (640, 1152, 5, 1, "", 0, 385),         # 25 tokens per attention block
 ])
 def test_prefill_chunk_edges(hidden, inter, nq, nkv, kv, ctx, n):
@@ -121,13 +121,14 @@ def test_prefill_reports_a_bad_token_of_any_chunk():
 
 
 @pytest.mark.parametrize("hidden,inter,n", [
-    (1280, 3072, 2048),   # QKV and gate/up: 256 x 256 tiles, more than one a pair
-    (2432, 1024, 300),    # every GEMM in 128 x 128 tiles; ragged last token tile
-    (2432, 1152, 2048),   # O and down: two 128 x 128 tiles a block
-    (2432, 4096, 1700),   # down: 256 x 256 tiles, the last cut by the matrix and the prompt
+    (1280, 3072, 2048),   # narrow: few k-blocks a segment
+    (2432, 1024, 300),    # a ragged last token tile of every kind
+    (2432, 1152, 2048),
+    (2432, 4096, 1700),   # many gate/up tiles a pair, the last cut by the prompt
 ])
 def test_prefill_wide_tiles(hidden, inter, n):
-    """Sizes on both sides of the choice of tiles, one layer."""
+    """One layer, seen through q/k/v and the last token; test_gpu_prefill_tiles.py has
+    two, and says which tiles it reaches."""
     over = dict(hidden=hidden, intermediate=inter, n_q_heads=16, n_kv_heads=8, n_layers=1, vocab=700,
                 init_std=1.0 / hidden ** 0.5)
     case = build_case("mini-bf16", 6, T=4, plant=0, ctx_len=0, cfg_overrides=over, gain_std=0.1, prefill=False)
