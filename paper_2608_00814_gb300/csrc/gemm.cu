@@ -1328,13 +1328,13 @@ cudaError_t launch_gemm_gu(Model& m, int layer, int T, cudaStream_t st) {
   GemmArgs a = base_args(m, m.g_gu[layer], T, layer * 4 + 2);
   a.ss_chunks = m.g_o[layer].plan.n_work;
   a.act_out = (__nv_bfloat16*)m.ws.act;
-  // Above 64 tokens, where tiles of 64 tokens x 128 rows fit the SMs at once: chains of
+  // Above 64 tokens, where tiles of 64 tokens x 128 rows leave SMs free: chains of
   // k_chain, where a pair's single accumulator collects all of K (an MLP's error, its
-  // attention off: 2048 x 6144 6.3e-6, of which 5.6e-6 so; trees of 64 5.7e-6), and
-  // twice the CTAs (a layer at T = 65 / 128: 9728 rows 92.0 -> 90.1 / 107.2 -> 101.4 us,
-  // 6144 69.3 -> 67.2 / 82.4 -> 79.9, 3072 52.7 -> 54.3 / 64.1 -> 64.4).
+  // attention off: 2048 x 6144 6.3e-6 in pairs, 5.6e-6 so, 5.7e-6 in trees of 64; from 76
+  // tiles on the pairs' is no larger than the even deal's would be).  A layer at T = 65 / 128:
+  // 6144 rows 69.3 -> 67.2 / 82.4 -> 79.9 us, 3072 52.7 -> 54.3 / 64.1 -> 64.4.
   const int tiles = a.N / kTile;
-  if (T > 64 && 2 * tiles <= m.num_sms) {
+  if (T > 64 && 2 * tiles < m.num_sms) {
     a.rows = kTile;
     a.n_work = tiles;
     a.ldr = kMaxT;
