@@ -54,7 +54,7 @@ OOS_DEV void f32_dots_of(const float* const (&w)[R], const float* x, const float
   float acc[kDots<R, NORM, TOK>];
 #pragma unroll
   for (int i = 0; i < kDots<R, NORM, TOK>; ++i) acc[i] = 0.f;
-#pragma unroll(TOK <= 2 ? 16 / (TOK * V) : 2)
+#pragma unroll(TOK <= 2 ? 16 / V : 2)
   for (int k = lane * V; k < K; k += 32 * V) {
     F32Vec<V> wv[R], g;
 #pragma unroll
